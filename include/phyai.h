@@ -229,6 +229,10 @@ phyai_status_t phyai_poll_status(phyai_expert_t *h);
  * epilogue under the next tile's main loop); 0 keeps them on the one-tile-per-CTA kernel.
  * key "use_attn_splits": 1 (default) lets calls of few requests (at most a quarter of the SMs' worth of head-pair
  * CTAs) split every request's key tiles over up to 8 CTAs of the tcgen05 attention kernel, merged by a second launch.
+ * key "use_pair_gemm": 1 (default) runs the projections of calls with more than 64 suffix tokens on the CTA-pair GEMM
+ * with the norms folded in (together with use_cluster_gemm and the two use_persistent options); 0 keeps the general kernels.
+ * key "use_pair_attention": 1 (default) lets those calls of few requests use the CTA-pair attention kernel (caches of at
+ * least 256 tokens); key "pair_attn_ranges": key ranges per request (1..4, 0 = choose) of that kernel.
  * key "trace": see phyai_read_trace.
  * key "wait_limit": iteration bound of the device-side waits on other agents' progress (testing).
  * Unknown key -> INVALID_ARG. */

@@ -153,9 +153,11 @@ size_t attention_scratch_floats(const Dims& d, int batch, int splits) {
 
 cudaError_t launch_attention_mma(const Request* rq, int* status, const float* qkv, const float2* rope, int layer,
                                  __nv_bfloat16* out_tiled, int rows_pad, int num_splits, float* scratch, const Dims& d,
-                                 int batch, unsigned wait_limit, cudaStream_t st) {
+                                 int batch, unsigned wait_limit, cudaStream_t st, const __nv_bfloat16* qr,
+                                 const __nv_bfloat16* kr, const __nv_bfloat16* vr) {
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qkv = qkv, a.rope = rope, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
+  a.qr = qr, a.kr = kr, a.vr = vr;   // when set: rotated bf16 operands instead of the fp32 QKV output
   a.num_splits = num_splits, a.d = d, a.wait_limit = wait_limit;
   a.part_o = scratch;
   a.part_ml = scratch ? scratch + (size_t)batch * d.Hq * num_splits * QROWS * d.dh : nullptr;

@@ -114,7 +114,8 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
 
   // (the request block is written before the captured loop starts: safe to read ahead of the dependency wait)
   const Request r = *a.rq;
-  const int p0 = r.cu_lens[b], P = r.cu_lens[b + 1] - p0;
+  // (a call whose lengths are invalid stores nothing; the clamps keep its loads inside the cache)
+  const int p0 = min(max(r.cu_lens[b], 0), (int)r.kv_tokens), P = min(max(r.cu_lens[b + 1] - p0, 0), (int)r.kv_tokens - p0);
   // Keys of this CTA: an eighth of the prefix keys followed by an eighth of the request's own (suffix) keys -- the
   // suffix rows only exist after the dependency wait, so every CTA fetches its share of them then, not one CTA all.
   const int pre_lo = (int)(((long long)P * rank) / 8), n_pre = (int)(((long long)P * (rank + 1)) / 8) - pre_lo;

@@ -1,0 +1,616 @@
+// Suffix -> (prefix U suffix) attention on CTA pairs (tcgen05 cta_group::2), for calls of several requests.
+//
+// A pair of SMs takes four query heads of one request that share a kv head (each CTA two of them: 2 x 64 padded rows = its
+// 128 rows of the 256-row MMAs).  What bounds the one-CTA form of this kernel (attention_tc.cu) is the key / value stream
+// -- every CTA reads all of K and V of its request -- and the tensor pipe at N = 64, which runs at half rate.  In a pair
+// every CTA fetches half: of a 128-key tile its 64 keys of K and its DH / 2 channels of all 128 rows of V; the tensor cores
+// read the other half from the peer's shared memory, and both products run at N = 128 / DH.  64 KB per CTA and tile of
+// 2048 tensor clocks (head_dim 256): 32 bytes per clock, half of what an SM takes in.
+//   S = Q K^T   M = 256, N = 128 keys, K = head_dim; Q (the QKV projection wrote it as this kernel's operand tile) and K in
+//               shared memory; two S buffers in tensor memory, so that the logits of the next tile exist before the
+//               softmax of this one is done
+//   softmax     two threads per row (half of the columns each), straight from tensor memory; P (bf16) over the S buffer
+//   O += P V    M = 256, N = head_dim, K = 128 keys; P is the tensor-memory A operand, V an MN-major B operand; rescaled
+//               only when a row's maximum grows by more than 2^8
+// Small calls split the keys of a request over C = 2 to 4 pairs of one cluster (each range: its share of the prefix and of
+// the suffix keys); the partial results, rounded to bf16, are merged over distributed shared memory: row range p of every
+// head belongs to pair p, which adds the C partials in range order.  No partials in global memory, no merge launch.
+//
+// Warps of a CTA: 0-1 load K, 2-3 load V (full prefix tiles with tensor-map copies -- the map of the call's cache sits in
+// the request block --, the rest row by row with cp.async; prefix rows before the dependency wait), 4 issues the MMAs (leader CTA), 5-12 softmax, correction, output.  Every wait is bounded; after a
+// give-up the protocol runs to its end and only the global stores are skipped.
+#include "attention.cuh"
+#include "tc.cuh"
+#include "tmap.h"
+
+namespace phyai {
+namespace {
+
+constexpr int KB = 128;                       // keys per tile
+constexpr int AP_THREADS = 13 * 32;
+constexpr int BAR_ROWS = 1, BAR_K = 2, BAR_V = 3;
+constexpr float RESCALE_THRESHOLD = 8.0f;     // log2 units
+
+template <int DH, int C>
+struct ApLayout {
+  static constexpr int KBLOCK = 64 * 128;                    // one 64-channel block of this CTA's 64 keys
+  static constexpr int KTILE = (DH / 64) * KBLOCK;
+  static constexpr int PIECE = (DH / 128) * KBLOCK;          // one tensor-map copy: 64 keys x DH / 2 channels
+  static constexpr int VTILE = 2 * PIECE;                    // V: two halves of 64 keys, this CTA's DH / 2 channels
+  static constexpr int QTILE = 128 * DH * 2;
+  static constexpr int OWN = (64 + C - 1) / C;                         // rows per head a pair finishes
+  static constexpr int PITCH = DH * 2 + 16;                  // bf16 partial row, padded against bank conflicts
+  static constexpr int SLOT = 2 * OWN * (PITCH + 16);        // one owner's block: 2 heads x OWN rows, then (max, sum) entries
+  static constexpr int RECV = C > 1 ? C * SLOT : 0;          // [C sources] partials for my rows; first holds Q
+  static constexpr int KV = 2 * (KTILE + VTILE);             // two buffers each; later the outgoing partials [C owners][SLOT]
+  static constexpr size_t SMEM = 1024 + (size_t)KV + (QTILE > RECV ? QTILE : RECV);
+  static_assert(C == 1 || C * SLOT <= KV, "partials exceed the key / value buffers");
+};
+
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void remote_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void umma2_ss(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void umma2_ts(uint32_t d, uint32_t ta, uint64_t db, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d), "r"(ta), "l"(db), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// arrives on the barrier at this offset in the CTAs of `mask` once every MMA issued so far has completed
+__device__ __forceinline__ void umma2_commit(uint32_t bar, uint16_t mask) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(mask)
+               : "memory");
+}
+// the two warps that share the rows of a tensor-memory lane quarter
+__device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+template <int DH, int C>
+__global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
+  using L = ApLayout<DH, C>;
+  constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(KB >> 3) << 17) | ((256u >> 4) << 24);
+  constexpr uint32_t IDESC_PV = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(DH >> 3) << 17) | ((256u >> 4) << 24);
+
+  extern __shared__ uint8_t smem_raw[];
+  // leader: operands of a buffer complete in both CTAs; P of a buffer complete in both.  Each CTA: logits / P V complete.
+  __shared__ __align__(8) uint64_t k_full[2], v_full[2], p_full[2][2], s_full[2], pv_done[2], mrg_bar, q_bar, q_ready;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag, mrg_ok;
+  __shared__ float xch[2][2][128];       // the two half-row threads of a row exchange their maximum (by tile parity) and, at the end, sum
+  __shared__ float wtab[C > 1 ? 2 * L::OWN : 1][C]; // merge: weight of partial s for each of my rows
+
+  const Dims& d = a.d;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int crank = blockIdx.x, pr = crank >> 1, half = crank & 1;     // key range, CTA of the pair
+  const int b = a.order ? a.order[blockIdx.z] : (int)blockIdx.z;       // longest requests first
+  const int head0 = (int)blockIdx.y * 4 + half * 2;
+  const int hk = head0 / (d.Hq / d.Hkv);
+  const int S = d.S;
+  unsigned long long* const trc = a.trace ? a.trace + (size_t)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 16 : nullptr;
+  if (tid == 0) trace_stamp(trc, 0);
+  pdl_launch_dependents();
+
+  const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  const uint32_t Ks = base, Vs = base + 2 * L::KTILE, Qs = base + L::KV;
+  const uint32_t stg = base, recv = Qs;                                // merge: outgoing blocks by owner; [C sources] mine
+  const int own_lo = pr * L::OWN, n_me = max(0, min(L::OWN, S - own_lo));   // suffix rows (per head) this CTA finishes
+
+  if (tid == 0) {
+    abort_flag = 0;
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&k_full[i]), 2), mbar_init(smem_u32(&v_full[i]), 2), mbar_init(smem_u32(&p_full[i][0]), 8), mbar_init(smem_u32(&p_full[i][1]), 8);
+      mbar_init(smem_u32(&s_full[i]), 1), mbar_init(smem_u32(&pv_done[i]), 1);
+    }
+    mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 1), mbar_init(smem_u32(&q_ready), 2);
+    if (C > 1 && n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * (L::PITCH + 16)));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 4) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    tc_fence_before();
+  }
+  __syncthreads();
+  cluster_arrive();                                 // every CTA's barriers exist before a peer can signal them
+  cluster_wait();
+  tc_fence_after();
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(&tmem_slot), 0);
+  const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + 2 * KB;
+  const WaitCtx wc{a.status, &abort_flag, a.wait_limit, true};
+
+  // Keys of this range: a share of the prefix keys followed by a share of the request's own (suffix) keys.  (The request
+  // block is written before the captured loop starts: safe to read ahead of the dependency wait.  A call whose lengths are
+  // invalid stores nothing; the clamps keep its loads inside the cache.)
+  const Request r = *a.rq;
+  const int kvt = (int)r.kv_tokens;
+  const int p0 = min(max(r.cu_lens[b], 0), kvt), P = min(max(r.cu_lens[b + 1] - p0, 0), kvt - p0);
+  const int pre_lo = (int)(((long long)P * pr) / C), n_pre = (int)(((long long)P * (pr + 1)) / C) - pre_lo;
+  const int suf_lo = (S * pr) / C, n_suf = (S * (pr + 1)) / C - suf_lo;
+  // Tiles: first the mixed ones (the last n_pre % 128 prefix keys, then the suffix keys; at most two tiles, gathered row by
+  // row), then the full prefix tiles (tensor-map copies).  Softmax does not care about the order.
+  const int n_full = n_pre / KB, rem = n_pre - n_full * KB, n_mix = (rem + n_suf + KB - 1) / KB;
+  const int T = n_mix + n_full;
+  const int lead_rank = crank & ~1;
+  const uint16_t pair_mask = (uint16_t)(3u << lead_rank);
+
+  if (warp < 4) {
+    // =========================== loaders: warps 0-1 K, 2-3 V =======================================================
+    // Buffer t & 1 is free again once the logits of tile t (K), P V of tile t (V) exist: both commits reach both CTAs.
+    // (16-byte cp.async for every row, the first form of this loader, took 3 us to issue 64 KB: the requests of a tile did
+    // not fit the load / store unit's queue.)
+    const bool is_v = warp >= 2;
+    const int lt = tid & 63;
+    const uint32_t buf0 = is_v ? Vs : Ks, tile_bytes = is_v ? L::VTILE : L::KTILE;
+    const uint32_t full_own = smem_u32(is_v ? &v_full[0] : &k_full[0]);
+    const uint32_t full0 = map_rank(full_own, lead_rank);
+    // ---- full prefix tiles: two tensor-map copies per stream and CTA, counted on the leader's barrier
+    auto issue_full = [&](int t) {
+      const int row0 = p0 + pre_lo + (t - n_mix) * KB, plane = a.layer * 2 + (is_v ? 1 : 0);
+      const uint32_t bar = full_own + (uint32_t)(t & 1) * 8u, dst = buf0 + (uint32_t)(t & 1) * tile_bytes;
+      if (half == 0) mbar_expect_tx(bar, 4u * L::PIECE);
+      else remote_arrive(full0 + (uint32_t)(t & 1) * 8u);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        // K: my 64 keys, channel halves u; V: key halves u, my channel half
+        const int row = row0 + 64 * (is_v ? u : half), blk = hk * (DH / 64) + (is_v ? half : u) * (DH / 128);
+        asm volatile(
+            "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(
+                dst + (uint32_t)u * L::PIECE),
+            "l"(a.rq->kv_map), "r"(0), "r"(row), "r"(blk), "r"(plane), "r"(bar & 0xFEFFFFFFu)
+            : "memory");
+      }
+    };
+    if (lt == 0) {
+      // (the map was written into the request block by the kernel at the head of the call)
+      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(a.rq->kv_map) : "memory");
+      for (int t = n_mix; t < 2 && t < T; ++t) issue_full(t);        // constants of the call: ahead of the dependency wait
+    }
+    // ---- mixed tiles: row by row
+    const int chunks = is_v ? DH / 16 : DH / 8, rstep = 64 / chunks;     // 16-byte chunks per row of this stream
+    const int lc = lt % chunks, r0 = lt / chunks;
+    const int rows = is_v ? KB : 64, key0 = is_v ? 0 : half * 64;        // my rows are keys key0 .. key0 + rows - 1 of a tile
+    const uint32_t src_off = (uint32_t)(is_v ? half * DH : 0) + (uint32_t)lc * 16;
+    const size_t kv_stride = (size_t)d.Hkv * DH * 2;
+    const uint8_t* Gp = reinterpret_cast<const uint8_t*>(r.prefix_kv) +
+                        (((size_t)(a.layer * 2 + (is_v ? 1 : 0)) * r.kv_tokens + p0 + pre_lo + n_full * KB) * d.Hkv + hk) * (DH * 2) + src_off;
+    const uint8_t* Gs = reinterpret_cast<const uint8_t*>(is_v ? a.vr : a.kr) + ((size_t)(b * d.Hkv + hk) * S + suf_lo) * (DH * 2) + src_off;
+    auto dst_of = [&](int t, int row) {
+      return buf0 + (uint32_t)t * tile_bytes + (is_v ? (uint32_t)(row >> 6) * L::PIECE : 0u) + (uint32_t)(lc >> 3) * L::KBLOCK +
+             (uint32_t)(row & 63) * 128 + (uint32_t)(((lc & 7) ^ (row & 7)) << 4);
+    };
+    // the prefix rows of mixed tile t, or its suffix rows and, for V, zeros past the range (their probabilities are 0, but
+    // 0 x stale shared memory must stay 0; K rows past the range only give logits that the softmax masks)
+    auto gather = [&](int t, bool prefix) {
+      const int k0 = t * KB + key0;                                      // first key of my rows within the mixed keys
+      const int np = max(0, min(rows, rem - k0)), nv = max(0, min(rows, rem + n_suf - k0));
+      if (prefix) {
+        const uint8_t* src = Gp + (size_t)(k0 + r0) * kv_stride;
+#pragma unroll 4
+        for (int row = r0; row < np; row += rstep, src += (size_t)rstep * kv_stride) cp_async16(dst_of(t, row), src, 16u);
+      } else {
+        int row = r0 + (np > r0 ? (np - r0 + rstep - 1) / rstep * rstep : 0);      // my first row >= np
+        for (; row < nv; row += rstep) cp_async16(dst_of(t, row), Gs + (size_t)(k0 + row - rem) * (DH * 2), 16u);
+        if (is_v)
+          for (; row < rows; row += rstep) asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst_of(t, row)), "r"(0u) : "memory");
+      }
+    };
+    for (int t = 0; t < n_mix; ++t) gather(t, true);
+    pdl_wait();
+    if (T > 0) {
+      if (lane == 0) {
+        // Q (rotated, scaled) was written by the QKV projection as this CTA's operand tile: eight bulk copies
+        if (warp == 0) mbar_expect_tx(smem_u32(&q_bar), L::QTILE);
+        const uint8_t* qt = reinterpret_cast<const uint8_t*>(a.qr) + (size_t)(b * (d.Hq >> 1) + (head0 >> 1)) * L::QTILE;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          constexpr uint32_t QP = L::QTILE / 8;
+          bulk_g2s(Qs + (uint32_t)(2 * warp + u) * QP, qt + (size_t)(2 * warp + u) * QP, QP, smem_u32(&q_bar));
+        }
+      }
+      for (int t = 0; t < n_mix; ++t) gather(t, false);
+      if (n_mix > 0) {
+        cp_async_commit();
+        cp_async_wait<0>();
+        fence_async_smem();                    // generic-proxy writes, read next by the tensor cores
+        if (is_v) group_sync<BAR_V, 64>(); else group_sync<BAR_K, 64>();
+      }
+      if (lt == 0) {
+        for (int t = 0; t < n_mix; ++t) remote_arrive(full0 + (uint32_t)t * 8u);
+        if (!is_v) {
+          mbar_wait_drain(smem_u32(&q_bar), 0u, wc);
+          remote_arrive(map_rank(smem_u32(&q_ready), lead_rank));
+        }
+        for (int t = n_mix > 2 ? n_mix : 2; t < T; ++t) {
+          mbar_wait_drain(smem_u32(is_v ? &pv_done[t & 1] : &s_full[t & 1]), (uint32_t)((t - 2) >> 1) & 1u, wc);
+          issue_full(t);
+        }
+      }
+      __syncwarp();
+    }
+    if (C > 1) cluster_arrive();
+  } else if (warp == 4) {
+    // =========================== MMA issuer (leader CTA): S(0), S(1), then P(t) V(t), S(t + 2) ======================
+    pdl_wait();
+    if (lane == 0) {
+      trace_stamp(trc, 1), trace_stamp(trc, 2);
+      if (half == 1) trace_stamp(trc, 3), trace_stamp(trc, 4), trace_stamp(trc, 5);
+    }
+    if (half == 0) {
+      auto issue_s = [&](int t) {
+        mbar_wait_drain(smem_u32(&k_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        tc_fence_after();
+        const uint32_t kb = Ks + (uint32_t)(t & 1) * L::KTILE;
+#pragma unroll
+        for (int kk = 0; kk < DH / 16; ++kk) {
+          const uint64_t da = make_desc(Qs + (uint32_t)(kk >> 2) * (128 * 128) + (uint32_t)(kk & 3) * 32);
+          const uint64_t db = make_desc(kb + (uint32_t)(kk >> 2) * L::KBLOCK + (uint32_t)(kk & 3) * 32);
+          if (elect_one()) umma2_ss(tmem_s + (uint32_t)(t & 1) * KB, da, db, IDESC_S, kk > 0 ? 1u : 0u);
+        }
+        if (elect_one()) umma2_commit(smem_u32(&s_full[t & 1]), pair_mask);
+        __syncwarp();
+      };
+      if (T > 0) {
+        mbar_wait_drain(smem_u32(&q_ready), 0u, wc);      // both CTAs' Q tiles have landed
+        issue_s(0);
+      }
+      if (lane == 0) trace_stamp(trc, 3);
+      if (T > 1) issue_s(1);
+      for (int t = 0; t < T; ++t) {
+        mbar_wait_drain(smem_u32(&v_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        const uint32_t vb = Vs + (uint32_t)(t & 1) * L::VTILE;
+        // (the first 64 keys' probabilities are ready before the others': their half of the product hides under the rest of
+        // the softmax)
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh) {
+          mbar_wait_drain(smem_u32(&p_full[t & 1][kh]), (uint32_t)(t >> 1) & 1u, wc);
+          tc_fence_after();
+#pragma unroll
+          for (int kj = 0; kj < KB / 32; ++kj) {
+            // A = P of this tile: bf16 pairs in the first 64 columns of its S buffer
+            const uint64_t db = make_desc_mn(vb + (uint32_t)kh * L::PIECE + (uint32_t)kj * (16 * 128), L::KBLOCK, 1024);
+            if (elect_one())
+              umma2_ts(tmem_o, tmem_s + (uint32_t)(t & 1) * KB + (uint32_t)(kh * 4 + kj) * 8, db, IDESC_PV, (t > 0 || kh > 0 || kj > 0) ? 1u : 0u);
+          }
+        }
+        if (elect_one()) umma2_commit(smem_u32(&pv_done[t & 1]), pair_mask);
+        __syncwarp();
+        if (t + 2 < T) issue_s(t + 2);
+        if (t == 0 && lane == 0) trace_stamp(trc, 4);
+      }
+      if (lane == 0) trace_stamp(trc, 5);
+    }
+    __syncwarp();
+    if (C > 1) cluster_arrive();
+  } else {
+    // =========================== softmax / correction / output =====================================================
+    const int g = (warp - 5) >> 2;            // which half of a row's columns
+    const int q = warp & 3;
+    const int row = q * 32 + lane;            // accumulator row = tensor-memory lane
+    const int hl = row >> 6, i = row & 63;
+    const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+    const bool causal_row = d.block_causal && d.ns && i == 0;
+    const uint32_t pfull0 = map_rank(smem_u32(&p_full[0][g]), lead_rank);
+    float m = -INFINITY, l = 0.f;             // running maximum (log2 units) and sum
+    pdl_wait();
+    const bool skip = status_set(a.status);
+    for (int t = 0; t < T; ++t) {
+      const uint32_t sb = tmem_s + (uint32_t)(t & 1) * KB + lane_addr;
+      if (lane == 0) mbar_wait_drain(smem_u32(&s_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+      __syncwarp();
+      tc_fence_after();
+      if (C > 1 && t == T - 1) cluster_arrive();     // (the last logits exist: Q is dead, its area may receive partials)
+      // the visible keys of a row form a prefix of a mixed tile: the keys that exist, and for the state-token row under the
+      // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
+      int nvis = t < n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - t * KB) : KB;
+      nvis -= g * 64;
+      float s[64];
+      tmem_ld64(sb + (uint32_t)(g * 64), s);
+      if (nvis < 64) {
+#pragma unroll
+        for (int c = 0; c < 64; ++c) s[c] = c < nvis ? s[c] : -INFINITY;
+      }
+      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+      for (int c = 0; c < 64; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], s[c]);
+      xch[t & 1][g][row] = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      quarter_sync(q);                        // (also: both halves of these S rows have been read -> P may overwrite them)
+      const float mx = fmaxf(xch[t & 1][0][row], xch[t & 1][1][row]) * LOG2E;
+      // keep the old maximum unless the new one exceeds it by more than the threshold (exact algebra, no rescaling)
+      float m_new = m;
+      if (mx > m + RESCALE_THRESHOLD || m == -INFINITY) m_new = fmaxf(m, mx);
+      const bool rescale = m_new != m && m != -INFINITY;
+      const float corr = rescale ? exp2f(m - m_new) : 1.0f;
+      const float nsub = m_new == -INFINITY ? 0.f : -m_new;
+      float rs4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int c16 = 0; c16 < 2; ++c16) {
+        uint32_t w[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const int c = c16 * 32 + 2 * e;
+          const float e0 = ex2_fast(fmaf(s[c], LOG2E, nsub)), e1 = ex2_fast(fmaf(s[c + 1], LOG2E, nsub));
+          rs4[e & 3] += e0 + e1;
+          w[e] = pack_bf16(e0, e1);
+        }
+        tmem_st16u(sb + (uint32_t)(g * 32 + c16 * 16), w);
+      }
+      if (__any_sync(0xffffffffu, rescale)) {     // rare: rescale this warp's half rows of the accumulator
+        if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(t - 1) & 1]), (uint32_t)((t - 1) >> 1) & 1u, wc);   // every P V so far
+        __syncwarp();
+        tc_fence_after();
+#pragma unroll 1
+        for (int c = g * (DH / 2); c < (g + 1) * (DH / 2); c += 16) {
+          float o[16];
+          tmem_ld16(tmem_o + lane_addr + (uint32_t)c, o);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) o[e] *= corr;
+          tmem_st16(tmem_o + lane_addr + (uint32_t)c, o);
+        }
+      }
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) remote_arrive(pfull0 + (uint32_t)(t & 1) * 16u);
+      l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);      // (of this thread's half of the columns)
+      m = m_new;
+    }
+    if (C > 1 && T == 0) cluster_arrive();
+    xch[T & 1][g][row] = l;
+    quarter_sync(q);
+    l = xch[T & 1][0][row] + xch[T & 1][1][row];
+    if (T > 0 && warp == 5) mbar_wait_drain(smem_u32(&pv_done[(T - 1) & 1]), (uint32_t)((T - 1) >> 1) & 1u, wc);
+    group_sync<BAR_ROWS, 256>();
+    tc_fence_after();
+    if (warp == 5 && lane == 0) trace_stamp(trc, 6);
+    if constexpr (C == 1) {
+      // O / l -> bf16, the O projection's tiled operand: a thread's 128 bytes of a 64-channel chunk go to a staging block of
+      // the warp (the K / V buffers are dead) at the position they have in global memory, then out with coalesced stores
+      const bool okf = !skip && !*reinterpret_cast<volatile int*>(&abort_flag);
+      const float inv = 1.0f / l;
+      const int i0 = (q * 32) & 63, orow = b * S + i0 + lane;
+      const int nrow = okf ? max(0, min(32, S - i0)) : 0;
+      const uint32_t ostage = stg + (uint32_t)(warp - 5) * 4096u;
+#pragma unroll 1
+      for (int c = g * (DH / 2); c < (g + 1) * (DH / 2); c += 64) {
+        float o[64];
+        tmem_ld64(tmem_o + lane_addr + (uint32_t)c, o);
+#pragma unroll
+        for (int e = 0; e < 64; e += 8)
+          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ostage + (uint32_t)lane * 128u + (uint32_t)(((e >> 3) ^ (orow & 7)) << 4)),
+                       "r"(pack_bf16(o[e] * inv, o[e + 1] * inv)), "r"(pack_bf16(o[e + 2] * inv, o[e + 3] * inv)),
+                       "r"(pack_bf16(o[e + 4] * inv, o[e + 5] * inv)), "r"(pack_bf16(o[e + 6] * inv, o[e + 7] * inv))
+                       : "memory");
+        __syncwarp();
+        uint4* dst = reinterpret_cast<uint4*>(a.out + ((size_t)(((head0 + hl) * DH + c) >> 6) * a.rows_pad + (size_t)(b * S + i0)) * 64);
+        for (int idx = lane; idx < nrow * 8; idx += 32) {
+          uint4 v;
+          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(ostage + (uint32_t)idx * 16u) : "memory");
+          dst[idx] = v;
+        }
+        __syncwarp();
+      }
+    } else {
+      // ---- partial out: half an O row -> bf16 into the owner's block of the staging area; half 0 adds (max, sum) -------
+      const int c = i / L::OWN, il = i - c * L::OWN, n_c = max(0, min(L::OWN, S - c * L::OWN));
+      const bool wr = i < S;
+      const uint32_t blk = stg + (uint32_t)c * L::SLOT, rowp = blk + (uint32_t)(hl * n_c + il) * L::PITCH;
+#pragma unroll 1
+      for (int c0 = g * (DH / 2); c0 < (g + 1) * (DH / 2); c0 += 64) {
+        float o[64];
+        if (T > 0) {
+          tmem_ld64(tmem_o + lane_addr + (uint32_t)c0, o);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 64; ++e) o[e] = 0.f;
+        }
+        if (wr) {
+#pragma unroll
+          for (int e = 0; e < 64; e += 8)
+            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)(c0 + e) * 2), "r"(pack_bf16(o[e], o[e + 1])),
+                         "r"(pack_bf16(o[e + 2], o[e + 3])), "r"(pack_bf16(o[e + 4], o[e + 5])), "r"(pack_bf16(o[e + 6], o[e + 7]))
+                         : "memory");
+        }
+      }
+      if (wr && g == 0)
+        asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(blk + (uint32_t)(2 * n_c) * L::PITCH + (uint32_t)(hl * n_c + il) * 16), "f"(m), "f"(l)
+                     : "memory");
+      fence_async_smem();                      // generic writes -> visible to the bulk-copy engine
+      group_sync<BAR_ROWS, 256>();
+      cluster_wait();                          // every CTA's Q is dead
+      const int peer = warp - 5;               // (one copy per warp: the bulk copies of one warp complete one after the other)
+      if (lane == 0 && peer < C && peer != pr) {
+        const int n_p = max(0, min(L::OWN, S - peer * L::OWN));
+        if (n_p > 0)
+          asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                           map_rank(recv + (uint32_t)pr * L::SLOT, peer * 2 + half)),
+                       "r"(stg + (uint32_t)peer * L::SLOT), "r"((uint32_t)(2 * n_p * (L::PITCH + 16))),
+                       "r"(map_rank(smem_u32(&mrg_bar), peer * 2 + half))
+                       : "memory");
+      }
+      if (warp == 5) {
+        bool ok = true;
+        if (n_me > 0) ok = mbar_wait_drain(smem_u32(&mrg_bar), 0u, wc) > 0;
+        if (lane == 0) mrg_ok = ok && !skip ? 1 : 0;
+      }
+    }
+    tc_fence_before();
+  }
+  if (C > 1 && warp < 5) cluster_wait();
+  __syncthreads();
+  // From here on this CTA no longer needs its peers; it may leave once every peer says the same (the leader's MMAs have
+  // read both CTAs' shared memory, every partial copied out of its staging area has landed).
+  cluster_arrive();
+  if constexpr (C > 1) {
+    // ---- merge my rows: the C partials in range order, normalise, store as the output projection's operand ------------
+    const bool store = !*reinterpret_cast<volatile int*>(&abort_flag) && *reinterpret_cast<volatile int*>(&mrg_ok);
+    auto blk_of = [&](int s) { return s == pr ? stg + (uint32_t)pr * L::SLOT : recv + (uint32_t)s * L::SLOT; };
+    if (tid < 2 * n_me) {
+      float ms[C], ls[C], mm = -INFINITY, w[C], ll = 0.f;
+#pragma unroll
+      for (int s = 0; s < C; ++s) {
+        asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(ms[s]), "=f"(ls[s]) : "r"(blk_of(s) + (uint32_t)(2 * n_me) * L::PITCH + (uint32_t)tid * 16) : "memory");
+        mm = fmaxf(mm, ms[s]);
+      }
+#pragma unroll
+      for (int s = 0; s < C; ++s) {
+        w[s] = ms[s] == -INFINITY ? 0.f : exp2f(ms[s] - mm);
+        ll = fmaf(w[s], ls[s], ll);
+      }
+      const float inv = 1.0f / ll;
+#pragma unroll
+      for (int s = 0; s < C; ++s) wtab[tid][s] = w[s] * inv;
+    }
+    __syncthreads();
+    if (store) {
+      constexpr int CH = DH / 8;               // 16-byte chunks per row
+#pragma unroll 1
+      for (int idx = tid; idx < 2 * n_me * CH; idx += AP_THREADS) {
+        const int rr = idx / CH, ch = idx - rr * CH;       // rr = hl * n_me + il
+        const int hl = rr >= n_me ? 1 : 0, il = rr - hl * n_me;
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int s = 0; s < C; ++s) {
+          const float w = wtab[rr][s];
+          uint32_t uu[4];
+          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(uu[0]), "=r"(uu[1]), "=r"(uu[2]), "=r"(uu[3]) : "r"(blk_of(s) + (uint32_t)rr * L::PITCH + (uint32_t)ch * 16) : "memory");
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&uu[e]);
+            acc[2 * e] = fmaf(w, __low2float(p), acc[2 * e]);
+            acc[2 * e + 1] = fmaf(w, __high2float(p), acc[2 * e + 1]);
+          }
+        }
+        const int orow = b * S + own_lo + il, col = (head0 + hl) * DH + ch * 8;
+        *reinterpret_cast<uint4*>(a.out + tiled_index(orow, col, a.rows_pad)) =
+            make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+      }
+    }
+  }
+  cluster_wait();
+  if (warp == 4) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+    if (lane == 0 && trc) {
+      unsigned long long t;
+      unsigned sm;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)::"memory");
+      asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+      trc[8] = t, trc[7] = sm, trc[9] = (unsigned long long)T, trc[10] = 1;   // ([10]: marks an attention slot)
+    }
+  }
+}
+
+template <int DH, int C>
+cudaError_t setup_one() {
+  static PerDeviceOnce once;
+  if (!once.needed()) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k_attn_pair<DH, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ApLayout<DH, C>::SMEM);
+  if (e == cudaSuccess) once.done();
+  return e;
+}
+// clusters of this kernel that are resident at a time (0 on an error)
+template <int DH, int C>
+int max_clusters_one() {
+  if (setup_one<DH, C>() != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(2 * C, 1, 64), cfg.blockDim = dim3(AP_THREADS), cfg.dynamicSmemBytes = ApLayout<DH, C>::SMEM;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2 * C, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
+  cfg.attrs = at, cfg.numAttrs = 1;
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, k_attn_pair<DH, C>, &cfg) == cudaSuccess ? n : 0;
+}
+int max_clusters(int dh, int c) {
+  if (dh == 256) return c == 1 ? max_clusters_one<256, 1>() : c == 2 ? max_clusters_one<256, 2>() : c == 3 ? max_clusters_one<256, 3>() : max_clusters_one<256, 4>();
+  return c == 1 ? max_clusters_one<128, 1>() : c == 2 ? max_clusters_one<128, 2>() : c == 3 ? max_clusters_one<128, 3>() : max_clusters_one<128, 4>();
+}
+
+template <int DH, int C>
+cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st) {
+  cudaError_t e = setup_one<DH, C>();
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(2 * C, a.d.Hq / 4, batch), cfg.blockDim = dim3(AP_THREADS), cfg.dynamicSmemBytes = ApLayout<DH, C>::SMEM, cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2 * C, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at, cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_attn_pair<DH, C>, a);
+}
+
+}  // namespace
+
+// Tensor map over a prefix cache [planes][tokens][Hkv * dh / 64 blocks][64]: copies of 64 tokens x dh / 128 blocks (64-channel
+// blocks of 128-byte rows, 128-byte swizzle: the operand layout of the MMAs).
+bool prefix_kv_map(unsigned char* map, const void* kv, uint64_t kv_tokens, const Dims& d) {
+  const EncodeTiled enc = encode_tiled();
+  if (!enc) return false;
+  const cuuint64_t row = (cuuint64_t)d.Hkv * d.dh * 2;
+  const cuuint64_t dims[4] = {64, kv_tokens, (cuuint64_t)(d.Hkv * d.dh / 64), (cuuint64_t)(2 * d.L)}, strides[3] = {row, 128, kv_tokens * row};
+  const cuuint32_t box[4] = {64, 64, (cuuint32_t)(d.dh / 128), 1}, es[4] = {1, 1, 1, 1};
+  return enc(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(kv), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool attention_pair_supported(const Dims& d) {
+  return (d.dh == 256 || d.dh == 128) && d.S <= 64 && d.Hq % 4 == 0 && (d.Hq / d.Hkv) % 4 == 0;
+}
+
+// Key ranges per request: 1 to 4, the least of waves x (fixed cost + tiles of a range), in tiles of 128 keys.  How many
+// clusters of 2 C CTAs the device holds at a time decides the waves (a cluster of 8 needs 8 free SMs in one GPC: 15 on a
+// B200, not 18).
+int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
+  static std::atomic<int> cached[2][5];
+  const int dh = d.dh == 256 ? 1 : 0, items = batch * (d.Hq / 4);
+  int best_c = 1;
+  double best = 1e30;
+  for (int c = 1; c <= 4; ++c) {
+    int n = cached[dh][c].load();
+    if (n == 0) {
+      n = max_clusters(d.dh, c);
+      cached[dh][c].store(n > 0 ? n : -1);
+    }
+    if (n <= 0) continue;
+    const double cost = (double)((items + n - 1) / n) * ((c > 1 ? 5.5 : 4.0) + (max_prefix + d.S + c * KB - 1) / (c * KB));
+    if (cost < best) best = cost, best_c = c;
+  }
+  return best_c;
+}
+
+cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
+                                  const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
+                                  int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace) {
+  AttnArgs a{};
+  a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
+  a.num_splits = ranges, a.d = d, a.wait_limit = wait_limit, a.order = order, a.trace = trace;
+  switch (ranges + (d.dh == 256 ? 4 : 0)) {
+    case 1: return launch_one<128, 1>(a, batch, st);
+    case 2: return launch_one<128, 2>(a, batch, st);
+    case 3: return launch_one<128, 3>(a, batch, st);
+    case 4: return launch_one<128, 4>(a, batch, st);
+    case 5: return launch_one<256, 1>(a, batch, st);
+    case 6: return launch_one<256, 2>(a, batch, st);
+    case 7: return launch_one<256, 3>(a, batch, st);
+    default: return launch_one<256, 4>(a, batch, st);
+  }
+}
+
+}  // namespace phyai

@@ -50,7 +50,7 @@ __device__ __forceinline__ void trace_stamp(unsigned long long* slot, int i) {
 // of the loop.  Keeping the per-request pointers and lengths here (not in kernel arguments) lets
 // one captured CUDA graph serve every request of the same (batch, n_steps).
 // ---------------------------------------------------------------------------------------------
-struct Request {
+struct alignas(128) Request {
   const void* prefix_kv;   // [L][2][kv_tokens][Hkv][dh], fp32 or bf16
   uint64_t kv_tokens;      // token capacity of prefix_kv (stride between K and V planes)
   const int* cu_lens;      // device [batch+1]
@@ -59,6 +59,7 @@ struct Request {
   float* x;                // [batch][H][A]: the Euler state, = out_actions
   int batch;
   int single_len;          // prefix_len of the single-request entry point
+  alignas(128) unsigned char kv_map[128];   // CUtensorMap over prefix_kv for the pair attention kernel (see prefix_kv_map)
 };
 
 // ---------------------------------------------------------------------------------------------

@@ -77,6 +77,7 @@ struct phyai_expert {
   std::vector<uint8_t*> b_qkv, b_o, b_gu, b_d;                   // e4m3 byte blocks for the cluster GEMM (W8 experts)
 
   float2* rope = nullptr;
+  float2* rope_il = nullptr;   // the same with interleaved channels, for the pair GEMM's rotary epilogue
 
   // workspace
   float *h = nullptr, *qkv = nullptr, *state_tok = nullptr;
@@ -109,6 +110,12 @@ struct phyai_expert {
   __nv_bfloat16* p_gu16 = nullptr;          // gate/up interleaved in groups of 16 channels (persistent tile GEMM)
   __nv_bfloat16* p_qkv16 = nullptr;         // q|k|v with the rows of every tile interleaved in groups of 16 (the same kernel)
   int use_persistent_gu = 1, use_persistent_qkv = 1, use_attn_splits = 1;
+  bool pair_ok = false;        // the CTA-pair GEMMs (norms folded in) cover this expert's shapes
+  int use_pair_gemm = 1, use_pair_attention = 1;
+  int pair_ranges = 0;         // key ranges of the pair attention kernel (0 = choose)
+  __nv_bfloat16* q_tiles_pair = nullptr;   // q as operand tiles [max_batch][Hq / 2][128 rows][dh] for the pair / cluster attention
+  float *ss_ta = nullptr, *ss_tb = nullptr;   // their [D/128][Mpad] partial sums of squares of h (after O / after down)
+  __nv_bfloat16 *pq_all = nullptr, *po_all = nullptr, *pd_all = nullptr;   // bases of the packed images of all layers
   float *s_qkv_all = nullptr, *s_o_all = nullptr, *s_g_all = nullptr, *s_u_all = nullptr, *s_d_all = nullptr;
   __nv_bfloat16 *xn64 = nullptr, *attn64 = nullptr, *m64 = nullptr, *u64 = nullptr;
   __nv_bfloat16 *qr64 = nullptr, *kr64 = nullptr, *vr64 = nullptr;
@@ -220,7 +227,7 @@ phyai_status_t build_tables(phyai_expert* h, int n, cudaStream_t st, Tables** ou
       launch_rows_gemm(t.cvec, D, reinterpret_cast<const uint8_t*>(h->wmod) + s * wsite, h->wmod_kind, 0, 3 * D, D,
                        h->bmod + (size_t)s * 3 * D, nullptr, 0, t.mod + (size_t)s * 3 * D, h->sites * 3 * D, n, st);
     launch_mod_finish(t.mod, n * h->sites, D, st);
-    if (h->b1_ok) {
+    if (h->b1_ok || h->pair_ok) {
       // the shift of a folded norm enters the projection after it as a per-channel constant shift . W
       const int L = h->d.L, Nqkv = h->d.Nqkv, F2 = 2 * h->d.F;
       ST(h->alloc(&t.shw_qkv, (size_t)n * L * Nqkv));
@@ -460,6 +467,97 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     return PHYAI_OK;
   };
 
+  // More than one 64-token tile: every projection on the CTA-pair GEMM, the norms folded in as on the cluster path (QKV,
+  // attention, O, gate/up, down: five kernels per layer).
+  const bool pair = h->pair_ok && h->use_pair_gemm && h->use_cluster_gemm && h->use_persistent_gu && h->use_persistent_qkv && M > 64;
+  auto pair_gemm = [&](PairGemm g) -> phyai_status_t {
+    g.rows_pad = h->Mpad, g.M = M, g.ss_n = ss_n, g.inv_D = 1.0f / (float)D, g.eps = d.eps, g.gelu_exact = d.gelu_exact;
+    g.wait_limit = h->wait_limit;
+    g.trace = (h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from) ? h->trace : nullptr;
+    cudaError_t e = launch_pair_gemm(h->status, g, h->n_sm, st);
+    if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "pair GEMM launch failed: %s", cudaGetErrorString(e));
+    ++cnt;
+    return PHYAI_OK;
+  };
+  // Attention of the pair path.  Caches of fewer than 256 tokens keep the one-CTA kernel: with at most four 64-key tiles
+  // there is nothing to share or split.
+  const int pr_ranges = h->pair_ranges ? h->pair_ranges : (pair && h->q_tiles_pair ? attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len) : 1);
+  const bool attn_pair = pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair && h->cfg.max_prefix_len >= 256 && (pr_ranges > 1 || h->pair_ranges);
+  auto attention_rot = [&](int l) -> phyai_status_t {   // from rotated bf16 q / k / v to the output projection's operand
+    cudaError_t e;
+    const bool tr1 = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from;
+    if (attn_pair) {
+      e = launch_attention_pair(h->rq, h->status, h->q_tiles_pair, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch,
+                                pr_ranges, h->order, h->wait_limit, st,
+                                tr1 ? h->trace : nullptr);
+      ++cnt;
+    } else if (h->use_tc_attention && attention_tc_supported(d) && batch * (d.Hq / 2) >= ATTN_TC_MIN_CTAS) {
+      const int tsp = (h->use_attn_splits && h->attn_scratch) ? attention_tc_splits(d, batch, h->n_sm, (int)h->cfg.max_prefix_len) : 1;
+      const bool tr = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from && batch * (d.Hq / 2) * tsp <= TRACE_SLOTS;
+      e = launch_attention_tc(h->rq, h->status, h->qr_big, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch, h->order,
+                              h->wait_limit, st, tr ? h->trace : nullptr, tsp, h->attn_scratch);
+      cnt += tsp > 1 ? 2 : 1;
+    } else if (h->use_cluster_attention && batch * d.Hq * 8 <= 2 * h->n_sm) {
+      e = launch_attention_cluster(h->rq, h->status, nullptr, h->rope, h->qr_big, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch,
+                                   h->wait_limit, st);
+      ++cnt;
+    } else {
+      const int splits = attention_pick_splits(d, batch, (int)h->cfg.max_prefix_len);
+      e = launch_attention_mma(h->rq, h->status, nullptr, h->rope, l, h->attn_t, h->Mpad, splits, h->attn_scratch, d, batch, h->wait_limit,
+                               st, h->qr_big, h->kr_big, h->vr_big);
+      cnt += splits > 1 ? 2 : 1;
+    }
+    if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "attention launch failed: %s", cudaGetErrorString(e));
+    return PHYAI_OK;
+  };
+  auto pair_layer = [&](int k, int l) -> phyai_status_t {
+    const float *gain, *shift, *gate, *gain2, *shift2, *gate2;
+    site(k, 2 * l, &gain, &shift, &gate);
+    site(k, 2 * l + 1, &gain2, &shift2, &gate2);
+    PairGemm q{};
+    q.epi = PG_QKV, q.W = h->p_qkv16, q.w_rows = (uint64_t)d.L * d.Nqkv * (D / 64), q.w_row0 = l * d.Nqkv * (D / 64);
+    q.X = h->xn_t, q.N = d.Nqkv, q.K = D, q.scale = h->s_qkv[l], q.ss_in = h->ss_tb;
+    q.shift = h->ada ? t.shw_qkv + ((size_t)k * d.L + l) * d.Nqkv : nullptr;
+    q.rq = h->rq, q.rope = h->rope_il, q.q_tiles = attn_pair ? h->q_tiles_pair : nullptr, q.qr = h->qr_big, q.kr = h->kr_big, q.vr = h->vr_big;
+    q.S = d.S, q.Hq = d.Hq, q.Hkv = d.Hkv, q.dh = d.dh;
+    ST(pair_gemm(q));
+    ST(attention_rot(l));
+    PairGemm o{};
+    o.epi = PG_RESID, o.W = h->po_all, o.w_rows = (uint64_t)d.L * D * (d.Nq / 64), o.w_row0 = l * D * (d.Nq / 64);
+    o.X = h->attn_t, o.N = D, o.K = d.Nq, o.scale = h->s_o[l], o.gate = gate, o.h = h->h;
+    o.gain_next = gain2, o.out = h->xn_t, o.ss_out = h->ss_ta;
+    ST(pair_gemm(o));
+    PairGemm gu{};
+    gu.epi = PG_GEGLU, gu.W = h->p_gu16, gu.w_rows = (uint64_t)d.L * 2 * d.F * (D / 64), gu.w_row0 = l * 2 * d.F * (D / 64);
+    gu.X = h->xn_t, gu.N = 2 * d.F, gu.K = D, gu.scale = h->s_g[l], gu.scale2 = h->s_u[l], gu.ss_in = h->ss_ta, gu.out = h->m_t;
+    gu.shift = h->ada ? t.shw_gu + ((size_t)k * d.L + l) * 2 * d.F : nullptr;
+    ST(pair_gemm(gu));
+    PairGemm dn{};
+    dn.epi = PG_RESID, dn.W = h->pd_all, dn.w_rows = (uint64_t)d.L * D * (d.F / 64), dn.w_row0 = l * D * (d.F / 64);
+    dn.X = h->m_t, dn.N = D, dn.K = d.F, dn.scale = h->s_d[l], dn.gate = gate2, dn.h = h->h;
+    if (l + 1 < d.L) {
+      const float *shift3, *gate3;
+      site(k, 2 * l + 2, &dn.gain_next, &shift3, &gate3);
+      dn.out = h->xn_t, dn.ss_out = h->ss_tb;
+    }
+    return pair_gemm(dn);
+  };
+  auto pair_embed = [&](int k) -> phyai_status_t {
+    const float *gain0, *shift0, *gate0;
+    site(k, 0, &gain0, &shift0, &gate0);
+    if (h->ada) {
+      launch_embed_tokens(h->rq, h->status, h->Wc, h->bcfold, h->state_tok, gain0, h->h, h->xn_t, h->ss_tb, h->Mpad, d, batch, st);
+      ++cnt;
+      return PHYAI_OK;
+    }
+    launch_embed_tokens(h->rq, h->status, h->Wc, t.tb + (size_t)k * D, h->state_tok, nullptr, nullptr, h->u_t, nullptr, h->Mpad, d, batch, st);
+    ++cnt;
+    PairGemm e{};
+    e.epi = PG_RESID, e.W = h->W2p, e.w_rows = (uint64_t)D * (D / 64), e.X = h->u_t, e.N = D, e.K = D, e.h = h->h;
+    e.bias = h->b2, e.state_tok = h->state_tok, e.ns = d.ns, e.S = d.S, e.gain_next = gain0, e.out = h->xn_t, e.ss_out = h->ss_tb;
+    return pair_gemm(e);
+  };
+
   launch_begin(h->rq, h->status, h->state_w, h->state_b, h->state_tok, d0, batch, st);
   ++cnt;
   if (cache_state) {
@@ -499,7 +597,9 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   };
   for (int k = 0; k < n; ++k) {
     // ---- suffix embedding ----
-    if (b1_step) {
+    if (pair) {
+      ST(pair_embed(k));
+    } else if (b1_step) {
       ST(step_kernel(k, k == 0, false));
       if (!h->ada) {
         B1Gemm e{};
@@ -536,6 +636,10 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     }
     // ---- transformer layers ----
     for (int l = 0; l < d.L; ++l) {
+      if (pair) {
+        ST(pair_layer(k, l));
+        continue;
+      }
       const float *gain, *shift, *gate;
       site(k, 2 * l, &gain, &shift, &gate);
       if (b1) {
@@ -698,8 +802,10 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   return PHYAI_OK;
 }
 
-phyai_status_t run(phyai_expert* h, const Request& r, int n, cudaStream_t st) {
+phyai_status_t run(phyai_expert* h, Request& r, int n, cudaStream_t st) {
   Tables* t = nullptr;
+  if (h->q_tiles_pair && r.kv_tokens > 0 && !prefix_kv_map(r.kv_map, r.prefix_kv, r.kv_tokens, h->d))
+    return fail(PHYAI_ERR_CUDA, "tensor map of the prefix cache could not be encoded");
   ST(build_tables(h, n, st, &t));
   launch_set_request(h->rq, r, h->cu_internal, st, h->order);
   if (r.cu_lens != nullptr) launch_validate(h->rq, h->status, (int)h->cfg.max_prefix_len, h->order, st);
@@ -910,10 +1016,13 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
       ST(h->alloc(&pq_all, (size_t)L * D * Nqkv)); ST(h->alloc(&po_all, (size_t)L * Nq * D));
       ST(h->alloc(&pg_all, (size_t)L * D * F)); ST(h->alloc(&pu_all, (size_t)L * D * F));
       ST(h->alloc(&pd_all, (size_t)L * F * D));
+      h->pq_all = pq_all, h->po_all = po_all, h->pd_all = pd_all;
       h->il_ok = F % 64 == 0 && !a8;   // (W8A8 keeps to the general kernels: no interleaved image, no cluster path)
       if (h->il_ok) ST(h->alloc(&h->p_gu_all, (size_t)L * D * 2 * F));
-      // token counts that use 256-token tiles: the persistent gate / up kernel and its weight image
-      if (pick_nt((int)(cfg->max_batch * d.S)) == 256 && persist_gemm_supported((int)(cfg->max_batch * d.S), 2 * F, D, h->Mpad, a8)) {
+      h->pair_ok = h->il_ok && (d.dh == 128 || d.dh == 256) && d.S <= 64 && cfg->max_batch * d.S > 64 && attention_mma_supported(d) &&
+                   pair_gemm_supported(Nqkv, D) && pair_gemm_supported(D, Nq) && pair_gemm_supported(2 * F, D) && pair_gemm_supported(D, F);
+      // token counts that use 256-token tiles: the persistent gate / up kernel and its weight image (the pair GEMMs' too)
+      if (h->pair_ok || (pick_nt((int)(cfg->max_batch * d.S)) == 256 && persist_gemm_supported((int)(cfg->max_batch * d.S), 2 * F, D, h->Mpad, a8))) {
         ST(h->alloc(&h->p_gu16, (size_t)L * D * 2 * F / (a8 ? 2 : 1)));
         if ((d.dh == 128 || d.dh == 256) && d.S <= 64) ST(h->alloc(&h->p_qkv16, (size_t)L * D * Nqkv / (a8 ? 2 : 1)));
       }
@@ -1041,6 +1150,10 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
       const int npos = (int)cfg->max_prefix_len + d.S;
       ST(h->alloc(&h->rope, (size_t)npos * (d.dh / 2)));
       launch_rope_table(h->rope, npos, d.dh, (double)cfg->rope_theta, st);
+      if (h->pair_ok) {
+        ST(h->alloc(&h->rope_il, (size_t)npos * (d.dh / 2)));
+        launch_rope_table(h->rope_il, npos, d.dh, (double)cfg->rope_theta, st, 1);
+      }
     }
     // ---- workspace (zeroed: padding rows of the tiled buffers stay finite) ----
     ST(h->alloc(&h->h, Mp * D, true));
@@ -1085,6 +1198,11 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
           ST(h->alloc(&h->kr_st, (size_t)L * per_layer, true));
           ST(h->alloc(&h->vr_st, (size_t)L * per_layer, true));
         }
+      }
+      if (h->pair_ok) {
+        ST(h->alloc(&h->ss_ta, (size_t)(D / 128) * Mp, true));
+        ST(h->alloc(&h->ss_tb, (size_t)(D / 128) * Mp, true));
+        if (attention_pair_supported(d)) ST(h->alloc(&h->q_tiles_pair, (size_t)cfg->max_batch * (d.Hq / 2) * 128 * d.dh, true));
       }
       ST(h->alloc(&h->xn_t, Mp * D, true));
       ST(h->alloc(&h->attn_t, Mp * Nq, true));
@@ -1304,6 +1422,19 @@ phyai_status_t phyai_set_option(phyai_expert_t* h, const char* key, int64_t valu
     }
     if (!h->trace_buf) ST(h->alloc(&h->trace_buf, (size_t)TRACE_SLOTS * TRACE_STAMPS, true));
     h->trace = h->trace_buf;
+    return PHYAI_OK;
+  }
+  if (!strcmp(key, "pair_attn_ranges")) {
+    if (value < 0 || value > 4) return fail(PHYAI_ERR_INVALID_ARG, "pair_attn_ranges is 0 (choose) or 1..4");
+    h->pair_ranges = (int)value;
+    for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
+    h->graphs.clear();
+    return PHYAI_OK;
+  }
+  if (!strcmp(key, "use_pair_gemm") || !strcmp(key, "use_pair_attention")) {
+    (!strcmp(key, "use_pair_gemm") ? h->use_pair_gemm : h->use_pair_attention) = value != 0;
+    for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
+    h->graphs.clear();
     return PHYAI_OK;
   }
   if (!strcmp(key, "use_persistent_gu") || !strcmp(key, "use_persistent_qkv") || !strcmp(key, "use_attn_splits")) {

@@ -1,0 +1,562 @@
+// bf16 tile GEMM on CTA pairs (tcgen05 cta_group::2) for calls of more than 64 tokens: a pair of SMs works on one tile of
+// 256 output channels x NT tokens, a persistent grid of pairs walks all tiles, the epilogue of a tile runs under the
+// main loop of the next.
+//
+// What bounds it.  An SM takes in about 62 bytes per clock from the L2 while all SMs stream (measured), its tensor
+// core multiplies 128 x 256 x 16 in 128 clocks.  A 64-element k-chunk of a 128-row x 256-token tile is 48 KB for 512
+// clocks of tensor work: 96 bytes per clock, ingest bound.  A 256 x 256 tile per SM needs 64 bytes per clock, but its
+// accumulators fill the 512 tensor-memory columns, so that nothing overlaps its epilogue.  The pair has both: every SM
+// holds 128 of the 256 weight rows and half of the tokens (the tensor cores read the other half from the peer's
+// shared memory): 32 KB per k-chunk and SM at NT = 256, 64 bytes per clock, and 256 accumulator columns per tile, two
+// tiles in tensor memory.
+//
+// Operands: the packed 128 x 64 weight blocks and the tiled activations are contiguous runs of 128-byte rows in their
+// final (128-byte-swizzled) image, so two-dimensional tensor maps of 64-element rows fetch them; the copies of both
+// SMs signal the leader's barrier (.cta_group::2), which alone issues the MMAs.
+//
+// Norms are folded into the projections either side, as in gemm_b1.cu: X holds bf16(h * gain), the accumulator columns
+// are multiplied by rsqrt(mean h^2 + eps) of their token (from partial sums of squares), a shift enters as the
+// per-channel constant shift . W; the residual epilogue writes h, the next projection's operand and its partial sums of
+// squares (one per 128 channels and token).  No split-K and no atomics: a request gives the same bits every time.
+//
+// Roles: warps 0-3 issue the copies (k-step i by warp i % 4), warp 4 issues the MMAs (leader CTA), the 16 warps from 5
+// on are the epilogue (tensor-memory lane quarter = warp % 4).  Every wait is
+// bounded; after a give-up copies, MMAs, commits and barriers go on and only the stores are skipped.
+#include <algorithm>
+
+#include "kernels.h"
+#include "ptx.cuh"
+#include "tc.cuh"
+#include "tmap.h"
+
+namespace phyai {
+namespace {
+
+constexpr int PG_PROD = 4;
+constexpr int PG_EPI = 512, PG_THREADS = (PG_PROD + 1) * 32 + PG_EPI;
+// tokens an epilogue warp takes at a time: 16 for the rotary epilogue, which then has the registers to hold the (cos, sin)
+// of the next two blocks (one 32-token block ahead on 8 warps: 7 us per tile, bound by the table's latency), else 32
+template <int EPI> constexpr int PG_TB = EPI == PG_QKV ? 16 : 32;
+constexpr int PG_MAXST = 12;
+constexpr int PG_A_BYTES = 128 * 128;             // one CTA's weight block: 128 rows x 64 k
+constexpr int BAR_EPI = 1;
+constexpr int PG_PITCH = 36, PG_STG = 16 * PG_PITCH;      // staging block of an epilogue warp: [16 tokens][32 rows + 4] floats
+constexpr size_t PG_STG_BYTES = (size_t)16 * PG_STG * 4;
+constexpr size_t PG_SMEM_MAX = 227 * 1024 - 11 * 1024;   // dynamic shared memory (the static tables take the rest)
+constexpr uint32_t LEADER_MASK = 0xFEFFFFFFu;     // clears the CTA-rank bit of a shared::cluster address: the pair's even CTA
+
+__device__ __forceinline__ void tma2d(uint32_t dst, const CUtensorMap* map, int row, uint32_t bar_leader) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(bar_leader)
+      : "memory");
+}
+__device__ __forceinline__ void umma2_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "setp.ne.b32 p, %4, 0;\n"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// arrives on the barrier at this offset in both CTAs once every MMA issued so far has completed
+__device__ __forceinline__ void umma2_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+__device__ __forceinline__ void pair_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&v);
+}
+// 32 columns of 16 tensor-memory lanes in the fragment order of the matrix instructions: registers 4 k .. 4 k + 3 of lane T
+// hold (row T / 4, columns 8 k + 2 (T % 4), + 1) and the same columns of row T / 4 + 8
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, float* v) {    // 16 columns
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait16(float* a, float* b) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]), "+f"(b[0]), "+f"(b[1]),
+                 "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait32(float* a, float* b) {    // the registers pass through, so that no use moves up
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]), "+f"(a[8]), "+f"(a[9]),
+                 "+f"(a[10]), "+f"(a[11]), "+f"(a[12]), "+f"(a[13]), "+f"(a[14]), "+f"(a[15]), "+f"(b[0]), "+f"(b[1]), "+f"(b[2]),
+                 "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7]), "+f"(b[8]), "+f"(b[9]), "+f"(b[10]), "+f"(b[11]),
+                 "+f"(b[12]), "+f"(b[13]), "+f"(b[14]), "+f"(b[15])
+               :
+               : "memory");
+}
+// four 8 x 8 bf16 matrices in fragment order -> shared memory, transposed (a memory row = a fragment column)
+__device__ __forceinline__ void stmatrix4_t(uint32_t addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
+    k_gemm_pair(int* status, const PairGemm g, const __grid_constant__ CUtensorMap tmw, const __grid_constant__ CUtensorMap tmx) {
+  constexpr int EPIW = PG_EPI / 32, TB = PG_TB<EPI>, K8 = TB / 8;
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(8) uint64_t bar_full[PG_MAXST];    // leader: both CTAs' operands of a stage have landed
+  __shared__ __align__(8) uint64_t bar_empty[PG_MAXST];   // each CTA: the MMAs have read the stage
+  __shared__ __align__(8) uint64_t bar_tfull[2];          // each CTA: accumulator complete
+  __shared__ __align__(8) uint64_t bar_tempty[2];         // leader: accumulator read out by the epilogue warps of both
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag;
+  __shared__ __align__(16) float rs_tab[2][256];                        // per token: the folded norm's 1 / rms
+  // QKV: (position x dh / 2, element offset of the token's row in q without the head term, the same in k / v, suffix row)
+  __shared__ int4 tok_tab[EPI == PG_QKV ? 2 : 1][EPI == PG_QKV ? 256 : 1];
+  __shared__ float ss_tab[EPI == PG_RESID ? 4 : 1][EPI == PG_RESID ? 256 : 1];   // partial sums of squares per lane quarter
+
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
+  const int KC = g.K >> 6, NT = g.NT, ST = g.stages;
+  const int n_n = g.N >> 8;                               // tiles of 256 channels
+  const int n_tiles = n_n * ((g.M + NT - 1) / NT);
+  const int n_my = pair < n_tiles ? (n_tiles - pair + n_pairs - 1) / n_pairs : 0;
+  const int steps = n_my * KC;
+  const uint32_t stage_bytes = (uint32_t)(PG_A_BYTES + NT * 64);
+
+  pdl_launch_dependents();
+  unsigned long long* const trc = g.trace ? g.trace + (size_t)blockIdx.x * 16 : nullptr;
+  if (threadIdx.x == 0) trace_stamp(trc, 0);
+  const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < ST; ++s) {
+      mbar_init(smem_u32(&bar_full[s]), 1);
+      mbar_init(smem_u32(&bar_empty[s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&bar_tfull[b]), 1);
+      mbar_init(smem_u32(&bar_tempty[b]), 2 * EPIW);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == PG_PROD) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    tc_fence_before();
+  }
+  __syncthreads();
+  pair_sync();                                            // the peer's barriers exist before anything signals them
+  tc_fence_after();
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(&tmem_slot), 0);
+  const WaitCtx wc{status, &abort_flag, g.wait_limit, true};
+  if (threadIdx.x == 0) trace_stamp(trc, 1);
+
+  if (warp < PG_PROD) {
+    // ---------------- copy issuers -------------------------------------------------------------------------------
+    if (lane == 0) {
+      auto load_w = [&](int gi, int s) {
+        const int ct = ((pair + (gi / KC) * n_pairs) % n_n) * 2 + rank;      // this CTA's 128-row weight tile
+        const uint32_t full = smem_u32(&bar_full[s]);
+        if (rank == 0) mbar_expect_tx(full, 2 * stage_bytes);
+        tma2d(tiles + (uint32_t)s * stage_bytes, &tmw, g.w_row0 + (ct * KC + gi % KC) * 128, full & LEADER_MASK);
+      };
+      auto load_x = [&](int gi, int s) {
+        const int tt = (pair + (gi / KC) * n_pairs) / n_n;
+        tma2d(tiles + (uint32_t)s * stage_bytes + PG_A_BYTES, &tmx, (gi % KC) * g.rows_pad + tt * NT + rank * (NT >> 1),
+              smem_u32(&bar_full[s]) & LEADER_MASK);
+      };
+      // Programmatic dependent launch: the weight blocks of the first stages are on their way before the kernel that
+      // produces the activations has finished.
+      const int n_early = steps < ST ? steps : ST;
+      for (int gi = warp; gi < n_early; gi += PG_PROD) load_w(gi, gi);
+      pdl_wait();
+      if (warp == 0) {
+        trace_stamp(trc, 2);
+        if (rank == 1) trace_stamp(trc, 3), trace_stamp(trc, 4);             // (only the leader issues MMAs)
+      }
+      for (int gi = warp; gi < n_early; gi += PG_PROD) load_x(gi, gi);
+      for (int gi = warp; gi < steps; gi += PG_PROD) {
+        if (gi < n_early) continue;
+        const int s = gi % ST;
+        if (mbar_wait_drain(smem_u32(&bar_empty[s]), ((uint32_t)(gi / ST) & 1u) ^ 1u, wc) < 0) break;
+        load_w(gi, s);
+        load_x(gi, s);
+      }
+    }
+  } else if (warp == PG_PROD) {
+    // ---------------- MMA issuer (whole warp in the loop, one elected lane issues) --------------------------------
+    if (rank == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((256u >> 4) << 24);
+      int s = 0, gi = 0;
+      uint32_t ph = 0;
+      bool dead = false;
+      for (int i = 0; i < n_my && !dead; ++i) {
+        const int buf = i & 1;
+        // the epilogue warps of both CTAs have read the accumulator that this tile overwrites (two tiles ago)
+        if (mbar_wait_drain(smem_u32(&bar_tempty[buf]), (((uint32_t)i >> 1) & 1u) ^ 1u, wc) < 0) break;
+        tc_fence_after();
+        const uint32_t tacc = tmem_base + (uint32_t)buf * 256u;
+        for (int k = 0; k < KC; ++k, ++gi) {
+          if (mbar_wait_drain(smem_u32(&bar_full[s]), ph, wc) < 0) {
+            dead = true;   // (copies that never landed: nothing more can be done with this pipeline)
+            break;
+          }
+          if (gi == 0 && lane == 0) trace_stamp(trc, 3);
+          const uint32_t a0 = tiles + (uint32_t)s * stage_bytes;
+          const uint64_t da = make_desc(a0), db = make_desc(a0 + PG_A_BYTES);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            if (elect_one()) umma2_bf16(tacc, da + 2 * kk, db + 2 * kk, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+          if (elect_one()) umma2_commit(smem_u32(&bar_empty[s]));
+          __syncwarp();
+          if (++s == ST) s = 0, ph ^= 1u;
+        }
+        if (!dead && elect_one()) umma2_commit(smem_u32(&bar_tfull[buf]));
+        __syncwarp();
+      }
+      if (lane == 0) trace_stamp(trc, 4);
+    }
+  } else {
+    // ---------------- epilogue: tensor memory -> registers -> global ---------------------------------------------
+    // The code is kept short: in a captured loop a kernel's code has left the instruction caches by the next layer, and a
+    // first version, unrolled per element (one row per thread, 2- and 4-byte stores), spent 14 us on a residual tile.
+    // Shared memory is used sparingly: while the main loop runs, the tensor core's operand reads and the copies take most
+    // of its bandwidth.
+    const int ew = warp - (PG_PROD + 1);
+    const int q = warp & 3, cg = ew >> 2;    // tensor-memory lane quarter; column blocks cg, cg + 4, ...
+    const int et = ew * 32 + lane;
+    const uint32_t tl_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+    float* const stg = reinterpret_cast<float*>(smem_raw + (tiles - smem_u32(smem_raw)) + (size_t)ST * stage_bytes) + ew * PG_STG;
+    uint32_t tempty0;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(tempty0) : "r"(smem_u32(&bar_tempty[0])));
+    bool dead = false;
+    pdl_wait();
+    const bool skip = status_set(status);
+    for (int i = 0; i < n_my; ++i) {
+      const int buf = i & 1;
+      const int t = pair + i * n_pairs;
+      const int ct = (t % n_n) * 2 + rank, tok_base = (t / n_n) * NT;      // this CTA's 128 channels; first token
+      const int n_tok = min(NT, g.M - tok_base), n0 = ct * 128;
+      // ---- before the accumulator is complete: per-token and per-channel factors
+      if (EPI == PG_GEGLU || EPI == PG_QKV) {
+        if (et < NT) {      // (NT <= 256 <= threads of the epilogue)
+          float ss = 0.f;
+#pragma unroll 8
+          for (int j = 0; j < g.ss_n; ++j) ss += __ldg(g.ss_in + (size_t)j * g.rows_pad + min(tok_base + et, g.M - 1));
+          rs_tab[buf][et] = 1.0f / sqrtf(ss * g.inv_D + g.eps);
+        }
+      }
+      if constexpr (EPI == PG_QKV) {
+        if (et < n_tok) {
+          const int tok = tok_base + et, b = tok / g.S, ii = tok - b * g.S;
+          const int* cu = g.rq->cu_lens;
+          const int qo = g.q_tiles ? b * g.Hq * 64 * g.dh + ii * 64 : (b * g.Hq * g.S + ii) * g.dh;
+          tok_tab[buf][et] = make_int4((cu[b + 1] - cu[b] + ii) * (g.dh >> 1), qo, (b * g.Hkv * g.S + ii) * g.dh, ii);
+        }
+      }
+      // (a warp can be at most one tile ahead of the slowest: it passes this barrier only after every warp has left the
+      // tile before, so the tables of the tile before that are free to be overwritten)
+      asm volatile("bar.sync %0, %1;" ::"n"(BAR_EPI), "n"(PG_EPI) : "memory");
+      // GEGLU / QKV / PLANES: a warp's 32 rows are two groups of 16: gate (first-half, first) rows and the up (partner, next)
+      // rows; in fragment order a lane holds channels lane / 4 and + 8 of both groups, i.e. the pairs that are combined.
+      // Their weight scales and shifts: [group][channel lane / 4 or + 8]
+      float sc[2][2] = {{1.f, 1.f}, {1.f, 1.f}}, sh[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, scr = 1.0f;
+      if constexpr (EPI == PG_GEGLU || EPI == PG_QKV) {
+        const float osc = (EPI == PG_QKV && n0 < g.Hq * g.dh) ? rsqrtf((float)g.dh) : 1.0f;   // q leaves scaled by 1 / sqrt(dh)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int gr = e >> 1, cl = 16 * q + (lane >> 2) + 8 * (e & 1), row = n0 + 64 * gr + cl;
+          const float* sp = EPI == PG_QKV ? g.scale : (gr ? g.scale2 : g.scale);
+          if (sp) sc[gr][e & 1] = sp[EPI == PG_QKV ? row : ct * 64 + cl];
+          if (g.shift) sh[gr][e & 1] = g.shift[row] * osc;
+          sc[gr][e & 1] *= osc;
+        }
+      } else if constexpr (EPI == PG_RESID) {
+        if (g.scale) scr = g.scale[n0 + q * 32 + lane];
+        if (g.gate) scr *= g.gate[n0 + q * 32 + lane];
+      }
+      // where a lane's 16-byte pieces go: tokens lane / 2 and + 16 of a 32-token block, channels 8 (lane & 1) .. of a group
+      const int p8 = 16 * q + 8 * (lane & 1);
+      __nv_bfloat16* obase = nullptr;
+      int off2 = 0, rope_c = 0;
+      bool isq = false, rot = false, qt = false;
+      if constexpr (EPI == PG_GEGLU) {
+        obase = g.out + (size_t)ct * g.rows_pad * 64;
+      } else if constexpr (EPI == PG_QKV) {
+        const int Nq = g.Hq * g.dh, Nqk = Nq + g.Hkv * g.dh;
+        isq = n0 < Nq, rot = n0 < Nqk;
+        const int nn = isq ? n0 : (rot ? n0 - Nq : n0 - Nqk), head = nn / g.dh, coff = nn - head * g.dh;
+        // q / k: channels coff / 2 + .. and their partners dh / 2 further; v: coff + .. and + 64
+        rope_c = (coff >> 1) + 16 * q + 2 * (lane >> 2), off2 = rot ? g.dh >> 1 : 64;
+        obase = (isq ? g.qr : (rot ? g.kr : g.vr)) + (size_t)head * g.S * g.dh + (rot ? coff >> 1 : coff) + p8;
+        qt = isq && g.q_tiles;
+        if (qt) {     // operand tiles: (request, head pair) -> dh / 64 blocks of [64 (head & 1) + row][64 channels], swizzled
+          obase = g.q_tiles + (size_t)(head >> 1) * 128 * g.dh + (head & 1) * 4096 + (size_t)(coff >> 7) * 8192;
+          off2 = (g.dh >> 7) * 8192;
+        }
+      } else if constexpr (EPI == PG_PLANES) {
+        // K | V projections of all layers: row n of layer n / (2 nkv): nkv K channels, then nkv V channels
+        const int n = n0 + 32 * q, layer = n / (2 * g.nkv), c = n - layer * 2 * g.nkv, v = c >= g.nkv ? 1 : 0;
+        obase = g.out + (size_t)(layer * 2 + v) * g.plane_rows * g.nkv + (c - v * g.nkv) + 8 * (lane & 1), off2 = 16;
+      }
+      // RESID: in the transposed view a lane takes 4 channels of tokens lane / 8, + 4, + 8, + 12 of the chunk; what is added
+      // to (the residual stream, or the MLP's bias / the state token) is requested one chunk ahead
+      const int n4 = n0 + q * 32 + (lane & 7) * 4;
+      float4 old[2][4], gain4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      auto fetch_old = [&](int c0, float4* o) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int tok = min(tok_base + c0 + 4 * u + (lane >> 3), g.M - 1);
+          const float* src = g.h + (size_t)tok * g.N + n4;
+          if (g.bias) src = (tok % g.S) < g.ns ? g.state_tok + (size_t)(tok / g.S) * g.N + n4 : g.bias + n4;
+          o[u] = *reinterpret_cast<const float4*>(src);
+        }
+      };
+      if constexpr (EPI == PG_RESID) {
+        if (g.gain_next) gain4 = __ldg(reinterpret_cast<const float4*>(g.gain_next + n4));
+        if (cg * 16 < n_tok) fetch_old(cg * 16, old[0]);
+        if (cg * 16 + 64 < n_tok) fetch_old(cg * 16 + 64, old[1]);
+      }
+      // q / k: (cos, sin) of this lane's rotary pairs at its tokens, two 16-token blocks ahead
+      float2 cs[2][EPI == PG_QKV ? 8 : 1];
+      auto fetch_cs = [&](int c0, float2* o) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(g.rope + tok_tab[buf][min(c0 + 2 * (lane & 3) + 8 * k + e, n_tok - 1)].x + rope_c));
+            o[4 * k + e] = make_float2(x.x, x.y), o[4 * k + 2 + e] = make_float2(x.z, x.w);
+          }
+      };
+      const bool do_rot = EPI == PG_QKV && rot && g.rope && !skip;
+      if constexpr (EPI == PG_QKV) {
+        if (do_rot) fetch_cs(cg * 16, cs[0]), fetch_cs(cg * 16 + 64, cs[1]);
+      }
+      // ---- the accumulator
+      int r = 0;
+      if (!dead) {
+        if (lane == 0) r = mbar_wait_drain(smem_u32(&bar_tfull[buf]), ((uint32_t)i >> 1) & 1u, wc);
+        r = __shfl_sync(0xffffffffu, r, 0);
+        if (r < 0) dead = true;
+      }
+      const bool ok = !skip && !dead && r > 0 && !*reinterpret_cast<volatile int*>(&abort_flag);
+      tc_fence_after();
+      if (i == 0 && et == 0) trace_stamp(trc, 5);
+      if constexpr (EPI == PG_RESID) {
+        // 16 token columns at a time: the lane that holds a row scales it and puts it into the warp's staging block [16
+        // tokens][32 rows + 4]; then 8 lanes take the 32 channels (128 bytes of h) of one token
+#pragma unroll 1
+        for (int c0 = cg * 16; c0 < n_tok; c0 += 64) {
+          float v[16];
+          tmem_ld16(tl_addr + (uint32_t)(buf * 256 + c0), v);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) stg[j * PG_PITCH + lane] = v[j] * scr;
+          __syncwarp();
+          const float* sp = stg + (lane >> 3) * PG_PITCH + (lane & 7) * 4;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int tl = c0 + 4 * u + (lane >> 3), tok = tok_base + tl;
+            const float4 a = *reinterpret_cast<const float4*>(sp + 4 * u * PG_PITCH);
+            const bool live = !(g.bias && (tok % g.S) < g.ns);       // (state rows do not pass through the MLP)
+            float4 hv = old[0][u];
+            if (live) hv.x += a.x, hv.y += a.y, hv.z += a.z, hv.w += a.w;
+            if (ok && tl < n_tok) {
+              *reinterpret_cast<float4*>(g.h + (size_t)tok * g.N + n4) = hv;
+              if (g.gain_next)
+                *reinterpret_cast<uint2*>(g.out + tiled_index(tok, n4, g.rows_pad)) =
+                    make_uint2(pack_bf16x2(hv.x * gain4.x, hv.y * gain4.y), pack_bf16x2(hv.z * gain4.z, hv.w * gain4.w));
+            }
+            float s2 = hv.x * hv.x + hv.y * hv.y + hv.z * hv.z + hv.w * hv.w;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+            if ((lane & 7) == 0) ss_tab[q][tl] = s2;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) old[0][u] = old[1][u];
+          if (c0 + 128 < n_tok) fetch_old(c0 + 128, old[1]);
+          __syncwarp();
+        }
+      } else {
+        // TB token columns at a time, both row groups in fragment order; the bf16 results go through the warp's staging
+        // block [TB tokens][16 channels] (16-byte chunks swapped in every other group of four tokens against bank
+        // conflicts) by transposing matrix stores and leave as 16-byte pieces, two lanes to a 32-byte sector
+        const uint32_t st_s = smem_u32(stg);
+        const uint32_t st_w = st_s + (uint32_t)((8 * (lane >> 4) + (lane & 7)) * 32 + ((((lane >> 3) & 1) ^ ((lane >> 2) & 1)) << 4));
+        const uint32_t st_r = st_s + (uint32_t)((lane >> 1) * 32 + (((lane & 1) ^ ((lane >> 3) & 1)) << 4));
+#pragma unroll 1
+        for (int c0 = cg * TB; c0 < n_tok; c0 += 4 * TB) {
+          float a[4 * K8], b[4 * K8];
+          const uint32_t ta = tl_addr + (uint32_t)(buf * 256 + c0), tb = ta + (16u << 16);
+          if constexpr (TB == 32) {
+            tmem_ld_frag(ta, a), tmem_ld_frag(tb, b);
+            tmem_ld_wait32(a, b);
+          } else {
+            tmem_ld_frag16(ta, a), tmem_ld_frag16(tb, b);
+            tmem_ld_wait16(a, b);
+          }
+          const int t2 = c0 + 2 * (lane & 3);            // this lane's tokens: t2 + 8 k and + 1
+          if (EPI == PG_GEGLU || EPI == PG_QKV) {
+#pragma unroll
+            for (int k = 0; k < K8; ++k) {
+              const float2 rs = *reinterpret_cast<const float2*>(&rs_tab[buf][t2 + 8 * k]);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {              // e: channel e / 2, token e % 2
+                const float r1 = (e & 1) ? rs.y : rs.x;
+                a[4 * k + e] = fmaf(a[4 * k + e] * sc[0][e >> 1], r1, sh[0][e >> 1]);
+                b[4 * k + e] = fmaf(b[4 * k + e] * sc[1][e >> 1], r1, sh[1][e >> 1]);
+              }
+            }
+          }
+          if constexpr (EPI == PG_GEGLU) {
+#pragma unroll
+            for (int e = 0; e < 16; ++e) a[e] = gelu_fast(a[e], g.gelu_exact) * b[e];
+          } else if constexpr (EPI == PG_QKV) {
+            if (do_rot) {
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                const float l0 = a[e], u0 = b[e];
+                a[e] = l0 * cs[0][e].x - u0 * cs[0][e].y, b[e] = u0 * cs[0][e].x + l0 * cs[0][e].y;
+                cs[0][e] = cs[1][e];
+              }
+              if (c0 + 128 < n_tok) fetch_cs(c0 + 128, cs[1]);
+            }
+          }
+#pragma unroll
+          for (int m = 0; m < (EPI == PG_GEGLU ? 1 : 2); ++m) {      // the two row groups one after the other
+            const float* x = m ? b : a;
+#pragma unroll
+            for (int k = 0; k < K8; k += 2)
+              stmatrix4_t(st_w + (uint32_t)k * 256, pack_bf16x2(x[4 * k], x[4 * k + 1]), pack_bf16x2(x[4 * k + 2], x[4 * k + 3]),
+                          pack_bf16x2(x[4 * k + 4], x[4 * k + 5]), pack_bf16x2(x[4 * k + 6], x[4 * k + 7]));
+            __syncwarp();
+#pragma unroll
+            for (int it = 0; it < TB / 16; ++it) {
+              const int tl = c0 + (lane >> 1) + 16 * it, tok = tok_base + tl;
+              uint4 w;
+              asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(st_r + (uint32_t)it * 512) : "memory");
+              if (ok && tl < n_tok) {
+                __nv_bfloat16* dst = obase;
+                if constexpr (EPI == PG_GEGLU) dst += (size_t)tok * 64 + (((p8 >> 3) ^ (tok & 7)) << 3);
+                else if constexpr (EPI == PG_QKV) {
+                  const int4 e4 = tok_tab[buf][tl];
+                  dst += (isq ? e4.y : e4.z) + m * off2 + (qt ? ((p8 >> 3) ^ (e4.w & 7)) << 3 : 0);
+                }
+                else dst += (size_t)tok * g.nkv + m * off2;
+                *reinterpret_cast<uint4*>(dst) = w;
+              }
+            }
+            __syncwarp();
+          }
+        }
+      }
+      // this warp has read its part of the accumulator: the MMAs of the tile after next may overwrite it
+      tc_fence_before();
+      if (lane == 0)
+        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(tempty0 + (uint32_t)buf * 8u) : "memory");
+      if constexpr (EPI == PG_RESID) {
+        if (g.ss_out) {
+          asm volatile("bar.sync %0, %1;" ::"n"(BAR_EPI + 1), "n"(PG_EPI) : "memory");
+          if (ok && et < n_tok)
+            g.ss_out[(size_t)ct * g.rows_pad + tok_base + et] = (ss_tab[0][et] + ss_tab[1][et]) + (ss_tab[2][et] + ss_tab[3][et]);
+        }
+      }
+    }
+    if (et == 0 && trc) {
+      unsigned long long tt;
+      unsigned sm;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(tt)::"memory");
+      asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+      trc[6] = tt, trc[7] = sm, trc[9] = (unsigned long long)n_my;
+    }
+  }
+
+  __syncthreads();
+  // Neither CTA leaves (or gives its tensor memory back) while the other still works: the leader's MMAs read both CTAs'
+  // shared memory and write both tensor memories.
+  pair_sync();
+  if (warp == PG_PROD) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+    if (lane == 0 && trc) {
+      unsigned long long tt;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(tt)::"memory");
+      trc[8] = tt;
+    }
+  }
+}
+
+// `rows` rows of 64 bf16 (128 bytes), fetched `box` rows at a time
+bool row_map(CUtensorMap* m, const void* base, uint64_t rows, uint32_t box) {
+  const EncodeTiled enc = encode_tiled();
+  if (!enc) return false;
+  const cuuint64_t dims[2] = {64, rows}, strides[1] = {128};
+  const cuuint32_t bx[2] = {64, box}, es[2] = {1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int EPI>
+cudaError_t launch_one(int* status, const PairGemm& g, int grid, size_t smem, const CUtensorMap& tw, const CUtensorMap& tx, cudaStream_t st) {
+  static PerDeviceOnce once;
+  if (once.needed()) {
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    once.done();
+  }
+  return launch_pdl(k_gemm_pair<EPI>, dim3(grid), dim3(PG_THREADS), smem, st, status, g, tw, tx);
+}
+
+}  // namespace
+
+bool pair_gemm_supported(int N, int K) { return N % 256 == 0 && K % 64 == 0 && K > 0; }
+
+// Token-tile width: the one with the least work on the busiest pair.  A k-chunk of a tile costs the larger of the tensor
+// time (2 NT clocks: four MMAs of NT / 2) and the ingest of an SM (16 KB of weights + 64 NT bytes of activations at 62
+// bytes per clock); the last tile's epilogue is exposed (about 14 clocks per token column).
+int pair_gemm_pick_nt(int M, int N, int K, int n_sm) {
+  double best = 1e30;
+  int nt_best = 256;
+  for (int nt = 256; nt >= 32; nt -= 32) {
+    const int tiles = (N / 256) * ((M + nt - 1) / nt), pairs = n_sm / 2;
+    const double chunk = std::max(2.0 * nt, (PG_A_BYTES + 64.0 * nt) / 62.0);
+    const double cost = (double)((tiles + pairs - 1) / pairs) * (K / 64) * chunk + 14.0 * nt;
+    if (cost < best * 0.999) best = cost, nt_best = nt;
+  }
+  return nt_best;
+}
+
+cudaError_t launch_pair_gemm(int* status, const PairGemm& g_in, int n_sm, cudaStream_t st) {
+  PairGemm g = g_in;
+  if (!pair_gemm_supported(g.N, g.K) || g.M < 1) return cudaErrorInvalidValue;
+  if (g.NT <= 0) g.NT = pair_gemm_pick_nt(g.M, g.N, g.K, n_sm);
+  const size_t stage = (size_t)PG_A_BYTES + 64 * g.NT;
+  g.stages = (int)std::min<size_t>((PG_SMEM_MAX - 1024 - PG_STG_BYTES) / stage, PG_MAXST);
+  CUtensorMap tw, tx;
+  if (!row_map(&tw, g.W, g.w_rows, 128) || !row_map(&tx, g.X, (uint64_t)(g.K / 64) * g.rows_pad, (uint32_t)(g.NT / 2)))
+    return cudaErrorInvalidValue;
+  const int n_tiles = (g.N / 256) * ((g.M + g.NT - 1) / g.NT);
+  const int grid = 2 * std::min(n_tiles, n_sm / 2);
+  const size_t smem = (size_t)g.stages * stage + 1024 + PG_STG_BYTES;
+  switch (g.epi) {
+    case PG_QKV: return launch_one<PG_QKV>(status, g, grid, smem, tw, tx, st);
+    case PG_GEGLU: return launch_one<PG_GEGLU>(status, g, grid, smem, tw, tx, st);
+    case PG_RESID: return launch_one<PG_RESID>(status, g, grid, smem, tw, tx, st);
+    default: return launch_one<PG_PLANES>(status, g, grid, smem, tw, tx, st);
+  }
+}
+
+}  // namespace phyai

@@ -92,7 +92,8 @@ void launch_permute_scales(const float* src, float* dst, int N, int n_off, int p
 void launch_rows_gemm(const float* X, int ldx, const void* W, int w_kind, int w_row_off, int N, int K, const float* bias,
                       const float* add, int act_swish, float* Y, int ldy, int R, cudaStream_t st);
 void launch_sinusoid(float* tau, int n_steps, int D, double min_period, double max_period, cudaStream_t st);
-void launch_rope_table(float2* tab, int n_pos, int dh, double theta, cudaStream_t st);
+// (interleave8: the dh / 2 entries of a position in the order 0, 8, 1, 9, ..., 7, 15 of every 16)
+void launch_rope_table(float2* tab, int n_pos, int dh, double theta, cudaStream_t st, int interleave8 = 0);
 // gains[d] = 1 + gamma[d]
 void launch_one_plus(const float* gamma, float* out, int n, cudaStream_t st);
 // mod rows [R][3D] (scale|shift|gate) -> in place (1+scale|shift|gate)
@@ -108,6 +109,12 @@ void launch_embed_pi0(const Request* rq, const int* status, const float* Wc, con
 // pi0.5: h[b*S+ns+i][n] = x . Wa[:,n] + ba[n] (+ state rows)
 void launch_embed_pi05(const Request* rq, const int* status, const float* Wa, const float* ba, const float* state_tok,
                        float* h, const Dims& d, int batch, cudaStream_t st);
+// Embedding ahead of the pair GEMMs: gain null (pi0): u = swish(x Wc + bias) -> tiled bf16 `out` at token rows; gain set
+// (pi0.5): h = x Wc + bias (state rows: state_tok), out = bf16(h * gain), ss_out [D/128][rows_pad] partial sums of squares.
+// D a multiple of 128.
+void launch_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias, const float* state_tok,
+                         const float* gain, float* h, __nv_bfloat16* out, float* ss_out, int rows_pad, const Dims& d, int batch,
+                         cudaStream_t st);
 // n = h * rsqrt(mean h^2 + eps) * gain + shift  -> fp32 row-major or tiled bf16
 // Pending split-K partial sums of the residual stream: n slabs of [M][D] floats, `stride` floats apart.  The kernel
 // that reads h next adds them to each row in slab order (a fixed order: results are reproducible run to run) and,
@@ -155,7 +162,8 @@ int attention_pick_splits(const Dims& d, int batch, int max_prefix);
 size_t attention_scratch_floats(const Dims& d, int batch, int splits);  // split-KV partials (O, m, l)
 cudaError_t launch_attention_mma(const Request* rq, int* status, const float* qkv, const float2* rope, int layer,
                                  __nv_bfloat16* out_tiled, int rows_pad, int num_splits, float* scratch, const Dims& d,
-                                 int batch, unsigned wait_limit, cudaStream_t st);
+                                 int batch, unsigned wait_limit, cudaStream_t st, const __nv_bfloat16* qr = nullptr,
+                                 const __nv_bfloat16* kr = nullptr, const __nv_bfloat16* vr = nullptr);
 
 // ---- tcgen05 attention (large batches: two heads per CTA, whole key range, no split) ------------------
 bool attention_tc_supported(const Dims& d);
@@ -190,6 +198,15 @@ int attention_tc_splits(const Dims& d, int batch, int n_sm, int max_prefix);
 // combines split-KV partials ([b][head][split][64][dh] unnormalised rows, then [..][64][2] (max in log2 units, sum))
 cudaError_t launch_attention_merge(int* status, const float* part_o, const float* part_ml, __nv_bfloat16* out, int rows_pad,
                                    int num_splits, const Dims& d, int batch, cudaStream_t st);
+
+// ---- tcgen05 attention on CTA pairs (attention_pair.cu): several requests; q as operand tiles (see k_attn_b1), key ranges
+// of a request over up to 4 pairs of a cluster
+bool attention_pair_supported(const Dims& d);
+bool prefix_kv_map(unsigned char* map, const void* kv, uint64_t kv_tokens, const Dims& d);   // fills Request::kv_map
+int attention_pair_ranges(const Dims& d, int batch, int max_prefix);
+cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
+                                  const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
+                                  int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr);
 
 // ---- tcgen05 GEMM ------------------------------------------------------------------------------
 enum : int { TC_STORE = 0, TC_RESID = 1, TC_GEGLU = 2, TC_BIAS_ROWMAP = 3, TC_QKV_ROT = 4, TC_GEGLU_IL = 5 };
@@ -262,6 +279,53 @@ bool persist_gemm_supported(int M, int N, int K, int rows_pad, bool fp8);
 int persist_gemm_ctas(const PersistGemm& g, int n_sm);
 cudaError_t persist_gemm_setup();
 cudaError_t launch_persist_gemm(int* status, const PersistGemm& g, int n_sm, cudaStream_t st);
+// ---- tile GEMM on CTA pairs (gemm_pair.cu): calls of more than 64 tokens, norms folded in ------------------------
+enum : int { PG_QKV = 0, PG_GEGLU = 1, PG_RESID = 2, PG_PLANES = 3 };
+struct PairGemm {
+  const __nv_bfloat16* W;    // base of the packed weight image (blocks [N/128][K/64][128 x 64]), w_rows rows of 64 in total
+  uint64_t w_rows;
+  int w_row0;                // first row of this matrix in it
+  const __nv_bfloat16* X;    // tiled activations [K/64][rows_pad][64]
+  int rows_pad, M, N, K;
+  int NT;                    // token-tile width: a multiple of 32 up to 256, 0 = choose
+  int stages;                // (set by the launcher)
+  int epi;
+  const float* scale;        // per packed row weight scale or null (GEGLU: per gate channel; scale2: per up channel; QKV:
+  const float* scale2;       // un-interleaved packed order)
+  const float* shift;        // QKV / GEGLU: per packed row (un-interleaved; GEGLU: 64 gate rows, then 64 up rows) shift . W
+  // QKV / GEGLU: partial sums of squares of the tokens, [ss_n][rows_pad]: columns are multiplied by 1 / rms
+  const float* ss_in;
+  int ss_n;
+  float inv_D, eps;
+  int gelu_exact;
+  __nv_bfloat16* out;        // GEGLU: tiled [N/128][rows_pad][64] (W rows interleaved as for PersistGemm, gate / up);
+                             // RESID: tiled [N/64][rows_pad][64] bf16(h * gain_next), or unused; PLANES: [L][2][plane_rows][nkv]
+  // RESID: h[token][n] += gate[n] * scale[n] * acc (row stride N); with gain_next the operands of the norm that follows:
+  // `out` and ss_out[N/128][rows_pad].  With `bias` (second layer of the action MLP): h = bias + acc for action rows, the
+  // state token's embedding for the first ns of every request's S rows.
+  float* h;
+  const float* gate;
+  const float* gain_next;
+  float* ss_out;
+  const float* bias;
+  const float* state_tok;
+  int ns;
+  // QKV: see TcGemm (TC_QKV_ROT); W rows interleaved as for PersistGemm (qkv = 1)
+  const Request* rq;
+  const float2* rope;        // [pos][dh/2] with the channels of every 16 in the order 0, 8, 1, 9, ... (what a lane of the
+                             // fragment order combines is one 16-byte load), or null
+  __nv_bfloat16 *qr, *kr, *vr;
+  __nv_bfloat16* q_tiles;    // set: q goes out as the operand tiles of the pair / cluster attention kernels instead of rows
+  int S, Hq, Hkv, dh;
+  // PLANES: row n of layer n / (2 nkv): nkv K channels, nkv V channels
+  int nkv;
+  uint64_t plane_rows;
+  unsigned wait_limit;
+  unsigned long long* trace; // or null: CTA b stamps slot b (16 words)
+};
+bool pair_gemm_supported(int N, int K);
+int pair_gemm_pick_nt(int M, int N, int K, int n_sm);
+cudaError_t launch_pair_gemm(int* status, const PairGemm& g, int n_sm, cudaStream_t st);
 // ---- cluster split-K GEMM for a single 64-token tile (gemm_b1.cu) --------------------------------------------
 enum : int { B1_QKV = 0, B1_GEGLU = 1, B1_RESID = 2 };
 struct B1Gemm {

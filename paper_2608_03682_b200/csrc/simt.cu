@@ -10,6 +10,7 @@ namespace phyai {
 // =============================================================================================
 // request block
 // =============================================================================================
+static_assert(sizeof(Request) == 256, "the operator entry points reserve 256 bytes for the request block");
 __global__ void k_set_request(Request* dst, Request src, int* cu_internal, int* order) {
   if (threadIdx.x == 0) {
     if (src.cu_lens == nullptr) {  // single-request entry point: build cu = {0, prefix_len}
@@ -348,17 +349,18 @@ void launch_sinusoid(float* tau, int n_steps, int D, double pmin, double pmax, c
   k_sinusoid<<<(n + 127) / 128, 128, 0, st>>>(tau, n_steps, D, pmin, pmax);
 }
 
-__global__ void k_rope_table(float2* tab, int n_pos, int dh, double theta) {
+__global__ void k_rope_table(float2* tab, int n_pos, int dh, double theta, int interleave8) {
   const int half = dh / 2;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= n_pos * half) return;
   const int pos = idx / half, j = idx % half;
   const double phi = (double)pos * pow(theta, -2.0 * (double)j / (double)dh);
-  tab[idx] = make_float2((float)cos(phi), (float)sin(phi));
+  const int slot = interleave8 ? (j & ~15) + 2 * (j & 7) + ((j >> 3) & 1) : j;
+  tab[idx - j + slot] = make_float2((float)cos(phi), (float)sin(phi));
 }
-void launch_rope_table(float2* tab, int n_pos, int dh, double theta, cudaStream_t st) {
+void launch_rope_table(float2* tab, int n_pos, int dh, double theta, cudaStream_t st, int interleave8) {
   const int n = n_pos * (dh / 2);
-  k_rope_table<<<(n + 127) / 128, 128, 0, st>>>(tab, n_pos, dh, theta);
+  k_rope_table<<<(n + 127) / 128, 128, 0, st>>>(tab, n_pos, dh, theta, interleave8);
 }
 
 __global__ void k_one_plus(const float* g, float* out, int n) {
@@ -515,6 +517,81 @@ void launch_embed_pi05(const Request* rq, const int* status, const float* Wa, co
                        float* h, const Dims& d, int batch, cudaStream_t st) {
   k_embed_pi05<<<batch * d.H, 256, d.A * sizeof(float), st>>>(rq, status, Wa, ba, state_tok, h, d.A, d.H, d.D, d.S,
                                                               d.ns);
+}
+
+
+// Suffix embedding ahead of the pair GEMMs (norms folded in): one block takes ER action rows, a thread four consecutive
+// channels of all of them.  ADA = false (pi0): u = swish(x Wc + tb) -> bf16 operand of the MLP's second layer, at token
+// rows (the state rows' operand is never used).  ADA = true (pi0.5): h = x Wa + ba (state rows: the state token), the first
+// norm's operand bf16(h * gain) and, per 128 channels (one warp), the row's partial sum of squares.  ER = 4 keeps small
+// calls on many SMs, ER = 16 reads Wc once per 16 rows.
+template <int ER, bool ADA>
+__global__ void __launch_bounds__(256) k_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias,
+                                                      const float* state_tok, const float* gain, float* h, __nv_bfloat16* out,
+                                                      float* ss_out, int rows_pad, int A, int H, int D, int S, int ns, int rows_total) {
+  extern __shared__ float xs[];            // ER x A
+  pdl_enter();
+  if (status_set(status)) return;
+  const int r0 = blockIdx.x * ER, lane = threadIdx.x & 31;
+  for (int idx = threadIdx.x; idx < ER * A; idx += blockDim.x) {
+    const int r = r0 + idx / A;
+    xs[idx] = r < rows_total ? rq->x[(size_t)r * A + idx % A] : 0.f;
+  }
+  __syncthreads();
+  auto emit = [&](int row, int n, float4 v, float4 g4) {
+    *reinterpret_cast<float4*>(h + (size_t)row * D + n) = v;
+    __nv_bfloat162 lo = __floats2bfloat162_rn(v.x * g4.x, v.y * g4.y), hi = __floats2bfloat162_rn(v.z * g4.z, v.w * g4.w);
+    uint2 pk;
+    pk.x = *reinterpret_cast<uint32_t*>(&lo), pk.y = *reinterpret_cast<uint32_t*>(&hi);
+    *reinterpret_cast<uint2*>(out + tiled_index(row, n, rows_pad)) = pk;
+    const float ss = warp_sum(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
+    if (lane == 0) ss_out[(size_t)(n >> 7) * rows_pad + row] = ss;
+  };
+  for (int n = threadIdx.x * 4; n < D; n += blockDim.x * 4) {      // (D a multiple of 128: a warp is in or out as a whole)
+    float4 acc[ER];
+#pragma unroll
+    for (int e = 0; e < ER; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+    for (int a = 0; a < A; ++a) {
+      const float4 w = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)a * D + n));
+#pragma unroll
+      for (int e = 0; e < ER; ++e) {
+        const float x = xs[e * A + a];
+        acc[e].x = fmaf(x, w.x, acc[e].x), acc[e].y = fmaf(x, w.y, acc[e].y);
+        acc[e].z = fmaf(x, w.z, acc[e].z), acc[e].w = fmaf(x, w.w, acc[e].w);
+      }
+    }
+    const float4 t4 = __ldg(reinterpret_cast<const float4*>(bias + n));
+    float4 g4 = t4;
+    if constexpr (ADA) g4 = __ldg(reinterpret_cast<const float4*>(gain + n));
+#pragma unroll
+    for (int e = 0; e < ER; ++e) {
+      const int r = r0 + e;
+      if (r >= rows_total) break;
+      const int b = r / H, i = r - b * H, row = b * S + ns + i;
+      const float4 v = make_float4(acc[e].x + t4.x, acc[e].y + t4.y, acc[e].z + t4.z, acc[e].w + t4.w);
+      if constexpr (ADA) {
+        emit(row, n, v, g4);
+        if (ns && i == 0) emit(b * S, n, __ldg(reinterpret_cast<const float4*>(state_tok + (size_t)b * D + n)), g4);
+      } else {
+        __nv_bfloat162 lo = __floats2bfloat162_rn(swish_precise(v.x), swish_precise(v.y));
+        __nv_bfloat162 hi = __floats2bfloat162_rn(swish_precise(v.z), swish_precise(v.w));
+        uint2 pk;
+        pk.x = *reinterpret_cast<uint32_t*>(&lo), pk.y = *reinterpret_cast<uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(out + tiled_index(row, n, rows_pad)) = pk;
+      }
+    }
+  }
+}
+void launch_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias, const float* state_tok,
+                         const float* gain, float* h, __nv_bfloat16* out, float* ss_out, int rows_pad, const Dims& d, int batch,
+                         cudaStream_t st) {
+  const int rows = batch * d.H;
+  const bool wide = rows >= 2048, ada = gain != nullptr;
+  const int er = wide ? 16 : 4;
+  auto k = ada ? (wide ? k_embed_tokens<16, true> : k_embed_tokens<4, true>) : (wide ? k_embed_tokens<16, false> : k_embed_tokens<4, false>);
+  launch_pdl(k, dim3((rows + er - 1) / er), dim3(256), (size_t)er * d.A * sizeof(float), st, rq, status, Wc, bias, state_tok, gain, h, out,
+             ss_out, rows_pad, d.A, d.H, d.D, d.S, d.ns, rows);
 }
 
 // =============================================================================================

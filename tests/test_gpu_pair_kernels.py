@@ -1,0 +1,48 @@
+"""The kernels on CTA pairs (calls of more than 64 suffix tokens) against the oracle, at the edges of their tiles: token
+counts around the 32-token steps of the tile width, one and several tiles per pair, every key-range split of the attention
+kernel, prefixes with no full key tile, exactly one, and empty ranges; reproducible to the bit."""
+import pytest
+import torch
+
+from oracle import expert_oracle as O
+from paper_2608_03682_b200 import binding, synth
+from tests.helpers import BAR, rel_err, small_bf16_config
+
+pytestmark = pytest.mark.gpu
+
+
+def check(cfg, lens, n_steps, which, cfg_id=51, std=0.05, **options):
+    batch = len(lens)
+    W = synth.make_weights(cfg, cfg_id, std=std)
+    kvs = [synth.make_prefix_kv(cfg, cfg_id, p, b) for b, p in enumerate(lens)]
+    packed, cu = synth.pack_prefix_kv(kvs)
+    states = torch.stack([synth.make_state(cfg, cfg_id, b) for b in range(batch)]) if cfg.has_state_token else None
+    noise = torch.stack([synth.make_noise(cfg, cfg_id, b) for b in range(batch)])
+    args = (packed.cuda(), torch.from_numpy(cu).cuda(), None if states is None else states.cuda(), noise.cuda(), n_steps)
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        for k, v in options.items():
+            ex.set_option(k, v)
+        out = ex.denoise_batched(*args).clone()
+        again = ex.denoise_batched(*args)
+        torch.cuda.synchronize()
+        assert ex.poll_status() == 0 and torch.equal(out, again)
+    Wf = O.Weights(W)
+    for b in which:
+        ref = O.denoise(cfg, Wf, kvs[b], lens[b], None if states is None else states[b], noise[b], n_steps)
+        err = rel_err(out[b].double().cpu().numpy(), ref)
+        assert err <= BAR["bf16"], (b, lens[b], err)
+
+
+@pytest.mark.parametrize("cond,dtype,horizon,batch", [("pi0", "bf16", 12, 5), ("pi0", "bf16", 31, 3), ("pi05", "bf16", 33, 2),
+                                                       ("pi05", "w8e4m3", 43, 3), ("pi0", "w4a16", 50, 11), ("pi0", "bf16", 63, 33)])
+def test_pair_gemms_at_the_edges_of_their_token_tiles(cond, dtype, horizon, batch):
+    cfg = small_bf16_config(cond, dtype=dtype, horizon=horizon, max_batch=batch, max_prefix_len=120, n_q_heads=4, mlp_dim=1024)
+    check(cfg, [(37 * b) % 121 for b in range(batch)], 2, {0, batch // 2, batch - 1})
+
+
+@pytest.mark.parametrize("head_dim,n_q,n_kv", [(256, 4, 1), (128, 8, 2)])
+@pytest.mark.parametrize("ranges", [1, 2, 3, 4])
+def test_pair_attention_key_ranges(head_dim, n_q, n_kv, ranges):
+    cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=9, max_prefix_len=700, n_layers=2,
+                            suffix_block_causal=ranges % 2 == 0)
+    check(cfg, [700, 0, 1, 127, 128, 129, 512, 64, 386], 1, range(9), pair_attn_ranges=ranges)
