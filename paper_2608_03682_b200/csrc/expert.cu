@@ -354,10 +354,13 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   };
   auto simt_gemm = [&](SimtGemm g) {
     if (!g.rows_in) g.rows_in = g.rows_out = 1 << 30, g.row_off = 0;
-    g.gelu_exact = d.gelu_exact;
-    launch_simt_gemm(h->status, g, st);
+    g.gelu_exact = d.gelu_exact, g.eps = d.eps;
+    if (simt_rows_supported(g.M, g.K)) launch_simt_rows(h->status, g, st);
+    else launch_simt_gemm(h->status, g, st);
     ++cnt;
   };
+  // CUDA-core path with few rows: the projections normalise their input rows themselves
+  const bool simt_norm = !h->tc && simt_rows_supported(M, D);
 
   const int kcb = h->a8 ? 128 : 64;   // contraction elements per 128-byte operand row (k-chunk of the tile GEMM)
   const int ss_n = D / 128;
@@ -647,9 +650,11 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
                     cache_state ? h->vr_st + (size_t)l * kv_layer : h->vr_big, b1_step));
         continue;
       }
-      launch_rmsnorm(h->status, h->h, gain, shift, h->xn_f, h->xn_t, h->Mpad, M, D, d.eps, st, take_slabs(),
-                     norm_q8 ? h->xq : nullptr, norm_q8 ? h->xs : nullptr);
-      ++cnt;
+      if (!simt_norm) {
+        launch_rmsnorm(h->status, h->h, gain, shift, h->xn_f, h->xn_t, h->Mpad, M, D, d.eps, st, take_slabs(),
+                       norm_q8 ? h->xq : nullptr, norm_q8 ? h->xs : nullptr);
+        ++cnt;
+      }
       const bool attn_tc = h->attn_mma && h->use_tc_attention && h->qr_big && attention_tc_supported(d) &&
                            batch * (d.Hq / 2) >= ATTN_TC_MIN_CTAS;
       const bool attn_cluster = !attn_tc && h->attn_mma && h->use_cluster_attention && batch * d.Hq * 8 <= 2 * h->n_sm;
@@ -691,6 +696,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
       } else {
         SimtGemm g{};
         g.A = h->xn_f, g.lda = D, g.B = h->f_qkv[l], g.M = M, g.N = d.Nqkv, g.K = D, g.epi = EPI_STORE;
+        if (simt_norm) g.A = h->h, g.norm_gain = gain, g.norm_shift = shift;
         g.out = h->qkv, g.ldo = d.Nqkv;
         simt_gemm(g);
       }
@@ -718,8 +724,12 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
         if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "attention launch failed: %s", cudaGetErrorString(e));
         cnt += splits > 1 ? 2 : 1;
       } else {
-        launch_attention_simt(h->rq, h->status, h->qkv, h->rope, l, h->cfg.dtype != PHYAI_F32, h->attn_f, h->attn_t,
-                              h->Mpad, d, batch, st);
+        if (!h->tc && attention_row_supported(d, (int)h->cfg.max_prefix_len))
+          launch_attention_row(h->rq, h->status, h->qkv, h->rope, l, h->cfg.dtype != PHYAI_F32, h->attn_f, d, batch,
+                               (int)h->cfg.max_prefix_len, st);
+        else
+          launch_attention_simt(h->rq, h->status, h->qkv, h->rope, l, h->cfg.dtype != PHYAI_F32, h->attn_f, h->attn_t,
+                                h->Mpad, d, batch, st);
         ++cnt;
       }
       if (fuse_o) {
@@ -737,9 +747,11 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
         simt_gemm(g);
       }
       site(k, 2 * l + 1, &gain, &shift, &gate);
-      launch_rmsnorm(h->status, h->h, gain, shift, h->xn_f, h->xn_t, h->Mpad, M, D, d.eps, st, take_slabs(),
-                     norm_q8 ? h->xq : nullptr, norm_q8 ? h->xs : nullptr);
-      ++cnt;
+      if (!simt_norm) {
+        launch_rmsnorm(h->status, h->h, gain, shift, h->xn_f, h->xn_t, h->Mpad, M, D, d.eps, st, take_slabs(),
+                       norm_q8 ? h->xq : nullptr, norm_q8 ? h->xs : nullptr);
+        ++cnt;
+      }
       if (h->tc) {
         TcGemm g{};
         g.W = h->p_g[l], g.W2 = h->p_u[l], g.X = h->xn_t, g.N = d.F, g.K = D, g.epi = TC_GEGLU;
@@ -774,6 +786,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
       } else {
         SimtGemm g{};
         g.A = h->xn_f, g.lda = D, g.B = h->f_g[l], g.B2 = h->f_u[l], g.M = M, g.N = d.F, g.K = D, g.epi = EPI_GEGLU;
+        if (simt_norm) g.A = h->h, g.norm_gain = gain, g.norm_shift = shift;
         g.out = h->m_f, g.ldo = d.F;
         simt_gemm(g);
         SimtGemm g2{};

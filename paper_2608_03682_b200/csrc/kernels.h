@@ -148,7 +148,16 @@ struct SimtGemm {
   float* out; int ldo;
   int rows_in, rows_out, row_off; // output row = (m / rows_in) * rows_out + row_off + m % rows_in
   int gelu_exact;
+  const float* norm_gain;         // few-row kernel: RMSNorm of the A rows first (A rms(a)^-1 gain + shift), or null
+  const float* norm_shift;
+  float eps;
 };
+// few token rows (simt_rows.cu)
+bool simt_rows_supported(int M, int K);
+cudaError_t launch_simt_rows(const int* status, const SimtGemm& g, cudaStream_t st);
+bool attention_row_supported(const Dims& d, int max_prefix);
+cudaError_t launch_attention_row(const Request* rq, const int* status, const float* qkv, const float2* rope, int layer, int kv_is_bf16,
+                                 float* out, const Dims& d, int batch, int max_prefix, cudaStream_t st);
 void launch_simt_gemm(const int* status, const SimtGemm& g, cudaStream_t st);
 
 // ---- CUDA-core attention -----------------------------------------------------------------------

@@ -418,6 +418,7 @@ void launch_begin(const Request* rq, const int* status, const float* Ws, const f
 template <class Writer>
 __global__ void k_embed_pi0(const Request* rq, const int* status, const float* Wc, const float* tb,
                             const float* state_tok, float* h, Writer u, int A, int H, int D, int S, int ns) {
+  pdl_enter();
   if (status_set(status)) return;
   extern __shared__ float xs[];
   const int r = blockIdx.x;  // action row b*H + i
@@ -489,11 +490,11 @@ void launch_embed_pi0(const Request* rq, const int* status, const float* Wc, con
     return;
   }
   if (u_tiled)
-    k_embed_pi0<<<rows, 256, d.A * sizeof(float), st>>>(rq, status, Wc, tb, state_tok, h, TiledBf16{u_tiled, rows_pad},
-                                                        d.A, d.H, d.D, d.S, d.ns);
+    launch_pdl(k_embed_pi0<TiledBf16>, dim3(rows), dim3(256), d.A * sizeof(float), st, rq, status, Wc, tb, state_tok, h,
+               TiledBf16{u_tiled, rows_pad}, d.A, d.H, d.D, d.S, d.ns);
   else
-    k_embed_pi0<<<rows, 256, d.A * sizeof(float), st>>>(rq, status, Wc, tb, state_tok, h, RowMajorF32{u_f32, d.D}, d.A,
-                                                        d.H, d.D, d.S, d.ns);
+    launch_pdl(k_embed_pi0<RowMajorF32>, dim3(rows), dim3(256), d.A * sizeof(float), st, rq, status, Wc, tb, state_tok, h,
+               RowMajorF32{u_f32, d.D}, d.A, d.H, d.D, d.S, d.ns);
 }
 
 __global__ void k_embed_pi05(const Request* rq, const int* status, const float* Wa, const float* ba,
