@@ -286,8 +286,8 @@ uint64_t phyai_launches_per_call(phyai_expert_t *h, uint32_t batch, uint32_t n_s
  *   status_word     device int32, zeroed by the caller; stays 0 on success, becomes PHYAI_ERR_INVALID_ARG
  *                   (cu_prefix_lens) or PHYAI_ERR_TIMEOUT (a bounded wait inside the kernel expired)
  *
- * Split-KV partial results need scratch memory: this entry point takes it from the stream-ordered
- * allocator (cudaMallocAsync / cudaFreeAsync on `stream`).  Only enqueues work.  Errors: INVALID_ARG,
+ * bf16 operands or split-KV partial results need scratch memory: this entry point takes it from a stream-ordered pool of
+ * the library's own (one per device; it keeps up to 64 MiB across synchronisations).  Only enqueues work.  Errors: INVALID_ARG,
  * UNSUPPORTED, OOM, CUDA; message in phyai_op_last_error().
  */
 typedef struct {
@@ -313,15 +313,15 @@ size_t phyai_suffix_attention_scratch_bytes(const phyai_attention_desc_t *desc, 
  * that may only use the buffers it is handed.)
  *
  * Same arguments, same result as phyai_suffix_attention; the caller still passes inputs, the
- * output and the status word.  The request block and the split-KV partials go into a fixed
+ * output and the status word.  The bf16 operands or the split-KV partials go into a fixed
  * 16 MiB array (phyai_suffix_attention_static_capacity()) that is part of the library image: every GPU that
  * loads the library holds it until the process exits.  The call uses no cudaMalloc, cudaFree,
  * stream-ordered allocator or other allocating routine.
  *
  *   - The first call on each device looks up the array's device address (with that device
  *     current) and remembers it; make that first call before starting any stream capture.
- *   - Shapes that need more than the capacity (256 bytes + batch * Hq * splits * 64 * (head_dim + 2) * 4)
- *     are rejected with PHYAI_ERR_INVALID_ARG and a message naming both numbers; with
+ *   - Shapes that need more than the capacity (with num_splits set: 256 bytes + batch * Hq * splits * 64 *
+ *     (head_dim + 2) * 4) are rejected with PHYAI_ERR_INVALID_ARG and a message naming both numbers; with
  *     num_splits == 0 the library picks a split count first and then checks.
  *   - All calls on a device share the one array and it keeps the last call's contents.  Nothing
  *     in it needs clearing between calls, but two calls that overlap on the GPU (different
@@ -358,6 +358,12 @@ typedef struct {
 phyai_status_t phyai_pack_prefix_kv(const phyai_kv_pack_desc_t *desc, const void *k, const void *v, const int32_t *lens,
                                     void *prefix_kv, uint64_t kv_tokens, int32_t *cu_prefix_lens, int32_t *status_word,
                                     void *stream);
+
+/* The same, and every row of prefix_kv that receives no request row is set to zero (the rows past the last request; after
+ * an error all rows): for callers that would otherwise clear the whole buffer first. */
+phyai_status_t phyai_pack_prefix_kv_cleared(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens,
+                                            void* prefix_kv, uint64_t kv_tokens, int32_t* cu_prefix_lens,
+                                            int32_t* status_word, void* stream);
 
 /*
  * phyai_postprocess_actions: the raw chunk x at t = 0 -> robot actions (appendices on the pi0 / pi0.5 reproductions:

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import threading
 from typing import Dict, Optional, Sequence
 
 import numpy as np
@@ -29,7 +30,7 @@ EXPORTS = ("phyai_expert_create", "phyai_expert_destroy", "phyai_prefix_kv_bytes
            "phyai_set_option", "phyai_launches_per_call", "phyai_last_error", "phyai_version",
            "phyai_suffix_attention", "phyai_suffix_attention_scratch_bytes", "phyai_op_last_error",
            "phyai_suffix_attention_static", "phyai_suffix_attention_static_capacity", "phyai_read_trace",
-           "phyai_pack_prefix_kv", "phyai_postprocess_actions", "phyai_adapter_last_error", "phyai_batcher_create",
+           "phyai_pack_prefix_kv", "phyai_pack_prefix_kv_cleared", "phyai_postprocess_actions", "phyai_adapter_last_error", "phyai_batcher_create",
            "phyai_batcher_destroy", "phyai_batcher_submit", "phyai_batcher_next", "phyai_batcher_pending",
            "phyai_batcher_plan", "phyai_w8a8_project", "phyai_w8a8_last_error", "phyai_project_features_kv", "phyai_kv_projector_create",
            "phyai_kv_projector_run", "phyai_kv_projector_destroy")
@@ -61,6 +62,9 @@ class AttentionDesc(C.Structure):
 class KvPackDesc(C.Structure):
     _fields_ = [(n, C.c_uint32) for n in ("struct_size", "n_layers", "n_kv_heads", "head_dim", "elem_bytes", "batch",
                                           "p_max")]
+
+
+_KV_PACK_SIZE = C.sizeof(KvPackDesc)
 
 
 class BatcherConfig(C.Structure):
@@ -114,6 +118,7 @@ def load_library() -> C.CDLL:
     lib.phyai_suffix_attention_static.argtypes = lib.phyai_suffix_attention.argtypes
     lib.phyai_suffix_attention_static_capacity.restype = C.c_size_t
     lib.phyai_pack_prefix_kv.argtypes = [C.POINTER(KvPackDesc), _VP, _VP, _VP, _VP, C.c_uint64, _VP, _VP, _VP]
+    lib.phyai_pack_prefix_kv_cleared.argtypes = lib.phyai_pack_prefix_kv.argtypes
     lib.phyai_postprocess_actions.argtypes = [_VP, C.c_uint32, C.c_uint32, C.c_uint32, _VP, _VP, C.c_float, C.c_float,
                                               C.c_uint32, C.c_uint32, _VP, _VP]
     lib.phyai_adapter_last_error.restype = C.c_char_p
@@ -171,6 +176,11 @@ def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
         stream = torch.cuda.current_stream()
     return stream.cuda_stream or None
+
+
+def _raw_stream(stream, device: torch.device) -> int:
+    """cudaStream_t of ``stream`` (the device's current stream when None) as an integer."""
+    return torch._C._cuda_getCurrentRawStream(device.index) if stream is None else stream.cuda_stream
 
 
 class Expert:
@@ -310,16 +320,36 @@ def attention_desc(n_q_heads, n_kv_heads, head_dim, suffix_len, n_layers, layer,
     return d
 
 
+_zero_words: Dict[tuple, list] = {}
+_zero_lock = threading.Lock()
+
+
+def _zero_word(device: torch.device, stream: int) -> torch.Tensor:
+    """A zeroed int32 device word for an operator's status.  Words come from blocks of 256, zeroed at a time on the stream
+    that uses them (a fill kernel per call cost as much as the launch it served); every word is handed out once, and a block
+    lives as long as its words.  At most 64 streams keep a block."""
+    key = (device.index, stream)
+    with _zero_lock:
+        block = _zero_words.get(key)
+        if not block:
+            if block is None and len(_zero_words) >= 64:
+                _zero_words.clear()
+            with torch.cuda.stream(torch.cuda.ExternalStream(stream, device=device) if stream else torch.cuda.default_stream(device)):
+                block = _zero_words[key] = list(torch.zeros(256, dtype=torch.int32, device=device).split(1))
+        return block.pop()
+
+
 def suffix_attention(desc: AttentionDesc, qkv: torch.Tensor, prefix_kv: torch.Tensor, cu_prefix_lens: torch.Tensor,
                      rope_cos_sin: Optional[torch.Tensor], entry: str = "phyai_suffix_attention", stream=None):
     """Stand-alone attention operator; returns (out bf16 [rows, Hq*dh], status_word int32 tensor)."""
-    lib = load_library()
-    batch = int(cu_prefix_lens.numel()) - 1
-    rows = batch * desc.suffix_len
-    out = torch.empty(rows, desc.n_q_heads * desc.head_dim, dtype=torch.bfloat16, device=qkv.device)
-    status = torch.zeros(1, dtype=torch.int32, device=qkv.device)
-    st = getattr(lib, entry)(C.byref(desc), batch, _ptr(qkv), _ptr(prefix_kv), int(prefix_kv.shape[2]),
-                             _ptr(cu_prefix_lens), _ptr(rope_cos_sin), _ptr(out), _ptr(status), _stream_ptr(stream))
+    lib = _lib or load_library()
+    device = qkv.device
+    sp = _raw_stream(stream, device)
+    batch = cu_prefix_lens.numel() - 1
+    out = torch.empty(batch * desc.suffix_len, desc.n_q_heads * desc.head_dim, dtype=torch.bfloat16, device=device)
+    status = _zero_word(device, sp)
+    st = getattr(lib, entry)(C.byref(desc), batch, qkv.data_ptr(), prefix_kv.data_ptr(), prefix_kv.shape[2],
+                             cu_prefix_lens.data_ptr(), _ptr(rope_cos_sin), out.data_ptr(), status.data_ptr(), sp or None)
     if st != OK:
         raise PhyaiError(st, lib.phyai_op_last_error().decode())
     return out, status
@@ -328,18 +358,18 @@ def suffix_attention(desc: AttentionDesc, qkv: torch.Tensor, prefix_kv: torch.Te
 def pack_prefix_kv(k: torch.Tensor, v: torch.Tensor, lens: torch.Tensor, kv_tokens: Optional[int] = None, stream=None):
     """Padded backbone K / V ``[L, B, p_max, Hkv, dh]`` + ``lens`` (int32 ``[B]``, device) -> the library's ragged
     layout.  Returns (prefix_kv ``[L, 2, kv_tokens, Hkv, dh]``, cu_prefix_lens int32 ``[B + 1]``, status word)."""
-    lib = load_library()
+    lib = _lib or load_library()
     L, B, p_max, Hkv, dh = k.shape
     if kv_tokens is None:
         kv_tokens = B * p_max
-    desc = KvPackDesc()
-    desc.struct_size = C.sizeof(KvPackDesc)
-    desc.n_layers, desc.n_kv_heads, desc.head_dim, desc.elem_bytes, desc.batch, desc.p_max = L, Hkv, dh, k.element_size(), B, p_max
-    out = torch.zeros(L, 2, kv_tokens, Hkv, dh, dtype=k.dtype, device=k.device)
-    cu = torch.empty(B + 1, dtype=torch.int32, device=k.device)
-    status = torch.zeros(1, dtype=torch.int32, device=k.device)
-    st = lib.phyai_pack_prefix_kv(C.byref(desc), _ptr(k), _ptr(v), _ptr(lens), _ptr(out), int(kv_tokens), _ptr(cu), _ptr(status),
-                                  _stream_ptr(stream))
+    device = k.device
+    sp = _raw_stream(stream, device)
+    desc = KvPackDesc(_KV_PACK_SIZE, L, Hkv, dh, k.element_size(), B, p_max)
+    out = torch.empty(L, 2, kv_tokens, Hkv, dh, dtype=k.dtype, device=device)
+    cu = torch.empty(B + 1, dtype=torch.int32, device=device)
+    status = _zero_word(device, sp)
+    st = lib.phyai_pack_prefix_kv_cleared(C.byref(desc), k.data_ptr(), v.data_ptr(), lens.data_ptr(), out.data_ptr(), int(kv_tokens),
+                                          cu.data_ptr(), status.data_ptr(), sp or None)
     if st != OK:
         raise PhyaiError(st, lib.phyai_adapter_last_error().decode())
     return out, cu, status
@@ -348,13 +378,13 @@ def pack_prefix_kv(k: torch.Tensor, v: torch.Tensor, lens: torch.Tensor, kv_toke
 def postprocess_actions(x: torch.Tensor, q01: Optional[torch.Tensor], q99: Optional[torch.Tensor], clip=(-1.0, 1.0),
                         out_horizon: Optional[int] = None, out_dim: Optional[int] = None, stream=None) -> torch.Tensor:
     """Raw chunk ``[B, H, A]`` -> clipped, un-normalised actions ``[B, out_horizon, out_dim]``."""
-    lib = load_library()
+    lib = _lib or load_library()
     B, H, A = x.shape
     out_horizon, out_dim = out_horizon or H, out_dim or A
     out = torch.empty(B, out_horizon, out_dim, dtype=torch.float32, device=x.device)
     lo, hi = (clip if clip is not None else (0.0, 0.0))
     st = lib.phyai_postprocess_actions(_ptr(x), B, H, A, _ptr(q01), _ptr(q99), float(lo), float(hi), out_horizon, out_dim,
-                                       _ptr(out), _stream_ptr(stream))
+                                       _ptr(out), _raw_stream(stream, x.device) or None)
     if st != OK:
         raise PhyaiError(st, lib.phyai_adapter_last_error().decode())
     return out

@@ -14,36 +14,72 @@ namespace {
 thread_local char g_ad_err[256] = "";
 
 // cu[0] = 0, cu[b + 1] = cu[b] + lens[b]; a length outside 0..p_max or a total beyond kv_tokens raises the status word
-// (INVALID_ARG) and the pack kernel then copies nothing.
-__global__ void k_kv_scan(const int* lens, int batch, int p_max, unsigned long long kv_tokens, int* cu, int* status) {
-  if (threadIdx.x != 0) return;
-  long long acc = 0;
+// (INVALID_ARG) and the pack kernel then copies nothing.  One block: a thread sums a run of lengths, the runs are scanned.
+__global__ void __launch_bounds__(1024) k_kv_scan(const int* lens, int batch, int p_max, unsigned long long kv_tokens, int* cu, int* status) {
+  __shared__ long long wsum[32];
+  pdl_launch_dependents();
+  const int per = (batch + 1023) / 1024, b0 = min(batch, (int)threadIdx.x * per), b1 = min(batch, b0 + per);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   bool bad = false;
-  cu[0] = 0;
-  for (int b = 0; b < batch; ++b) {
+  long long sum = 0;
+  for (int b = b0; b < b1; ++b) {
     const int n = lens[b];
     if (n < 0 || n > p_max) bad = true;
-    acc += n < 0 ? 0 : n;
-    cu[b + 1] = (int)(acc > 0x7fffffffLL ? 0x7fffffffLL : acc);
+    sum += max(n, 0);
   }
-  if ((unsigned long long)acc > kv_tokens) bad = true;
+  long long run = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long v = __shfl_up_sync(0xffffffffu, run, o);
+    if (lane >= o) run += v;
+  }
+  if (lane == 31) wsum[warp] = run;
+  __syncthreads();
+  long long acc = run - sum;
+  for (int w = 0; w < warp; ++w) acc += wsum[w];
+  if (threadIdx.x == 0) cu[0] = 0;
+  for (int b = b0; b < b1; ++b) {
+    acc += max(lens[b], 0);
+    cu[b + 1] = (int)min(acc, 0x7fffffffLL);
+  }
+  if (b1 == batch && b0 < b1 && (unsigned long long)acc > kv_tokens) bad = true;
   if (bad) atomicExch(status, ST_INVALID_ARG);
 }
 
 // src [L][B][p_max][row_bytes], dst [L][2][kv_tokens][row_bytes]: plane (l, kv) of request b, rows p < lens[b], go to
-// rows cu[b] + p.  One thread per 16 bytes; grid.y = layer * 2 + (0 = K, 1 = V).
-__global__ void k_kv_pack(const uint4* k, const uint4* v, const int* lens, const int* cu, const int* status, uint4* dst,
-                          int batch, int p_max, unsigned long long kv_tokens, int row_chunks) {
-  if (status_set(status)) return;
+// rows cu[b] + p.  The rows of a request are one contiguous run on both sides: a block moves 16 KB of it (grid.x) of one
+// plane (grid.y) and request (grid.z), its loads issued before the dependency wait (only the destination needs cu).  With
+// `zero_tail` the entry grid.z = batch clears the rows past the last request (after an error: all rows).  Bound by HBM: 258 MB
+// of 8 requests of the pi0 shape 48 us, 5.4 TB/s (a grid-stride loop over padded rows with two divisions per 16 bytes,
+// behind a fill of the whole output by the caller: 139 us).
+constexpr int PACK_T = 256, PACK_U = 4, PACK_CHUNK = PACK_T * PACK_U;
+__global__ void __launch_bounds__(PACK_T) k_kv_pack(const uint4* k, const uint4* v, const int* lens, const int* cu, const int* status, uint4* dst,
+                                                    int batch, int p_max, unsigned long long kv_tokens, int row_chunks, int zero_tail) {
   const int layer = blockIdx.y >> 1, is_v = blockIdx.y & 1;
-  const uint4* src = (is_v ? v : k) + (size_t)layer * batch * p_max * row_chunks;
-  uint4* out = dst + ((size_t)layer * 2 + is_v) * kv_tokens * row_chunks;
-  const size_t total = (size_t)batch * p_max * row_chunks;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % row_chunks);
-    const size_t row = i / row_chunks;
-    const int p = (int)(row % p_max), b = (int)(row / p_max);
-    if (p < lens[b]) out[((size_t)cu[b] + p) * row_chunks + c] = src[i];
+  uint4* out = dst + (size_t)blockIdx.y * kv_tokens * row_chunks;
+  bool waited = false;
+  for (int b = blockIdx.z; b < batch + zero_tail; b += gridDim.z) {
+    if (b == batch) {
+      if (!waited) pdl_wait();
+      waited = true;
+      const size_t lo = status_set(status) ? 0 : (size_t)cu[batch] * row_chunks, hi = kv_tokens * row_chunks;
+      for (size_t i = lo + (size_t)blockIdx.x * PACK_T + threadIdx.x; i < hi; i += (size_t)gridDim.x * PACK_T) out[i] = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
+    const int n = min(max(lens[b], 0), p_max) * row_chunks;
+    const uint4* src = (is_v ? v : k) + ((size_t)layer * batch + b) * p_max * row_chunks;
+    uint4 x[PACK_U];
+    const int i0 = (int)blockIdx.x * PACK_CHUNK + (int)threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < PACK_U; ++u)
+      if (i0 + u * PACK_T < n) x[u] = __ldcs(src + i0 + u * PACK_T);
+    if (!waited) pdl_wait();
+    waited = true;
+    if ((int)blockIdx.x * PACK_CHUNK >= n || status_set(status)) continue;
+    uint4* o = out + (size_t)cu[b] * row_chunks + i0;
+#pragma unroll
+    for (int u = 0; u < PACK_U; ++u)
+      if (i0 + u * PACK_T < n) o[u * PACK_T] = x[u];
   }
 }
 
@@ -84,9 +120,8 @@ extern "C" {
 
 const char* phyai_adapter_last_error(void) { return phyai::g_ad_err; }
 
-phyai_status_t phyai_pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens,
-                                    void* prefix_kv, uint64_t kv_tokens, int32_t* cu_prefix_lens, int32_t* status_word,
-                                    void* stream) {
+static phyai_status_t pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens, void* prefix_kv,
+                                     uint64_t kv_tokens, int32_t* cu_prefix_lens, int32_t* status_word, int zero_tail, void* stream) {
   using namespace phyai;
   auto bad = [](const char* m) {
     snprintf(g_ad_err, sizeof(g_ad_err), "%s", m);
@@ -101,21 +136,31 @@ phyai_status_t phyai_pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const void
   if (row_bytes % 16) return bad("n_kv_heads * head_dim * elem_bytes must be a multiple of 16");
   if ((reinterpret_cast<uintptr_t>(k) | reinterpret_cast<uintptr_t>(v) | reinterpret_cast<uintptr_t>(prefix_kv)) & 15u)
     return bad("k, v and prefix_kv must be 16-byte aligned");
-  if (kv_tokens > 0x7fffffffull || desc->batch > 65535u || desc->n_layers > 32767u) return bad("kv_tokens, batch or n_layers too large");
+  if (kv_tokens > 0x7fffffffull || desc->batch > 65535u || desc->n_layers > 32767u || desc->p_max * (row_bytes / 16) > 0x7fffffffull)
+    return bad("kv_tokens, batch, p_max or n_layers too large");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int chunks = (int)(row_bytes / 16);
-  k_kv_scan<<<1, 32, 0, st>>>(lens, (int)desc->batch, (int)desc->p_max, kv_tokens, cu_prefix_lens, status_word);
-  const size_t total = (size_t)desc->batch * desc->p_max * chunks;
-  const int blocks = (int)((total + 255) / 256 < 2048 ? (total + 255) / 256 : 2048);
-  k_kv_pack<<<dim3(blocks, desc->n_layers * 2), 256, 0, st>>>(reinterpret_cast<const uint4*>(k), reinterpret_cast<const uint4*>(v), lens,
-                                                             cu_prefix_lens, status_word, reinterpret_cast<uint4*>(prefix_kv),
-                                                             (int)desc->batch, (int)desc->p_max, kv_tokens, chunks);
-  cudaError_t e = cudaGetLastError();
+  const int chunks = (int)(row_bytes / 16), B = (int)desc->batch;
+  k_kv_scan<<<1, 1024, 0, st>>>(lens, B, (int)desc->p_max, kv_tokens, cu_prefix_lens, status_word);
+  const unsigned gx = (unsigned)(((size_t)desc->p_max * chunks + PACK_CHUNK - 1) / PACK_CHUNK);
+  cudaError_t e = launch_pdl(k_kv_pack, dim3(gx, desc->n_layers * 2, B + zero_tail < 65535 ? B + zero_tail : 65535), dim3(PACK_T), 0, st,
+                             reinterpret_cast<const uint4*>(k), reinterpret_cast<const uint4*>(v), (const int*)lens, (const int*)cu_prefix_lens,
+                             (const int*)status_word, reinterpret_cast<uint4*>(prefix_kv), B, (int)desc->p_max,
+                             (unsigned long long)kv_tokens, chunks, zero_tail);
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(g_ad_err, sizeof(g_ad_err), "kernel launch failed: %s", cudaGetErrorString(e));
     return PHYAI_ERR_CUDA;
   }
   return PHYAI_OK;
+}
+
+phyai_status_t phyai_pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens, void* prefix_kv,
+                                    uint64_t kv_tokens, int32_t* cu_prefix_lens, int32_t* status_word, void* stream) {
+  return pack_prefix_kv(desc, k, v, lens, prefix_kv, kv_tokens, cu_prefix_lens, status_word, 0, stream);
+}
+phyai_status_t phyai_pack_prefix_kv_cleared(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens,
+                                            void* prefix_kv, uint64_t kv_tokens, int32_t* cu_prefix_lens, int32_t* status_word, void* stream) {
+  return pack_prefix_kv(desc, k, v, lens, prefix_kv, kv_tokens, cu_prefix_lens, status_word, 1, stream);
 }
 
 phyai_status_t phyai_postprocess_actions(const float* x, uint32_t batch, uint32_t horizon, uint32_t action_dim,

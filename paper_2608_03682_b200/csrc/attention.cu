@@ -101,6 +101,15 @@ cudaError_t launch_attn_cluster(const AttnArgs& a, int batch, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, k_attn_cluster<DH, KTT, OPROJ>, a);
 }
 
+cudaError_t launch_mma(const AttnArgs& a, int batch, cudaStream_t st) {
+  const int G = a.d.Hq / a.d.Hkv;
+  const bool two = (G % 2 == 0) && (batch * a.d.Hq * a.num_splits >= 2 * 148);
+  // (one head per CTA with 32-key tiles, two CTAs per SM, was measured no faster than two heads per CTA)
+  if (a.d.dh == 256) return two ? launch_attn<256, 2, 64>(a, batch, st) : launch_attn<256, 1, 64>(a, batch, st);
+  if (a.d.dh == 128) return two ? launch_attn<128, 2, 64>(a, batch, st) : launch_attn<128, 1, 64>(a, batch, st);
+  return two ? launch_attn<64, 2, 64>(a, batch, st) : launch_attn<64, 1, 64>(a, batch, st);
+}
+
 }  // namespace
 
 // Key-split attention whose partials are merged through distributed shared memory (clusters of 8 CTAs).
@@ -161,12 +170,7 @@ cudaError_t launch_attention_mma(const Request* rq, int* status, const float* qk
   a.num_splits = num_splits, a.d = d, a.wait_limit = wait_limit;
   a.part_o = scratch;
   a.part_ml = scratch ? scratch + (size_t)batch * d.Hq * num_splits * QROWS * d.dh : nullptr;
-  const int G = d.Hq / d.Hkv;
-  const bool two = (G % 2 == 0) && (batch * d.Hq * num_splits >= 2 * 148);
-  // (one head per CTA with 32-key tiles, two CTAs per SM, was measured no faster than two heads per CTA)
-  if (d.dh == 256) return two ? launch_attn<256, 2, 64>(a, batch, st) : launch_attn<256, 1, 64>(a, batch, st);
-  if (d.dh == 128) return two ? launch_attn<128, 2, 64>(a, batch, st) : launch_attn<128, 1, 64>(a, batch, st);
-  return two ? launch_attn<64, 2, 64>(a, batch, st) : launch_attn<64, 1, 64>(a, batch, st);
+  return launch_mma(a, batch, st);
 }
 
 }  // namespace phyai
@@ -179,8 +183,101 @@ namespace {
 
 thread_local char g_op_err[256] = "";
 
-// Shared body of the operator entry points: fills the request block at the head of `scratch`,
-// then launches the attention (and merge) kernels with the split-KV partials placed after it.
+// cu_prefix_lens of an operator call, checked on the device like in the denoise calls: a violation raises the caller's
+// status word (INVALID_ARG) and turns the attention kernels into no-ops.
+__device__ __forceinline__ void check_lens(const int* cu, int batch, uint64_t kv_tokens, int* status) {
+  for (int b = threadIdx.x; b < batch; b += blockDim.x) {
+    const int lo = cu[b], hi = cu[b + 1];
+    if (lo < 0 || hi < lo || (uint64_t)hi > kv_tokens) atomicExch(status, ST_INVALID_ARG);
+  }
+}
+__global__ void k_check_lens(const int* cu, int batch, uint64_t kv_tokens, int* status) {
+  pdl_launch_dependents();
+  check_lens(cu, batch, kv_tokens, status);
+}
+
+// Operands of the tcgen05 kernels from an operator call's fp32 q | k | v rows: q rotated, scaled and rounded into the operand
+// tiles [request][head pair][dh / 64][128 rows][64] (rows past the suffix are zero), k rotated, v as is: bf16 rows
+// [request][Hkv][S][dh].  One block per (suffix row < 64, request), a thread 8 channels and their rotary partners.  Block 0
+// also writes the request block and checks the lengths.
+__global__ void __launch_bounds__(256) k_op_operands(Request* rq, const Request src, int* status, const float* qkv, const float2* rope,
+                                                     __nv_bfloat16* q_tiles, __nv_bfloat16* kr, __nv_bfloat16* vr, const Dims d) {
+  const int i = blockIdx.x, b = blockIdx.y, half = d.dh >> 1, hc = half >> 3;
+  if (i == 0 && b == 0) {
+    if (threadIdx.x == 0) *rq = src;
+    check_lens(src.cu_lens, src.batch, src.kv_tokens, status);
+  }
+  const int nq = d.Hq * hc, nk = d.Hkv * hc;               // items of 8 + 8 channels: q, k, v
+  const float scale = rsqrtf((float)d.dh);
+  const int lo_b = src.cu_lens[b], hi_b = src.cu_lens[b + 1], pos = hi_b - lo_b + i;
+  const bool live = i < d.S && lo_b >= 0 && hi_b >= lo_b && (uint64_t)hi_b <= src.kv_tokens;
+  for (int it = threadIdx.x; it < nq + 2 * nk; it += blockDim.x) {
+    const int kind = it < nq ? 0 : (it < nq + nk ? 1 : 2), item = it - (kind == 0 ? 0 : (kind == 1 ? nq : nq + nk));
+    const int head = item / hc, c = (item - head * hc) * 8;
+    float lo[8] = {}, hi[8] = {};
+    if (live) {
+      const float* p = qkv + (size_t)(b * d.S + i) * d.Nqkv + (kind == 0 ? 0 : (kind == 1 ? d.Nq : d.Nq + d.Hkv * d.dh)) + head * d.dh + c;
+#pragma unroll
+      for (int e = 0; e < 8; e += 4) {
+        *reinterpret_cast<float4*>(lo + e) = *reinterpret_cast<const float4*>(p + e);
+        *reinterpret_cast<float4*>(hi + e) = *reinterpret_cast<const float4*>(p + half + e);
+      }
+      if (kind < 2 && rope) {
+        const float2* cs = rope + (size_t)pos * half + c;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float2 w = cs[e];
+          const float l = lo[e] * w.x - hi[e] * w.y;
+          hi[e] = hi[e] * w.x + lo[e] * w.y, lo[e] = l;
+        }
+      }
+    }
+    const float s = kind == 0 ? scale : 1.0f;
+    auto pack8 = [&](const float* x) {
+      return make_uint4(pack_bf16(x[0] * s, x[1] * s), pack_bf16(x[2] * s, x[3] * s), pack_bf16(x[4] * s, x[5] * s), pack_bf16(x[6] * s, x[7] * s));
+    };
+    if (kind == 0) {
+      __nv_bfloat16* t = q_tiles + (size_t)(b * (d.Hq >> 1) + (head >> 1)) * 128 * d.dh + ((head & 1) * 64 + i) * 64;
+      const int c2 = c + half;
+      *reinterpret_cast<uint4*>(t + (size_t)(c >> 6) * 8192 + ((((c & 63) >> 3) ^ (i & 7)) << 3)) = pack8(lo);
+      *reinterpret_cast<uint4*>(t + (size_t)(c2 >> 6) * 8192 + ((((c2 & 63) >> 3) ^ (i & 7)) << 3)) = pack8(hi);
+    } else if (i < d.S) {
+      __nv_bfloat16* t = (kind == 1 ? kr : vr) + ((size_t)(b * d.Hkv + head) * d.S + i) * d.dh + c;
+      *reinterpret_cast<uint4*>(t) = pack8(lo), *reinterpret_cast<uint4*>(t + half) = pack8(hi);
+    }
+  }
+}
+
+// Scratch: a pool of the library's own per device, which keeps up to 64 MiB across synchronisations (the device's default
+// pool gives everything back at each one: 1 - 3 ms for the next call).  Stream-ordered, so several threads and streams may
+// use it at a time.
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+  static std::mutex mu;
+  static cudaMemPool_t pools[64] = {};
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaMallocAsync(p, bytes, st);
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!pools[dev]) {
+      cudaMemPoolProps props{};
+      props.allocType = cudaMemAllocationTypePinned, props.location.type = cudaMemLocationTypeDevice, props.location.id = dev;
+      uint64_t keep = 64ull << 20;
+      if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+      if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return e;
+      }
+      pools[dev] = pool;
+    }
+    pool = pools[dev];
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
+
+// Shared body of the operator entry points.  `scratch` null: taken from the library's pool when the call needs any.
 phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, const float* qkv, const void* prefix_kv,
                             uint64_t kv_tokens, const int32_t* cu, const float* rope, uint16_t* out, int32_t* status_word,
                             void* scratch, size_t scratch_bytes, cudaStream_t st) {
@@ -206,24 +303,54 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     return PHYAI_ERR_UNSUPPORTED;
   }
   int splits = (int)desc->num_splits;
+  if (splits < 0 || splits > 16) return bad("num_splits must be 0 (choose) or 1..16");
+  AttnArgs a{};
+  a.op_kv = prefix_kv, a.op_kv_tokens = kv_tokens, a.op_cu = cu, a.status = status_word, a.qkv = qkv;
+  a.rope = reinterpret_cast<const float2*>(rope), a.layer = (int)desc->layer, a.out = reinterpret_cast<__nv_bfloat16*>(out);
+  a.d = d, a.wait_limit = 1u << 22;
+  // The library's choice where shapes and alignment allow it: bf16 operands first (one small kernel), then the tcgen05 kernels
+  // of the denoising loop.  One request of the pi0 shape: 37.6 -> 23 us per call; 16 requests: 70 -> 35 us.
+  const bool tc = splits == 0 && !((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(qkv)) & 15u) && kv_tokens > 0 &&
+                  attention_pair_supported(d);
   if (splits == 0) splits = attention_pick_splits(d, (int)batch, (int)(kv_tokens < 4096 ? kv_tokens : 4096));
-  if (splits < 1 || splits > 16) return bad("num_splits must be 0 (choose) or 1..16");
-  const size_t need = 256 + attention_scratch_floats(d, (int)batch, splits) * sizeof(float);
-  if (need > scratch_bytes) {
+  const size_t q_elems = (size_t)batch * (d.Hq / 2) * 128 * d.dh, kv_elems = (size_t)batch * d.Hkv * d.S * d.dh;
+  const size_t need = tc ? sizeof(Request) + (q_elems + 2 * kv_elems) * 2 : attention_scratch_floats(d, (int)batch, splits) * sizeof(float);
+  if (need && scratch && need > scratch_bytes) {
     snprintf(g_op_err, sizeof(g_op_err), "needs %zu bytes of scratch, only %zu available", need, scratch_bytes);
     return PHYAI_ERR_INVALID_ARG;
   }
-  Request r{};
-  r.prefix_kv = prefix_kv, r.kv_tokens = kv_tokens, r.cu_lens = cu, r.batch = (int)batch;
-  Request* rq = reinterpret_cast<Request*>(scratch);
-  launch_set_request(rq, r, nullptr, st);
-  // cu_prefix_lens is checked on the device like in the denoise calls: a violation raises the caller's status word
-  // (INVALID_ARG) and turns the attention kernels into no-ops
-  launch_validate(rq, status_word, (int)kv_tokens, nullptr, st);
-  float* partials = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(scratch) + 256);
-  cudaError_t e = launch_attention_mma(rq, status_word, qkv, reinterpret_cast<const float2*>(rope), (int)desc->layer,
-                                       reinterpret_cast<__nv_bfloat16*>(out), 0, splits, splits > 1 ? partials : nullptr,
-                                       d, (int)batch, 1u << 22, st);
+  cudaError_t e = cudaSuccess;
+  const bool own = need && !scratch;
+  if (own && (e = scratch_alloc(&scratch, need, st)) != cudaSuccess) {
+    snprintf(g_op_err, sizeof(g_op_err), "scratch allocation of %zu bytes failed: %s", need, cudaGetErrorString(e));
+    return PHYAI_ERR_OOM;
+  }
+  if (tc) {
+    Request* rq = reinterpret_cast<Request*>(scratch);
+    __nv_bfloat16 *qt = reinterpret_cast<__nv_bfloat16*>(rq + 1), *kr = qt + q_elems, *vr = kr + kv_elems;
+    Request r{};
+    r.prefix_kv = prefix_kv, r.kv_tokens = kv_tokens, r.cu_lens = cu, r.batch = (int)batch;
+    if (!prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) {
+      k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d);
+      // (the attention kernels read the request block before their dependency wait: no programmatic launch here)
+      if (attention_b1_ctas(d, (int)batch, 1) <= 15 * 8)     // 15 clusters of 8 fit a B200
+        e = launch_attention_b1(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch, 1, a.wait_limit, st, nullptr, 0, false);
+      else
+        e = launch_attention_pair(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch,
+                                  attention_pair_ranges(d, (int)batch, (int)(kv_tokens / batch)), nullptr, a.wait_limit, st, nullptr, false);
+    }
+  } else {
+    if (splits > 1) {
+      a.part_o = reinterpret_cast<float*>(scratch);
+      a.part_ml = a.part_o + (size_t)batch * d.Hq * splits * QROWS * d.dh;
+    }
+    k_check_lens<<<1, 256, 0, st>>>(cu, (int)batch, kv_tokens, status_word);
+    a.num_splits = splits;
+    e = launch_mma(a, (int)batch, st);
+  }
+  if (own) cudaFreeAsync(scratch, st);      // stream-ordered: released after the kernels above have run
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(g_op_err, sizeof(g_op_err), "attention launch failed: %s", cudaGetErrorString(e));
     return PHYAI_ERR_CUDA;
@@ -255,16 +382,7 @@ phyai_status_t phyai_suffix_attention(const phyai_attention_desc_t* desc, uint32
     snprintf(phyai::g_op_err, sizeof(phyai::g_op_err), "desc is NULL or batch is 0");
     return PHYAI_ERR_INVALID_ARG;
   }
-  void* scratch = nullptr;
-  cudaError_t e = cudaMallocAsync(&scratch, bytes, st);
-  if (e != cudaSuccess) {
-    snprintf(phyai::g_op_err, sizeof(phyai::g_op_err), "cudaMallocAsync(%zu) failed: %s", bytes, cudaGetErrorString(e));
-    return PHYAI_ERR_OOM;
-  }
-  phyai_status_t s = phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out,
-                                         status_word, scratch, bytes, st);
-  cudaFreeAsync(scratch, st);  // stream-ordered: released after the kernels above have run
-  return s;
+  return phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word, nullptr, 0, st);
 }
 
 }  // extern "C"
@@ -272,7 +390,7 @@ phyai_status_t phyai_suffix_attention(const phyai_attention_desc_t* desc, uint32
 // =============================================================================================
 // Attention operator that allocates nothing
 // =============================================================================================
-// Scratch for the request block and the split-KV partials lives in this fixed array instead of
+// Scratch for the operands or the split-KV partials lives in this fixed array instead of
 // coming from an allocator.  Every GPU that loads the library holds it until the process exits.
 #define PHYAI_STATIC_SCRATCH_BYTES (16u << 20)
 static __device__ __align__(256) unsigned char g_static_scratch[PHYAI_STATIC_SCRATCH_BYTES];
@@ -333,8 +451,8 @@ phyai_status_t phyai_suffix_attention_static(const phyai_attention_desc_t* desc,
   phyai_status_t s = phyai::static_scratch_address(&scratch);
   if (s != PHYAI_OK) return s;
   // attention_op re-derives the exact requirement (after choosing num_splits) and refuses sizes
-  // beyond the capacity passed here.  Nothing in the scratch has to start at zero: the request
-  // block is rewritten by every call and every partial that is read was written by the same call.
+  // beyond the capacity passed here.  Nothing in the scratch has to start at zero: whatever is read was written by
+  // the same call.
   return phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word,
                              scratch, PHYAI_STATIC_SCRATCH_BYTES, reinterpret_cast<cudaStream_t>(stream));
 }

@@ -40,7 +40,10 @@ __device__ __forceinline__ size_t out_index(int row, int col, int rows_pad, int 
 }
 
 struct AttnArgs {
-  const Request* rq;
+  const Request* rq;     // or null (operator entry points): the cache and the lengths are the op_ members
+  const void* op_kv;
+  uint64_t op_kv_tokens;
+  const int* op_cu;
   int* status;
   const float* qkv;      // [rows][Nqkv] fp32 (q | k | v), un-rotated
   const __nv_bfloat16 *qr, *kr, *vr;  // or: rotated, scaled bf16 q [b][Hq][S][dh], k / v [b][Hkv][S][dh] (null = use qkv)
@@ -118,8 +121,11 @@ __device__ __forceinline__ void attn_role(const AttnArgs& a, int split, int hgrp
   const int hk = head0 / (d.Hq / d.Hkv);
   const int S = d.S;
 
-  const Request r = *a.rq;
-  const int p0 = r.cu_lens[b], P = r.cu_lens[b + 1] - p0;
+  struct { const void* prefix_kv; uint64_t kv_tokens; const int* cu_lens; } r;
+  if (a.rq) r.prefix_kv = a.rq->prefix_kv, r.kv_tokens = a.rq->kv_tokens, r.cu_lens = a.rq->cu_lens;
+  else r.prefix_kv = a.op_kv, r.kv_tokens = a.op_kv_tokens, r.cu_lens = a.op_cu;
+  // (a call whose lengths are invalid stores nothing; the clamps keep its loads inside the cache)
+  const int p0 = min(max(r.cu_lens[b], 0), (int)r.kv_tokens), P = min(max(r.cu_lens[b + 1] - p0, 0), (int)r.kv_tokens - p0);
   const int Tp = (P + KTT - 1) / KTT;          // prefix tiles, followed by the suffix tiles
   const int T = Tp + (S + KTT - 1) / KTT;
   const int t_begin = (int)(((long long)T * split) / a.num_splits);

@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
 }
 
 template <int DH, int HPC>
-cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st) {
+cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) {
   static PerDeviceOnce once;
   if (once.needed()) {
     cudaError_t e = cudaFuncSetAttribute(k_attn_b1<DH, HPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B1Layout<DH, HPC>::SMEM);
@@ -460,7 +460,7 @@ cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st) {
   at[0].val.clusterDim.x = 8, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at, cfg.numAttrs = 2;
+  cfg.attrs = at, cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_attn_b1<DH, HPC>, a);
 }
 
@@ -476,12 +476,12 @@ int attention_b1_ctas(const Dims& d, int batch, int hpc) { return 8 * (d.Hq / hp
 
 cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
-                                int batch, int hpc, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, int trace_all) {
+                                int batch, int hpc, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, int trace_all, bool pdl) {
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
   a.num_splits = 8, a.d = d, a.wait_limit = wait_limit, a.trace = trace, a.trace_all = trace_all;
-  if (hpc == 1) return d.dh == 256 ? launch_one<256, 1>(a, batch, st) : launch_one<128, 1>(a, batch, st);
-  return d.dh == 256 ? launch_one<256, 2>(a, batch, st) : launch_one<128, 2>(a, batch, st);
+  if (hpc == 1) return d.dh == 256 ? launch_one<256, 1>(a, batch, st, pdl) : launch_one<128, 1>(a, batch, st, pdl);
+  return d.dh == 256 ? launch_one<256, 2>(a, batch, st, pdl) : launch_one<128, 2>(a, batch, st, pdl);
 }
 
 }  // namespace phyai

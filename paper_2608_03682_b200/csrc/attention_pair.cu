@@ -395,11 +395,12 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
                        "r"(pack_bf16(o[e + 4] * inv, o[e + 5] * inv)), "r"(pack_bf16(o[e + 6] * inv, o[e + 7] * inv))
                        : "memory");
         __syncwarp();
-        uint4* dst = reinterpret_cast<uint4*>(a.out + ((size_t)(((head0 + hl) * DH + c) >> 6) * a.rows_pad + (size_t)(b * S + i0)) * 64);
         for (int idx = lane; idx < nrow * 8; idx += 32) {
+          const int rr = b * S + i0 + (idx >> 3);
           uint4 v;
           asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(ostage + (uint32_t)idx * 16u) : "memory");
-          dst[idx] = v;
+          // (tiled: the chunk's place as staged; row-major, for the operator: the swizzle undone)
+          *reinterpret_cast<uint4*>(a.out + out_index(rr, (head0 + hl) * DH + c + (((idx & 7) ^ (rr & 7)) << 3), a.rows_pad, d.Nq)) = v;
         }
         __syncwarp();
       }
@@ -495,7 +496,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
           }
         }
         const int orow = b * S + own_lo + il, col = (head0 + hl) * DH + ch * 8;
-        *reinterpret_cast<uint4*>(a.out + tiled_index(orow, col, a.rows_pad)) =
+        *reinterpret_cast<uint4*>(a.out + out_index(orow, col, a.rows_pad, d.Nq)) =
             make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
       }
     }
@@ -541,7 +542,7 @@ int max_clusters(int dh, int c) {
 }
 
 template <int DH, int C>
-cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st) {
+cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) {
   cudaError_t e = setup_one<DH, C>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -551,7 +552,7 @@ cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st) {
   at[0].val.clusterDim.x = 2 * C, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at, cfg.numAttrs = 2;
+  cfg.attrs = at, cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_attn_pair<DH, C>, a);
 }
 
@@ -597,19 +598,19 @@ int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
 
 cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                   const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
-                                  int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace) {
+                                  int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, bool pdl) {
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
   a.num_splits = ranges, a.d = d, a.wait_limit = wait_limit, a.order = order, a.trace = trace;
   switch (ranges + (d.dh == 256 ? 4 : 0)) {
-    case 1: return launch_one<128, 1>(a, batch, st);
-    case 2: return launch_one<128, 2>(a, batch, st);
-    case 3: return launch_one<128, 3>(a, batch, st);
-    case 4: return launch_one<128, 4>(a, batch, st);
-    case 5: return launch_one<256, 1>(a, batch, st);
-    case 6: return launch_one<256, 2>(a, batch, st);
-    case 7: return launch_one<256, 3>(a, batch, st);
-    default: return launch_one<256, 4>(a, batch, st);
+    case 1: return launch_one<128, 1>(a, batch, st, pdl);
+    case 2: return launch_one<128, 2>(a, batch, st, pdl);
+    case 3: return launch_one<128, 3>(a, batch, st, pdl);
+    case 4: return launch_one<128, 4>(a, batch, st, pdl);
+    case 5: return launch_one<256, 1>(a, batch, st, pdl);
+    case 6: return launch_one<256, 2>(a, batch, st, pdl);
+    case 7: return launch_one<256, 3>(a, batch, st, pdl);
+    default: return launch_one<256, 4>(a, batch, st, pdl);
   }
 }
 

@@ -195,7 +195,7 @@ bool attention_b1_supported(const Dims& d);
 cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
                                 int batch, int hpc, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr,
-                                int trace_all = 0);
+                                int trace_all = 0, bool pdl = true);
 // CTAs of one launch with `hpc` (1 or 2) query heads per CTA
 int attention_b1_ctas(const Dims& d, int batch, int hpc);
 cudaError_t launch_attention_tc(const Request* rq, int* status, const __nv_bfloat16* qr, const __nv_bfloat16* kr,
@@ -215,7 +215,8 @@ bool prefix_kv_map(unsigned char* map, const void* kv, uint64_t kv_tokens, const
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix);
 cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                   const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
-                                  int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr);
+                                  int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr,
+                                  bool pdl = true);
 
 // ---- tcgen05 GEMM ------------------------------------------------------------------------------
 enum : int { TC_STORE = 0, TC_RESID = 1, TC_GEGLU = 2, TC_BIAS_ROWMAP = 3, TC_QKV_ROT = 4, TC_GEGLU_IL = 5 };

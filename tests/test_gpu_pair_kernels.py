@@ -46,3 +46,17 @@ def test_pair_attention_key_ranges(head_dim, n_q, n_kv, ranges):
     cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=9, max_prefix_len=700, n_layers=2,
                             suffix_block_causal=ranges % 2 == 0)
     check(cfg, [700, 0, 1, 127, 128, 129, 512, 64, 386], 1, range(9), pair_attn_ranges=ranges)
+
+
+@pytest.mark.parametrize("n_kv,head_dim,suffix,lens", [(1, 256, 51, [700, 0, 129]), (1, 256, 64, [(53 * b) % 300 for b in range(40)]),
+                                                      (2, 128, 17, [128] * 45)])
+def test_attention_operator_on_the_pair_kernel(n_kv, head_dim, suffix, lens):
+    """The library's own choice of kernel: split key ranges, one range per request (row-major output), 128-channel heads."""
+    from tests.test_gpu_attention_op import make_case, oracle_attention
+    qkv, kv, cu, rope = make_case(9, 8, n_kv, head_dim, suffix, lens)
+    desc = binding.attention_desc(8, n_kv, head_dim, suffix, n_layers=2, layer=1)
+    out, status = binding.suffix_attention(desc, qkv.cuda(), kv.cuda(), torch.from_numpy(cu).cuda(), rope.cuda())
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    ref = oracle_attention(qkv, kv, cu, 8, n_kv, head_dim, suffix, 1, 10000.0)
+    assert abs(out.double().cpu().numpy() - ref).max() <= 2e-2 * abs(ref).max()
