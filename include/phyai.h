@@ -195,6 +195,19 @@ phyai_status_t phyai_denoise_batched_host(phyai_expert_t *h, uint32_t batch, con
                                           const float *noise, uint32_t n_steps, float *out_actions, void *stream);
 
 /*
+ * Requests as they arrive at a serving rank: every request's tensors in ordinary (pageable) host memory of its own.
+ *   prefix_kvs   HOST array of HOST pointers, [n_layers][2][prefix_lens[b]][n_kv_heads][head_dim] (NULL for an empty prefix)
+ *   states, noises  HOST arrays of HOST pointers, float32 [state_dim] / [horizon, action_dim]; a NULL entry means zeros
+ *   out_actions  HOST, float32 [batch, horizon, action_dim] (pinned memory makes the copy asynchronous)
+ * The call gathers the requests into page-locked staging of the handle (on a few threads of the handle's own, the copies
+ * to the device following plane by plane), runs the batched kernels and copies the actions back on `stream`.  The inputs
+ * are not read after it returns; the result is valid after the stream is synchronised.
+ */
+phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, const void* const* prefix_kvs,
+                                           const uint32_t* prefix_lens, const float* const* states,
+                                           const float* const* noises, uint32_t n_steps, float* out_actions, void* stream);
+
+/*
  * After the stream has been synchronised: read and clear the handle's device status word.
  * PHYAI_OK, PHYAI_ERR_TIMEOUT (a bounded wait inside a kernel expired; results are invalid) or
  * PHYAI_ERR_INVALID_ARG (device-side validation of cu_prefix_lens failed).  Synchronises the

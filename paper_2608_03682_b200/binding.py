@@ -26,7 +26,7 @@ BIG = ("wq", "wk", "wv", "wo", "wgate", "wup", "wdown")
 
 #: every symbol the header declares
 EXPORTS = ("phyai_expert_create", "phyai_expert_destroy", "phyai_prefix_kv_bytes", "phyai_denoise",
-           "phyai_denoise_batched", "phyai_denoise_host", "phyai_denoise_batched_host", "phyai_poll_status",
+           "phyai_denoise_batched", "phyai_denoise_host", "phyai_denoise_batched_host", "phyai_denoise_requests_host", "phyai_poll_status",
            "phyai_set_option", "phyai_launches_per_call", "phyai_last_error", "phyai_version",
            "phyai_suffix_attention", "phyai_suffix_attention_scratch_bytes", "phyai_op_last_error",
            "phyai_suffix_attention_static", "phyai_suffix_attention_static_capacity", "phyai_read_trace",
@@ -105,6 +105,7 @@ def load_library() -> C.CDLL:
     lib.phyai_denoise_host.argtypes = single
     lib.phyai_denoise_batched.argtypes = batched
     lib.phyai_denoise_batched_host.argtypes = batched
+    lib.phyai_denoise_requests_host.argtypes = [_VP, C.c_uint32, _VP, _VP, _VP, _VP, C.c_uint32, _VP, _VP]
     lib.phyai_poll_status.argtypes = [_VP]
     lib.phyai_set_option.argtypes = [_VP, C.c_char_p, C.c_int64]
     lib.phyai_read_trace.argtypes = [_VP, _VP, C.c_size_t, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)]
@@ -280,6 +281,19 @@ class Expert:
         _check(self.lib.phyai_denoise_batched_host(self._handle, batch, _ptr(prefix_kv), int(prefix_kv.shape[2]),
                                                    _ptr(cu_prefix_lens), _ptr(states), _ptr(noise), int(n_steps),
                                                    _ptr(out), _stream_ptr(stream)))
+        return out
+
+    def denoise_requests_host(self, requests, n_steps: int, out: torch.Tensor, stream=None) -> torch.Tensor:
+        """phyai_denoise_requests_host: ``requests`` = (prefix_kv or None, state or None, noise or None) per request, contiguous
+        host tensors of the expert's storage types; ``out`` [B,H,A] (ideally pinned) is complete once the stream is."""
+        B = len(requests)
+        kv, st, nz = (_VP * B)(), (_VP * B)(), (_VP * B)()
+        lens = (C.c_uint32 * B)()
+        for b, (k, s, z) in enumerate(requests):
+            if k is not None and k.shape[2]:
+                kv[b], lens[b] = k.data_ptr(), k.shape[2]
+            st[b], nz[b] = _ptr(s), _ptr(z)
+        _check(self.lib.phyai_denoise_requests_host(self._handle, B, kv, lens, st, nz, int(n_steps), _ptr(out), _stream_ptr(stream)))
         return out
 
     def poll_status(self) -> int:

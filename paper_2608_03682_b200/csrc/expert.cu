@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/phyai.h"
+#include "host_pack.h"
 #include "kernels.h"
 
 using namespace phyai;
@@ -140,6 +141,12 @@ struct phyai_expert {
   void* stg_kv = nullptr; size_t stg_kv_bytes = 0;
   float *stg_states = nullptr, *stg_noise = nullptr, *stg_out = nullptr;
   int* stg_cu = nullptr;
+
+  // requests in ordinary host memory: page-locked staging (grown on demand, freed with the handle) and the gather threads
+  void* pin_kv = nullptr; size_t pin_kv_bytes = 0;
+  float* pin_small = nullptr;            // cu | states | noise of max_batch requests
+  cudaEvent_t pin_free = nullptr;        // the last call's copies out of the staging have completed
+  phyai::HostPacker* packer = nullptr;
 
   int use_graph = 1;
   unsigned wait_limit = 1u << 22;
@@ -1249,6 +1256,10 @@ void phyai_expert_destroy(phyai_expert_t* h) {
   cudaDeviceSynchronize();
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+  delete h->packer;
+  if (h->pin_kv) cudaFreeHost(h->pin_kv);
+  if (h->pin_small) cudaFreeHost(h->pin_small);
+  if (h->pin_free) cudaEventDestroy(h->pin_free);
   for (void* p : h->allocs) cudaFree(p);
   delete h;
 }
@@ -1314,6 +1325,80 @@ phyai_status_t phyai_denoise_batched_host(phyai_expert_t* h, uint32_t batch, con
   r.noise = h->stg_noise, r.x = h->stg_out, r.batch = (int)batch, r.single_len = 0;
   ST(run(h, r, (int)n_steps, st));
   CU(cudaMemcpyAsync(out, h->stg_out, ha, cudaMemcpyDeviceToHost, st));
+  return PHYAI_OK;
+}
+
+phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, const void* const* prefix_kvs,
+                                           const uint32_t* prefix_lens, const float* const* states, const float* const* noises,
+                                           uint32_t n_steps, float* out, void* stream) {
+  if (!h) return fail(PHYAI_ERR_INVALID_ARG, "handle is NULL");
+  if (batch == 0 || batch > h->cfg.max_batch)
+    return fail(PHYAI_ERR_INVALID_ARG, "batch %u outside 1..max_batch (%u)", batch, h->cfg.max_batch);
+  if (!prefix_kvs || !prefix_lens || !noises || !out || (h->cfg.has_state_token && !states))
+    return fail(PHYAI_ERR_INVALID_ARG, "prefix_kvs / prefix_lens / noises / out_actions (or states) is NULL");
+  if (n_steps == 0 || n_steps > 1000) return fail(PHYAI_ERR_INVALID_ARG, "n_steps must be in 1..1000");
+  size_t total = 0;
+  for (uint32_t b = 0; b < batch; ++b) {
+    if (prefix_lens[b] > h->cfg.max_prefix_len) return fail(PHYAI_ERR_INVALID_ARG, "prefix_lens[%u] exceeds max_prefix_len", b);
+    if (prefix_lens[b] && !prefix_kvs[b]) return fail(PHYAI_ERR_INVALID_ARG, "prefix_kvs[%u] is NULL", b);
+    total += prefix_lens[b];
+  }
+  ST(ensure_staging(h));
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const size_t B = h->cfg.max_batch, ha = (size_t)h->d.H * h->d.A, Ds = h->d.Ds;
+  const size_t kvb = phyai_prefix_kv_bytes(&h->cfg, total);
+  if (!h->pin_free) CU(cudaEventCreateWithFlags(&h->pin_free, cudaEventDisableTiming));
+  if (!h->pin_small) CU(cudaHostAlloc(reinterpret_cast<void**>(&h->pin_small), (B + 1 + B * Ds + B * ha) * 4, cudaHostAllocDefault));
+  CU(cudaEventSynchronize(h->pin_free));         // the last call's copies (complete unless that call is still in flight)
+  if (kvb > h->pin_kv_bytes) {
+    if (h->pin_kv) CU(cudaFreeHost(h->pin_kv));
+    h->pin_kv = nullptr, h->pin_kv_bytes = 0;
+    const size_t want = std::min(kvb + kvb / 4, h->stg_kv_bytes);
+    CU(cudaHostAlloc(&h->pin_kv, want, cudaHostAllocDefault));
+    h->pin_kv_bytes = want;
+  }
+  const int planes = 2 * h->d.L;
+  const size_t plane = kvb / planes;
+  if (kvb) {
+    if (!h->packer) h->packer = new (std::nothrow) phyai::HostPacker();
+    if (!h->packer) return fail(PHYAI_ERR_OOM, "host allocation failed");
+    h->packer->start(static_cast<uint8_t*>(h->pin_kv), prefix_kvs, prefix_lens, (int)batch, planes, plane / total);
+  }
+  int32_t* cu = reinterpret_cast<int32_t*>(h->pin_small);
+  float *ps = h->pin_small + B + 1, *pn = ps + B * Ds;
+  cu[0] = 0;
+  for (uint32_t b = 0; b < batch; ++b) {
+    cu[b + 1] = cu[b] + (int32_t)prefix_lens[b];
+    if (h->cfg.has_state_token) {
+      if (states[b]) memcpy(ps + b * Ds, states[b], Ds * 4);
+      else memset(ps + b * Ds, 0, Ds * 4);
+    }
+    if (noises[b]) memcpy(pn + b * ha, noises[b], ha * 4);
+    else memset(pn + b * ha, 0, ha * 4);
+  }
+  phyai_status_t s = [&]() -> phyai_status_t {
+    CU(cudaMemcpyAsync(h->stg_cu, cu, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, st));
+    if (h->cfg.has_state_token) CU(cudaMemcpyAsync(h->stg_states, ps, batch * Ds * 4, cudaMemcpyHostToDevice, st));
+    CU(cudaMemcpyAsync(h->stg_noise, pn, batch * ha * 4, cudaMemcpyHostToDevice, st));
+    // several copies: the engine works on the first planes while the rest is gathered
+    const int pieces = std::min(planes, 12);
+    for (int q = 0; kvb && q < pieces; ++q) {
+      const int p0 = planes * q / pieces, p1 = planes * (q + 1) / pieces;
+      if (p1 == p0) continue;
+      h->packer->wait(p1);
+      CU(cudaMemcpyAsync(static_cast<uint8_t*>(h->stg_kv) + p0 * plane, static_cast<uint8_t*>(h->pin_kv) + p0 * plane, (p1 - p0) * plane,
+                         cudaMemcpyHostToDevice, st));
+    }
+    CU(cudaEventRecord(h->pin_free, st));
+    return PHYAI_OK;
+  }();
+  if (kvb) h->packer->wait(planes);              // (the caller's memory is not read after this call returns)
+  ST(s);
+  Request r{};
+  r.prefix_kv = h->stg_kv, r.kv_tokens = total, r.cu_lens = h->stg_cu, r.states = h->cfg.has_state_token ? h->stg_states : nullptr;
+  r.noise = h->stg_noise, r.x = h->stg_out, r.batch = (int)batch, r.single_len = 0;
+  ST(run(h, r, (int)n_steps, st));
+  CU(cudaMemcpyAsync(out, h->stg_out, batch * ha * 4, cudaMemcpyDeviceToHost, st));
   return PHYAI_OK;
 }
 

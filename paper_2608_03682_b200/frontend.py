@@ -36,25 +36,16 @@ class ExpertWorker:
         if self.stream is None:
             self.stream = torch.cuda.Stream(device=self.device)
         kv_dtype = torch.float32 if cfg.dtype == "f32" else torch.bfloat16
-        empty = torch.zeros(cfg.n_layers, 2, 0, cfg.n_kv_heads, cfg.head_dim, dtype=kv_dtype)
-        kvs = [empty if r is None else r["prefix_kv"] for r in requests]
-        cu = np.zeros(len(requests) + 1, dtype=np.int32)
-        cu[1:] = np.cumsum([kv.shape[2] for kv in kvs])
-        packed = torch.cat(kvs, dim=2).contiguous()
-        if packed.shape[2] == 0:                       # an all-padding batch still needs a valid (non-null) buffer
-            packed = torch.zeros(cfg.n_layers, 2, 1, cfg.n_kv_heads, cfg.head_dim, dtype=kv_dtype)
-        noise = torch.stack([torch.zeros(cfg.horizon, cfg.action_dim) if r is None else r["noise"] for r in requests])
-        states = None
-        if cfg.has_state_token:
-            states = torch.stack([torch.zeros(cfg.state_dim) if r is None else r["state"] for r in requests])
-        host = [packed.pin_memory(), torch.from_numpy(cu).pin_memory(), None if states is None else states.pin_memory(),
-                noise.pin_memory()]
+        host = lambda t, dtype: None if t is None else t.to(device="cpu", dtype=dtype).contiguous()   # (no copy in the usual case)
+        reqs = [(None, None, None) if r is None else
+                (host(r["prefix_kv"], kv_dtype), host(r["state"], torch.float32) if cfg.has_state_token else None,
+                 host(r["noise"], torch.float32)) for r in requests]
+        out = torch.empty(len(reqs), cfg.horizon, cfg.action_dim, pin_memory=True)
         with torch.cuda.stream(self.stream):
-            dev = [None if t is None else t.to(self.device, non_blocking=True) for t in host]
-            out = self.ex.denoise_batched(dev[0], dev[1], dev[2], dev[3], self.n_steps, stream=self.stream)
+            self.ex.denoise_requests_host(reqs, self.n_steps, out, stream=self.stream)
             done = torch.cuda.Event()
             done.record(self.stream)
-        return {"out": out, "done": done, "keep": (host, dev)}
+        return {"out": out, "done": done}
 
     def collect(self, pending) -> List[np.ndarray]:
         """Wait for a launched batch and return its action chunks."""
@@ -62,7 +53,7 @@ class ExpertWorker:
         status = self.ex.poll_status()
         if status != 0:
             raise RuntimeError(f"device status {status}")
-        return [o.cpu().numpy() for o in pending["out"]]
+        return list(pending["out"].numpy().copy())
 
     def __call__(self, requests: List[Optional[dict]]) -> List[np.ndarray]:
         return self.collect(self.launch(requests))
