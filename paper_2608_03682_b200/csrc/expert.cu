@@ -115,7 +115,7 @@ struct phyai_expert {
   int use_pair_gemm = 1, use_pair_attention = 1;
   int pair_ranges = 0;         // key ranges of the pair attention kernel (0 = choose)
   __nv_bfloat16* q_tiles_pair = nullptr;   // q as operand tiles [max_batch][Hq / 2][128 rows][dh] for the pair / cluster attention
-  float *ss_ta = nullptr, *ss_tb = nullptr;   // their [D/128][Mpad] partial sums of squares of h (after O / after down)
+  float *ss_ta = nullptr, *ss_tb = nullptr;   // their [D/64][Mpad] partial sums of squares of h (after O / after down)
   __nv_bfloat16 *pq_all = nullptr, *po_all = nullptr, *pd_all = nullptr;   // bases of the packed images of all layers
   float *s_qkv_all = nullptr, *s_o_all = nullptr, *s_g_all = nullptr, *s_u_all = nullptr, *s_d_all = nullptr;
   __nv_bfloat16 *xn64 = nullptr, *attn64 = nullptr, *m64 = nullptr, *u64 = nullptr;
@@ -480,11 +480,12 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   // More than one 64-token tile: every projection on the CTA-pair GEMM, the norms folded in as on the cluster path (QKV,
   // attention, O, gate/up, down: five kernels per layer).
   const bool pair = h->pair_ok && h->use_pair_gemm && h->use_cluster_gemm && h->use_persistent_gu && h->use_persistent_qkv && M > 64;
+  int busy = 0;      // SMs that the kernel launched last occupies
   auto pair_gemm = [&](PairGemm g) -> phyai_status_t {
-    g.rows_pad = h->Mpad, g.M = M, g.ss_n = ss_n, g.inv_D = 1.0f / (float)D, g.eps = d.eps, g.gelu_exact = d.gelu_exact;
+    g.rows_pad = h->Mpad, g.M = M, g.ss_n = D / 64, g.inv_D = 1.0f / (float)D, g.eps = d.eps, g.gelu_exact = d.gelu_exact;
     g.wait_limit = h->wait_limit;
     g.trace = (h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from) ? h->trace : nullptr;
-    cudaError_t e = launch_pair_gemm(h->status, g, h->n_sm, st);
+    cudaError_t e = launch_pair_gemm(h->status, g, h->n_sm, &busy, st);
     if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "pair GEMM launch failed: %s", cudaGetErrorString(e));
     ++cnt;
     return PHYAI_OK;
@@ -500,12 +501,14 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
       e = launch_attention_pair(h->rq, h->status, h->q_tiles_pair, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch,
                                 pr_ranges, h->order, h->wait_limit, st,
                                 tr1 ? h->trace : nullptr);
+      busy = std::min(h->n_sm, 2 * pr_ranges * (d.Hq / 4) * batch);
       ++cnt;
     } else if (h->use_tc_attention && attention_tc_supported(d) && batch * (d.Hq / 2) >= ATTN_TC_MIN_CTAS) {
       const int tsp = (h->use_attn_splits && h->attn_scratch) ? attention_tc_splits(d, batch, h->n_sm, (int)h->cfg.max_prefix_len) : 1;
       const bool tr = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from && batch * (d.Hq / 2) * tsp <= TRACE_SLOTS;
       e = launch_attention_tc(h->rq, h->status, h->qr_big, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch, h->order,
                               h->wait_limit, st, tr ? h->trace : nullptr, tsp, h->attn_scratch);
+      busy = tsp > 1 ? 0 : std::min(h->n_sm, batch * (d.Hq / 2));
       cnt += tsp > 1 ? 2 : 1;
     } else if (h->use_cluster_attention && batch * d.Hq * 8 <= 2 * h->n_sm) {
       e = launch_attention_cluster(h->rq, h->status, nullptr, h->rope, h->qr_big, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch,
@@ -1220,8 +1223,8 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
         }
       }
       if (h->pair_ok) {
-        ST(h->alloc(&h->ss_ta, (size_t)(D / 128) * Mp, true));
-        ST(h->alloc(&h->ss_tb, (size_t)(D / 128) * Mp, true));
+        ST(h->alloc(&h->ss_ta, (size_t)(D / 64) * Mp, true));
+        ST(h->alloc(&h->ss_tb, (size_t)(D / 64) * Mp, true));
         if (attention_pair_supported(d)) ST(h->alloc(&h->q_tiles_pair, (size_t)cfg->max_batch * (d.Hq / 2) * 128 * d.dh, true));
       }
       ST(h->alloc(&h->xn_t, Mp * D, true));

@@ -37,8 +37,9 @@ constexpr int PG_EPI = 512, PG_THREADS = (PG_PROD + 1) * 32 + PG_EPI;
 // tokens an epilogue warp takes at a time: 16 for the rotary epilogue, which then has the registers to hold the (cos, sin)
 // of the next two blocks (one 32-token block ahead on 8 warps: 7 us per tile, bound by the table's latency), else 32
 template <int EPI> constexpr int PG_TB = EPI == PG_QKV ? 16 : 32;
-constexpr int PG_MAXST = 12;
-constexpr int PG_A_BYTES = 128 * 128;             // one CTA's weight block: 128 rows x 64 k
+constexpr int PG_MAXST = 20;
+// one CTA's weight block: 128 rows x 64 k; 64 rows in the half-height form (residual projections of few tokens)
+template <bool HALF> constexpr int PG_A_BYTES = (HALF ? 64 : 128) * 128;
 constexpr int BAR_EPI = 1;
 constexpr int PG_PITCH = 36, PG_STG = 16 * PG_PITCH;      // staging block of an epilogue warp: [16 tokens][32 rows + 4] floats
 constexpr size_t PG_STG_BYTES = (size_t)16 * PG_STG * 4;
@@ -112,10 +113,13 @@ __device__ __forceinline__ void stmatrix4_t(uint32_t addr, uint32_t r0, uint32_t
   asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
 }
 
-template <int EPI>
+// CPS: k-chunks of 64 per ring stage.  A stage costs the MMA issuer a wait and a commit on top of the chunks' copies; with few
+// tokens per tile that, not bytes or tensor time, set the pace (290 clocks per chunk whatever its size; with four chunks per
+// stage 165, the ingest of the SM: down projection of 204 tokens 9.9 -> 5.6 us).
+template <int EPI, bool HALF, int CPS>
 __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
     k_gemm_pair(int* status, const PairGemm g, const __grid_constant__ CUtensorMap tmw, const __grid_constant__ CUtensorMap tmx) {
-  constexpr int EPIW = PG_EPI / 32, TB = PG_TB<EPI>, K8 = TB / 8;
+  constexpr int EPIW = PG_EPI / 32, TB = PG_TB<EPI>, K8 = TB / 8, A_BYTES = PG_A_BYTES<HALF>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_full[PG_MAXST];    // leader: both CTAs' operands of a stage have landed
   __shared__ __align__(8) uint64_t bar_empty[PG_MAXST];   // each CTA: the MMAs have read the stage
@@ -130,16 +134,20 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
-  const int KC = g.K >> 6, NT = g.NT, ST = g.stages;
-  const int n_n = g.N >> 8;                               // tiles of 256 channels
+  const int KC = g.K >> 6, NT = g.NT, ST = g.stages, KS = KC / CPS;   // CPS k-chunks per stage, KS stages per tile
+  const int n_n = HALF ? g.N >> 7 : g.N >> 8;             // tiles of 256 (128) channels
   const int n_tiles = n_n * ((g.M + NT - 1) / NT);
   const int n_my = pair < n_tiles ? (n_tiles - pair + n_pairs - 1) / n_pairs : 0;
-  const int steps = n_my * KC;
-  const uint32_t stage_bytes = (uint32_t)(PG_A_BYTES + NT * 64);
+  const int steps = n_my * KS;
+  const uint32_t chunk_bytes = (uint32_t)(A_BYTES + NT * 64), stage_bytes = chunk_bytes * (uint32_t)CPS;
 
   pdl_launch_dependents();
   unsigned long long* const trc = g.trace ? g.trace + (size_t)blockIdx.x * 16 : nullptr;
   if (threadIdx.x == 0) trace_stamp(trc, 0);
+  if (threadIdx.x == 32) {      // (the first copy would otherwise wait for its map)
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmw)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
+  }
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -169,15 +177,16 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
     // ---------------- copy issuers -------------------------------------------------------------------------------
     if (lane == 0) {
       auto load_w = [&](int gi, int s) {
-        const int ct = ((pair + (gi / KC) * n_pairs) % n_n) * 2 + rank;      // this CTA's 128-row weight tile
+        const int ct = ((pair + (gi / KS) * n_pairs) % n_n) * 2 + rank, kc = (gi % KS) * CPS;      // this CTA's 128-row (64-row) weight tile
         const uint32_t full = smem_u32(&bar_full[s]);
         if (rank == 0) mbar_expect_tx(full, 2 * stage_bytes);
-        tma2d(tiles + (uint32_t)s * stage_bytes, &tmw, g.w_row0 + (ct * KC + gi % KC) * 128, full & LEADER_MASK);
+        const int row = g.w_row0 + (HALF ? ((ct >> 1) * KC + kc) * 128 + rank * 64 : (ct * KC + kc) * 128);
+        for (int c = 0; c < CPS; ++c) tma2d(tiles + (uint32_t)s * stage_bytes + (uint32_t)c * chunk_bytes, &tmw, row + c * 128, full & LEADER_MASK);
       };
       auto load_x = [&](int gi, int s) {
-        const int tt = (pair + (gi / KC) * n_pairs) / n_n;
-        tma2d(tiles + (uint32_t)s * stage_bytes + PG_A_BYTES, &tmx, (gi % KC) * g.rows_pad + tt * NT + rank * (NT >> 1),
-              smem_u32(&bar_full[s]) & LEADER_MASK);
+        const int row = (gi % KS) * CPS * g.rows_pad + (pair + (gi / KS) * n_pairs) / n_n * NT + rank * (NT >> 1);
+        for (int c = 0; c < CPS; ++c)
+          tma2d(tiles + (uint32_t)s * stage_bytes + (uint32_t)c * chunk_bytes + A_BYTES, &tmx, row + c * g.rows_pad, smem_u32(&bar_full[s]) & LEADER_MASK);
       };
       // Programmatic dependent launch: the weight blocks of the first stages are on their way before the kernel that
       // produces the activations has finished.
@@ -200,7 +209,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
   } else if (warp == PG_PROD) {
     // ---------------- MMA issuer (whole warp in the loop, one elected lane issues) --------------------------------
     if (rank == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((256u >> 4) << 24);
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((HALF ? 128u : 256u) >> 4) << 24;
       int s = 0, gi = 0;
       uint32_t ph = 0;
       bool dead = false;
@@ -210,17 +219,20 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
         if (mbar_wait_drain(smem_u32(&bar_tempty[buf]), (((uint32_t)i >> 1) & 1u) ^ 1u, wc) < 0) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + (uint32_t)buf * 256u;
-        for (int k = 0; k < KC; ++k, ++gi) {
+        for (int k = 0; k < KS; ++k, ++gi) {
           if (mbar_wait_drain(smem_u32(&bar_full[s]), ph, wc) < 0) {
             dead = true;   // (copies that never landed: nothing more can be done with this pipeline)
             break;
           }
           if (gi == 0 && lane == 0) trace_stamp(trc, 3);
-          const uint32_t a0 = tiles + (uint32_t)s * stage_bytes;
-          const uint64_t da = make_desc(a0), db = make_desc(a0 + PG_A_BYTES);
+          uint32_t a0 = tiles + (uint32_t)s * stage_bytes;
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            if (elect_one()) umma2_bf16(tacc, da + 2 * kk, db + 2 * kk, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+          for (int c = 0; c < CPS; ++c, a0 += chunk_bytes) {
+            const uint64_t da = make_desc(a0), db = make_desc(a0 + A_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              if (elect_one()) umma2_bf16(tacc, da + 2 * kk, db + 2 * kk, idesc, (k > 0 || c > 0 || kk > 0) ? 1u : 0u);
+          }
           if (elect_one()) umma2_commit(smem_u32(&bar_empty[s]));
           __syncwarp();
           if (++s == ST) s = 0, ph ^= 1u;
@@ -250,7 +262,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       const int buf = i & 1;
       const int t = pair + i * n_pairs;
       const int ct = (t % n_n) * 2 + rank, tok_base = (t / n_n) * NT;      // this CTA's 128 channels; first token
-      const int n_tok = min(NT, g.M - tok_base), n0 = ct * 128;
+      const int n_tok = min(NT, g.M - tok_base), n0 = ct * (HALF ? 64 : 128);
+      // half height: 64 rows, the second half of the token columns in lanes 64..127
+      const int th = HALF ? (q >> 1) * (NT >> 1) : 0, tl_end = HALF ? min(n_tok, th + (NT >> 1)) : n_tok;
       // ---- before the accumulator is complete: per-token and per-channel factors
       if (EPI == PG_GEGLU || EPI == PG_QKV) {
         if (et < NT) {      // (NT <= 256 <= threads of the epilogue)
@@ -286,8 +300,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
           sc[gr][e & 1] *= osc;
         }
       } else if constexpr (EPI == PG_RESID) {
-        if (g.scale) scr = g.scale[n0 + q * 32 + lane];
-        if (g.gate) scr *= g.gate[n0 + q * 32 + lane];
+        const int n = n0 + (HALF ? q & 1 : q) * 32 + lane;
+        if (g.scale) scr = g.scale[n];
+        if (g.gate) scr *= g.gate[n];
       }
       // where a lane's 16-byte pieces go: tokens lane / 2 and + 16 of a 32-token block, channels 8 (lane & 1) .. of a group
       const int p8 = 16 * q + 8 * (lane & 1);
@@ -315,7 +330,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       }
       // RESID: in the transposed view a lane takes 4 channels of tokens lane / 8, + 4, + 8, + 12 of the chunk; what is added
       // to (the residual stream, or the MLP's bias / the state token) is requested one chunk ahead
-      const int n4 = n0 + q * 32 + (lane & 7) * 4;
+      const int n4 = n0 + (HALF ? q & 1 : q) * 32 + (lane & 7) * 4;
       float4 old[2][4], gain4 = make_float4(0.f, 0.f, 0.f, 0.f);
       auto fetch_old = [&](int c0, float4* o) {
 #pragma unroll
@@ -328,8 +343,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       };
       if constexpr (EPI == PG_RESID) {
         if (g.gain_next) gain4 = __ldg(reinterpret_cast<const float4*>(g.gain_next + n4));
-        if (cg * 16 < n_tok) fetch_old(cg * 16, old[0]);
-        if (cg * 16 + 64 < n_tok) fetch_old(cg * 16 + 64, old[1]);
+        if (th + cg * 16 < tl_end) fetch_old(th + cg * 16, old[0]);
+        if (th + cg * 16 + 64 < tl_end) fetch_old(th + cg * 16 + 64, old[1]);
       }
       // q / k: (cos, sin) of this lane's rotary pairs at its tokens, two 16-token blocks ahead
       float2 cs[2][EPI == PG_QKV ? 8 : 1];
@@ -360,9 +375,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
         // 16 token columns at a time: the lane that holds a row scales it and puts it into the warp's staging block [16
         // tokens][32 rows + 4]; then 8 lanes take the 32 channels (128 bytes of h) of one token
 #pragma unroll 1
-        for (int c0 = cg * 16; c0 < n_tok; c0 += 64) {
+        for (int c0 = th + cg * 16; c0 < tl_end; c0 += 64) {
           float v[16];
-          tmem_ld16(tl_addr + (uint32_t)(buf * 256 + c0), v);
+          tmem_ld16(tl_addr + (uint32_t)(buf * 256 + c0 - th), v);
 #pragma unroll
           for (int j = 0; j < 16; ++j) stg[j * PG_PITCH + lane] = v[j] * scr;
           __syncwarp();
@@ -374,7 +389,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
             const bool live = !(g.bias && (tok % g.S) < g.ns);       // (state rows do not pass through the MLP)
             float4 hv = old[0][u];
             if (live) hv.x += a.x, hv.y += a.y, hv.z += a.z, hv.w += a.w;
-            if (ok && tl < n_tok) {
+            if (ok && tl < tl_end) {
               *reinterpret_cast<float4*>(g.h + (size_t)tok * g.N + n4) = hv;
               if (g.gain_next)
                 *reinterpret_cast<uint2*>(g.out + tiled_index(tok, n4, g.rows_pad)) =
@@ -383,11 +398,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
             float s2 = hv.x * hv.x + hv.y * hv.y + hv.z * hv.z + hv.w * hv.w;
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-            if ((lane & 7) == 0) ss_tab[q][tl] = s2;
+            if ((lane & 7) == 0 && tl < tl_end) ss_tab[q][tl] = s2;
           }
 #pragma unroll
           for (int u = 0; u < 4; ++u) old[0][u] = old[1][u];
-          if (c0 + 128 < n_tok) fetch_old(c0 + 128, old[1]);
+          if (c0 + 128 < tl_end) fetch_old(c0 + 128, old[1]);
           __syncwarp();
         }
       } else {
@@ -470,8 +485,12 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       if constexpr (EPI == PG_RESID) {
         if (g.ss_out) {
           asm volatile("bar.sync %0, %1;" ::"n"(BAR_EPI + 1), "n"(PG_EPI) : "memory");
-          if (ok && et < n_tok)
-            g.ss_out[(size_t)ct * g.rows_pad + tok_base + et] = (ss_tab[0][et] + ss_tab[1][et]) + (ss_tab[2][et] + ss_tab[3][et]);
+          if (ok && et < n_tok) {     // one partial sum per 64 channels and token
+            float* so = g.ss_out + tok_base + et;
+            const int q0 = HALF && et >= (NT >> 1) ? 2 : 0;
+            so[(size_t)(HALF ? ct : 2 * ct) * g.rows_pad] = ss_tab[q0][et] + ss_tab[q0 + 1][et];
+            if (!HALF) so[(size_t)(2 * ct + 1) * g.rows_pad] = ss_tab[2][et] + ss_tab[3][et];
+          }
         }
       }
     }
@@ -509,48 +528,73 @@ bool row_map(CUtensorMap* m, const void* base, uint64_t rows, uint32_t box) {
              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int EPI>
-cudaError_t launch_one(int* status, const PairGemm& g, int grid, size_t smem, const CUtensorMap& tw, const CUtensorMap& tx, cudaStream_t st) {
+template <int EPI, bool HALF, int CPS>
+cudaError_t launch_cps(int* status, const PairGemm& g, int grid, size_t smem, const CUtensorMap& tw, const CUtensorMap& tx, cudaStream_t st) {
   static PerDeviceOnce once;
   if (once.needed()) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_MAX);
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_pair<EPI, HALF, CPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM_MAX);
     if (e != cudaSuccess) return e;
     once.done();
   }
-  return launch_pdl(k_gemm_pair<EPI>, dim3(grid), dim3(PG_THREADS), smem, st, status, g, tw, tx);
+  return launch_pdl(k_gemm_pair<EPI, HALF, CPS>, dim3(grid), dim3(PG_THREADS), smem, st, status, g, tw, tx);
+}
+
+template <int EPI, bool HALF = false>
+cudaError_t launch_one(int* status, const PairGemm& g, int grid, size_t smem, const CUtensorMap& tw, const CUtensorMap& tx, cudaStream_t st) {
+  if (g.cps == 4) return launch_cps<EPI, HALF, 4>(status, g, grid, smem, tw, tx, st);
+  if (g.cps == 2) return launch_cps<EPI, HALF, 2>(status, g, grid, smem, tw, tx, st);
+  return launch_cps<EPI, HALF, 1>(status, g, grid, smem, tw, tx, st);
 }
 
 }  // namespace
 
 bool pair_gemm_supported(int N, int K) { return N % 256 == 0 && K % 64 == 0 && K > 0; }
 
-// Token-tile width: the one with the least work on the busiest pair.  A k-chunk of a tile costs the larger of the tensor
-// time (2 NT clocks: four MMAs of NT / 2) and the ingest of an SM (16 KB of weights + 64 NT bytes of activations at 62
-// bytes per clock); the last tile's epilogue is exposed (about 14 clocks per token column).
-int pair_gemm_pick_nt(int M, int N, int K, int n_sm) {
+// Tile of a projection: the token width and, for residual projections, the height (256 or 128 channels per pair) with the
+// least work on the busiest pair, in clocks.  A k-chunk of a tile costs the larger of the tensor time (2 NT: four MMAs of
+// NT / 2) and the ingest of an SM (16 or 8 KB of weights + 64 NT bytes of activations at 62 bytes per clock); the last tile's
+// epilogue is exposed (30 - 60 per token column).  A grid that does not fit beside the kernel before it (`busy` CTAs, one per
+// SM) has CTAs that start only when that one ends, and then pay their set-up and the first weights' latency: about 3600
+// (measured: 1.9 us).  The half-height tile: few tokens against a long contraction leave 40 - 60 pairs whose SMs are bound
+// by the 16 KB of weights per chunk (down projection at 408 tokens: 10.2 us of main loop, 6.2 at half height).
+struct PairTile {
+  int nt;
+  bool half;
+};
+PairTile pick_tile(const PairGemm& g, int n_sm, int busy) {
   double best = 1e30;
-  int nt_best = 256;
-  for (int nt = 256; nt >= 32; nt -= 32) {
-    const int tiles = (N / 256) * ((M + nt - 1) / nt), pairs = n_sm / 2;
-    const double chunk = std::max(2.0 * nt, (PG_A_BYTES + 64.0 * nt) / 62.0);
-    const double cost = (double)((tiles + pairs - 1) / pairs) * (K / 64) * chunk + 14.0 * nt;
-    if (cost < best * 0.999) best = cost, nt_best = nt;
-  }
-  return nt_best;
+  PairTile t{256, false};
+  for (int half = 0; half <= (g.epi == PG_RESID ? 1 : 0); ++half)
+    for (int nt = 256; nt >= 32; nt -= 16) {
+      const int tiles = g.N / (half ? 128 : 256) * ((g.M + nt - 1) / nt), pairs = n_sm / 2;
+      const double chunk = std::max(2.0 * nt, ((half ? PG_A_BYTES<true> : PG_A_BYTES<false>) + 64.0 * nt) / 62.0);
+      const double epi = g.epi != PG_RESID ? 30.0 : half ? 30.0 : 60.0;
+      const double cost = (double)((tiles + pairs - 1) / pairs) * (g.K / 64) * chunk + epi * nt + (2 * std::min(tiles, pairs) + busy > n_sm ? 3600.0 : 0.0);
+      if (cost < best * 0.999) best = cost, t = PairTile{nt, half != 0};
+    }
+  return t;
 }
 
-cudaError_t launch_pair_gemm(int* status, const PairGemm& g_in, int n_sm, cudaStream_t st) {
+cudaError_t launch_pair_gemm(int* status, const PairGemm& g_in, int n_sm, int* busy, cudaStream_t st) {
   PairGemm g = g_in;
   if (!pair_gemm_supported(g.N, g.K) || g.M < 1) return cudaErrorInvalidValue;
-  if (g.NT <= 0) g.NT = pair_gemm_pick_nt(g.M, g.N, g.K, n_sm);
-  const size_t stage = (size_t)PG_A_BYTES + 64 * g.NT;
-  g.stages = (int)std::min<size_t>((PG_SMEM_MAX - 1024 - PG_STG_BYTES) / stage, PG_MAXST);
+  const PairTile t = pick_tile(g, n_sm, *busy);
+  g.NT = t.nt;
+  const size_t chunk = (size_t)(t.half ? PG_A_BYTES<true> : PG_A_BYTES<false>) + 64 * g.NT, ring = PG_SMEM_MAX - 1024 - PG_STG_BYTES;
+  // As many chunks per stage as leave a stage to each copy issuer (PG_PROD: with fewer, two issuers would meet in one stage
+  // and its parity could not tell their turns apart).
+  g.cps = 1;
+  while (g.cps < 4 && (g.K / 64) % (2 * g.cps) == 0 && 2 * g.cps * PG_PROD * chunk <= ring) g.cps *= 2;
+  const size_t stage = g.cps * chunk;
+  g.stages = (int)std::min<size_t>(ring / stage, PG_MAXST);
   CUtensorMap tw, tx;
-  if (!row_map(&tw, g.W, g.w_rows, 128) || !row_map(&tx, g.X, (uint64_t)(g.K / 64) * g.rows_pad, (uint32_t)(g.NT / 2)))
+  if (!row_map(&tw, g.W, g.w_rows, t.half ? 64 : 128) || !row_map(&tx, g.X, (uint64_t)(g.K / 64) * g.rows_pad, (uint32_t)(g.NT / 2)))
     return cudaErrorInvalidValue;
-  const int n_tiles = (g.N / 256) * ((g.M + g.NT - 1) / g.NT);
+  const int n_tiles = g.N / (t.half ? 128 : 256) * ((g.M + g.NT - 1) / g.NT);
   const int grid = 2 * std::min(n_tiles, n_sm / 2);
+  *busy = grid;
   const size_t smem = (size_t)g.stages * stage + 1024 + PG_STG_BYTES;
+  if (t.half) return launch_one<PG_RESID, true>(status, g, grid, smem, tw, tx, st);
   switch (g.epi) {
     case PG_QKV: return launch_one<PG_QKV>(status, g, grid, smem, tw, tx, st);
     case PG_GEGLU: return launch_one<PG_GEGLU>(status, g, grid, smem, tw, tx, st);

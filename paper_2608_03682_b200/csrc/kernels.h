@@ -110,7 +110,7 @@ void launch_embed_pi0(const Request* rq, const int* status, const float* Wc, con
 void launch_embed_pi05(const Request* rq, const int* status, const float* Wa, const float* ba, const float* state_tok,
                        float* h, const Dims& d, int batch, cudaStream_t st);
 // Embedding ahead of the pair GEMMs: gain null (pi0): u = swish(x Wc + bias) -> tiled bf16 `out` at token rows; gain set
-// (pi0.5): h = x Wc + bias (state rows: state_tok), out = bf16(h * gain), ss_out [D/128][rows_pad] partial sums of squares.
+// (pi0.5): h = x Wc + bias (state rows: state_tok), out = bf16(h * gain), ss_out [D/64][rows_pad] partial sums of squares.
 // D a multiple of 128.
 void launch_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias, const float* state_tok,
                          const float* gain, float* h, __nv_bfloat16* out, float* ss_out, int rows_pad, const Dims& d, int batch,
@@ -297,8 +297,8 @@ struct PairGemm {
   int w_row0;                // first row of this matrix in it
   const __nv_bfloat16* X;    // tiled activations [K/64][rows_pad][64]
   int rows_pad, M, N, K;
-  int NT;                    // token-tile width: a multiple of 32 up to 256, 0 = choose
-  int stages;                // (set by the launcher)
+  int NT, stages, cps;       // (set by the launcher) token-tile width: a multiple of 16 from 32 to 256; ring depth; k-chunks of
+                             // a ring stage
   int epi;
   const float* scale;        // per packed row weight scale or null (GEGLU: per gate channel; scale2: per up channel; QKV:
   const float* scale2;       // un-interleaved packed order)
@@ -311,7 +311,7 @@ struct PairGemm {
   __nv_bfloat16* out;        // GEGLU: tiled [N/128][rows_pad][64] (W rows interleaved as for PersistGemm, gate / up);
                              // RESID: tiled [N/64][rows_pad][64] bf16(h * gain_next), or unused; PLANES: [L][2][plane_rows][nkv]
   // RESID: h[token][n] += gate[n] * scale[n] * acc (row stride N); with gain_next the operands of the norm that follows:
-  // `out` and ss_out[N/128][rows_pad].  With `bias` (second layer of the action MLP): h = bias + acc for action rows, the
+  // `out` and ss_out[N/64][rows_pad].  With `bias` (second layer of the action MLP): h = bias + acc for action rows, the
   // state token's embedding for the first ns of every request's S rows.
   float* h;
   const float* gate;
@@ -334,8 +334,8 @@ struct PairGemm {
   unsigned long long* trace; // or null: CTA b stamps slot b (16 words)
 };
 bool pair_gemm_supported(int N, int K);
-int pair_gemm_pick_nt(int M, int N, int K, int n_sm);
-cudaError_t launch_pair_gemm(int* status, const PairGemm& g, int n_sm, cudaStream_t st);
+// busy: CTAs (one per SM) of the kernel before this one; receives this one's
+cudaError_t launch_pair_gemm(int* status, const PairGemm& g, int n_sm, int* busy, cudaStream_t st);
 // ---- cluster split-K GEMM for a single 64-token tile (gemm_b1.cu) --------------------------------------------
 enum : int { B1_QKV = 0, B1_GEGLU = 1, B1_RESID = 2 };
 struct B1Gemm {

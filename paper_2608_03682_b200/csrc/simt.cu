@@ -524,7 +524,7 @@ void launch_embed_pi05(const Request* rq, const int* status, const float* Wa, co
 // Suffix embedding ahead of the pair GEMMs (norms folded in): one block takes ER action rows, a thread four consecutive
 // channels of all of them.  ADA = false (pi0): u = swish(x Wc + tb) -> bf16 operand of the MLP's second layer, at token
 // rows (the state rows' operand is never used).  ADA = true (pi0.5): h = x Wa + ba (state rows: the state token), the first
-// norm's operand bf16(h * gain) and, per 128 channels (one warp), the row's partial sum of squares.  ER = 4 keeps small
+// norm's operand bf16(h * gain) and, per 64 channels (half a warp), the row's partial sum of squares.  ER = 4 keeps small
 // calls on many SMs, ER = 16 reads Wc once per 16 rows.
 template <int ER, bool ADA>
 __global__ void __launch_bounds__(256) k_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias,
@@ -545,8 +545,10 @@ __global__ void __launch_bounds__(256) k_embed_tokens(const Request* rq, const i
     uint2 pk;
     pk.x = *reinterpret_cast<uint32_t*>(&lo), pk.y = *reinterpret_cast<uint32_t*>(&hi);
     *reinterpret_cast<uint2*>(out + tiled_index(row, n, rows_pad)) = pk;
-    const float ss = warp_sum(v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
-    if (lane == 0) ss_out[(size_t)(n >> 7) * rows_pad + row] = ss;
+    float ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;      // (16 lanes = 64 channels)
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((lane & 15) == 0) ss_out[(size_t)(n >> 6) * rows_pad + row] = ss;
   };
   for (int n = threadIdx.x * 4; n < D; n += blockDim.x * 4) {      // (D a multiple of 128: a warp is in or out as a whole)
     float4 acc[ER];
