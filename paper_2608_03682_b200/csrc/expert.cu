@@ -555,20 +555,29 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     }
     return pair_gemm(dn);
   };
-  auto pair_embed = [&](int k) -> phyai_status_t {
-    const float *gain0, *shift0, *gate0;
-    site(k, 0, &gain0, &shift0, &gate0);
-    if (h->ada) {
-      launch_embed_tokens(h->rq, h->status, h->Wc, h->bcfold, h->state_tok, gain0, h->h, h->xn_t, h->ss_tb, h->Mpad, d, batch, st);
-      ++cnt;
-      return PHYAI_OK;
+  // step boundary: velocity head of step k - 1 (k > 0), embedding of step k (k < n); pi0: then the MLP's second layer
+  auto pair_step = [&](int k) -> phyai_status_t {
+    StepTokens p{};
+    const float *gain0 = nullptr, *shift0, *gate0;
+    if (k > 0) {
+      site(k - 1, 2 * d.L, &p.gain_f, &p.shift_f, &gate0);
+      p.Wout = h->Wout, p.bout = h->bout, p.dt = dt;
     }
-    launch_embed_tokens(h->rq, h->status, h->Wc, t.tb + (size_t)k * D, h->state_tok, nullptr, nullptr, h->u_t, nullptr, h->Mpad, d, batch, st);
+    if (k < n) {
+      site(k, 0, &gain0, &shift0, &gate0);
+      p.Wc = h->Wc, p.state_tok = h->state_tok;
+      p.bias = h->ada ? h->bcfold : t.tb + (size_t)k * D, p.gain_next = h->ada ? gain0 : nullptr;
+      p.out = h->ada ? h->xn_t : h->u_t, p.ss_out = h->ss_tb;
+    }
+    p.h = h->h, p.rows = batch * d.H, p.rows_pad = h->Mpad, p.A = d.A, p.H = d.H, p.D = D, p.S = d.S, p.ns = d.ns, p.eps = d.eps;
+    cudaError_t e = launch_step_tokens(h->rq, h->status, p, h->n_sm, st);
+    if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "step boundary launch failed: %s", cudaGetErrorString(e));
     ++cnt;
-    PairGemm e{};
-    e.epi = PG_RESID, e.W = h->W2p, e.w_rows = (uint64_t)D * (D / 64), e.X = h->u_t, e.N = D, e.K = D, e.h = h->h;
-    e.bias = h->b2, e.state_tok = h->state_tok, e.ns = d.ns, e.S = d.S, e.gain_next = gain0, e.out = h->xn_t, e.ss_out = h->ss_tb;
-    return pair_gemm(e);
+    if (k == n || h->ada) return PHYAI_OK;
+    PairGemm g{};
+    g.epi = PG_RESID, g.W = h->W2p, g.w_rows = (uint64_t)D * (D / 64), g.X = h->u_t, g.N = D, g.K = D, g.h = h->h;
+    g.bias = h->b2, g.state_tok = h->state_tok, g.ns = d.ns, g.S = d.S, g.gain_next = gain0, g.out = h->xn_t, g.ss_out = h->ss_tb;
+    return pair_gemm(g);
   };
 
   launch_begin(h->rq, h->status, h->state_w, h->state_b, h->state_tok, d0, batch, st);
@@ -611,7 +620,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   for (int k = 0; k < n; ++k) {
     // ---- suffix embedding ----
     if (pair) {
-      ST(pair_embed(k));
+      ST(pair_step(k));
     } else if (b1_step) {
       ST(step_kernel(k, k == 0, false));
       if (!h->ada) {
@@ -806,6 +815,10 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
       }
     }
     // ---- final norm, velocity head, Euler update ----
+    if (pair) {
+      if (k + 1 == n) ST(pair_step(n));
+      continue;
+    }
     if (b1_step) {
       if (k + 1 == n) ST(step_kernel(n, false, true));
       continue;

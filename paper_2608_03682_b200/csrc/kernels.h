@@ -109,12 +109,21 @@ void launch_embed_pi0(const Request* rq, const int* status, const float* Wc, con
 // pi0.5: h[b*S+ns+i][n] = x . Wa[:,n] + ba[n] (+ state rows)
 void launch_embed_pi05(const Request* rq, const int* status, const float* Wa, const float* ba, const float* state_tok,
                        float* h, const Dims& d, int batch, cudaStream_t st);
-// Embedding ahead of the pair GEMMs: gain null (pi0): u = swish(x Wc + bias) -> tiled bf16 `out` at token rows; gain set
-// (pi0.5): h = x Wc + bias (state rows: state_tok), out = bf16(h * gain), ss_out [D/64][rows_pad] partial sums of squares.
+// Step boundary around the pair GEMMs: velocity head and Euler update of the step that ends (gain_f set), embedding of the
+// step that begins (out set): gain_next null (pi0): u = swish(x Wc + bias) -> tiled bf16 `out` at token rows; gain_next set
+// (pi0.5): h = x Wc + bias (state rows: state_tok), out = bf16(h * gain_next), ss_out [D/64][rows_pad] partial sums of squares.
 // D a multiple of 128.
-void launch_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias, const float* state_tok,
-                         const float* gain, float* h, __nv_bfloat16* out, float* ss_out, int rows_pad, const Dims& d, int batch,
-                         cudaStream_t st);
+struct StepTokens {
+  const float *gain_f, *shift_f, *Wout, *bout;    // final norm's scale and shift, velocity head
+  float dt;
+  const float *Wc, *bias, *state_tok, *gain_next;
+  float* h;                                       // [tokens][D]
+  __nv_bfloat16* out;
+  float* ss_out;
+  int rows, rows_pad, A, H, D, S, ns;             // rows: action rows of all requests
+  float eps;
+};
+cudaError_t launch_step_tokens(const Request* rq, const int* status, const StepTokens& p, int n_sm, cudaStream_t st);
 // n = h * rsqrt(mean h^2 + eps) * gain + shift  -> fp32 row-major or tiled bf16
 // Pending split-K partial sums of the residual stream: n slabs of [M][D] floats, `stride` floats apart.  The kernel
 // that reads h next adds them to each row in slab order (a fixed order: results are reproducible run to run) and,

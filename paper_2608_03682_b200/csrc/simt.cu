@@ -521,80 +521,167 @@ void launch_embed_pi05(const Request* rq, const int* status, const float* Wa, co
 }
 
 
-// Suffix embedding ahead of the pair GEMMs (norms folded in): one block takes ER action rows, a thread four consecutive
-// channels of all of them.  ADA = false (pi0): u = swish(x Wc + tb) -> bf16 operand of the MLP's second layer, at token
-// rows (the state rows' operand is never used).  ADA = true (pi0.5): h = x Wa + ba (state rows: the state token), the first
-// norm's operand bf16(h * gain) and, per 64 channels (half a warp), the row's partial sum of squares.  ER = 4 keeps small
-// calls on many SMs, ER = 16 reads Wc once per 16 rows.
+// Step boundary around the pair GEMMs (norms folded in), one block per ER action rows, which stay in shared memory between
+// the halves (either may be left out):
+//   velocity head of the step that ends: x += dt ((norm(h) gain + shift) . Wout + bout), one warp normalises a row, the
+//     contraction is split over the 16 warps (lane = action channel; a weight is read once per block, the rows as float4) and
+//     their sums are added in warp order;
+//   embedding of the step that begins, a thread four consecutive channels: ADA = false (pi0): u = swish(x Wc + tb) -> bf16
+//     operand of the MLP's second layer, at token rows (the state rows' operand is never used).  ADA = true (pi0.5):
+//     h = x Wa + ba (state rows: the state token), the first norm's operand bf16(h * gain) and, per 64 channels (half a warp),
+//     the row's partial sum of squares.
+// A chain of loads from L2 bounds it: the weights are read 32 (16) rows ahead, the first ones before the dependency wait.  As
+// two kernels of 8 warps with 4 - 8 loads in flight and 16 rows per block it took 27 + 11 us at 400 rows.
+// ER = 4 keeps small calls on many SMs, ER = 16 reads the weights once per 16 rows (from two blocks of four rows per SM on).
+constexpr int STEP_W = 16;
 template <int ER, bool ADA>
-__global__ void __launch_bounds__(256) k_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias,
-                                                      const float* state_tok, const float* gain, float* h, __nv_bfloat16* out,
-                                                      float* ss_out, int rows_pad, int A, int H, int D, int S, int ns, int rows_total) {
-  extern __shared__ float xs[];            // ER x A
-  pdl_enter();
+__global__ void __launch_bounds__(STEP_W * 32) k_step_tokens(const Request* rq, const int* status, const StepTokens p) {
+  extern __shared__ __align__(16) float step_sm[];
+  const int A = p.A, D = p.D;
+  float* nrm = step_sm;                                   // ER x D normalised rows
+  float* part = nrm + (p.gain_f ? (size_t)ER * D : 0);    // STEP_W x ER x 32 partial sums
+  float* xs = part + (p.gain_f ? STEP_W * ER * 32 : 0);   // ER x A action rows
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r0 = blockIdx.x * ER;
+  const int dper = D / STEP_W, d_lo = warp * dper;        // (D a multiple of 128)
+  pdl_launch_dependents();
+  float w_first[32];
+  if (p.gain_f)
+#pragma unroll
+    for (int j = 0; j < 32; ++j) w_first[j] = (lane < A && j < dper) ? __ldg(p.Wout + (size_t)(d_lo + j) * A + lane) : 0.f;
+  pdl_wait();
   if (status_set(status)) return;
-  const int r0 = blockIdx.x * ER, lane = threadIdx.x & 31;
-  for (int idx = threadIdx.x; idx < ER * A; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < ER * A; idx += STEP_W * 32) {
     const int r = r0 + idx / A;
-    xs[idx] = r < rows_total ? rq->x[(size_t)r * A + idx % A] : 0.f;
+    xs[idx] = r < p.rows ? rq->x[(size_t)r * A + idx % A] : 0.f;
   }
-  __syncthreads();
+  if (p.gain_f) {
+    if (warp < ER) {
+      const int r = r0 + warp, b = r / p.H;
+      const float4* x = reinterpret_cast<const float4*>(p.h + (size_t)(b * p.S + p.ns + r - b * p.H) * D);
+      const bool live = r < p.rows;
+      float ss = 0.f;
+#pragma unroll 8
+      for (int d = lane; d < D / 4; d += 32) {
+        const float4 v = live ? x[d] : make_float4(0.f, 0.f, 0.f, 0.f);
+        reinterpret_cast<float4*>(nrm + (size_t)warp * D)[d] = v;
+        ss = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss))));
+      }
+      const float rs = 1.0f / sqrtf(warp_sum(ss) / (float)D + p.eps);
+#pragma unroll 4
+      for (int d = lane; d < D / 4; d += 32) {
+        const float4 g4 = __ldg(reinterpret_cast<const float4*>(p.gain_f) + d);
+        const float4 s4 = p.shift_f ? __ldg(reinterpret_cast<const float4*>(p.shift_f) + d) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4& v = reinterpret_cast<float4*>(nrm + (size_t)warp * D)[d];
+        v = make_float4(fmaf(v.x * rs, g4.x, s4.x), fmaf(v.y * rs, g4.y, s4.y), fmaf(v.z * rs, g4.z, s4.z), fmaf(v.w * rs, g4.w, s4.w));
+      }
+    }
+    __syncthreads();
+    for (int a0 = 0; a0 < A; a0 += 32) {
+      const int a = a0 + lane;
+      float acc[ER];
+#pragma unroll
+      for (int e = 0; e < ER; ++e) acc[e] = 0.f;
+#pragma unroll 1
+      for (int j0 = 0; j0 < dper; j0 += 32) {
+        if (a0 > 0 || j0 > 0)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) w_first[j] = (a < A && j0 + j < dper) ? __ldg(p.Wout + (size_t)(d_lo + j0 + j) * A + a) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          if (j0 + j >= dper) break;
+#pragma unroll
+          for (int e = 0; e < ER; ++e) {
+            const float4 n4 = *reinterpret_cast<const float4*>(nrm + (size_t)e * D + d_lo + j0 + j);
+            acc[e] = fmaf(n4.x, w_first[j], fmaf(n4.y, w_first[j + 1], fmaf(n4.z, w_first[j + 2], fmaf(n4.w, w_first[j + 3], acc[e]))));
+          }
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < ER; ++e) part[(warp * ER + e) * 32 + lane] = acc[e];
+      __syncthreads();
+      for (int idx = threadIdx.x; idx < ER * 32; idx += STEP_W * 32) {
+        const int e = idx >> 5, r = r0 + e, aa = a0 + (idx & 31);
+        if (r < p.rows && aa < A) {
+          float v = 0.f;
+#pragma unroll
+          for (int w = 0; w < STEP_W; ++w) v += part[(w * ER + e) * 32 + (idx & 31)];
+          const float xn = xs[e * A + aa] + p.dt * (v + p.bout[aa]);
+          xs[e * A + aa] = xn;
+          rq->x[(size_t)r * A + aa] = xn;
+        }
+      }
+      __syncthreads();
+    }
+  } else {
+    __syncthreads();
+  }
+  if (!p.out) return;
   auto emit = [&](int row, int n, float4 v, float4 g4) {
-    *reinterpret_cast<float4*>(h + (size_t)row * D + n) = v;
+    *reinterpret_cast<float4*>(p.h + (size_t)row * D + n) = v;
     __nv_bfloat162 lo = __floats2bfloat162_rn(v.x * g4.x, v.y * g4.y), hi = __floats2bfloat162_rn(v.z * g4.z, v.w * g4.w);
     uint2 pk;
     pk.x = *reinterpret_cast<uint32_t*>(&lo), pk.y = *reinterpret_cast<uint32_t*>(&hi);
-    *reinterpret_cast<uint2*>(out + tiled_index(row, n, rows_pad)) = pk;
+    *reinterpret_cast<uint2*>(p.out + tiled_index(row, n, p.rows_pad)) = pk;
     float ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;      // (16 lanes = 64 channels)
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if ((lane & 15) == 0) ss_out[(size_t)(n >> 6) * rows_pad + row] = ss;
+    if ((lane & 15) == 0) p.ss_out[(size_t)(n >> 6) * p.rows_pad + row] = ss;
   };
-  for (int n = threadIdx.x * 4; n < D; n += blockDim.x * 4) {      // (D a multiple of 128: a warp is in or out as a whole)
-    float4 acc[ER];
+  // an item: four consecutive channels of half the block's rows (D a multiple of 128: a warp is in or out as a whole)
+  constexpr int EH = ER / 2;
+  for (int it = threadIdx.x; it < D / 2; it += STEP_W * 32) {
+    const int half = it >= D / 4 ? 1 : 0, n = (it - half * (D / 4)) * 4, e0 = half * EH;
+    float4 acc[EH];
 #pragma unroll
-    for (int e = 0; e < ER; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 8
+    for (int e = 0; e < EH; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 16
     for (int a = 0; a < A; ++a) {
-      const float4 w = __ldg(reinterpret_cast<const float4*>(Wc + (size_t)a * D + n));
+      const float4 w = __ldg(reinterpret_cast<const float4*>(p.Wc + (size_t)a * D + n));
 #pragma unroll
-      for (int e = 0; e < ER; ++e) {
-        const float x = xs[e * A + a];
+      for (int e = 0; e < EH; ++e) {
+        const float x = xs[(e0 + e) * A + a];
         acc[e].x = fmaf(x, w.x, acc[e].x), acc[e].y = fmaf(x, w.y, acc[e].y);
         acc[e].z = fmaf(x, w.z, acc[e].z), acc[e].w = fmaf(x, w.w, acc[e].w);
       }
     }
-    const float4 t4 = __ldg(reinterpret_cast<const float4*>(bias + n));
+    const float4 t4 = __ldg(reinterpret_cast<const float4*>(p.bias + n));
     float4 g4 = t4;
-    if constexpr (ADA) g4 = __ldg(reinterpret_cast<const float4*>(gain + n));
+    if constexpr (ADA) g4 = __ldg(reinterpret_cast<const float4*>(p.gain_next + n));
 #pragma unroll
-    for (int e = 0; e < ER; ++e) {
-      const int r = r0 + e;
-      if (r >= rows_total) break;
-      const int b = r / H, i = r - b * H, row = b * S + ns + i;
+    for (int e = 0; e < EH; ++e) {
+      const int r = r0 + e0 + e;
+      if (r >= p.rows) break;
+      const int b = r / p.H, i = r - b * p.H, row = b * p.S + p.ns + i;
       const float4 v = make_float4(acc[e].x + t4.x, acc[e].y + t4.y, acc[e].z + t4.z, acc[e].w + t4.w);
       if constexpr (ADA) {
         emit(row, n, v, g4);
-        if (ns && i == 0) emit(b * S, n, __ldg(reinterpret_cast<const float4*>(state_tok + (size_t)b * D + n)), g4);
+        if (p.ns && i == 0) emit(b * p.S, n, __ldg(reinterpret_cast<const float4*>(p.state_tok + (size_t)b * D + n)), g4);
       } else {
         __nv_bfloat162 lo = __floats2bfloat162_rn(swish_precise(v.x), swish_precise(v.y));
         __nv_bfloat162 hi = __floats2bfloat162_rn(swish_precise(v.z), swish_precise(v.w));
         uint2 pk;
         pk.x = *reinterpret_cast<uint32_t*>(&lo), pk.y = *reinterpret_cast<uint32_t*>(&hi);
-        *reinterpret_cast<uint2*>(out + tiled_index(row, n, rows_pad)) = pk;
+        *reinterpret_cast<uint2*>(p.out + tiled_index(row, n, p.rows_pad)) = pk;
       }
     }
   }
 }
-void launch_embed_tokens(const Request* rq, const int* status, const float* Wc, const float* bias, const float* state_tok,
-                         const float* gain, float* h, __nv_bfloat16* out, float* ss_out, int rows_pad, const Dims& d, int batch,
-                         cudaStream_t st) {
-  const int rows = batch * d.H;
-  const bool wide = rows >= 2048, ada = gain != nullptr;
-  const int er = wide ? 16 : 4;
-  auto k = ada ? (wide ? k_embed_tokens<16, true> : k_embed_tokens<4, true>) : (wide ? k_embed_tokens<16, false> : k_embed_tokens<4, false>);
-  launch_pdl(k, dim3((rows + er - 1) / er), dim3(256), (size_t)er * d.A * sizeof(float), st, rq, status, Wc, bias, state_tok, gain, h, out,
-             ss_out, rows_pad, d.A, d.H, d.D, d.S, d.ns, rows);
+cudaError_t launch_step_tokens(const Request* rq, const int* status, const StepTokens& p, int n_sm, cudaStream_t st) {
+  constexpr size_t SMEM = 200 * 1024;
+  static PerDeviceOnce once;
+  if (once.needed()) {
+    cudaError_t e = cudaSuccess;
+    for (auto f : {k_step_tokens<4, false>, k_step_tokens<4, true>, k_step_tokens<16, false>, k_step_tokens<16, true>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+    if (e != cudaSuccess) return e;
+    once.done();
+  }
+  const bool ada = p.gain_next != nullptr;
+  auto smem = [&](int er) { return ((p.gain_f ? (size_t)er * p.D + STEP_W * er * 32 : 0) + (size_t)er * p.A) * sizeof(float); };
+  const int er = p.rows > 2 * 4 * n_sm && smem(16) <= SMEM ? 16 : 4;
+  if (smem(er) > SMEM) return cudaErrorInvalidValue;
+  auto k = ada ? (er == 16 ? k_step_tokens<16, true> : k_step_tokens<4, true>) : (er == 16 ? k_step_tokens<16, false> : k_step_tokens<4, false>);
+  return launch_pdl(k, dim3((p.rows + er - 1) / er), dim3(STEP_W * 32), smem(er), st, rq, status, p);
 }
 
 // =============================================================================================

@@ -40,6 +40,13 @@ def test_pair_gemms_at_the_edges_of_their_token_tiles(cond, dtype, horizon, batc
     check(cfg, [(37 * b) % 121 for b in range(batch)], 2, {0, batch // 2, batch - 1})
 
 
+@pytest.mark.parametrize("cond,action_dim,width,horizon,batch", [("pi05", 33, 768, 60, 20), ("pi0", 7, 1280, 37, 32), ("pi05", 1, 256, 61, 2)])
+def test_step_boundary_row_groups(cond, action_dim, width, horizon, batch):
+    """Sixteen rows per block from 1185 action rows on, four below; ragged last groups; action widths around a warp's lanes."""
+    cfg = small_bf16_config(cond, action_dim=action_dim, width=width, horizon=horizon, max_batch=batch, max_prefix_len=40, n_layers=2)
+    check(cfg, [(13 * b) % 41 for b in range(batch)], 3, {0, batch - 1})
+
+
 @pytest.mark.parametrize("head_dim,n_q,n_kv", [(256, 4, 1), (128, 8, 2)])
 @pytest.mark.parametrize("ranges", [1, 2, 3, 4])
 def test_pair_attention_key_ranges(head_dim, n_q, n_kv, ranges):
