@@ -448,7 +448,7 @@ class KvProjector:
     def run(self, features: torch.Tensor, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
         tokens = features.shape[0]
         if out is None:
-            out = torch.zeros(self.L, 2, tokens, self.n_kv_heads, self.head_dim, dtype=torch.bfloat16, device=features.device)
+            out = torch.empty(self.L, 2, tokens, self.n_kv_heads, self.head_dim, dtype=torch.bfloat16, device=features.device)
         st = self.lib.phyai_kv_projector_run(self._h, _ptr(features), tokens, out.shape[2], _ptr(out), _stream_ptr(stream))
         if st != OK:
             raise PhyaiError(st, self.lib.phyai_adapter_last_error().decode())

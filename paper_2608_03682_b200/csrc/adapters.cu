@@ -96,23 +96,6 @@ __global__ void k_postprocess(const float* x, const float* q01, const float* q99
   }
 }
 
-
-// fp32 [tokens][2 * nkv] (K channels, then V channels) -> bf16 rows of the K plane and the V plane of one layer
-__global__ void k_kv_planes(const float* src, __nv_bfloat16* kplane, __nv_bfloat16* vplane, int tokens, int nkv) {
-  const size_t n = (size_t)tokens * (nkv >> 2) * 2;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const int per_row = (nkv >> 2) * 2;
-    const int t = (int)(i / per_row), c4 = (int)(i % per_row);
-    const float4 v = *reinterpret_cast<const float4*>(src + (size_t)t * 2 * nkv + c4 * 4);
-    const int col = c4 * 4;
-    __nv_bfloat16* dst = col < nkv ? kplane + (size_t)t * nkv + col : vplane + (size_t)t * nkv + (col - nkv);
-    __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-    uint2 pk;
-    pk.x = *reinterpret_cast<uint32_t*>(&lo), pk.y = *reinterpret_cast<uint32_t*>(&hi);
-    *reinterpret_cast<uint2*>(dst) = pk;
-  }
-}
-
 }  // namespace
 }  // namespace phyai
 
@@ -187,14 +170,14 @@ phyai_status_t phyai_postprocess_actions(const float* x, uint32_t batch, uint32_
 
 }  // extern "C"
 
-// Request-local K / V projections of a feature-handoff head: per layer one tcgen05 GEMM of the (tiled) feature rows
-// against [Wk | Wv], fp32 out, then the bf16 rows of the two planes.  The projector handle owns the packed weight
-// images and the workspace, so that a run only enqueues kernels.
+// Request-local K / V projections of a feature-handoff head: one GEMM on CTA pairs of the (tiled) feature rows against
+// [Wk | Wv] of all layers, whose epilogue writes the bf16 rows of every layer's two planes.  The projector handle owns the
+// packed weight images and the workspace, so that a run only enqueues kernels.  640 rows of 2048 features, 16 layers of
+// 2 x 256 channels: 27 us (a 128-row tile GEMM with fp32 output and a conversion kernel per layer, 32 launches: 260 us).
 struct phyai_kv_projector {
-  int L = 0, nkv = 0, Dv = 0, max_tokens = 0, rows_pad = 0;
-  __nv_bfloat16* wp = nullptr;    // [L] packed [Wk | Wv] images, Dv x 2 nkv each
+  int L = 0, nkv = 0, Dv = 0, max_tokens = 0, rows_pad = 0, N = 0, n_sm = 0;   // N: rows of the image, a multiple of 256
+  __nv_bfloat16* wp = nullptr;    // packed [Wk | Wv] of layer 0, of layer 1, ...: blocks [N/128][Dv/64][128 x 64]
   __nv_bfloat16* xt = nullptr;    // tiled features [Dv / 64][rows_pad][64]
-  float* y = nullptr;             // [max_tokens][2 nkv]
   int* status = nullptr;
 };
 
@@ -209,7 +192,7 @@ phyai_status_t proj_fail(phyai_status_t st, const char* msg, cudaError_t e = cud
 
 extern "C" void phyai_kv_projector_destroy(phyai_kv_projector_t* p) {
   if (!p) return;
-  cudaFree(p->wp), cudaFree(p->xt), cudaFree(p->y), cudaFree(p->status);
+  cudaFree(p->wp), cudaFree(p->xt), cudaFree(p->status);
   delete p;
 }
 
@@ -228,22 +211,30 @@ extern "C" phyai_status_t phyai_kv_projector_create(const phyai_kv_proj_desc_t* 
   for (int l = 0; l < L; ++l)
     if (!wk[l] || !wv[l]) return proj_fail(PHYAI_ERR_INVALID_ARG, "a per-layer weight pointer is NULL");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  cudaError_t e = tc_gemm_setup();
-  if (e != cudaSuccess) return proj_fail(PHYAI_ERR_CUDA, "tc_gemm_setup", e);
+  cudaError_t e = cudaSuccess;
   phyai_kv_projector* p = new (std::nothrow) phyai_kv_projector();
   if (!p) return proj_fail(PHYAI_ERR_OOM, "host allocation failed");
   p->L = L, p->nkv = nkv, p->Dv = Dv, p->max_tokens = (int)max_tokens, p->rows_pad = ((int)max_tokens + 255) / 256 * 256;
-  const size_t N = 2 * (size_t)nkv;
-  if ((e = cudaMalloc(&p->wp, (size_t)L * Dv * N * 2)) != cudaSuccess || (e = cudaMalloc(&p->xt, (size_t)p->rows_pad * Dv * 2)) != cudaSuccess ||
-      (e = cudaMalloc(&p->y, (size_t)max_tokens * N * 4)) != cudaSuccess || (e = cudaMalloc(&p->status, 4)) != cudaSuccess) {
+  const size_t per_layer = 2 * (size_t)nkv, n_rows = (size_t)L * per_layer;
+  p->N = (int)((n_rows + 255) / 256 * 256);
+  if ((e = cudaMalloc(&p->wp, (size_t)Dv * p->N * 2)) != cudaSuccess || (e = cudaMalloc(&p->xt, (size_t)p->rows_pad * Dv * 2)) != cudaSuccess ||
+      (e = cudaMalloc(&p->status, 4)) != cudaSuccess) {
     phyai_kv_projector_destroy(p);
     return proj_fail(PHYAI_ERR_OOM, "cudaMalloc", e);
   }
   cudaMemsetAsync(p->xt, 0, (size_t)p->rows_pad * Dv * 2, st);
   cudaMemsetAsync(p->status, 0, 4, st);
+  cudaMemsetAsync(p->wp + n_rows * Dv, 0, (p->N - n_rows) * Dv * 2, st);
+  int dev = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) {
+    phyai_kv_projector_destroy(p);
+    return proj_fail(PHYAI_ERR_CUDA, "device attributes", e);
+  }
   for (int l = 0; l < L; ++l) {
-    launch_pack_tiled(wk[l], 1, p->wp + (size_t)l * Dv * N, Dv, nkv, 0, st);
-    launch_pack_tiled(wv[l], 1, p->wp + (size_t)l * Dv * N, Dv, nkv, nkv, st);
+    launch_pack_tiled(wk[l], 1, p->wp + (size_t)l * Dv * per_layer, Dv, nkv, 0, st);
+    launch_pack_tiled(wv[l], 1, p->wp + (size_t)l * Dv * per_layer, Dv, nkv, nkv, st);
   }
   e = cudaStreamSynchronize(st);
   if (e == cudaSuccess) e = cudaGetLastError();
@@ -263,20 +254,16 @@ extern "C" phyai_status_t phyai_kv_projector_run(phyai_kv_projector_t* p, const 
   if (tokens == 0 || tokens > (uint64_t)p->max_tokens || tokens > kv_tokens)
     return proj_fail(PHYAI_ERR_INVALID_ARG, "need 1 <= tokens <= max_tokens and tokens <= kv_tokens");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int M = (int)tokens, N = 2 * p->nkv;
+  const int M = (int)tokens;
   launch_rows_to_tiled(reinterpret_cast<const __nv_bfloat16*>(features), p->xt, M, p->Dv, p->rows_pad, st);
-  __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(prefix_kv);
-  for (int l = 0; l < p->L; ++l) {
-    TcGemm g{};
-    g.W = p->wp + (size_t)l * p->Dv * N, g.X = p->xt, g.M = M, g.N = N, g.K = p->Dv, g.epi = TC_STORE, g.out_f32 = p->y, g.ldo = N;
-    g.splits = 1, g.rows_pad = p->rows_pad, g.wait_limit = 1u << 28;
-    cudaError_t e = launch_tc_gemm(p->status, g, M <= 64 ? 64 : (M <= 1024 ? 128 : 256), st);
-    if (e != cudaSuccess) return proj_fail(PHYAI_ERR_CUDA, "projection GEMM launch", e);
-    const size_t n = (size_t)M * (p->nkv >> 2) * 2;
-    k_kv_planes<<<(int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096), 256, 0, st>>>(
-        p->y, out + ((size_t)l * 2) * kv_tokens * p->nkv, out + ((size_t)l * 2 + 1) * kv_tokens * p->nkv, M, p->nkv);
-  }
-  cudaError_t e = cudaGetLastError();
+  PairGemm g{};
+  g.epi = PG_PLANES, g.W = p->wp, g.w_rows = (uint64_t)p->N * (p->Dv / 64), g.X = p->xt, g.rows_pad = p->rows_pad;
+  g.M = M, g.N = p->N, g.K = p->Dv, g.out = reinterpret_cast<__nv_bfloat16*>(prefix_kv), g.nkv = p->nkv, g.n_planes = 2 * p->L;
+  g.plane_rows = kv_tokens, g.wait_limit = 1u << 28;
+  int busy = 0;
+  cudaError_t e = launch_pair_gemm(p->status, g, p->n_sm, &busy, st);
+  if (e != cudaSuccess) return proj_fail(PHYAI_ERR_CUDA, "projection GEMM launch", e);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return proj_fail(PHYAI_ERR_CUDA, "kernel launch failed", e);
   return PHYAI_OK;
 }

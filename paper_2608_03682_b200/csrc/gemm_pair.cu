@@ -324,9 +324,10 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
           off2 = (g.dh >> 7) * 8192;
         }
       } else if constexpr (EPI == PG_PLANES) {
-        // K | V projections of all layers: row n of layer n / (2 nkv): nkv K channels, then nkv V channels
-        const int n = n0 + 32 * q, layer = n / (2 * g.nkv), c = n - layer * 2 * g.nkv, v = c >= g.nkv ? 1 : 0;
-        obase = g.out + (size_t)(layer * 2 + v) * g.plane_rows * g.nkv + (c - v * g.nkv) + 8 * (lane & 1), off2 = 16;
+        // K | V projections of all layers: row n belongs to plane n / nkv (a warp's 32 rows to one: nkv is a multiple of 64)
+        const int n = n0 + 32 * q, plane = n / g.nkv;
+        if (plane < g.n_planes) obase = g.out + (size_t)plane * g.plane_rows * g.nkv + (n - plane * g.nkv) + 8 * (lane & 1);
+        off2 = 16;
       }
       // RESID: in the transposed view a lane takes 4 channels of tokens lane / 8, + 4, + 8, + 12 of the chunk; what is added
       // to (the residual stream, or the MLP's bias / the state token) is requested one chunk ahead
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
               const int tl = c0 + (lane >> 1) + 16 * it, tok = tok_base + tl;
               uint4 w;
               asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "r"(st_r + (uint32_t)it * 512) : "memory");
-              if (ok && tl < n_tok) {
+              if (ok && tl < n_tok && (EPI != PG_PLANES || obase)) {
                 __nv_bfloat16* dst = obase;
                 if constexpr (EPI == PG_GEGLU) dst += (size_t)tok * 64 + (((p8 >> 3) ^ (tok & 7)) << 3);
                 else if constexpr (EPI == PG_QKV) {
@@ -471,7 +472,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
                   dst += (isq ? e4.y : e4.z) + m * off2 + (qt ? ((p8 >> 3) ^ (e4.w & 7)) << 3 : 0);
                 }
                 else dst += (size_t)tok * g.nkv + m * off2;
-                *reinterpret_cast<uint4*>(dst) = w;
+                if (EPI == PG_PLANES && (reinterpret_cast<uintptr_t>(dst) & 15u)) {      // (planes at a caller's address)
+                  reinterpret_cast<uint2*>(dst)[0] = make_uint2(w.x, w.y), reinterpret_cast<uint2*>(dst)[1] = make_uint2(w.z, w.w);
+                } else {
+                  *reinterpret_cast<uint4*>(dst) = w;
+                }
               }
             }
             __syncwarp();

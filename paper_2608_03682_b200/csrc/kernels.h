@@ -336,8 +336,9 @@ struct PairGemm {
   __nv_bfloat16 *qr, *kr, *vr;
   __nv_bfloat16* q_tiles;    // set: q goes out as the operand tiles of the pair / cluster attention kernels instead of rows
   int S, Hq, Hkv, dh;
-  // PLANES: row n of layer n / (2 nkv): nkv K channels, nkv V channels
-  int nkv;
+  // PLANES: rows n_plane nkv .. + nkv - 1 go to plane n_plane (a layer's K plane, then its V plane); rows past the last plane
+  // are padding
+  int nkv, n_planes;
   uint64_t plane_rows;
   unsigned wait_limit;
   unsigned long long* trace; // or null: CTA b stamps slot b (16 words)

@@ -67,3 +67,22 @@ def test_attention_operator_on_the_pair_kernel(n_kv, head_dim, suffix, lens):
     assert int(status.item()) == 0
     ref = oracle_attention(qkv, kv, cu, 8, n_kv, head_dim, suffix, 1, 10000.0)
     assert abs(out.double().cpu().numpy() - ref).max() <= 2e-2 * abs(ref).max()
+
+
+@pytest.mark.parametrize("tokens,n_kv,dh,layers,shift", [(1, 1, 64, 3, 0), (65, 3, 64, 1, 4), (641, 1, 128, 5, 0), (200, 1, 192, 2, 4)])
+def test_feature_projection_of_all_layers(tokens, n_kv, dh, layers, shift):
+    """Row counts that leave the last 256 padded, warps whose 32 rows end a plane, planes at an 8-byte-aligned address."""
+    from oracle import adapter_oracle as A
+    F = synth.make_features(44, tokens, 192)
+    g = torch.Generator().manual_seed(44)
+    wk, wv = ([torch.randn(192, n_kv * dh, generator=g).mul(192 ** -0.5).bfloat16() for _ in range(layers)] for _ in range(2))
+    n = layers * 2 * (tokens + 3) * n_kv * dh
+    out = torch.full((n + 2 * shift,), 7.0, dtype=torch.bfloat16, device="cuda")
+    planes = out[shift:shift + n].view(layers, 2, tokens + 3, n_kv, dh)
+    with binding.KvProjector([w.cuda() for w in wk], [w.cuda() for w in wv], n_kv, dh, max_tokens=tokens) as proj:
+        proj.run(F.cuda(), out=planes)
+        torch.cuda.synchronize()
+    ref = torch.from_numpy(A.project_features_kv(F.double().numpy(), [w.double().numpy() for w in wk], [w.double().numpy() for w in wv], n_kv, dh))
+    got = planes.double().cpu()
+    assert (got[:, :, tokens:] == 7).all() and (out[:shift] == 7).all() and (out[shift + n:] == 7).all()
+    assert ((got[:, :, :tokens] - ref).abs() <= ref.abs() * 2.0 ** -8 + 1e-4).all()
