@@ -98,8 +98,9 @@ struct phyai_expert {
                                // one request the 18-layer state pass costs more than the 51st row it saves (measured)
   __nv_bfloat16 *kr_st = nullptr, *vr_st = nullptr;   // [L][max 64 tokens worth of requests][Hkv][S][dh] suffix K / V per layer
   int use_w8_inkernel = 1;     // e4m3 experts: the cluster GEMM decodes byte blocks itself (0: bf16 images made at create)    // tcgen05 attention with the key range split over a cluster (few requests)
+  int use_b1_pair = 1;         // single-tile calls: projections on CTA pairs where they fit
   int b1_c[4] = {0, 0, 0, 0};  // cluster sizes of the QKV / O / gate-up / down projections (0 = choose)
-  float *ss_a = nullptr, *ss_b = nullptr;   // [D/128][64] partial sums of squares of h (after O / after down)
+  float *ss_a = nullptr, *ss_b = nullptr;   // [D/128 or D/64][64] partial sums of squares of h (after O / after down)
   unsigned long long* trace_buf = nullptr;
   int trace_all_from = 0;                   // > 0: launches [from, from + 5) of a call trace every CTA
   unsigned long long* trace = nullptr;      // [TRACE_SLOTS][8] timer stamps of the traced launches of one call, or null
@@ -370,7 +371,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   const bool simt_norm = !h->tc && simt_rows_supported(M, D);
 
   const int kcb = h->a8 ? 128 : 64;   // contraction elements per 128-byte operand row (k-chunk of the tile GEMM)
-  const int ss_n = D / 128;
+  int ss_na = D / 128, ss_nb = D / 128;   // partial sums of squares per token that the last writer of ss_a / ss_b left
   int trace_cursor = 0;
   const bool use_w8 = h->use_w8_inkernel && !h->b_qkv.empty();
   auto b1_gemm = [&](B1Gemm g, int which, int Mloc) -> phyai_status_t {
@@ -390,16 +391,19 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
       if (c6 >= 1 && c6 < C && b1_gemm_supported(g.N, g.K, c6, h->n_sm, true)) C = c6;
     }
     if (h->b1_c[which] > 0 && b1_gemm_supported(g.N, g.K, h->b1_c[which], h->n_sm, which == 0)) C = h->b1_c[which];
+    // (a cluster size chosen by hand keeps to the kernel that has one)
+    const int pairs = h->use_b1_pair && h->b1_c[which] == 0 ? b1_pair_ranges(g.N, g.K, h->n_sm, g.epi) : 0;
+    if (g.ss_out) (g.ss_out == h->ss_a ? ss_na : ss_nb) = pairs ? g.N / 64 : g.N / 128;
     if (h->trace && h->trace_all_from > 0) {
       // every CTA of five consecutive launches stamps, one slot per CTA in launch order
       g.trace = nullptr;
-      const int n_cta = C * (g.N / 128);
+      const int n_cta = (pairs ? 2 * pairs : C) * (g.N / 128);
       if (cnt >= h->trace_all_from && cnt < h->trace_all_from + 5 && trace_cursor + n_cta <= TRACE_SLOTS) {
         g.trace = h->trace + (size_t)trace_cursor * TRACE_STAMPS, g.trace_all = 1;
         trace_cursor += n_cta;
       }
     }
-    cudaError_t e = launch_b1_gemm(h->status, g, C, st);
+    const cudaError_t e = pairs ? launch_b1_pair_gemm(h->status, g, pairs, st) : launch_b1_gemm(h->status, g, C, st);
     if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "cluster GEMM launch failed: %s", cudaGetErrorString(e));
     ++cnt;
     return PHYAI_OK;
@@ -421,7 +425,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     B1Gemm q{};
     q.W = h->p_qkv[l], q.W8 = use_w8 ? h->b_qkv[l] : nullptr, q.X = h->xn64, q.N = dd.Nqkv, q.K = D, q.epi = B1_QKV, q.wscale = h->s_qkv[l];
     if (l > 0 || folded_first) {
-      q.ss_part = h->ss_b, q.ss_n = ss_n;
+      q.ss_part = h->ss_b, q.ss_n = ss_nb;
       q.shift_row = h->ada ? t.shw_qkv + ((size_t)k * dd.L + l) * dd.Nqkv : nullptr;
     }
     q.rq = h->rq, q.rope = h->rope, q.qr = h->qr_big, q.kr = kr, q.vr = vr;
@@ -460,7 +464,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     // ---- gate / up + GeGLU
     B1Gemm gu{};
     gu.W = h->p_gu_all + (size_t)l * D * 2 * dd.F, gu.W8 = use_w8 ? h->b_gu[l] : nullptr, gu.X = h->xn64, gu.N = 2 * dd.F, gu.K = D, gu.epi = B1_GEGLU;
-    gu.wscale = h->s_g[l], gu.wscale2 = h->s_u[l], gu.ss_part = h->ss_a, gu.ss_n = ss_n;
+    gu.wscale = h->s_g[l], gu.wscale2 = h->s_u[l], gu.ss_part = h->ss_a, gu.ss_n = ss_na;
     gu.shift_row = h->ada ? t.shw_gu + ((size_t)k * dd.L + l) * 2 * dd.F : nullptr;
     gu.out_tiled = h->m64;
     ST(b1_gemm(gu, 2, Mloc));
@@ -606,7 +610,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
       if (h->ada) {
         const float *shift0, *gate0;
         site(k, 0, &p.gain_next, &shift0, &gate0);
-        p.bias = h->bcfold, p.h_out = h->h, p.xn_out = h->xn64, p.ss_out = h->ss_b;
+        p.bias = h->bcfold, p.h_out = h->h, p.xn_out = h->xn64, p.ss_out = h->ss_b, ss_nb = D / 128;
       } else {
         p.bias = t.tb + (size_t)k * D, p.u = h->m64;
       }
@@ -1224,8 +1228,8 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
         ST(h->alloc(&h->xn64, (size_t)64 * D, true));
         ST(h->alloc(&h->attn64, (size_t)64 * Nq, true));
         ST(h->alloc(&h->m64, (size_t)64 * F, true));
-        ST(h->alloc(&h->ss_a, (size_t)(D / 128) * 64, true));
-        ST(h->alloc(&h->ss_b, (size_t)(D / 128) * 64, true));
+        ST(h->alloc(&h->ss_a, (size_t)(D / 64) * 64, true));
+        ST(h->alloc(&h->ss_b, (size_t)(D / 64) * 64, true));
         if (attention_b1_supported(d) && d.Hq >= 2)   // q as operand tiles of the cluster attention kernel: up to 64 query rows
           ST(h->alloc(&h->q_tiles, (size_t)64 * (d.Hq / 2) * 128 * d.dh, true));
         if (d.block_causal && d.ns && !ada) {
@@ -1499,6 +1503,12 @@ phyai_status_t phyai_set_option(phyai_expert_t* h, const char* key, int64_t valu
   }
   if (!strcmp(key, "use_state_cache")) {
     h->use_state_cache = value != 0;
+    for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
+    h->graphs.clear();
+    return PHYAI_OK;
+  }
+  if (!strcmp(key, "use_b1_pair")) {
+    h->use_b1_pair = value != 0;
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();
     return PHYAI_OK;

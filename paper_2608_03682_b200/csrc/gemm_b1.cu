@@ -27,6 +27,7 @@
 // token) and the per-channel tables are read as 16-byte vectors.  Waits: see mbar_wait_drain -- a given-up
 // wait suppresses the global stores but never the copy / reduce protocol, so peers are not left waiting and
 // nothing is in flight at exit.
+#include "decode.cuh"
 #include "kernels.h"
 #include "ptx.cuh"
 #include "tc.cuh"
@@ -60,24 +61,6 @@ __device__ __forceinline__ float4 lds4(uint32_t addr) {
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
-}
-
-// Four e4m3 codes (one 32-bit word) -> two bf16 pairs, exactly, without the (slow-rate) conversion instructions.
-// A code is S EEEE MMM (bias 7).  Its byte goes to the high byte of a 16-bit half (byte permute): the sign is then
-// in place; the magnitude, moved down by four bits, puts EEEE into the low bits of bf16's exponent field and MMM
-// at the top of its mantissa, i.e. the bf16 number 2^(E - 127) (1 + M/8) -- for E = 0 the bf16 subnormal
-// 2^-126 (M/8).  One exact bf16x2 multiplication by 2^120 restores the bias: 2^(E - 7)(1 + M/8), and for E = 0
-// 2^-6 (M/8), which is the value of e4m3's subnormals; zero stays zero.  (bf16 multiplication has no flush-to-zero
-// mode: subnormal inputs are honoured.)  Five full-rate instructions per pair.
-__device__ __forceinline__ void e4m3x4_to_bf16x4(uint32_t w, uint32_t& lo, uint32_t& hi) {
-  uint32_t x0, x1;
-  asm("prmt.b32 %0, %1, 0, 0x1404;" : "=r"(x0) : "r"(w));   // [b1 0 b0 0]
-  asm("prmt.b32 %0, %1, 0, 0x3424;" : "=r"(x1) : "r"(w));   // [b3 0 b2 0]
-  const uint32_t t0 = (x0 & 0x80008000u) | ((x0 >> 4) & 0x07F007F0u);
-  const uint32_t t1 = (x1 & 0x80008000u) | ((x1 >> 4) & 0x07F007F0u);
-  const uint32_t c = 0x7B807B80u;   // (2^120, 2^120)
-  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(lo) : "r"(t0), "r"(c));
-  asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(hi) : "r"(t1), "r"(c));
 }
 
 // WB: bits per streamed weight -- 0 = the bf16 operand image itself, 8 = e4m3 codes, 4 = int4 codes; the codes are
@@ -211,58 +194,7 @@ __global__ void __launch_bounds__(NT, 1) k_gemm_b1(int* status, const B1Gemm g) 
     if (s < nk) {
       mbar_wait_drain(smem_u32(&bar_w8[s]), 0u, wc);
       const uint32_t slot0 = tiles + (uint32_t)s * STAGE;
-      const int r0 = hf * 64 + (lane >> 2), cq = lane & 3;       // my row of every group of 8 rows, my quarter of a row
-      if constexpr (WB == 8) {
-        uint4 raw[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint32_t src = slot0 + W_BYTES - CODE_BYTES + (uint32_t)(r0 + 8 * j) * 64 + (uint32_t)cq * 16;
-          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(raw[j].x), "=r"(raw[j].y), "=r"(raw[j].z), "=r"(raw[j].w) : "r"(src) : "memory");
-        }
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int r = r0 + 8 * j;
-          const uint32_t words[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {       // 16-byte chunk 2 cq + c of the row: 8 codes = words[2c], words[2c + 1]
-            uint32_t o0, o1, o2, o3;
-            e4m3x4_to_bf16x4(words[2 * c], o0, o1);
-            e4m3x4_to_bf16x4(words[2 * c + 1], o2, o3);
-            const uint32_t dst = slot0 + (uint32_t)r * 128 + (uint32_t)((((2 * cq + c) ^ (r & 7))) << 4);
-            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(o0), "r"(o1), "r"(o2), "r"(o3) : "memory");
-          }
-        }
-      } else {
-        // int4: a row of the block is 32 bytes = 64 codes, byte j = codes (k = 2j in the low nibble, 2j + 1 in the
-        // high one).  A nibble c becomes the bf16 number 128 + c by bit insertion (0x4300 | c: the unit of the mantissa
-        // at 128 is 1), and one exact bf16x2 subtraction of 136 makes it c - 8.
-        uint2 raw[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint32_t src = slot0 + W_BYTES - CODE_BYTES + (uint32_t)(r0 + 8 * j) * 32 + (uint32_t)cq * 8;
-          asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(raw[j].x), "=r"(raw[j].y) : "r"(src) : "memory");
-        }
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory");
-        auto pair = [](uint32_t byte) -> uint32_t {       // one byte -> (bf16(lo - 8), bf16(hi - 8))
-          uint32_t w = 0x43004300u | (byte & 15u) | ((byte & 0xF0u) << 12), o;
-          asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(o) : "r"(w), "r"(0x43084308u));
-          return o;
-        };
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int r = r0 + 8 * j;
-          const uint32_t words[2] = {raw[j].x, raw[j].y};
-#pragma unroll
-          for (int c = 0; c < 2; ++c) {       // 16-byte chunk 2 cq + c: codes of bytes 4c .. 4c + 3 of my 8
-            const uint32_t w4 = words[c];
-            const uint32_t dst = slot0 + (uint32_t)r * 128 + (uint32_t)((((2 * cq + c) ^ (r & 7))) << 4);
-            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(pair(w4 & 0xFFu)), "r"(pair((w4 >> 8) & 0xFFu)),
-                         "r"(pair((w4 >> 16) & 0xFFu)), "r"(pair(w4 >> 24))
-                         : "memory");
-          }
-        }
-      }
+      decode_rows64<WB>(slot0 + W_BYTES - CODE_BYTES, slot0, hf * 64, lane, [&] { asm volatile("bar.sync %0, 64;" ::"r"(1 + s) : "memory"); });
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the tensor core's reads
     __syncthreads();

@@ -27,7 +27,7 @@
 #include "kernels.h"
 #include "ptx.cuh"
 #include "tc.cuh"
-#include "tmap.h"
+#include "tc_pair.cuh"
 
 namespace phyai {
 namespace {
@@ -44,31 +44,6 @@ constexpr int BAR_EPI = 1;
 constexpr int PG_PITCH = 36, PG_STG = 16 * PG_PITCH;      // staging block of an epilogue warp: [16 tokens][32 rows + 4] floats
 constexpr size_t PG_STG_BYTES = (size_t)16 * PG_STG * 4;
 constexpr size_t PG_SMEM_MAX = 227 * 1024 - 11 * 1024;   // dynamic shared memory (the static tables take the rest)
-constexpr uint32_t LEADER_MASK = 0xFEFFFFFFu;     // clears the CTA-rank bit of a shared::cluster address: the pair's even CTA
-
-__device__ __forceinline__ void tma2d(uint32_t dst, const CUtensorMap* map, int row, uint32_t bar_leader) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(bar_leader)
-      : "memory");
-}
-__device__ __forceinline__ void umma2_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// arrives on the barrier at this offset in both CTAs once every MMA issued so far has completed
-__device__ __forceinline__ void umma2_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-               "h"((uint16_t)3)
-               : "memory");
-}
-__device__ __forceinline__ void pair_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -145,8 +120,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
   unsigned long long* const trc = g.trace ? g.trace + (size_t)blockIdx.x * 16 : nullptr;
   if (threadIdx.x == 0) trace_stamp(trc, 0);
   if (threadIdx.x == 32) {      // (the first copy would otherwise wait for its map)
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmw)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
+    prefetch_tmap(&tmw), prefetch_tmap(&tmx);
   }
   const uint32_t tiles = (smem_u32(smem_raw) + 1023u) & ~1023u;
   if (threadIdx.x == 0) {
@@ -162,8 +136,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == PG_PROD) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    tmem_alloc2(smem_u32(&tmem_slot), 512);
     tc_fence_before();
   }
   __syncthreads();
@@ -514,23 +487,13 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
   pair_sync();
   if (warp == PG_PROD) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+    tmem_dealloc2(tmem_base, 512);
     if (lane == 0 && trc) {
       unsigned long long tt;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(tt)::"memory");
       trc[8] = tt;
     }
   }
-}
-
-// `rows` rows of 64 bf16 (128 bytes), fetched `box` rows at a time
-bool row_map(CUtensorMap* m, const void* base, uint64_t rows, uint32_t box) {
-  const EncodeTiled enc = encode_tiled();
-  if (!enc) return false;
-  const cuuint64_t dims[2] = {64, rows}, strides[1] = {128};
-  const cuuint32_t bx[2] = {64, box}, es[2] = {1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int EPI, bool HALF, int CPS>

@@ -427,6 +427,9 @@ cudaError_t launch_step_b1(int* status, const StepB1& p, cudaStream_t st);
 int b1_pick_cluster(int tiles, int KC, int n_sm);
 bool b1_gemm_supported(int N, int K, int C, int n_sm, bool qkv);
 cudaError_t launch_b1_gemm(int* status, const B1Gemm& g, int C, cudaStream_t st);
+// The same projections on CTA pairs (gemm_b1_pair.cu); ss_out then holds [N/64][64] partial sums.  Ranges: see there.
+int b1_pair_ranges(int N, int K, int n_sm, int epi);
+cudaError_t launch_b1_pair_gemm(int* status, const B1Gemm& g, int ranges, cudaStream_t st);
 // out[n] = scale(n) * sum_k shift[k] * W[n][k] for the packed rows n < N of a packed matrix with K / 64 chunks.
 // interleaved = 1: the rows are gate / up channels interleaved in groups of 64 (scale per gate channel f = wscale[f],
 // per up channel wscale2[f]); otherwise scale(n) = wscale[n].  Null scales mean 1.

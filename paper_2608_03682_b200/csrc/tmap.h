@@ -21,4 +21,14 @@ inline EncodeTiled encode_tiled() {
   return fn;
 }
 
+// `rows` rows of 64 bf16 (128 bytes), fetched `box` rows at a time
+inline bool row_map(CUtensorMap* m, const void* base, uint64_t rows, uint32_t box) {
+  const EncodeTiled enc = encode_tiled();
+  if (!enc) return false;
+  const cuuint64_t dims[2] = {64, rows}, strides[1] = {128};
+  const cuuint32_t bx[2] = {64, box}, es[2] = {1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace phyai

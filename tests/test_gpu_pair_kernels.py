@@ -40,6 +40,17 @@ def test_pair_gemms_at_the_edges_of_their_token_tiles(cond, dtype, horizon, batc
     check(cfg, [(37 * b) % 121 for b in range(batch)], 2, {0, batch // 2, batch - 1})
 
 
+@pytest.mark.parametrize("cond,dtype,width,mlp,horizon,batch", [
+    ("pi0", "bf16", 256, 512, 1, 1), ("pi05", "w8e4m3", 512, 1024, 16, 4), ("pi0", "w4a16", 384, 640, 15, 3),
+    ("pi05", "bf16", 1024, 4096, 33, 1), ("pi0", "w8e4m3", 1024, 1152, 63, 1), ("pi0", "bf16", 1152, 1280, 20, 3)])
+def test_single_tile_projections_on_pairs(cond, dtype, width, mlp, horizon, batch):
+    """Fewest and most tokens of the tile, uneven k-ranges, all three weight codings, contractions up to and past one pair's
+    (past it: both kernel families in one layer)."""
+    cfg = small_bf16_config(cond, dtype=dtype, width=width, mlp_dim=mlp, horizon=horizon, max_batch=batch, max_prefix_len=200)
+    for pair in (1, 0):
+        check(cfg, [(200, 77, 0, 128)[b] for b in range(batch)], 2, range(batch), use_b1_pair=pair)
+
+
 @pytest.mark.parametrize("cond,action_dim,width,horizon,batch", [("pi05", 33, 768, 60, 20), ("pi0", 7, 1280, 37, 32), ("pi05", 1, 256, 61, 2)])
 def test_step_boundary_row_groups(cond, action_dim, width, horizon, batch):
     """Sixteen rows per block from 1185 action rows on, four below; ragged last groups; action widths around a warp's lanes."""
