@@ -456,11 +456,11 @@ def main():
             name = f"C5b{b5}"
             r5 = run_workload(name, e5, c5, l5[:b5], n5, in5, Ko if b5 < 256 else min(Ko, 5), Wo, world, rank, local_rank,
                               e2e=(b5 <= 64))
-            if b5 == 1:   # the single-tile path streams the e4m3 bytes; for comparison: the bf16 images made at create
-                e5.set_option("use_w8_inkernel", 0)
-                r5["ms_per_step_bf16_images"] = run_workload(name, e5, c5, l5[:b5], n5, in5, Ko, Wo, world, rank, local_rank,
-                                                             e2e=False)["ms_per_step"]
+            if b5 == 1:   # the single-tile path reads the bf16 images made at create; for comparison: streaming the e4m3 codes
                 e5.set_option("use_w8_inkernel", 1)
+                r5["ms_per_step_codes"] = run_workload(name, e5, c5, l5[:b5], n5, in5, Ko, Wo, world, rank, local_rank,
+                                                             e2e=False)["ms_per_step"]
+                e5.set_option("use_w8_inkernel", 0)
             r5["workload"], r5["steps"], r5["warmup"] = describe(name, c5, b5, l5[:b5], n5), Ko, Wo
             r5["roofline"] = roofline_of(name, c5, l5[:b5], n5, b5, r5["ms_per_step"], peaks)
             others[name] = r5
@@ -479,13 +479,13 @@ def main():
         e6.close()
         del in5
         torch.cuda.empty_cache()
-        # the same expert with 4-bit integer weights at batch 1: the cluster path streams half a byte per weight
+        # the same expert with 4-bit integer weights at batch 1 (images; for comparison: half a byte per weight)
         c7, id7, _, l7, n7 = workload("C7b1")
         e7 = make_expert(c7, id7)
         in7 = Inputs(c7, id7, l7)
         r7 = run_workload("C7b1", e7, c7, l7, n7, in7, Ko, Wo, world, rank, local_rank, e2e=False)
-        e7.set_option("use_w8_inkernel", 0)
-        r7["ms_per_step_bf16_images"] = run_workload("C7b1", e7, c7, l7, n7, in7, Ko, Wo, world, rank, local_rank,
+        e7.set_option("use_w8_inkernel", 1)
+        r7["ms_per_step_codes"] = run_workload("C7b1", e7, c7, l7, n7, in7, Ko, Wo, world, rank, local_rank,
                                                      e2e=False)["ms_per_step"]
         r7["workload"], r7["steps"], r7["warmup"] = describe("C7b1", c7, 1, l7, n7), Ko, Wo
         r7["roofline"] = roofline_of("C7b1", c7, l7, n7, 1, r7["ms_per_step"], peaks)

@@ -230,8 +230,9 @@ phyai_status_t phyai_poll_status(phyai_expert_t *h);
  * the four projections on the cluster split-K kernel; key "use_b1_pair": 1 (default) runs those whose cluster size is not
  * chosen by hand on CTA pairs where they fit (one k-range up to a contraction of 1024).  key "use_b1_attention": 1 (default) lets those calls use
  * the cluster tcgen05 attention kernel (head_dim 128 / 256, even head and group counts), 0 keeps the mma.sync
- * cluster kernel.  key "use_w8_inkernel": 1 (default) streams PHYAI_DTYPE_FP8_E4M3 weights as bytes and decodes
- * them inside the cluster GEMM, 0 reads the bf16 images made at create (bit-identical results, twice the bytes).
+ * cluster kernel.  key "use_w8_inkernel": 1 streams weight codes (e4m3, int4) and decodes them inside the
+ * cluster GEMM, 0 (default) reads the bf16 images made at create (bit-identical results, faster, two to four times the
+ * bytes).
  * key "use_state_cache": 1 lets a block-causal expert (Sec. "adapters"; the state tokens see only the prefix and
  * themselves, so their keys and values do not change over the steps) run its state tokens once per call and the
  * loop on the action tokens only; 0 (default) runs every suffix token in every step, which is faster as long as the

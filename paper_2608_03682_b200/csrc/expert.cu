@@ -97,7 +97,12 @@ struct phyai_expert {
   int use_state_cache = 0;     // block-causal experts: state token computed once per call (single-tile calls); exact, but at
                                // one request the 18-layer state pass costs more than the 51st row it saves (measured)
   __nv_bfloat16 *kr_st = nullptr, *vr_st = nullptr;   // [L][max 64 tokens worth of requests][Hkv][S][dh] suffix K / V per layer
-  int use_w8_inkernel = 1;     // e4m3 experts: the cluster GEMM decodes byte blocks itself (0: bf16 images made at create)    // tcgen05 attention with the key range split over a cluster (few requests)
+  // Weight codes of single-tile calls: 0 = the bf16 images made at create (the other token counts need them as well), 1 = the
+  // GEMM kernels decode blocks of codes.  The loop is bound by its chain of kernels, not by bytes, and the decode (about 1 us
+  // of shared-memory traffic) lies on it for every CTA that starts late: pi0 with e4m3 codes 5.09 ms with images, 5.76 with
+  // codes, 5.15 with codes in the QKV projection alone.
+  int use_w8_inkernel = 0;
+    // tcgen05 attention with the key range split over a cluster (few requests)
   int use_b1_pair = 1;         // single-tile calls: projections on CTA pairs where they fit
   int b1_c[4] = {0, 0, 0, 0};  // cluster sizes of the QKV / O / gate-up / down projections (0 = choose)
   float *ss_a = nullptr, *ss_b = nullptr;   // [D/128 or D/64][64] partial sums of squares of h (after O / after down)
