@@ -132,6 +132,20 @@ __device__ __forceinline__ float gelu_fast(float z, int exact) {
   return fmaf(hz, t, hz);
 }
 
+// a[i] = GELU(a[i]) b[i].  One test of the form for all of them: tested per element, the erf code stood between the elements
+// and every one of them jumped across it (in a captured loop a kernel's code has left the instruction caches by the next
+// layer: ten-step loop of four requests 9.42 -> 9.21 ms, of 16 pi0.5 requests 12.70 -> 12.38).
+template <int N>
+__device__ __forceinline__ void gelu_mul(float (&a)[N], const float (&b)[N], int exact) {
+  if (__builtin_expect(exact != 0, 0)) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = gelu_erf_f(a[i]) * b[i];
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) a[i] = gelu_fast(a[i], 0) * b[i];
+  }
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -305,9 +305,10 @@ __global__ void __launch_bounds__(BP_THREADS, 1)
       float4 lo = fin4(lds4(sp), s0, rstd, h0), hi = fin4(lds4(sp + 128), s1, rstd, h1);
       if constexpr (EPI == B1_GEGLU) {
         // one 64-wide k-chunk (`tile`) of the down projection's activation tile, in halves of its swizzled 16-byte groups
-        const float4 m = make_float4(gelu_fast(lo.x, g.gelu_exact) * hi.x, gelu_fast(lo.y, g.gelu_exact) * hi.y,
-                                     gelu_fast(lo.z, g.gelu_exact) * hi.z, gelu_fast(lo.w, g.gelu_exact) * hi.w);
-        *reinterpret_cast<uint2*>(g.out_tiled + ((size_t)tile * 64 + tok) * 64 + (((j0 >> 3) ^ (tok & 7)) << 3) + (j0 & 7)) = pack4(m);
+        float m[4] = {lo.x, lo.y, lo.z, lo.w};
+        const float up[4] = {hi.x, hi.y, hi.z, hi.w};
+        gelu_mul(m, up, g.gelu_exact);
+        *reinterpret_cast<uint2*>(g.out_tiled + ((size_t)tile * 64 + tok) * 64 + (((j0 >> 3) ^ (tok & 7)) << 3) + (j0 & 7)) = make_uint2(pack2(m[0], m[1]), pack2(m[2], m[3]));
       } else if (rot_tile) {
         const int nn = isq ? n0 : n0 - Nq, head = nn / g.dh, t64 = (nn - head * g.dh) >> 7, half = g.dh >> 1;
         const float osc = isq ? rsqrtf((float)g.dh) : 1.0f;

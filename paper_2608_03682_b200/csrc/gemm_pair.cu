@@ -411,8 +411,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
             }
           }
           if constexpr (EPI == PG_GEGLU) {
-#pragma unroll
-            for (int e = 0; e < 16; ++e) a[e] = gelu_fast(a[e], g.gelu_exact) * b[e];
+            gelu_mul(a, b, g.gelu_exact);
           } else if constexpr (EPI == PG_QKV) {
             if (do_rot) {
 #pragma unroll
