@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       mbar_init(smem_u32(&k_full[i]), 2), mbar_init(smem_u32(&v_full[i]), 2), mbar_init(smem_u32(&p_full[i][0]), 8), mbar_init(smem_u32(&p_full[i][1]), 8);
       mbar_init(smem_u32(&s_full[i]), 1), mbar_init(smem_u32(&pv_done[i]), 1);
     }
-    mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 1), mbar_init(smem_u32(&q_ready), 2);
+    mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 8), mbar_init(smem_u32(&q_ready), 1);
     if (C > 1 && n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * (L::PITCH + 16)));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -174,11 +174,6 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
             : "memory");
       }
     };
-    if (lt == 0) {
-      // (the map was written into the request block by the kernel at the head of the call)
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(a.rq->kv_map) : "memory");
-      for (int t = n_mix; t < 2 && t < T; ++t) issue_full(t);        // constants of the call: ahead of the dependency wait
-    }
     // ---- mixed tiles: row by row
     const int chunks = is_v ? DH / 16 : DH / 8, rstep = 64 / chunks;     // 16-byte chunks per row of this stream
     const int lc = lt % chunks, r0 = lt / chunks;
@@ -208,19 +203,17 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
           for (; row < rows; row += rstep) asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(dst_of(t, row)), "r"(0u) : "memory");
       }
     };
+    // Constants of the call, ahead of the dependency wait, in the order of their use (an SM takes in 64 KB per 0.55 us: what
+    // is asked for first arrives first).
     for (int t = 0; t < n_mix; ++t) gather(t, true);
+    if (lt == 0) {
+      // (the map was written into the request block by the kernel at the head of the call)
+      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(a.rq->kv_map) : "memory");
+      for (int t = n_mix; t < 2 && t < T; ++t) issue_full(t);
+    }
+    __syncwarp();
     pdl_wait();
     if (T > 0) {
-      if (lane == 0) {
-        // Q (rotated, scaled) was written by the QKV projection as this CTA's operand tile: eight bulk copies
-        if (warp == 0) mbar_expect_tx(smem_u32(&q_bar), L::QTILE);
-        const uint8_t* qt = reinterpret_cast<const uint8_t*>(a.qr) + (size_t)(b * (d.Hq >> 1) + (head0 >> 1)) * L::QTILE;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          constexpr uint32_t QP = L::QTILE / 8;
-          bulk_g2s(Qs + (uint32_t)(2 * warp + u) * QP, qt + (size_t)(2 * warp + u) * QP, QP, smem_u32(&q_bar));
-        }
-      }
       for (int t = 0; t < n_mix; ++t) gather(t, false);
       if (n_mix > 0) {
         cp_async_commit();
@@ -230,10 +223,6 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       }
       if (lt == 0) {
         for (int t = 0; t < n_mix; ++t) remote_arrive(full0 + (uint32_t)t * 8u);
-        if (!is_v) {
-          mbar_wait_drain(smem_u32(&q_bar), 0u, wc);
-          remote_arrive(map_rank(smem_u32(&q_ready), lead_rank));
-        }
         for (int t = n_mix > 2 ? n_mix : 2; t < T; ++t) {
           mbar_wait_drain(smem_u32(is_v ? &pv_done[t & 1] : &s_full[t & 1]), (uint32_t)((t - 2) >> 1) & 1u, wc);
           issue_full(t);
@@ -243,6 +232,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     }
     if (C > 1) cluster_arrive();
   } else if (warp == 4) {
+    const WaitCtx wm{a.status, &abort_flag, a.wait_limit};
     // =========================== MMA issuer (leader CTA): S(0), S(1), then P(t) V(t), S(t + 2) ======================
     pdl_wait();
     if (lane == 0) {
@@ -251,7 +241,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     }
     if (half == 0) {
       auto issue_s = [&](int t) {
-        mbar_wait_drain(smem_u32(&k_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        mbar_wait_drain(smem_u32(&k_full[t & 1]), (uint32_t)(t >> 1) & 1u, wm);
         tc_fence_after();
         const uint32_t kb = Ks + (uint32_t)(t & 1) * L::KTILE;
 #pragma unroll
@@ -264,19 +254,20 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         __syncwarp();
       };
       if (T > 0) {
-        mbar_wait_drain(smem_u32(&q_ready), 0u, wc);      // both CTAs' Q tiles have landed
+        mbar_wait_drain(smem_u32(&q_bar), 0u, wm);        // both CTAs' Q tiles have landed
+        mbar_wait_drain(smem_u32(&q_ready), 0u, wm);
         issue_s(0);
       }
       if (lane == 0) trace_stamp(trc, 3);
       if (T > 1) issue_s(1);
       for (int t = 0; t < T; ++t) {
-        mbar_wait_drain(smem_u32(&v_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        mbar_wait_drain(smem_u32(&v_full[t & 1]), (uint32_t)(t >> 1) & 1u, wm);
         const uint32_t vb = Vs + (uint32_t)(t & 1) * L::VTILE;
         // (the first 64 keys' probabilities are ready before the others': their half of the product hides under the rest of
         // the softmax)
 #pragma unroll
         for (int kh = 0; kh < 2; ++kh) {
-          mbar_wait_drain(smem_u32(&p_full[t & 1][kh]), (uint32_t)(t >> 1) & 1u, wc);
+          mbar_wait_drain(smem_u32(&p_full[t & 1][kh]), (uint32_t)(t >> 1) & 1u, wm);
           tc_fence_after();
 #pragma unroll
           for (int kj = 0; kj < KB / 32; ++kj) {
@@ -292,6 +283,11 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         if (t == 0 && lane == 0) trace_stamp(trc, 4);
       }
       if (lane == 0) trace_stamp(trc, 5);
+    } else if (T > 0) {
+      if (lane == 0) {
+        mbar_wait_drain(smem_u32(&q_bar), 0u, wm);
+        remote_arrive(map_rank(smem_u32(&q_ready), lead_rank));
+      }
     }
     __syncwarp();
     if (C > 1) cluster_arrive();
@@ -306,6 +302,15 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     const uint32_t pfull0 = map_rank(smem_u32(&p_full[0][g]), lead_rank);
     float m = -INFINITY, l = 0.f;             // running maximum (log2 units) and sum
     pdl_wait();
+    if (T > 0 && lane == 0) {
+      // Q (rotated, scaled) was written by the QKV projection as this CTA's operand tile: an eighth per warp (the copies of
+      // one warp complete one after the other)
+      constexpr uint32_t QP = L::QTILE / 8;
+      const uint32_t off = (uint32_t)(warp - 5) * QP;
+      mbar_expect_tx(smem_u32(&q_bar), QP);
+      bulk_g2s(Qs + off, reinterpret_cast<const uint8_t*>(a.qr) + (size_t)(b * (d.Hq >> 1) + (head0 >> 1)) * L::QTILE + off, QP, smem_u32(&q_bar));
+    }
+    __syncwarp();
     const bool skip = status_set(a.status);
     for (int t = 0; t < T; ++t) {
       const uint32_t sb = tmem_s + (uint32_t)(t & 1) * KB + lane_addr;

@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       }
     }
   } else if (warp == PG_PROD) {
+    const WaitCtx wm{status, &abort_flag, g.wait_limit};
     // ---------------- MMA issuer (whole warp in the loop, one elected lane issues) --------------------------------
     if (rank == 0) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NT >> 3) << 17) | ((HALF ? 128u : 256u) >> 4) << 24;
@@ -189,11 +190,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       for (int i = 0; i < n_my && !dead; ++i) {
         const int buf = i & 1;
         // the epilogue warps of both CTAs have read the accumulator that this tile overwrites (two tiles ago)
-        if (mbar_wait_drain(smem_u32(&bar_tempty[buf]), (((uint32_t)i >> 1) & 1u) ^ 1u, wc) < 0) break;
+        if (mbar_wait_drain(smem_u32(&bar_tempty[buf]), (((uint32_t)i >> 1) & 1u) ^ 1u, wm) < 0) break;
         tc_fence_after();
         const uint32_t tacc = tmem_base + (uint32_t)buf * 256u;
         for (int k = 0; k < KS; ++k, ++gi) {
-          if (mbar_wait_drain(smem_u32(&bar_full[s]), ph, wc) < 0) {
+          if (mbar_wait_drain(smem_u32(&bar_full[s]), ph, wm) < 0) {
             dead = true;   // (copies that never landed: nothing more can be done with this pipeline)
             break;
           }
