@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(&tmem_slot), 0);
   const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + 2 * KB;
-  const WaitCtx wc{a.status, &abort_flag, a.wait_limit, true};
+  const WaitCtx wc{a.status, &abort_flag, a.wait_limit};
 
   // Keys of this range: a share of the prefix keys followed by a share of the request's own (suffix) keys.  (The request
   // block is written before the captured loop starts: safe to read ahead of the dependency wait.  A call whose lengths are
@@ -232,7 +232,6 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     }
     if (C > 1) cluster_arrive();
   } else if (warp == 4) {
-    const WaitCtx wm{a.status, &abort_flag, a.wait_limit};
     // =========================== MMA issuer (leader CTA): S(0), S(1), then P(t) V(t), S(t + 2) ======================
     pdl_wait();
     if (lane == 0) {
@@ -241,7 +240,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     }
     if (half == 0) {
       auto issue_s = [&](int t) {
-        mbar_wait_drain(smem_u32(&k_full[t & 1]), (uint32_t)(t >> 1) & 1u, wm);
+        mbar_wait_drain(smem_u32(&k_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
         tc_fence_after();
         const uint32_t kb = Ks + (uint32_t)(t & 1) * L::KTILE;
 #pragma unroll
@@ -254,20 +253,20 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         __syncwarp();
       };
       if (T > 0) {
-        mbar_wait_drain(smem_u32(&q_bar), 0u, wm);        // both CTAs' Q tiles have landed
-        mbar_wait_drain(smem_u32(&q_ready), 0u, wm);
+        mbar_wait_drain(smem_u32(&q_bar), 0u, wc);        // both CTAs' Q tiles have landed
+        mbar_wait_drain(smem_u32(&q_ready), 0u, wc);
         issue_s(0);
       }
       if (lane == 0) trace_stamp(trc, 3);
       if (T > 1) issue_s(1);
       for (int t = 0; t < T; ++t) {
-        mbar_wait_drain(smem_u32(&v_full[t & 1]), (uint32_t)(t >> 1) & 1u, wm);
+        mbar_wait_drain(smem_u32(&v_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
         const uint32_t vb = Vs + (uint32_t)(t & 1) * L::VTILE;
         // (the first 64 keys' probabilities are ready before the others': their half of the product hides under the rest of
         // the softmax)
 #pragma unroll
         for (int kh = 0; kh < 2; ++kh) {
-          mbar_wait_drain(smem_u32(&p_full[t & 1][kh]), (uint32_t)(t >> 1) & 1u, wm);
+          mbar_wait_drain(smem_u32(&p_full[t & 1][kh]), (uint32_t)(t >> 1) & 1u, wc);
           tc_fence_after();
 #pragma unroll
           for (int kj = 0; kj < KB / 32; ++kj) {
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       if (lane == 0) trace_stamp(trc, 5);
     } else if (T > 0) {
       if (lane == 0) {
-        mbar_wait_drain(smem_u32(&q_bar), 0u, wm);
+        mbar_wait_drain(smem_u32(&q_bar), 0u, wc);
         remote_arrive(map_rank(smem_u32(&q_ready), lead_rank));
       }
     }
