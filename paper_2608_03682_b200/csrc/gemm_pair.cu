@@ -17,7 +17,7 @@
 // Norms are folded into the projections either side, as in gemm_b1.cu: X holds bf16(h * gain), the accumulator columns
 // are multiplied by rsqrt(mean h^2 + eps) of their token (from partial sums of squares), a shift enters as the
 // per-channel constant shift . W; the residual epilogue writes h, the next projection's operand and its partial sums of
-// squares (one per 128 channels and token).  No split-K and no atomics: a request gives the same bits every time.
+// squares (one per 64 channels and token).  No split-K and no atomics: a request gives the same bits every time.
 //
 // Roles: warps 0-3 issue the copies (k-step i by warp i % 4), warp 4 issues the MMAs (leader CTA), the 16 warps from 5
 // on are the epilogue (tensor-memory lane quarter = warp % 4).  Every wait is
