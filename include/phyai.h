@@ -199,13 +199,17 @@ phyai_status_t phyai_denoise_batched_host(phyai_expert_t *h, uint32_t batch, con
  *   prefix_kvs   HOST array of HOST pointers, [n_layers][2][prefix_lens[b]][n_kv_heads][head_dim] (NULL for an empty prefix)
  *   states, noises  HOST arrays of HOST pointers, float32 [state_dim] / [horizon, action_dim]; a NULL entry means zeros
  *   out_actions  HOST, float32 [batch, horizon, action_dim] (pinned memory makes the copy asynchronous)
- * The call gathers the requests into page-locked staging of the handle (on a few threads of the handle's own, the copies
- * to the device following plane by plane), runs the batched kernels and copies the actions back on `stream`.  The inputs
- * are not read after it returns; the result is valid after the stream is synchronised.
+ *   staging      HOST, page-locked, phyai_requests_staging_bytes(h, batch, sum of prefix_lens) bytes: the caller's until the
+ *                call's copies have run on `stream` (a buffer per call lets the next call gather while this one computes)
+ * The call gathers the requests into `staging` (on a few threads of the handle's own, the copies to the device following
+ * plane by plane), runs the batched kernels and copies the actions back on `stream`.  The inputs are not read after it
+ * returns; the result is valid after the stream is synchronised.
  */
+uint64_t phyai_requests_staging_bytes(const phyai_expert_t* h, uint32_t batch, uint64_t kv_tokens);
 phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, const void* const* prefix_kvs,
                                            const uint32_t* prefix_lens, const float* const* states,
-                                           const float* const* noises, uint32_t n_steps, float* out_actions, void* stream);
+                                           const float* const* noises, uint32_t n_steps, float* out_actions, void* staging,
+                                           uint64_t staging_bytes, void* stream);
 
 /*
  * After the stream has been synchronised: read and clear the handle's device status word.

@@ -26,7 +26,7 @@ BIG = ("wq", "wk", "wv", "wo", "wgate", "wup", "wdown")
 
 #: every symbol the header declares
 EXPORTS = ("phyai_expert_create", "phyai_expert_destroy", "phyai_prefix_kv_bytes", "phyai_denoise",
-           "phyai_denoise_batched", "phyai_denoise_host", "phyai_denoise_batched_host", "phyai_denoise_requests_host", "phyai_poll_status",
+           "phyai_denoise_batched", "phyai_denoise_host", "phyai_denoise_batched_host", "phyai_denoise_requests_host", "phyai_requests_staging_bytes", "phyai_poll_status",
            "phyai_set_option", "phyai_launches_per_call", "phyai_last_error", "phyai_version",
            "phyai_suffix_attention", "phyai_suffix_attention_scratch_bytes", "phyai_op_last_error",
            "phyai_suffix_attention_static", "phyai_suffix_attention_static_capacity", "phyai_read_trace",
@@ -105,7 +105,8 @@ def load_library() -> C.CDLL:
     lib.phyai_denoise_host.argtypes = single
     lib.phyai_denoise_batched.argtypes = batched
     lib.phyai_denoise_batched_host.argtypes = batched
-    lib.phyai_denoise_requests_host.argtypes = [_VP, C.c_uint32, _VP, _VP, _VP, _VP, C.c_uint32, _VP, _VP]
+    lib.phyai_denoise_requests_host.argtypes = [_VP, C.c_uint32, _VP, _VP, _VP, _VP, C.c_uint32, _VP, _VP, C.c_uint64, _VP]
+    lib.phyai_requests_staging_bytes.argtypes, lib.phyai_requests_staging_bytes.restype = [_VP, C.c_uint32, C.c_uint64], C.c_uint64
     lib.phyai_poll_status.argtypes = [_VP]
     lib.phyai_set_option.argtypes = [_VP, C.c_char_p, C.c_int64]
     lib.phyai_read_trace.argtypes = [_VP, _VP, C.c_size_t, C.POINTER(C.c_uint32), C.POINTER(C.c_uint32)]
@@ -227,12 +228,14 @@ class Expert:
                 ws.scales[i] = C.cast(scale_arrays[m], _VPP)
         _check(self.lib.phyai_expert_create(C.byref(cs), C.byref(ws), _stream_ptr(stream), C.byref(self._handle)))
         del keep  # create has repacked everything and synchronised
+        self._staged = []  # (event, buffers) of host-request calls in flight
 
     # ------------------------------------------------------------------------------------------
     def close(self):
         if getattr(self, "_handle", None) is not None and self._handle.value:
             self.lib.phyai_expert_destroy(self._handle)
             self._handle = _VP()
+            self._staged = []
 
     def __del__(self):
         try:
@@ -285,7 +288,8 @@ class Expert:
 
     def denoise_requests_host(self, requests, n_steps: int, out: torch.Tensor, stream=None) -> torch.Tensor:
         """phyai_denoise_requests_host: ``requests`` = (prefix_kv or None, state or None, noise or None) per request, contiguous
-        host tensors of the expert's storage types; ``out`` [B,H,A] (ideally pinned) is complete once the stream is."""
+        host tensors of the expert's storage types; ``out`` [B,H,A] (ideally pinned) is complete once the stream is.  The staging
+        comes from torch's pool of page-locked memory (page-locking 60 MB anew for each handle takes 35 ms)."""
         B = len(requests)
         kv, st, nz = (_VP * B)(), (_VP * B)(), (_VP * B)()
         lens = (C.c_uint32 * B)()
@@ -293,7 +297,14 @@ class Expert:
             if k is not None and k.shape[2]:
                 kv[b], lens[b] = k.data_ptr(), k.shape[2]
             st[b], nz[b] = _ptr(s), _ptr(z)
-        _check(self.lib.phyai_denoise_requests_host(self._handle, B, kv, lens, st, nz, int(n_steps), _ptr(out), _stream_ptr(stream)))
+        # (the pool does not know of the library's copies: buffers stay referenced until they have run)
+        self._staged = [s for s in self._staged if not s[0].query()]
+        staging = torch.empty(self.lib.phyai_requests_staging_bytes(self._handle, B, sum(lens)), dtype=torch.uint8, pin_memory=True)
+        done = torch.cuda.Event()
+        _check(self.lib.phyai_denoise_requests_host(self._handle, B, kv, lens, st, nz, int(n_steps), _ptr(out), _ptr(staging),
+                                                    staging.numel(), _stream_ptr(stream)))
+        done.record(torch.cuda.current_stream() if stream is None else stream)
+        self._staged.append((done, staging, out))
         return out
 
     def poll_status(self) -> int:

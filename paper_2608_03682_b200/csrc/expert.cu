@@ -148,11 +148,7 @@ struct phyai_expert {
   float *stg_states = nullptr, *stg_noise = nullptr, *stg_out = nullptr;
   int* stg_cu = nullptr;
 
-  // requests in ordinary host memory: page-locked staging (grown on demand, freed with the handle) and the gather threads
-  void* pin_kv = nullptr; size_t pin_kv_bytes = 0;
-  float* pin_small = nullptr;            // cu | states | noise of max_batch requests
-  cudaEvent_t pin_free = nullptr;        // the last call's copies out of the staging have completed
-  phyai::HostPacker* packer = nullptr;
+  phyai::HostPacker* packer = nullptr;   // requests in ordinary host memory: the gather threads
 
   int use_graph = 1;
   unsigned wait_limit = 1u << 22;
@@ -1292,9 +1288,6 @@ void phyai_expert_destroy(phyai_expert_t* h) {
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   delete h->packer;
-  if (h->pin_kv) cudaFreeHost(h->pin_kv);
-  if (h->pin_small) cudaFreeHost(h->pin_small);
-  if (h->pin_free) cudaEventDestroy(h->pin_free);
   for (void* p : h->allocs) cudaFree(p);
   delete h;
 }
@@ -1363,14 +1356,20 @@ phyai_status_t phyai_denoise_batched_host(phyai_expert_t* h, uint32_t batch, con
   return PHYAI_OK;
 }
 
+// staging of a call: [planes][tokens][row] prefix caches, then states | noise | cumulative lengths
+uint64_t phyai_requests_staging_bytes(const phyai_expert_t* h, uint32_t batch, uint64_t kv_tokens) {
+  if (!h) return 0;
+  return phyai_prefix_kv_bytes(&h->cfg, kv_tokens) + (uint64_t)batch * (h->d.Ds + (uint64_t)h->d.H * h->d.A + 1) * 4 + 4;
+}
+
 phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, const void* const* prefix_kvs,
                                            const uint32_t* prefix_lens, const float* const* states, const float* const* noises,
-                                           uint32_t n_steps, float* out, void* stream) {
+                                           uint32_t n_steps, float* out, void* staging, uint64_t staging_bytes, void* stream) {
   if (!h) return fail(PHYAI_ERR_INVALID_ARG, "handle is NULL");
   if (batch == 0 || batch > h->cfg.max_batch)
     return fail(PHYAI_ERR_INVALID_ARG, "batch %u outside 1..max_batch (%u)", batch, h->cfg.max_batch);
-  if (!prefix_kvs || !prefix_lens || !noises || !out || (h->cfg.has_state_token && !states))
-    return fail(PHYAI_ERR_INVALID_ARG, "prefix_kvs / prefix_lens / noises / out_actions (or states) is NULL");
+  if (!prefix_kvs || !prefix_lens || !noises || !out || !staging || (h->cfg.has_state_token && !states))
+    return fail(PHYAI_ERR_INVALID_ARG, "prefix_kvs / prefix_lens / noises / out_actions / staging (or states) is NULL");
   if (n_steps == 0 || n_steps > 1000) return fail(PHYAI_ERR_INVALID_ARG, "n_steps must be in 1..1000");
   size_t total = 0;
   for (uint32_t b = 0; b < batch; ++b) {
@@ -1378,29 +1377,22 @@ phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, co
     if (prefix_lens[b] && !prefix_kvs[b]) return fail(PHYAI_ERR_INVALID_ARG, "prefix_kvs[%u] is NULL", b);
     total += prefix_lens[b];
   }
+  if ((reinterpret_cast<uintptr_t>(staging) & 3) || staging_bytes < phyai_requests_staging_bytes(h, batch, total))
+    return fail(PHYAI_ERR_INVALID_ARG, "staging is too small (phyai_requests_staging_bytes) or not aligned to 4 bytes");
   ST(ensure_staging(h));
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const size_t B = h->cfg.max_batch, ha = (size_t)h->d.H * h->d.A, Ds = h->d.Ds;
+  const size_t ha = (size_t)h->d.H * h->d.A, Ds = h->d.Ds;
   const size_t kvb = phyai_prefix_kv_bytes(&h->cfg, total);
-  if (!h->pin_free) CU(cudaEventCreateWithFlags(&h->pin_free, cudaEventDisableTiming));
-  if (!h->pin_small) CU(cudaHostAlloc(reinterpret_cast<void**>(&h->pin_small), (B + 1 + B * Ds + B * ha) * 4, cudaHostAllocDefault));
-  CU(cudaEventSynchronize(h->pin_free));         // the last call's copies (complete unless that call is still in flight)
-  if (kvb > h->pin_kv_bytes) {
-    if (h->pin_kv) CU(cudaFreeHost(h->pin_kv));
-    h->pin_kv = nullptr, h->pin_kv_bytes = 0;
-    const size_t want = std::min(kvb + kvb / 4, h->stg_kv_bytes);
-    CU(cudaHostAlloc(&h->pin_kv, want, cudaHostAllocDefault));
-    h->pin_kv_bytes = want;
-  }
+  uint8_t* const pin_kv = static_cast<uint8_t*>(staging);
   const int planes = 2 * h->d.L;
   const size_t plane = kvb / planes;
   if (kvb) {
     if (!h->packer) h->packer = new (std::nothrow) phyai::HostPacker();
     if (!h->packer) return fail(PHYAI_ERR_OOM, "host allocation failed");
-    h->packer->start(static_cast<uint8_t*>(h->pin_kv), prefix_kvs, prefix_lens, (int)batch, planes, plane / total);
+    h->packer->start(pin_kv, prefix_kvs, prefix_lens, (int)batch, planes, plane / total);
   }
-  int32_t* cu = reinterpret_cast<int32_t*>(h->pin_small);
-  float *ps = h->pin_small + B + 1, *pn = ps + B * Ds;
+  float *ps = reinterpret_cast<float*>(pin_kv + kvb), *pn = ps + batch * Ds;
+  int32_t* cu = reinterpret_cast<int32_t*>(pn + batch * ha);
   cu[0] = 0;
   for (uint32_t b = 0; b < batch; ++b) {
     cu[b + 1] = cu[b] + (int32_t)prefix_lens[b];
@@ -1421,10 +1413,8 @@ phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, co
       const int p0 = planes * q / pieces, p1 = planes * (q + 1) / pieces;
       if (p1 == p0) continue;
       h->packer->wait(p1);
-      CU(cudaMemcpyAsync(static_cast<uint8_t*>(h->stg_kv) + p0 * plane, static_cast<uint8_t*>(h->pin_kv) + p0 * plane, (p1 - p0) * plane,
-                         cudaMemcpyHostToDevice, st));
+      CU(cudaMemcpyAsync(static_cast<uint8_t*>(h->stg_kv) + p0 * plane, pin_kv + p0 * plane, (p1 - p0) * plane, cudaMemcpyHostToDevice, st));
     }
-    CU(cudaEventRecord(h->pin_free, st));
     return PHYAI_OK;
   }();
   if (kvb) h->packer->wait(planes);              // (the caller's memory is not read after this call returns)
