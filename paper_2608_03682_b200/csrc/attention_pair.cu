@@ -316,12 +316,16 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     }
     __syncwarp();
     const bool skip = status_set(a.status);
-    for (int t = 0; t < T; ++t) {
+    // Turn -1 is a rehearsal, without effect, in the 3 - 4 us until the first logits exist: in a captured loop a kernel's code
+    // has left the instruction caches by the next layer, and the first softmax took 3.4 us instead of 1.7.
+    for (int t = T > 0 ? -1 : 0; t < T; ++t) {
       const uint32_t sb = tmem_s + (uint32_t)(t & 1) * KB + lane_addr;
-      if (lane == 0) mbar_wait_drain(smem_u32(&s_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
-      __syncwarp();
+      if (t >= 0) {
+        if (lane == 0) mbar_wait_drain(smem_u32(&s_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        __syncwarp();
+      }
       tc_fence_after();
-      if (C > 1 && t == T - 1) cluster_arrive();     // (the last logits exist: Q is dead, its area may receive partials)
+      if (C > 1 && t >= 0 && t == T - 1) cluster_arrive();     // (the last logits exist: Q is dead, its area may receive partials)
       // the visible keys of a row form a prefix of a mixed tile: the keys that exist, and for the state-token row under the
       // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
       int nvis = t >= m0 && t < m0 + n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - (t - m0) * KB) : KB;
@@ -355,7 +359,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
           rs4[e & 3] += e0 + e1;
           w[e] = pack_bf16(e0, e1);
         }
-        tmem_st16u(sb + (uint32_t)(g * 32 + c16 * 16), w);
+        if (t >= 0) tmem_st16u(sb + (uint32_t)(g * 32 + c16 * 16), w);
       }
       if (__any_sync(0xffffffffu, rescale)) {     // rare: rescale this warp's half rows of the accumulator
         if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(t - 1) & 1]), (uint32_t)((t - 1) >> 1) & 1u, wc);   // every P V so far
@@ -373,6 +377,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
+      if (t < 0) continue;
       if (lane == 0) remote_arrive(pfull0 + (uint32_t)(t & 1) * 16u);
       l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);      // (of this thread's half of the columns)
       m = m_new;
