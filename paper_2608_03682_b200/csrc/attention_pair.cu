@@ -16,9 +16,13 @@
 // the suffix keys); the partial results, rounded to bf16, are merged over distributed shared memory: row range p of every
 // head belongs to pair p, which adds the C partials in range order.  No partials in global memory, no merge launch.
 //
+// Measured at 8 requests of 816 + 51 keys and 8 heads (C = 3), from the projection's end to the merged output: 14 us (split
+// ranges of the one-CTA kernel 21 us, their merge launch 8): operands 2 - 3, 1.2 - 2 per key tile, merge 3.5.
+//
 // Warps of a CTA: 0-1 load K, 2-3 load V (full prefix tiles with tensor-map copies -- the map of the call's cache sits in
-// the request block --, the rest row by row with cp.async; prefix rows before the dependency wait), 4 issues the MMAs (leader CTA), 5-12 softmax, correction, output.  Every wait is bounded; after a
-// give-up the protocol runs to its end and only the global stores are skipped.
+// the request block --, the rest row by row with cp.async; prefix rows before the dependency wait), 4 issues the MMAs
+// (leader CTA), 5-12 fetch Q, softmax, correction, output.  Every wait is bounded; after a give-up the protocol runs to its
+// end and only the global stores are skipped.
 #include "attention.cuh"
 #include "tc.cuh"
 #include "tmap.h"

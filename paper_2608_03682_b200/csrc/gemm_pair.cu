@@ -19,6 +19,9 @@
 // per-channel constant shift . W; the residual epilogue writes h, the next projection's operand and its partial sums of
 // squares (one per 64 channels and token).  No split-K and no atomics: a request gives the same bits every time.
 //
+// Measured in the captured ten-step loops, against the one-CTA tile GEMMs and their norm launches: 4 requests 11.0 -> 9.1 ms
+// (with the attention's gains), 8: 12.8 -> 10.4, 64: 32.7 -> 29.4 (power-capped), 256: 117.6 -> 106.
+//
 // Roles: warps 0-3 issue the copies (k-step i by warp i % 4), warp 4 issues the MMAs (leader CTA), the 16 warps from 5
 // on are the epilogue (tensor-memory lane quarter = warp % 4).  Every wait is
 // bounded; after a give-up copies, MMAs, commits and barriers go on and only the stores are skipped.
