@@ -31,18 +31,43 @@ __global__ void __launch_bounds__(RW * 32) k_rows_f32(const int* status, const S
     }
   };
   fetch(k_lo);
-  pdl_wait();
-  if (status_set(status)) return;
-  // ---- the rows (RW / RM warps each), with the norm applied in place
-  constexpr int WPR = RW / RM;
+  // Every load is asked for as early as its address allows (the norm's and the epilogue's constants ahead of the dependency
+  // wait, the row and what the result is added to right after it): each one left where it is used costs a round trip to the L2
+  // (55 launches of the tiny expert 274 -> 254 us).  Eight rows per block are for grids of several blocks per SM, which hide
+  // the trips themselves and need the registers: there the norm's constants stay where they are used.
+  constexpr int WPR = RW / RM, RU = RM == 4 ? 8 : 4, RG = RM == 4 ? RU : 0;
   const int row = warp / WPR, t = (warp % WPR) * 32 + lane, m = m0 + row;
+  float gn[RG + 1], sf[RG + 1];
+#pragma unroll
+  for (int u = 0; u < RG; ++u) {
+    const int k = t + u * WPR * 32;
+    gn[u] = g.norm_gain && k < g.K ? g.norm_gain[k] : 0.f;
+    sf[u] = g.norm_gain && g.norm_shift && k < g.K ? g.norm_shift[k] : 0.f;
+  }
+  const int mm = m0 + warp, orow = (mm / g.rows_in) * g.rows_out + g.row_off + mm % g.rows_in;
+  const bool mine = warp < RM && col && mm < g.M;           // one output per thread of the first RM warps
+  float* const o = g.out + (size_t)orow * g.ldo + n;
+  float cst = 0.f, old = 0.f;
+  if (mine && !DUAL) {
+    if (g.epi == EPI_RESID) cst = g.gate ? g.gate[n] : 1.f;
+    else if (g.bias) cst = g.bias[n];
+  }
+  pdl_wait();
+  if (mine && !DUAL && g.epi == EPI_RESID) old = *o;
+  // ---- the rows (RW / RM warps each), with the norm applied in place
   const float* a = g.A + (size_t)min(m, g.M - 1) * g.lda;
   float ss = 0.f;
-  for (int k = t; k < g.K; k += WPR * 32) {
-    const float x = a[k];
-    As[row * g.K + k] = x;
-    ss = fmaf(x, x, ss);
+  for (int k0 = t; k0 < g.K; k0 += RU * WPR * 32) {
+    float x[RU];
+#pragma unroll
+    for (int u = 0; u < RU; ++u) x[u] = k0 + u * WPR * 32 < g.K ? a[k0 + u * WPR * 32] : 0.f;
+#pragma unroll
+    for (int u = 0; u < RU; ++u) {
+      if (k0 + u * WPR * 32 < g.K) As[row * g.K + k0 + u * WPR * 32] = x[u];
+      ss = fmaf(x[u], x[u], ss);
+    }
   }
+  if (status_set(status)) return;
   if (g.norm_gain) {
     ss = warp_sum(ss);
     if (lane == 0) ssp[warp] = ss;
@@ -51,7 +76,12 @@ __global__ void __launch_bounds__(RW * 32) k_rows_f32(const int* status, const S
 #pragma unroll
     for (int w = 0; w < WPR; ++w) tot += ssp[row * WPR + w];
     const float r = 1.0f / sqrtf(tot / (float)g.K + g.eps);
-    for (int k = t; k < g.K; k += WPR * 32) {
+#pragma unroll
+    for (int u = 0; u < RG; ++u) {
+      const int k = t + u * WPR * 32;
+      if (k < g.K) As[row * g.K + k] = fmaf(As[row * g.K + k] * r, gn[u], sf[u]);
+    }
+    for (int k = t + RG * WPR * 32; k < g.K; k += WPR * 32) {
       float v = As[row * g.K + k] * r * g.norm_gain[k];
       if (g.norm_shift) v += g.norm_shift[k];
       As[row * g.K + k] = v;
@@ -100,19 +130,17 @@ __global__ void __launch_bounds__(RW * 32) k_rows_f32(const int* status, const S
   }
   __syncthreads();
   // ---- one output per thread: the partial sums in range order, epilogue
-  if (warp >= RM || !col || m0 + warp >= g.M) return;
+  if (!mine) return;
   float v = 0.f, v2 = 0.f;
 #pragma unroll
   for (int w = 0; w < RW; ++w) {
     v += red[0][w][warp][lane];
     if (DUAL) v2 += red[DUAL ? 1 : 0][w][warp][lane];
   }
-  const int mm = m0 + warp, orow = (mm / g.rows_in) * g.rows_out + g.row_off + mm % g.rows_in;
-  float* o = g.out + (size_t)orow * g.ldo + n;
   if (DUAL) *o = gelu_f(v, g.gelu_exact) * v2;
-  else if (g.epi == EPI_RESID) *o = *o + (g.gate ? g.gate[n] * v : v);
-  else if (g.epi == EPI_SWISH) *o = swish_precise(v + (g.bias ? g.bias[n] : 0.f));
-  else *o = v + (g.bias ? g.bias[n] : 0.f);
+  else if (g.epi == EPI_RESID) *o = fmaf(cst, v, old);
+  else if (g.epi == EPI_SWISH) *o = swish_precise(v + cst);
+  else *o = v + cst;
 }
 
 // One (suffix row, query head) per block of eight warps.  Scores: a lane takes a key and its whole dot product (the key's
