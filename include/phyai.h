@@ -321,6 +321,12 @@ phyai_status_t phyai_suffix_attention(const phyai_attention_desc_t *desc, uint32
                                       const void *prefix_kv, uint64_t kv_tokens, const int32_t *cu_prefix_lens,
                                       const float *rope_cos_sin, uint16_t *out, int32_t *status_word, void *stream);
 
+/* The same, and the call clears the status word itself (in its first kernel, also at every replay of a captured call): for
+ * callers with a fresh word per call. */
+phyai_status_t phyai_suffix_attention_cleared(const phyai_attention_desc_t *desc, uint32_t batch, const float *qkv,
+                                              const void *prefix_kv, uint64_t kv_tokens, const int32_t *cu_prefix_lens,
+                                              const float *rope_cos_sin, uint16_t *out, int32_t *status_word, void *stream);
+
 /* Scratch bytes phyai_suffix_attention uses for this shape and batch (upper bound when num_splits is 0). */
 size_t phyai_suffix_attention_scratch_bytes(const phyai_attention_desc_t *desc, uint32_t batch);
 
@@ -379,7 +385,8 @@ phyai_status_t phyai_pack_prefix_kv(const phyai_kv_pack_desc_t *desc, const void
                                     void *stream);
 
 /* The same, and every row of prefix_kv that receives no request row is set to zero (the rows past the last request; after
- * an error all rows): for callers that would otherwise clear the whole buffer first. */
+ * an error all rows), and the status word needs no clearing, which the call does itself: for callers that would otherwise
+ * clear both first. */
 phyai_status_t phyai_pack_prefix_kv_cleared(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens,
                                             void* prefix_kv, uint64_t kv_tokens, int32_t* cu_prefix_lens,
                                             int32_t* status_word, void* stream);

@@ -8,7 +8,6 @@ from __future__ import annotations
 
 import ctypes as C
 import os
-import threading
 from typing import Dict, Optional, Sequence
 
 import numpy as np
@@ -28,7 +27,7 @@ BIG = ("wq", "wk", "wv", "wo", "wgate", "wup", "wdown")
 EXPORTS = ("phyai_expert_create", "phyai_expert_destroy", "phyai_prefix_kv_bytes", "phyai_denoise",
            "phyai_denoise_batched", "phyai_denoise_host", "phyai_denoise_batched_host", "phyai_denoise_requests_host", "phyai_requests_staging_bytes", "phyai_poll_status",
            "phyai_set_option", "phyai_launches_per_call", "phyai_last_error", "phyai_version",
-           "phyai_suffix_attention", "phyai_suffix_attention_scratch_bytes", "phyai_op_last_error",
+           "phyai_suffix_attention", "phyai_suffix_attention_cleared", "phyai_suffix_attention_scratch_bytes", "phyai_op_last_error",
            "phyai_suffix_attention_static", "phyai_suffix_attention_static_capacity", "phyai_read_trace",
            "phyai_pack_prefix_kv", "phyai_pack_prefix_kv_cleared", "phyai_postprocess_actions", "phyai_adapter_last_error", "phyai_batcher_create",
            "phyai_batcher_destroy", "phyai_batcher_submit", "phyai_batcher_next", "phyai_batcher_pending",
@@ -118,6 +117,7 @@ def load_library() -> C.CDLL:
     lib.phyai_suffix_attention.argtypes = [C.POINTER(AttentionDesc), C.c_uint32, _VP, _VP, C.c_uint64, _VP, _VP, _VP,
                                            _VP, _VP]
     lib.phyai_suffix_attention_static.argtypes = lib.phyai_suffix_attention.argtypes
+    lib.phyai_suffix_attention_cleared.argtypes = lib.phyai_suffix_attention.argtypes
     lib.phyai_suffix_attention_static_capacity.restype = C.c_size_t
     lib.phyai_pack_prefix_kv.argtypes = [C.POINTER(KvPackDesc), _VP, _VP, _VP, _VP, C.c_uint64, _VP, _VP, _VP]
     lib.phyai_pack_prefix_kv_cleared.argtypes = lib.phyai_pack_prefix_kv.argtypes
@@ -345,25 +345,6 @@ def attention_desc(n_q_heads, n_kv_heads, head_dim, suffix_len, n_layers, layer,
     return d
 
 
-_zero_words: Dict[tuple, list] = {}
-_zero_lock = threading.Lock()
-
-
-def _zero_word(device: torch.device, stream: int) -> torch.Tensor:
-    """A zeroed int32 device word for an operator's status.  Words come from blocks of 256, zeroed at a time on the stream
-    that uses them (a fill kernel per call cost as much as the launch it served); every word is handed out once, and a block
-    lives as long as its words.  At most 64 streams keep a block."""
-    key = (device.index, stream)
-    with _zero_lock:
-        block = _zero_words.get(key)
-        if not block:
-            if block is None and len(_zero_words) >= 64:
-                _zero_words.clear()
-            with torch.cuda.stream(torch.cuda.ExternalStream(stream, device=device) if stream else torch.cuda.default_stream(device)):
-                block = _zero_words[key] = list(torch.zeros(256, dtype=torch.int32, device=device).split(1))
-        return block.pop()
-
-
 def suffix_attention(desc: AttentionDesc, qkv: torch.Tensor, prefix_kv: torch.Tensor, cu_prefix_lens: torch.Tensor,
                      rope_cos_sin: Optional[torch.Tensor], entry: str = "phyai_suffix_attention", stream=None):
     """Stand-alone attention operator; returns (out bf16 [rows, Hq*dh], status_word int32 tensor)."""
@@ -372,7 +353,11 @@ def suffix_attention(desc: AttentionDesc, qkv: torch.Tensor, prefix_kv: torch.Te
     sp = _raw_stream(stream, device)
     batch = cu_prefix_lens.numel() - 1
     out = torch.empty(batch * desc.suffix_len, desc.n_q_heads * desc.head_dim, dtype=torch.bfloat16, device=device)
-    status = _zero_word(device, sp)
+    if entry == "phyai_suffix_attention":        # (the form whose first kernel clears the word: a launch less per call)
+        entry, status = "phyai_suffix_attention_cleared", torch.empty(1, dtype=torch.int32, device=device)
+    else:
+        with torch.cuda.stream(stream):
+            status = torch.zeros(1, dtype=torch.int32, device=device)
     st = getattr(lib, entry)(C.byref(desc), batch, qkv.data_ptr(), prefix_kv.data_ptr(), prefix_kv.shape[2],
                              cu_prefix_lens.data_ptr(), _ptr(rope_cos_sin), out.data_ptr(), status.data_ptr(), sp or None)
     if st != OK:
@@ -392,7 +377,7 @@ def pack_prefix_kv(k: torch.Tensor, v: torch.Tensor, lens: torch.Tensor, kv_toke
     desc = KvPackDesc(_KV_PACK_SIZE, L, Hkv, dh, k.element_size(), B, p_max)
     out = torch.empty(L, 2, kv_tokens, Hkv, dh, dtype=k.dtype, device=device)
     cu = torch.empty(B + 1, dtype=torch.int32, device=device)
-    status = _zero_word(device, sp)
+    status = torch.empty(1, dtype=torch.int32, device=device)
     st = lib.phyai_pack_prefix_kv_cleared(C.byref(desc), k.data_ptr(), v.data_ptr(), lens.data_ptr(), out.data_ptr(), int(kv_tokens),
                                           cu.data_ptr(), status.data_ptr(), sp or None)
     if st != OK:

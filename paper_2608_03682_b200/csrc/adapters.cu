@@ -14,8 +14,8 @@ namespace {
 thread_local char g_ad_err[256] = "";
 
 // cu[0] = 0, cu[b + 1] = cu[b] + lens[b]; a length outside 0..p_max or a total beyond kv_tokens raises the status word
-// (INVALID_ARG) and the pack kernel then copies nothing.  One block: a thread sums a run of lengths, the runs are scanned.
-__global__ void __launch_bounds__(1024) k_kv_scan(const int* lens, int batch, int p_max, unsigned long long kv_tokens, int* cu, int* status) {
+// (INVALID_ARG) and the pack kernel then copies nothing; with `clear` the word is written either way.  One block: a thread sums a run of lengths, the runs are scanned.
+__global__ void __launch_bounds__(1024) k_kv_scan(const int* lens, int batch, int p_max, unsigned long long kv_tokens, int* cu, int* status, int clear) {
   __shared__ long long wsum[32];
   pdl_launch_dependents();
   const int per = (batch + 1023) / 1024, b0 = min(batch, (int)threadIdx.x * per), b1 = min(batch, b0 + per);
@@ -43,7 +43,8 @@ __global__ void __launch_bounds__(1024) k_kv_scan(const int* lens, int batch, in
     cu[b + 1] = (int)min(acc, 0x7fffffffLL);
   }
   if (b1 == batch && b0 < b1 && (unsigned long long)acc > kv_tokens) bad = true;
-  if (bad) atomicExch(status, ST_INVALID_ARG);
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x == 0 && (bad || clear)) atomicExch(status, bad ? ST_INVALID_ARG : 0);
 }
 
 // src [L][B][p_max][row_bytes], dst [L][2][kv_tokens][row_bytes]: plane (l, kv) of request b, rows p < lens[b], go to
@@ -104,7 +105,7 @@ extern "C" {
 const char* phyai_adapter_last_error(void) { return phyai::g_ad_err; }
 
 static phyai_status_t pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const void* k, const void* v, const int32_t* lens, void* prefix_kv,
-                                     uint64_t kv_tokens, int32_t* cu_prefix_lens, int32_t* status_word, int zero_tail, void* stream) {
+                                     uint64_t kv_tokens, int32_t* cu_prefix_lens, int32_t* status_word, int cleared, void* stream) {
   using namespace phyai;
   auto bad = [](const char* m) {
     snprintf(g_ad_err, sizeof(g_ad_err), "%s", m);
@@ -123,12 +124,12 @@ static phyai_status_t pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const voi
     return bad("kv_tokens, batch, p_max or n_layers too large");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int chunks = (int)(row_bytes / 16), B = (int)desc->batch;
-  k_kv_scan<<<1, 1024, 0, st>>>(lens, B, (int)desc->p_max, kv_tokens, cu_prefix_lens, status_word);
+  k_kv_scan<<<1, 1024, 0, st>>>(lens, B, (int)desc->p_max, kv_tokens, cu_prefix_lens, status_word, cleared);
   const unsigned gx = (unsigned)(((size_t)desc->p_max * chunks + PACK_CHUNK - 1) / PACK_CHUNK);
-  cudaError_t e = launch_pdl(k_kv_pack, dim3(gx, desc->n_layers * 2, B + zero_tail < 65535 ? B + zero_tail : 65535), dim3(PACK_T), 0, st,
+  cudaError_t e = launch_pdl(k_kv_pack, dim3(gx, desc->n_layers * 2, B + cleared < 65535 ? B + cleared : 65535), dim3(PACK_T), 0, st,
                              reinterpret_cast<const uint4*>(k), reinterpret_cast<const uint4*>(v), (const int*)lens, (const int*)cu_prefix_lens,
                              (const int*)status_word, reinterpret_cast<uint4*>(prefix_kv), B, (int)desc->p_max,
-                             (unsigned long long)kv_tokens, chunks, zero_tail);
+                             (unsigned long long)kv_tokens, chunks, cleared);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     snprintf(g_ad_err, sizeof(g_ad_err), "kernel launch failed: %s", cudaGetErrorString(e));

@@ -184,16 +184,20 @@ namespace {
 thread_local char g_op_err[256] = "";
 
 // cu_prefix_lens of an operator call, checked on the device like in the denoise calls: a violation raises the caller's
-// status word (INVALID_ARG) and turns the attention kernels into no-ops.
-__device__ __forceinline__ void check_lens(const int* cu, int batch, uint64_t kv_tokens, int* status) {
+// status word (INVALID_ARG) and turns the attention kernels into no-ops.  With `clear` the word is written either way, so that
+// the call needs no cleared word (and a captured call clears it at every replay).  One block.
+__device__ __forceinline__ void check_lens(const int* cu, int batch, uint64_t kv_tokens, int* status, int clear) {
+  bool bad = false;
   for (int b = threadIdx.x; b < batch; b += blockDim.x) {
     const int lo = cu[b], hi = cu[b + 1];
-    if (lo < 0 || hi < lo || (uint64_t)hi > kv_tokens) atomicExch(status, ST_INVALID_ARG);
+    bad |= lo < 0 || hi < lo || (uint64_t)hi > kv_tokens;
   }
+  bad = __syncthreads_or(bad);
+  if (threadIdx.x == 0 && (bad || clear)) atomicExch(status, bad ? ST_INVALID_ARG : 0);
 }
-__global__ void k_check_lens(const int* cu, int batch, uint64_t kv_tokens, int* status) {
+__global__ void k_check_lens(const int* cu, int batch, uint64_t kv_tokens, int* status, int clear) {
   pdl_launch_dependents();
-  check_lens(cu, batch, kv_tokens, status);
+  check_lens(cu, batch, kv_tokens, status, clear);
 }
 
 // Operands of the tcgen05 kernels from an operator call's fp32 q | k | v rows: q rotated, scaled and rounded into the operand
@@ -201,11 +205,11 @@ __global__ void k_check_lens(const int* cu, int batch, uint64_t kv_tokens, int* 
 // [request][Hkv][S][dh].  One block per (suffix row < 64, request), a thread 8 channels and their rotary partners.  Block 0
 // also writes the request block and checks the lengths.
 __global__ void __launch_bounds__(256) k_op_operands(Request* rq, const Request src, int* status, const float* qkv, const float2* rope,
-                                                     __nv_bfloat16* q_tiles, __nv_bfloat16* kr, __nv_bfloat16* vr, const Dims d) {
+                                                     __nv_bfloat16* q_tiles, __nv_bfloat16* kr, __nv_bfloat16* vr, const Dims d, int clear) {
   const int i = blockIdx.x, b = blockIdx.y, half = d.dh >> 1, hc = half >> 3;
   if (i == 0 && b == 0) {
     if (threadIdx.x == 0) *rq = src;
-    check_lens(src.cu_lens, src.batch, src.kv_tokens, status);
+    check_lens(src.cu_lens, src.batch, src.kv_tokens, status, clear);
   }
   const int nq = d.Hq * hc, nk = d.Hkv * hc;               // items of 8 + 8 channels: q, k, v
   const float scale = rsqrtf((float)d.dh);
@@ -277,10 +281,11 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
   return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
-// Shared body of the operator entry points.  `scratch` null: taken from the library's pool when the call needs any.
+// Shared body of the operator entry points.  `clear`: the call clears the status word itself.  `scratch` null: taken from the
+// library's pool when the call needs any.
 phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, const float* qkv, const void* prefix_kv,
                             uint64_t kv_tokens, const int32_t* cu, const float* rope, uint16_t* out, int32_t* status_word,
-                            void* scratch, size_t scratch_bytes, cudaStream_t st) {
+                            int clear, void* scratch, size_t scratch_bytes, cudaStream_t st) {
   auto bad = [](const char* m) {
     snprintf(g_op_err, sizeof(g_op_err), "%s", m);
     return PHYAI_ERR_INVALID_ARG;
@@ -332,7 +337,7 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     r.prefix_kv = prefix_kv, r.kv_tokens = kv_tokens, r.cu_lens = cu, r.batch = (int)batch;
     if (!prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) {
-      k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d);
+      k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
       // (the attention kernels read the request block before their dependency wait: no programmatic launch here)
       if (attention_b1_ctas(d, (int)batch, 1) <= 15 * 8)     // 15 clusters of 8 fit a B200
         e = launch_attention_b1(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch, 1, a.wait_limit, st, nullptr, 0, false);
@@ -345,7 +350,7 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
       a.part_o = reinterpret_cast<float*>(scratch);
       a.part_ml = a.part_o + (size_t)batch * d.Hq * splits * QROWS * d.dh;
     }
-    k_check_lens<<<1, 256, 0, st>>>(cu, (int)batch, kv_tokens, status_word);
+    k_check_lens<<<1, 256, 0, st>>>(cu, (int)batch, kv_tokens, status_word, clear);
     a.num_splits = splits;
     e = launch_mma(a, (int)batch, st);
   }
@@ -373,16 +378,27 @@ size_t phyai_suffix_attention_scratch_bytes(const phyai_attention_desc_t* desc, 
   return 256 + phyai::attention_scratch_floats(d, (int)batch, splits) * sizeof(float);
 }
 
-phyai_status_t phyai_suffix_attention(const phyai_attention_desc_t* desc, uint32_t batch, const float* qkv,
-                                      const void* prefix_kv, uint64_t kv_tokens, const int32_t* cu_prefix_lens,
-                                      const float* rope_cos_sin, uint16_t* out, int32_t* status_word, void* stream) {
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const size_t bytes = phyai_suffix_attention_scratch_bytes(desc, batch);
-  if (!bytes) {
+static phyai_status_t suffix_attention(const phyai_attention_desc_t* desc, uint32_t batch, const float* qkv, const void* prefix_kv,
+                                       uint64_t kv_tokens, const int32_t* cu_prefix_lens, const float* rope_cos_sin, uint16_t* out,
+                                       int32_t* status_word, int clear, void* stream) {
+  if (!phyai_suffix_attention_scratch_bytes(desc, batch)) {
     snprintf(phyai::g_op_err, sizeof(phyai::g_op_err), "desc is NULL or batch is 0");
     return PHYAI_ERR_INVALID_ARG;
   }
-  return phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word, nullptr, 0, st);
+  return phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word, clear, nullptr, 0,
+                             reinterpret_cast<cudaStream_t>(stream));
+}
+
+phyai_status_t phyai_suffix_attention(const phyai_attention_desc_t* desc, uint32_t batch, const float* qkv,
+                                      const void* prefix_kv, uint64_t kv_tokens, const int32_t* cu_prefix_lens,
+                                      const float* rope_cos_sin, uint16_t* out, int32_t* status_word, void* stream) {
+  return suffix_attention(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word, 0, stream);
+}
+
+phyai_status_t phyai_suffix_attention_cleared(const phyai_attention_desc_t* desc, uint32_t batch, const float* qkv,
+                                              const void* prefix_kv, uint64_t kv_tokens, const int32_t* cu_prefix_lens,
+                                              const float* rope_cos_sin, uint16_t* out, int32_t* status_word, void* stream) {
+  return suffix_attention(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word, 1, stream);
 }
 
 }  // extern "C"
@@ -453,7 +469,7 @@ phyai_status_t phyai_suffix_attention_static(const phyai_attention_desc_t* desc,
   // attention_op re-derives the exact requirement (after choosing num_splits) and refuses sizes
   // beyond the capacity passed here.  Nothing in the scratch has to start at zero: whatever is read was written by
   // the same call.
-  return phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word,
+  return phyai::attention_op(desc, batch, qkv, prefix_kv, kv_tokens, cu_prefix_lens, rope_cos_sin, out, status_word, 0,
                              scratch, PHYAI_STATIC_SCRATCH_BYTES, reinterpret_cast<cudaStream_t>(stream));
 }
 
