@@ -269,11 +269,14 @@ cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
       cudaMemPoolProps props{};
       props.allocType = cudaMemAllocationTypePinned, props.location.type = cudaMemLocationTypeDevice, props.location.id = dev;
       uint64_t keep = 64ull << 20;
-      if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
-      if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+      // (not a stream operation: a thread whose stream is being captured may create the pool as well)
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return e;
+      if ((e = cudaMemPoolCreate(&pool, &props)) == cudaSuccess &&
+          (e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess)
         cudaMemPoolDestroy(pool);
-        return e;
-      }
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e != cudaSuccess) return e;
       pools[dev] = pool;
     }
     pool = pools[dev];

@@ -1,5 +1,8 @@
 """Operator calls inside a captured CUDA graph: every call carries its own clearing of the status word, so that graphs may be
 replayed in any order, and an error of one replay does not stick to the next."""
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -68,3 +71,20 @@ def test_captured_operator_calls_clear_their_own_status_word(kind):
             assert status == (binding.ERR_INVALID_ARG if attempt == 1 else 0), (i, attempt)
             if attempt != 1:
                 check(results[i])
+
+
+def test_first_operator_call_of_a_process_may_be_a_captured_one():
+    code = """
+import torch
+from tests.test_gpu_capture import attention_call
+call, _, check = attention_call(3, 8, 1, 256, 17, [100])
+stream, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+with torch.cuda.graph(g, stream=stream):
+    result = call()
+g.replay()
+torch.cuda.synchronize()
+assert int(result[1].item()) == 0
+check(result)
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
