@@ -346,8 +346,10 @@ size_t phyai_suffix_attention_scratch_bytes(const phyai_attention_desc_t *desc, 
  *   - The first call on each device looks up the array's device address (with that device
  *     current) and remembers it; make that first call before starting any stream capture.
  *   - Shapes that need more than the capacity (with num_splits set: 256 bytes + batch * Hq * splits * 64 *
- *     (head_dim + 2) * 4) are rejected with PHYAI_ERR_INVALID_ARG and a message naming both numbers; with
- *     num_splits == 0 the library picks a split count first and then checks.
+ *     (head_dim + 2) * 4) are rejected with PHYAI_ERR_INVALID_ARG and a message naming both numbers.  With
+ *     num_splits == 0 the library picks a kernel and a split count that need less first: calls whose bf16 operands do not
+ *     fit (from 54 requests of 8 heads of 256 on) take a kernel that reads the fp32 rows, whose results differ from the
+ *     allocating entry point's by rounding; from 37 such requests on that kernel does not split the keys and needs nothing.
  *   - All calls on a device share the one array and it keeps the last call's contents.  Nothing
  *     in it needs clearing between calls, but two calls that overlap on the GPU (different
  *     streams, or different host threads) race on it: serialise them.

@@ -318,18 +318,26 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
   a.d = d, a.wait_limit = 1u << 22;
   // The library's choice where shapes and alignment allow it: bf16 operands first (one small kernel), then the tcgen05 kernels
   // of the denoising loop.  One request of the pi0 shape: 37.6 -> 23 us per call; 16 requests: 70 -> 35 us.
-  const bool tc = splits == 0 && !((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(qkv)) & 15u) && kv_tokens > 0 &&
-                  attention_pair_supported(d);
-  if (splits == 0) splits = attention_pick_splits(d, (int)batch, (int)(kv_tokens < 4096 ? kv_tokens : 4096));
   const size_t q_elems = (size_t)batch * (d.Hq / 2) * 128 * d.dh, kv_elems = (size_t)batch * d.Hkv * d.S * d.dh;
-  const size_t need = tc ? sizeof(Request) + (q_elems + 2 * kv_elems) * 2 : attention_scratch_floats(d, (int)batch, splits) * sizeof(float);
+  const size_t tc_need = sizeof(Request) + (q_elems + 2 * kv_elems) * 2;
+  // (a given scratch that cannot hold the operands leaves the call to the mma.sync kernel, which reads the fp32 rows itself)
+  bool tc = splits == 0 && !((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(qkv)) & 15u) && kv_tokens > 0 &&
+            attention_pair_supported(d) && (!scratch || tc_need <= scratch_bytes);
+  if (splits == 0) splits = attention_pick_splits(d, (int)batch, (int)(kv_tokens < 4096 ? kv_tokens : 4096));
+  const size_t mma_need = attention_scratch_floats(d, (int)batch, splits) * sizeof(float);
+  size_t need = tc ? tc_need : mma_need;
   if (need && scratch && need > scratch_bytes) {
     snprintf(g_op_err, sizeof(g_op_err), "needs %zu bytes of scratch, only %zu available", need, scratch_bytes);
     return PHYAI_ERR_INVALID_ARG;
   }
   cudaError_t e = cudaSuccess;
-  const bool own = need && !scratch;
-  if (own && (e = scratch_alloc(&scratch, need, st)) != cudaSuccess) {
+  const bool given = scratch != nullptr;
+  if (tc && !given && scratch_alloc(&scratch, tc_need, st) != cudaSuccess) {
+    cudaGetLastError();                     // (no room for the operands of a large batch: likewise)
+    scratch = nullptr, tc = false, need = mma_need;
+  }
+  const bool own = need && !given;
+  if (own && !scratch && (e = scratch_alloc(&scratch, need, st)) != cudaSuccess) {
     snprintf(g_op_err, sizeof(g_op_err), "scratch allocation of %zu bytes failed: %s", need, cudaGetErrorString(e));
     return PHYAI_ERR_OOM;
   }

@@ -74,3 +74,22 @@ def test_attention_operator_rejects_bad_arguments():
     with pytest.raises(binding.PhyaiError) as e:
         binding.suffix_attention(desc, qkv.cuda(), kv.cuda(), torch.from_numpy(cu).cuda(), None)
     assert e.value.status == binding.ERR_INVALID_ARG
+
+
+def test_attention_operator_without_room_for_the_operands():
+    """8192 requests: 2.1 GB of bf16 operands that a nearly full device has no room for; the kernel that needs no scratch serves."""
+    B = 8192
+    qkv, kv, cu, _ = make_case(9, 8, 1, 256, 1, [b % 3 for b in range(B)], theta=0.0)
+    desc = binding.attention_desc(8, 1, 256, 1, n_layers=2, layer=1)
+    args = (desc, qkv.cuda(), kv.cuda(), torch.from_numpy(cu).cuda(), None)
+    binding.suffix_attention(*args)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (1 << 30), dtype=torch.uint8, device="cuda")
+    out, status = binding.suffix_attention(*args)
+    torch.cuda.synchronize()
+    del filler
+    torch.cuda.empty_cache()
+    assert int(status.item()) == 0
+    ref = oracle_attention(qkv, kv, cu, 8, 1, 256, 1, 1, 0.0)
+    assert np.abs(out.double().cpu().numpy() - ref).max() <= 2e-2 * np.abs(ref).max()

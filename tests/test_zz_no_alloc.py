@@ -57,3 +57,17 @@ def test_static_scratch_entry_point_rejects_what_does_not_fit():
     out, st = binding.suffix_attention(desc, qkv, kv, cu, rope)
     torch.cuda.synchronize()
     assert int(st.item()) == 0 and bool(torch.isfinite(out.float()).all())
+
+
+@pytest.mark.parametrize("batch", [53, 54, 64])
+def test_static_scratch_entry_point_takes_batches_whose_operands_do_not_fit(batch):
+    """53 requests of this shape are the last whose bf16 operands fit the array; beyond, the kernel that needs none serves."""
+    qkv, kv, cu, rope = _case(4, 8, 1, 256, 51, [(29 * b) % 90 for b in range(batch)])
+    desc = binding.attention_desc(8, 1, 256, 51, n_layers=2, layer=1)
+    ref, st_ref = binding.suffix_attention(desc, qkv, kv, cu, rope)
+    got, st_got = binding.suffix_attention(desc, qkv, kv, cu, rope, entry="phyai_suffix_attention_static")
+    torch.cuda.synchronize()
+    assert int(st_ref.item()) == 0 and int(st_got.item()) == 0
+    ref, got = ref.double(), got.double()
+    assert (got - ref).abs().max() <= 2e-2 * ref.abs().max()
+    assert (batch > 53) or torch.equal(got, ref)
