@@ -17,10 +17,11 @@
 // CTA's share of the request's own (suffix) keys come right after it.
 //
 // Merge.  Every CTA holds an un-normalised partial (O, row max, row sum) of all HPC x S rows.  Row i of every head is
-// owned by CTA i / 8: each CTA writes its partial, rounded to bf16 and grouped by owner, into its own shared memory
-// and sends every owner one bulk copy over distributed shared memory (counted on the owner's mbarrier); the owner
-// combines the 8 partials of its rows in rank order and stores the normalised bf16 rows as the activation tile of
-// the output projection.  No partials in global memory, no merge kernel.
+// owned by CTA i / 8: each CTA writes its partial, grouped by owner, into its own shared memory and sends every owner one
+// bulk copy over distributed shared memory (counted on the owner's mbarrier); the owner combines the 8 partials of its rows
+// in rank order and stores the normalised bf16 rows as the activation tile of the output projection (or as rows of the
+// operator's output).  No partials in global memory, no merge kernel.  With F32 (the operator; one head per CTA) the partials
+// are sent as they are, single-tile calls of the loop round them to bf16.
 //
 // Warps: 4 issues the MMAs; the other eight are two threads per accumulator row (each half of the columns): the
 // softmax, partial out; warps 0-1 also load K, 2-3 V (16-byte cp.async into the swizzled block
@@ -42,21 +43,22 @@ __device__ __forceinline__ void named_arrive() {
   asm volatile("bar.arrive %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
 }
 
-template <int DH, int HPC>
+template <int DH, int HPC, bool F32>
 struct B1Layout {
   static constexpr int BLOCK = KB * 128;                     // one 64-channel block of a K / V tile: 128 keys x 128 bytes
   static constexpr int TILE = (DH / 64) * BLOCK;             // a K or V tile
-  static constexpr int PITCH = DH * 2 + 16;                  // bf16 partial row, padded against bank conflicts
+  static constexpr int PITCH = DH * (F32 ? 4 : 2) + 16;      // partial row, padded against bank conflicts
   static constexpr int SLOT = HPC * 8 * (PITCH + 16);        // one owner's block: HPC heads x 8 rows of O, then their (max, sum)
                                                              // in 16-byte entries (a bulk copy moves multiples of 16 bytes)
   static constexpr int QTILE = 128 * DH * 2;                 // the Q operand (128 rows; with one head the upper 64 idle)
   static constexpr int RECV = 8 * SLOT > QTILE ? 8 * SLOT : QTILE;   // receive area of the merge; first holds Q
   static constexpr size_t SMEM = 1024 + 2 * (size_t)TILE + (size_t)RECV;
+  static_assert(8 * SLOT <= 2 * TILE, "partials exceed the key / value tiles");
 };
 
-template <int DH, int HPC>
+template <int DH, int HPC, bool F32>
 __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
-  using L = B1Layout<DH, HPC>;
+  using L = B1Layout<DH, HPC, F32>;
   constexpr int COLS = 512;                   // S / P at columns [0, 128), O at [128, 128 + DH)
   constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(KB >> 3) << 17) | ((128u >> 4) << 24);
   constexpr uint32_t IDESC_PV =
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
       if (g == 1) cp_async_wait<0>();
       asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     }
-    // ---- partial out: half an O row -> bf16 into the owner's block of the staging area; group 0 adds (max, sum) ------
+    // ---- partial out: half an O row into the owner's block of the staging area; group 0 adds (max, sum) --------------
     if (T > 0 && warp == 5) mbar_wait_drain(smem_u32(&pv_done), (uint32_t)(T - 1) & 1u, wc);
     group_sync<BAR_ROWS, 256>();
     tc_fence_after();
@@ -339,7 +341,12 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
 #pragma unroll
           for (int e = 0; e < 64; ++e) o[e] = 0.f;
         }
-        if (wr) {
+        if (wr && F32) {
+#pragma unroll
+          for (int e = 0; e < 64; e += 4)
+            asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)(c0 + e) * 4), "f"(o[e]), "f"(o[e + 1]), "f"(o[e + 2]), "f"(o[e + 3])
+                         : "memory");
+        } else if (wr) {
 #pragma unroll
           for (int e = 0; e < 64; e += 8)
             asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)(c0 + e) * 2), "r"(pack_bf16(o[e], o[e + 1])),
@@ -420,14 +427,24 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
       for (int s = 0; s < 8; ++s) {
         const float w = wtab[rr][s];
         const uint32_t blk = (s == rank) ? stg + (uint32_t)rank * L::SLOT : recv + (uint32_t)s * L::SLOT;
-        uint32_t u0, u1, u2, u3;
-        asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(u0), "=r"(u1), "=r"(u2), "=r"(u3) : "r"(blk + (uint32_t)rr * L::PITCH + (uint32_t)ch * 16) : "memory");
-        const uint32_t uu[4] = {u0, u1, u2, u3};
+        const uint32_t src = blk + (uint32_t)rr * L::PITCH + (uint32_t)ch * (F32 ? 32 : 16);
+        if (F32) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&uu[e]);
-          acc[2 * e] = fmaf(w, __low2float(p), acc[2 * e]);
-          acc[2 * e + 1] = fmaf(w, __high2float(p), acc[2 * e + 1]);
+          for (int e = 0; e < 8; e += 4) {
+            float x[4];
+            asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]) : "r"(src + e * 4) : "memory");
+#pragma unroll
+            for (int f = 0; f < 4; ++f) acc[e + f] = fmaf(w, x[f], acc[e + f]);
+          }
+        } else {
+          uint32_t uu[4];
+          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(uu[0]), "=r"(uu[1]), "=r"(uu[2]), "=r"(uu[3]) : "r"(src) : "memory");
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&uu[e]);
+            acc[2 * e] = fmaf(w, __low2float(p), acc[2 * e]);
+            acc[2 * e + 1] = fmaf(w, __high2float(p), acc[2 * e + 1]);
+          }
         }
       }
       const int orow = b * S + rank * 8 + il, col = (head0 + hl) * DH + ch * 8;
@@ -445,23 +462,23 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
   (void)base_ptr;
 }
 
-template <int DH, int HPC>
+template <int DH, int HPC, bool F32>
 cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) {
   static PerDeviceOnce once;
   if (once.needed()) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_b1<DH, HPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B1Layout<DH, HPC>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_attn_b1<DH, HPC, F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B1Layout<DH, HPC, F32>::SMEM);
     if (e != cudaSuccess) return e;
     once.done();
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(8, a.d.Hq / HPC, batch), cfg.blockDim = dim3(288), cfg.dynamicSmemBytes = B1Layout<DH, HPC>::SMEM, cfg.stream = st;
+  cfg.gridDim = dim3(8, a.d.Hq / HPC, batch), cfg.blockDim = dim3(288), cfg.dynamicSmemBytes = B1Layout<DH, HPC, F32>::SMEM, cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 8, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at, cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_attn_b1<DH, HPC>, a);
+  return cudaLaunchKernelEx(&cfg, k_attn_b1<DH, HPC, F32>, a);
 }
 
 }  // namespace
@@ -476,12 +493,14 @@ int attention_b1_ctas(const Dims& d, int batch, int hpc) { return 8 * (d.Hq / hp
 
 cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
-                                int batch, int hpc, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, int trace_all, bool pdl) {
+                                int batch, int hpc, bool f32, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, int trace_all, bool pdl) {
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
   a.num_splits = 8, a.d = d, a.wait_limit = wait_limit, a.trace = trace, a.trace_all = trace_all;
-  if (hpc == 1) return d.dh == 256 ? launch_one<256, 1>(a, batch, st, pdl) : launch_one<128, 1>(a, batch, st, pdl);
-  return d.dh == 256 ? launch_one<256, 2>(a, batch, st, pdl) : launch_one<128, 2>(a, batch, st, pdl);
+  if (f32 && hpc != 1) return cudaErrorInvalidValue;
+  if (f32) return d.dh == 256 ? launch_one<256, 1, true>(a, batch, st, pdl) : launch_one<128, 1, true>(a, batch, st, pdl);
+  if (hpc == 1) return d.dh == 256 ? launch_one<256, 1, false>(a, batch, st, pdl) : launch_one<128, 1, false>(a, batch, st, pdl);
+  return d.dh == 256 ? launch_one<256, 2, false>(a, batch, st, pdl) : launch_one<128, 2, false>(a, batch, st, pdl);
 }
 
 }  // namespace phyai

@@ -13,11 +13,15 @@
 //   O += P V    M = 256, N = head_dim, K = 128 keys; P is the tensor-memory A operand, V an MN-major B operand; rescaled
 //               only when a row's maximum grows by more than 2^8
 // Small calls split the keys of a request over C = 2 to 4 pairs of one cluster (each range: its share of the prefix and of
-// the suffix keys); the partial results, rounded to bf16, are merged over distributed shared memory: row range p of every
-// head belongs to pair p, which adds the C partials in range order.  No partials in global memory, no merge launch.
+// the suffix keys); the fp32 partial results are merged over distributed shared memory: row range p of every head belongs to
+// pair p, which is sent its rows of the other C - 1 partials and adds the C in range order.  No partials in global memory, no
+// merge launch.  (Owners that read the partials from the other CTAs instead of being sent them: 4.2 us per launch more.)
 //
-// Measured at 8 requests of 816 + 51 keys and 8 heads (C = 3), from the projection's end to the merged output: 14 us (split
-// ranges of the one-CTA kernel 21 us, their merge launch 8): operands 2 - 3, 1.2 - 2 per key tile, merge 3.5.
+// Measured at 8 requests of 816 + 51 keys and 8 heads (C = 3), from the projection's end to the merged output: 15 us (split
+// ranges of the one-CTA kernel 21 us, their merge launch 8): operands 2 - 3, 1.2 - 2 per key tile, merge 4.7.  What bounds
+// the merge is the way between SMs, 28 bytes per ns for one: a CTA sends (C - 1) / C of its 102 KB, in two pieces, the first
+// while the second is staged (in one piece 0.7 us per launch more; as bf16, half the bytes, the merge took 3.7; through
+// global memory, which all clusters share, 3 us more at 8 requests).
 //
 // Warps of a CTA: 0-1 load K, 2-3 load V (full prefix tiles with tensor-map copies -- the map of the call's cache sits in
 // the request block --, the rest row by row with cp.async; prefix rows before the dependency wait), 4 issues the MMAs
@@ -42,13 +46,18 @@ struct ApLayout {
   static constexpr int PIECE = (DH / 128) * KBLOCK;          // one tensor-map copy: 64 keys x DH / 2 channels
   static constexpr int VTILE = 2 * PIECE;                    // V: two halves of 64 keys, this CTA's DH / 2 channels
   static constexpr int QTILE = 128 * DH * 2;
-  static constexpr int OWN = (64 + C - 1) / C;                         // rows per head a pair finishes
-  static constexpr int PITCH = DH * 2 + 16;                  // bf16 partial row, padded against bank conflicts
-  static constexpr int SLOT = 2 * OWN * (PITCH + 16);        // one owner's block: 2 heads x OWN rows, then (max, sum) entries
-  static constexpr int RECV = C > 1 ? C * SLOT : 0;          // [C sources] partials for my rows; first holds Q
-  static constexpr int KV = 2 * (KTILE + VTILE);             // two buffers each; later the outgoing partials [C owners][SLOT]
-  static constexpr size_t SMEM = 1024 + (size_t)KV + (QTILE > RECV ? QTILE : RECV);
-  static_assert(C == 1 || C * SLOT <= KV, "partials exceed the key / value buffers");
+  static constexpr int KV = 2 * (KTILE + VTILE);             // two buffers each
+  // Partials: staged over the (by then dead) K / V buffers in blocks by owner (2 heads x own rows of O, then their (max, sum)
+  // entries of 16 bytes: a bulk copy moves multiples of 16 bytes); behind them and behind K / V the blocks of the C - 1 peers,
+  // over Q and past it.  Of 256 channels three ranges fit up to 63 suffix rows, four up to 60.
+  static constexpr int S_MAX = DH != 256 || C < 3 ? 64 : (C == 3 ? 63 : 60);
+  static constexpr int OWN = (S_MAX + C - 1) / C;            // most rows per head a pair finishes
+  static constexpr int NP = DH / 128;                        // a block in pieces of 2 x 64 columns, sent as they are staged
+  static constexpr int PITCH = 512 + 16;                     // fp32 row of a piece, padded against bank conflicts
+  static constexpr int ROW = NP * PITCH + 16;
+  static constexpr int STG = 2 * C * OWN * ROW, RECV = (STG > KV ? STG : KV), PEERS = C > 1 ? 2 * (C - 1) * OWN * ROW : 0;
+  static constexpr size_t SMEM = 1024 + (size_t)(C > 1 && RECV + PEERS > KV + QTILE ? RECV + PEERS : KV + QTILE);
+  static_assert(SMEM + 3072 <= 227 * 1024, "partials exceed the shared memory");
 };
 
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
@@ -95,7 +104,6 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag, mrg_ok;
   __shared__ float xch[2][2][128];       // the two half-row threads of a row exchange their maximum (by tile parity) and, at the end, sum
-  __shared__ float wtab[C > 1 ? 2 * L::OWN : 1][C]; // merge: weight of partial s for each of my rows
 
   const Dims& d = a.d;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -110,8 +118,9 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t Ks = base, Vs = base + 2 * L::KTILE, Qs = base + L::KV;
-  const uint32_t stg = base, recv = Qs;                                // merge: outgoing blocks by owner; [C sources] mine
-  const int own_lo = pr * L::OWN, n_me = max(0, min(L::OWN, S - own_lo));   // suffix rows (per head) this CTA finishes
+  const int own = (S + C - 1) / C, own_lo = pr * own, n_me = max(0, min(own, S - own_lo));   // suffix rows (per head) this CTA finishes
+  const uint32_t slot = (uint32_t)(2 * own * L::ROW);
+  const uint32_t stg = base, recv = base + max((uint32_t)C * slot, (uint32_t)L::KV);   // merge: blocks by owner; [C - 1 peers] mine
 
   if (tid == 0) {
     abort_flag = 0;
@@ -120,7 +129,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       mbar_init(smem_u32(&s_full[i]), 1), mbar_init(smem_u32(&pv_done[i]), 1);
     }
     mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 8), mbar_init(smem_u32(&q_ready), 1);
-    if (C > 1 && n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * (L::PITCH + 16)));
+    if (C > 1 && n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * L::ROW));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 4) {
@@ -423,42 +432,45 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         __syncwarp();
       }
     } else {
-      // ---- partial out: half an O row -> bf16 into the owner's block of the staging area; half 0 adds (max, sum) -------
-      const int c = i / L::OWN, il = i - c * L::OWN, n_c = max(0, min(L::OWN, S - c * L::OWN));
+      // ---- partial out: half an O row into the owner's block of the staging area; half 0 adds (max, sum) ----------------
+      const int c = i / own, il = i - c * own, n_c = max(0, min(own, S - c * own));
       const bool wr = i < S;
-      const uint32_t blk = stg + (uint32_t)c * L::SLOT, rowp = blk + (uint32_t)(hl * n_c + il) * L::PITCH;
+      const uint32_t blk = stg + (uint32_t)c * slot;
+      constexpr int PARTS = 8 / (C - 1);       // warps per peer: the bulk copies of one warp complete one after the other
+      const int w8 = warp - 5, pi = w8 % (C - 1), peer = pi < pr ? pi : pi + 1, part = w8 / (C - 1);
+      const int n_p = max(0, min(own, S - peer * own));
 #pragma unroll 1
-      for (int c0 = g * (DH / 2); c0 < (g + 1) * (DH / 2); c0 += 64) {
+      for (int k = 0; k < L::NP; ++k) {
         float o[64];
         if (T > 0) {
-          tmem_ld64(tmem_o + lane_addr + (uint32_t)c0, o);
+          tmem_ld64(tmem_o + lane_addr + (uint32_t)(g * (DH / 2) + k * 64), o);
         } else {
 #pragma unroll
           for (int e = 0; e < 64; ++e) o[e] = 0.f;
         }
+        const uint32_t rowp = blk + (uint32_t)((k * 2 * n_c + hl * n_c + il) * L::PITCH + g * 256);
         if (wr) {
 #pragma unroll
-          for (int e = 0; e < 64; e += 8)
-            asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)(c0 + e) * 2), "r"(pack_bf16(o[e], o[e + 1])),
-                         "r"(pack_bf16(o[e + 2], o[e + 3])), "r"(pack_bf16(o[e + 4], o[e + 5])), "r"(pack_bf16(o[e + 6], o[e + 7]))
+          for (int e = 0; e < 64; e += 4)
+            asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)e * 4), "f"(o[e]), "f"(o[e + 1]), "f"(o[e + 2]), "f"(o[e + 3])
+                         : "memory");
+          if (k == 0 && g == 0)
+            asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(blk + (uint32_t)(L::NP * 2 * n_c * L::PITCH + (hl * n_c + il) * 16)), "f"(m), "f"(l)
                          : "memory");
         }
-      }
-      if (wr && g == 0)
-        asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(blk + (uint32_t)(2 * n_c) * L::PITCH + (uint32_t)(hl * n_c + il) * 16), "f"(m), "f"(l)
-                     : "memory");
-      fence_async_smem();                      // generic writes -> visible to the bulk-copy engine
-      group_sync<BAR_ROWS, 256>();
-      cluster_wait();                          // every CTA's Q is dead
-      const int peer = warp - 5;               // (one copy per warp: the bulk copies of one warp complete one after the other)
-      if (lane == 0 && peer < C && peer != pr) {
-        const int n_p = max(0, min(L::OWN, S - peer * L::OWN));
-        if (n_p > 0)
-          asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                           map_rank(recv + (uint32_t)pr * L::SLOT, peer * 2 + half)),
-                       "r"(stg + (uint32_t)peer * L::SLOT), "r"((uint32_t)(2 * n_p * (L::PITCH + 16))),
-                       "r"(map_rank(smem_u32(&mrg_bar), peer * 2 + half))
-                       : "memory");
+        fence_async_smem();                    // generic writes -> visible to the bulk-copy engine
+        group_sync<BAR_ROWS, 256>();
+        if (k == 0) cluster_wait();            // every CTA's Q is dead
+        if (lane == 0 && part < PARTS && n_p > 0) {
+          const uint32_t bytes = (uint32_t)(2 * n_p * (L::PITCH + (k == L::NP - 1 ? 16 : 0))), chunk = (bytes / PARTS + 15) & ~15u;
+          const uint32_t lo = (uint32_t)part * chunk, off = (uint32_t)(k * 2 * n_p * L::PITCH) + lo;
+          if (lo < bytes)
+            asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                             map_rank(recv + (uint32_t)(pr < peer ? pr : pr - 1) * slot + off, peer * 2 + half)),
+                         "r"(stg + (uint32_t)peer * slot + off), "r"(min(chunk, bytes - lo)), "r"(map_rank(smem_u32(&mrg_bar), peer * 2 + half))
+                         : "memory");
+        }
+        __syncwarp();
       }
       if (warp == 5) {
         bool ok = true;
@@ -475,47 +487,52 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   cluster_arrive();
   if constexpr (C > 1) {
     // ---- merge my rows: the C partials in range order, normalise, store as the output projection's operand ------------
+    // A warp per row (rr = hl * n_me + il, every 13th), lane l the four columns of every piece that its l-th 16 bytes hold;
+    // before that the weights of the warp's rows, a row per lane.
+    constexpr int NW = AP_THREADS / 32;
+    static_assert((2 * L::OWN + NW - 1) / NW <= 32, "more rows per warp than lanes");
     const bool store = !*reinterpret_cast<volatile int*>(&abort_flag) && *reinterpret_cast<volatile int*>(&mrg_ok);
-    auto blk_of = [&](int s) { return s == pr ? stg + (uint32_t)pr * L::SLOT : recv + (uint32_t)s * L::SLOT; };
-    if (tid < 2 * n_me) {
-      float ms[C], ls[C], mm = -INFINITY, w[C], ll = 0.f;
+    uint32_t blk[C];
+    float w[C], ls[C], mm = -INFINITY, ll = 0.f;
+    const int my = min(warp + NW * lane, max(0, 2 * n_me - 1));
 #pragma unroll
-      for (int s = 0; s < C; ++s) {
-        asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(ms[s]), "=f"(ls[s]) : "r"(blk_of(s) + (uint32_t)(2 * n_me) * L::PITCH + (uint32_t)tid * 16) : "memory");
-        mm = fmaxf(mm, ms[s]);
-      }
-#pragma unroll
-      for (int s = 0; s < C; ++s) {
-        w[s] = ms[s] == -INFINITY ? 0.f : exp2f(ms[s] - mm);
-        ll = fmaf(w[s], ls[s], ll);
-      }
-      const float inv = 1.0f / ll;
-#pragma unroll
-      for (int s = 0; s < C; ++s) wtab[tid][s] = w[s] * inv;
+    for (int s = 0; s < C; ++s) {
+      blk[s] = s == pr ? stg + (uint32_t)pr * slot : recv + (uint32_t)(s < pr ? s : s - 1) * slot;
+      asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(w[s]), "=f"(ls[s]) : "r"(blk[s] + (uint32_t)(L::NP * 2 * n_me * L::PITCH + my * 16)) : "memory");
+      mm = fmaxf(mm, w[s]);
     }
-    __syncthreads();
-    if (store) {
-      constexpr int CH = DH / 8;               // 16-byte chunks per row
+#pragma unroll
+    for (int s = 0; s < C; ++s) {
+      w[s] = w[s] == -INFINITY ? 0.f : exp2f(w[s] - mm);
+      ll = fmaf(w[s], ls[s], ll);
+    }
+    const float inv = 1.0f / ll;
+#pragma unroll
+    for (int s = 0; s < C; ++s) w[s] *= inv, blk[s] += (uint32_t)(warp * L::PITCH + lane * 16);
+    const int col = head0 * DH + (lane >> 4) * (DH / 2) + (lane & 15) * 4;
+    const bool tiled = a.rows_pad > 0;
+    const size_t kc = (size_t)(tiled ? a.rows_pad : 1) * 64;             // elements from one 64-column chunk to the next
+    __nv_bfloat16* const o0 = a.out + (tiled ? (size_t)(col >> 6) * kc + (col & 7) : (size_t)col);
 #pragma unroll 1
-      for (int idx = tid; idx < 2 * n_me * CH; idx += AP_THREADS) {
-        const int rr = idx / CH, ch = idx - rr * CH;       // rr = hl * n_me + il
-        const int hl = rr >= n_me ? 1 : 0, il = rr - hl * n_me;
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int j = 0, rr = warp; rr < 2 * n_me; ++j, rr += NW) {
+      const int hl = rr >= n_me ? 1 : 0, orow = b * S + own_lo + rr - hl * n_me;
+      float acc[L::NP][4] = {};
 #pragma unroll
-        for (int s = 0; s < C; ++s) {
-          const float w = wtab[rr][s];
-          uint32_t uu[4];
-          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(uu[0]), "=r"(uu[1]), "=r"(uu[2]), "=r"(uu[3]) : "r"(blk_of(s) + (uint32_t)rr * L::PITCH + (uint32_t)ch * 16) : "memory");
+      for (int s = 0; s < C; ++s) {
+        const float ws = __shfl_sync(0xffffffffu, w[s], j);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 p = *reinterpret_cast<const __nv_bfloat162*>(&uu[e]);
-            acc[2 * e] = fmaf(w, __low2float(p), acc[2 * e]);
-            acc[2 * e + 1] = fmaf(w, __high2float(p), acc[2 * e + 1]);
-          }
+        for (int k = 0; k < L::NP; ++k) {
+          float x[4];
+          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3])
+                       : "r"(blk[s] + (uint32_t)((k * 2 * n_me + j * NW) * L::PITCH)) : "memory");
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[k][e] = fmaf(ws, x[e], acc[k][e]);
         }
-        const int orow = b * S + own_lo + il, col = (head0 + hl) * DH + ch * 8;
-        *reinterpret_cast<uint4*>(a.out + out_index(orow, col, a.rows_pad, d.Nq)) =
-            make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+      }
+      __nv_bfloat16* const o = o0 + (tiled ? (size_t)orow * 64 + ((((col & 63) >> 3) ^ (orow & 7)) << 3) : (size_t)orow * d.Nq) + hl * (DH / 64) * kc;
+      if (store) {
+#pragma unroll
+        for (int k = 0; k < L::NP; ++k) *reinterpret_cast<uint2*>(o + k * kc) = make_uint2(pack_bf16(acc[k][0], acc[k][1]), pack_bf16(acc[k][2], acc[k][3]));
       }
     }
   }
@@ -593,6 +610,11 @@ bool attention_pair_supported(const Dims& d) {
   return (d.dh == 256 || d.dh == 128) && d.S <= 64 && d.Hq % 4 == 0 && (d.Hq / d.Hkv) % 4 == 0;
 }
 
+// (most ranges whose fp32 partials fit the shared memory)
+int attention_pair_max_ranges(const Dims& d) {
+  return d.dh != 256 || d.S <= ApLayout<256, 4>::S_MAX ? 4 : (d.S <= ApLayout<256, 3>::S_MAX ? 3 : 2);
+}
+
 // Key ranges per request: 1 to 4, the least of waves x (fixed cost + tiles of a range), in tiles of 128 keys.  How many
 // clusters of 2 C CTAs the device holds at a time decides the waves (a cluster of 8 needs 8 free SMs in one GPC: 15 on a
 // B200, not 18).
@@ -607,7 +629,7 @@ int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
       n = max_clusters(d.dh, c);
       cached[dh][c].store(n > 0 ? n : -1);
     }
-    if (n <= 0) continue;
+    if (n <= 0 || c > attention_pair_max_ranges(d)) continue;
     const double cost = (double)((items + n - 1) / n) * ((c > 1 ? 5.5 : 4.0) + (max_prefix + d.S + c * KB - 1) / (c * KB));
     if (cost < best) best = cost, best_c = c;
   }
@@ -617,6 +639,7 @@ int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
 cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                   const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
                                   int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, bool pdl) {
+  if (ranges > attention_pair_max_ranges(d)) return cudaErrorInvalidValue;
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
   a.num_splits = ranges, a.d = d, a.wait_limit = wait_limit, a.order = order, a.trace = trace;

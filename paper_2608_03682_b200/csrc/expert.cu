@@ -445,7 +445,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
         atr = h->trace + (size_t)trace_cursor * TRACE_STAMPS, all = 1;
         trace_cursor += n_cta;
       }
-      e = launch_attention_b1(h->rq, h->status, h->q_tiles, kr, vr, l, h->attn64, 64, dd, batch, b1_hpc, h->wait_limit, st, atr, all);
+      e = launch_attention_b1(h->rq, h->status, h->q_tiles, kr, vr, l, h->attn64, 64, dd, batch, b1_hpc, false, h->wait_limit, st, atr, all);
     }
     else if (b1_attn_tc)
       e = launch_attention_tc(h->rq, h->status, h->qr_big, kr, vr, l, h->attn64, 64, dd, batch, h->order, h->wait_limit, st);
@@ -497,22 +497,12 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   };
   // Attention of the pair path.  Caches of fewer than 256 tokens keep the one-CTA kernel: with at most four 64-key tiles
   // there is nothing to share or split.
-  const int pr_ranges = h->pair_ranges ? h->pair_ranges : (pair && h->q_tiles_pair ? attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len) : 1);
+  const int pr_ranges = h->pair_ranges ? std::min(h->pair_ranges, attention_pair_max_ranges(d)) : (pair && h->q_tiles_pair ? attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len) : 1);
   const bool attn_pair = pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair && h->cfg.max_prefix_len >= 256 && (pr_ranges > 1 || h->pair_ranges);
-  // Few requests: eight key ranges per head pair (the single-tile calls' kernel) instead of at most four per four heads, as
-  // long as its clusters of eight CTAs are resident at once (15 on a B200) and a range is one key tile.  Ten-step loop of two
-  // pi0 requests 8.46 -> 8.12 ms, of three 8.70 -> 8.60.
-  const bool attn_b1 = attn_pair && !h->pair_ranges && h->use_b1_attention && attention_b1_supported(d) &&
-                       attention_b1_ctas(d, batch, 2) <= 15 * 8 && h->cfg.max_prefix_len + d.S <= 1024;
   auto attention_rot = [&](int l) -> phyai_status_t {   // from rotated bf16 q / k / v to the output projection's operand
     cudaError_t e;
     const bool tr1 = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from;
-    if (attn_b1) {
-      e = launch_attention_b1(h->rq, h->status, h->q_tiles_pair, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch, 2, h->wait_limit,
-                              st);
-      busy = attention_b1_ctas(d, batch, 2);
-      ++cnt;
-    } else if (attn_pair) {
+    if (attn_pair) {
       e = launch_attention_pair(h->rq, h->status, h->q_tiles_pair, h->kr_big, h->vr_big, l, h->attn_t, h->Mpad, d, batch,
                                 pr_ranges, h->order, h->wait_limit, st,
                                 tr1 ? h->trace : nullptr);

@@ -203,8 +203,8 @@ cudaError_t launch_attention_cluster(const Request* rq, int* status, const float
 bool attention_b1_supported(const Dims& d);
 cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
-                                int batch, int hpc, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr,
-                                int trace_all = 0, bool pdl = true);
+                                int batch, int hpc, bool f32, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr,
+                                int trace_all = 0, bool pdl = true);   // f32: fp32 partial results (one head per CTA only)
 // CTAs of one launch with `hpc` (1 or 2) query heads per CTA
 int attention_b1_ctas(const Dims& d, int batch, int hpc);
 cudaError_t launch_attention_tc(const Request* rq, int* status, const __nv_bfloat16* qr, const __nv_bfloat16* kr,
@@ -221,6 +221,7 @@ cudaError_t launch_attention_merge(int* status, const float* part_o, const float
 // of a request over up to 4 pairs of a cluster
 bool attention_pair_supported(const Dims& d);
 bool prefix_kv_map(unsigned char* map, const void* kv, uint64_t kv_tokens, const Dims& d);   // fills Request::kv_map
+int attention_pair_max_ranges(const Dims& d);
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix);
 cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                   const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,

@@ -68,7 +68,8 @@ def test_pair_attention_key_ranges(head_dim, n_q, n_kv, ranges):
 
 @pytest.mark.parametrize("head_dim,n_q,n_kv,lens", [(256, 4, 1, [960, 0, 1, 7, 8, 511, 959]), (128, 8, 2, [700, 129, 64]), (128, 4, 1, [256] * 7)])
 def test_attention_of_a_few_requests(head_dim, n_q, n_kv, lens):
-    """Eight key ranges per head pair: as many clusters as are resident, empty and one-key ranges, a full last tile."""
+    """The library's own choice of key ranges for few requests (63 and 64 suffix rows: with 256 channels not four of them), empty and
+    one-key ranges, a full last tile."""
     cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=len(lens), max_prefix_len=max(lens),
                             n_layers=2, horizon=63, suffix_block_causal=n_kv == 2)
     check(cfg, lens, 1, range(len(lens)))
