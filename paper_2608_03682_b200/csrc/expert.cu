@@ -1378,8 +1378,8 @@ phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, co
   const size_t plane = kvb / planes;
   if (kvb) {
     if (!h->packer) h->packer = new (std::nothrow) phyai::HostPacker();
-    if (!h->packer) return fail(PHYAI_ERR_OOM, "host allocation failed");
-    h->packer->start(pin_kv, prefix_kvs, prefix_lens, (int)batch, planes, plane / total);
+    if (!h->packer || !h->packer->start(pin_kv, prefix_kvs, prefix_lens, (int)batch, planes, plane / total))
+      return fail(PHYAI_ERR_OOM, "host allocation failed");
   }
   float *ps = reinterpret_cast<float*>(pin_kv + kvb), *pn = ps + batch * Ds;
   int32_t* cu = reinterpret_cast<int32_t*>(pn + batch * ha);

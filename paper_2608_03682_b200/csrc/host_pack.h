@@ -7,6 +7,7 @@
 #include <condition_variable>
 #include <cstdint>
 #include <cstring>
+#include <exception>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -48,52 +49,62 @@ class HostPacker {
     for (auto& t : threads_) t.join();
   }
   // Starts the gather of `planes` planes: request b contributes lens[b] rows from src[b].  The arrays must stay valid until
-  // wait(planes) has returned.
-  void start(uint8_t* dst, const void* const* src, const uint32_t* lens, int batch, int planes, size_t row) {
+  // wait(planes) has returned.  False: out of memory, nothing was started.  (A process that may start no more threads has
+  // fewer, or none: wait() then gathers by itself.)
+  bool start(uint8_t* dst, const void* const* src, const uint32_t* lens, int batch, int planes, size_t row) noexcept {
     if (threads_.empty()) {
       const unsigned hw = std::thread::hardware_concurrency();
       const unsigned n = hw > 10 ? 8 : (hw > 3 ? hw - 2 : 1);
-      for (unsigned i = 0; i < n; ++i) threads_.emplace_back([this] { work(); });
+      try {
+        threads_.reserve(n);
+        for (unsigned i = 0; i < n; ++i) threads_.emplace_back([this] { work(); });
+      } catch (const std::exception&) {
+      }
     }
-    {
+    try {
       std::lock_guard<std::mutex> lock(mu_);
+      done_.assign(planes, 0);
       dst_ = dst, src_ = src, lens_ = lens, batch_ = batch, planes_ = planes, row_ = row;
       next_ = 0, ready_ = 0;
-      done_.assign(planes, 0);
       ++job_;
+    } catch (const std::exception&) {
+      return false;
     }
     cv_.notify_all();
+    return true;
   }
   // Blocks until the first `n` planes are complete.
   void wait(int n) {
     std::unique_lock<std::mutex> lock(mu_);
+    while (threads_.empty() && ready_ < n) gather_next(lock);
     cv_done_.wait(lock, [&] { return ready_ >= n; });
   }
 
  private:
+  void gather_next(std::unique_lock<std::mutex>& lock) {
+    const int p = next_++;
+    lock.unlock();
+    size_t total = 0;
+    for (int b = 0; b < batch_; ++b) total += lens_[b];
+    uint8_t* d = dst_ + (size_t)p * total * row_;
+    for (int b = 0; b < batch_; ++b) {
+      const size_t n = (size_t)lens_[b] * row_;
+      if (n) copy_streaming(d, static_cast<const uint8_t*>(src_[b]) + (size_t)p * n, n);
+      d += n;
+    }
+    lock.lock();
+    done_[p] = 1;
+    bool moved = false;
+    while (ready_ < planes_ && done_[ready_]) ++ready_, moved = true;
+    if (moved) cv_done_.notify_one();
+  }
   void work() {
     uint64_t seen = 0;
     for (;;) {
       std::unique_lock<std::mutex> lock(mu_);
       cv_.wait(lock, [&] { return stop_ || (job_ != seen && next_ < planes_); });
       if (stop_) return;
-      while (next_ < planes_) {
-        const int p = next_++;
-        lock.unlock();
-        size_t total = 0;
-        for (int b = 0; b < batch_; ++b) total += lens_[b];
-        uint8_t* d = dst_ + (size_t)p * total * row_;
-        for (int b = 0; b < batch_; ++b) {
-          const size_t n = (size_t)lens_[b] * row_;
-          if (n) copy_streaming(d, static_cast<const uint8_t*>(src_[b]) + (size_t)p * n, n);
-          d += n;
-        }
-        lock.lock();
-        done_[p] = 1;
-        bool moved = false;
-        while (ready_ < planes_ && done_[ready_]) ++ready_, moved = true;
-        if (moved) cv_done_.notify_one();
-      }
+      while (next_ < planes_) gather_next(lock);
       seen = job_;
     }
   }
