@@ -124,6 +124,34 @@ def test_two_workers_prepare_the_next_chunk_while_the_first_is_in_flight():
         assert np.array_equal(got, ref)
 
 
+def test_host_requests_arguments_are_checked():
+    """phyai_denoise_requests_host through the C ABI: every bad argument is a status code, and the handle still works."""
+    import ctypes as C
+    from tests.helpers import small_bf16_config
+    cfg = small_bf16_config("pi0", max_batch=2, max_prefix_len=60)
+    W = synth.make_weights(cfg, 28, std=0.05)
+    kvs = [synth.make_prefix_kv(cfg, 28, p, b) for b, p in enumerate([60, 7])]
+    states, noise = ([make(cfg, 28, b) for b in range(2)] for make in (synth.make_state, synth.make_noise))
+    ptrs = lambda ts: (C.c_void_p * len(ts))(*[t.data_ptr() for t in ts])
+    out = torch.empty(2, cfg.horizon, cfg.action_dim).pin_memory()
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        lib, need = ex.lib, ex.lib.phyai_requests_staging_bytes(ex._handle, 2, 67)
+        staging = torch.empty(need + 4, dtype=torch.uint8).pin_memory()
+        good = dict(h=ex._handle, batch=2, kvs=ptrs(kvs), lens=(C.c_uint32 * 2)(60, 7), states=ptrs(states), noises=ptrs(noise), n=3,
+                    out=out.data_ptr(), staging=staging.data_ptr(), bytes=need, stream=None)
+        call = lambda **kw: lib.phyai_denoise_requests_host(*{**good, **kw}.values())
+        for bad in (dict(h=None), dict(batch=0), dict(batch=3), dict(kvs=None), dict(lens=None), dict(states=None), dict(noises=None),
+                    dict(n=0), dict(n=1001), dict(out=None), dict(staging=None), dict(bytes=need - 1), dict(staging=staging.data_ptr() + 2),
+                    dict(lens=(C.c_uint32 * 2)(61, 6)), dict(kvs=(C.c_void_p * 2)(kvs[0].data_ptr(), None))):
+            assert call(**bad) == binding.ERR_INVALID_ARG, bad
+        assert call() == binding.OK
+        torch.cuda.synchronize()
+        assert ex.poll_status() == 0
+        packed, cu = synth.pack_prefix_kv(kvs)
+        dev = ex.denoise_batched(packed.cuda(), torch.from_numpy(cu).cuda(), torch.stack(states).cuda(), torch.stack(noise).cuda(), 3)
+        assert torch.equal(out, dev.cpu())
+
+
 # ------------------------------------------------------------------ feature-handoff head: request-local K / V projections
 @pytest.mark.parametrize("tokens,feat_dim,n_kv,dh,layers", [(300, 512, 2, 128, 3), (37, 1024, 1, 256, 2), (1500, 256, 2, 64, 2)])
 def test_feature_projection_matches_oracle(tokens, feat_dim, n_kv, dh, layers):
