@@ -350,7 +350,8 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     if (e == cudaSuccess) {
       k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
       // (the attention kernels read the request block before their dependency wait: no programmatic launch here)
-      if (attention_b1_ctas(d, (int)batch, 1) <= 15 * 8)     // 15 clusters of 8 fit a B200
+      // (one wave of clusters of eight, 15 on a B200: else CTA pairs with fewer key ranges)
+      if (attention_b1_ctas(d, (int)batch, 1) <= attention_b1_resident_ctas(d))
         e = launch_attention_b1(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch, 1, true, a.wait_limit, st, nullptr, 0, false);
       else
         e = launch_attention_pair(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch,

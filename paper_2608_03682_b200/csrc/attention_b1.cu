@@ -463,22 +463,40 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
 }
 
 template <int DH, int HPC, bool F32>
-cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) {
+cudaError_t setup_one() {
   static PerDeviceOnce once;
-  if (once.needed()) {
-    cudaError_t e = cudaFuncSetAttribute(k_attn_b1<DH, HPC, F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B1Layout<DH, HPC, F32>::SMEM);
-    if (e != cudaSuccess) return e;
-    once.done();
-  }
+  if (!once.needed()) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k_attn_b1<DH, HPC, F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B1Layout<DH, HPC, F32>::SMEM);
+  if (e == cudaSuccess) once.done();
+  return e;
+}
+template <int DH, int HPC, bool F32>
+cudaLaunchConfig_t config_one(const dim3& grid, cudaStream_t st, cudaLaunchAttribute* at, bool pdl) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(8, a.d.Hq / HPC, batch), cfg.blockDim = dim3(288), cfg.dynamicSmemBytes = B1Layout<DH, HPC, F32>::SMEM, cfg.stream = st;
-  cudaLaunchAttribute at[2];
+  cfg.gridDim = grid, cfg.blockDim = dim3(288), cfg.dynamicSmemBytes = B1Layout<DH, HPC, F32>::SMEM, cfg.stream = st;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 8, at[0].val.clusterDim.y = 1, at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at, cfg.numAttrs = pdl ? 2 : 1;
+  return cfg;
+}
+template <int DH, int HPC, bool F32>
+cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) {
+  cudaError_t e = setup_one<DH, HPC, F32>();
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t cfg = config_one<DH, HPC, F32>(dim3(8, a.d.Hq / HPC, batch), st, at, pdl);
   return cudaLaunchKernelEx(&cfg, k_attn_b1<DH, HPC, F32>, a);
+}
+// clusters of this kernel that are resident at a time (0 on an error)
+template <int DH, int HPC, bool F32>
+int max_clusters_one() {
+  if (setup_one<DH, HPC, F32>() != cudaSuccess) return 0;
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t cfg = config_one<DH, HPC, F32>(dim3(8, 1, 64), nullptr, at, false);
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, k_attn_b1<DH, HPC, F32>, &cfg) == cudaSuccess ? n : 0;
 }
 
 }  // namespace
@@ -490,6 +508,10 @@ bool attention_b1_supported(const Dims& d) {
 
 // CTAs of one launch with `hpc` (1 or 2) query heads per CTA
 int attention_b1_ctas(const Dims& d, int batch, int hpc) { return 8 * (d.Hq / hpc) * batch; }
+int attention_b1_resident_ctas(const Dims& d) {
+  static PerDeviceCount resident[2];
+  return 8 * (d.dh == 256 ? resident[1].get(max_clusters_one<256, 1, true>) : resident[0].get(max_clusters_one<128, 1, true>));
+}
 
 cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,

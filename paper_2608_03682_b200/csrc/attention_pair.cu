@@ -619,16 +619,12 @@ int attention_pair_max_ranges(const Dims& d) {
 // clusters of 2 C CTAs the device holds at a time decides the waves (a cluster of 8 needs 8 free SMs in one GPC: 15 on a
 // B200, not 18).
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
-  static std::atomic<int> cached[2][5];
+  static PerDeviceCount resident[2][5];
   const int dh = d.dh == 256 ? 1 : 0, items = batch * (d.Hq / 4);
   int best_c = 1;
   double best = 1e30;
   for (int c = 1; c <= 4; ++c) {
-    int n = cached[dh][c].load();
-    if (n == 0) {
-      n = max_clusters(d.dh, c);
-      cached[dh][c].store(n > 0 ? n : -1);
-    }
+    const int n = resident[dh][c].get([&] { return max_clusters(d.dh, c); });
     if (n <= 0 || c > attention_pair_max_ranges(d)) continue;
     const double cost = (double)((items + n - 1) / n) * ((c > 1 ? 5.5 : 4.0) + (max_prefix + d.S + c * KB - 1) / (c * KB));
     if (cost < best) best = cost, best_c = c;

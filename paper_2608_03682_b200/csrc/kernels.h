@@ -26,6 +26,24 @@ struct PerDeviceOnce {
   }
 };
 
+// A property of a kernel on the current device (how many of its clusters are resident at a time), asked once per device; <= 0:
+// none, or an error.
+struct PerDeviceCount {
+  std::atomic<int> n[64] = {};
+  template <typename F>
+  int get(F ask) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev > 63) return ask();
+    int v = n[dev].load(std::memory_order_acquire);
+    if (v == 0) {
+      v = ask();
+      if (v == 0) v = -1;
+      n[dev].store(v, std::memory_order_release);
+    }
+    return v;
+  }
+};
+
 // Launch with programmatic stream serialization (see pdl_enter in common.cuh): only for kernels that call
 // pdl_enter() before touching global memory.
 template <typename... KArgs, typename... Args>
@@ -205,8 +223,9 @@ cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloa
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
                                 int batch, int hpc, bool f32, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr,
                                 int trace_all = 0, bool pdl = true);   // f32: fp32 partial results (one head per CTA only)
-// CTAs of one launch with `hpc` (1 or 2) query heads per CTA
+// CTAs of one launch with `hpc` (1 or 2) query heads per CTA, and how many of the fp32 form are resident at a time
 int attention_b1_ctas(const Dims& d, int batch, int hpc);
+int attention_b1_resident_ctas(const Dims& d);
 cudaError_t launch_attention_tc(const Request* rq, int* status, const __nv_bfloat16* qr, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
                                 int batch, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace = nullptr,
