@@ -346,12 +346,13 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     __nv_bfloat16 *qt = reinterpret_cast<__nv_bfloat16*>(rq + 1), *kr = qt + q_elems, *vr = kr + kv_elems;
     Request r{};
     r.prefix_kv = prefix_kv, r.kv_tokens = kv_tokens, r.cu_lens = cu, r.batch = (int)batch;
-    if (!prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
+    // One wave of clusters of eight (15 on a B200), else CTA pairs with fewer key ranges, which read the cache through a tensor map.
+    const bool b1 = attention_b1_ctas(d, (int)batch, 1) <= attention_b1_resident_ctas(d);
+    if (!b1 && !prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) {
       k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
       // (the attention kernels read the request block before their dependency wait: no programmatic launch here)
-      // (one wave of clusters of eight, 15 on a B200: else CTA pairs with fewer key ranges)
-      if (attention_b1_ctas(d, (int)batch, 1) <= attention_b1_resident_ctas(d))
+      if (b1)
         e = launch_attention_b1(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch, 1, true, a.wait_limit, st, nullptr, 0, false);
       else
         e = launch_attention_pair(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch,
