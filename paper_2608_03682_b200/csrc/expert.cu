@@ -73,9 +73,10 @@ struct phyai_expert {
 
   // big matrices
   std::vector<float*> f_qkv, f_o, f_g, f_u, f_d;                 // SIMT fp32 row-major
-  std::vector<__nv_bfloat16*> p_qkv, p_o, p_g, p_u, p_d;         // TC packed
+  std::vector<__nv_bfloat16*> p_qkv, p_o, p_g, p_u, p_d;         // TC packed (p_g, p_u: entries null where no default kernel
+                                                                 // reads them, see split_gate_up)
   std::vector<float*> s_qkv, s_o, s_g, s_u, s_d;                 // TC per-channel scales (or null)
-  std::vector<uint8_t*> b_qkv, b_o, b_gu, b_d;                   // e4m3 byte blocks for the cluster GEMM (W8 experts)
+  std::vector<uint8_t*> b_qkv, b_o, b_gu, b_d;                   // code blocks for the cluster GEMM, see code_blocks
 
   float2* rope = nullptr;
   float2* rope_il = nullptr;   // the same with interleaved channels, for the pair GEMM's rotary epilogue
@@ -91,7 +92,7 @@ struct phyai_expert {
   bool il_ok = false;          // gate / up also packed interleaved (single-token-tile calls)
   bool b1_ok = false;          // the cluster split-K GEMM path covers this expert's shapes
   int use_cluster_gemm = 1;
-  int use_b1_attention = 1;
+  int use_b1_attention = 1;    // tcgen05 attention with the key range split over a cluster (few requests)
   int b1_attn_hpc = 0;         // query heads per CTA of the cluster attention kernel (0 = choose)
   int use_b1_step = 1;         // single-tile calls: velocity head + Euler update + next embedding as one cluster kernel
   int use_state_cache = 0;     // block-causal experts: state token computed once per call (single-tile calls); exact, but at
@@ -102,7 +103,6 @@ struct phyai_expert {
   // of shared-memory traffic) lies on it for every CTA that starts late: pi0 with e4m3 codes 5.09 ms with images, 5.76 with
   // codes, 5.15 with codes in the QKV projection alone.
   int use_w8_inkernel = 0;
-    // tcgen05 attention with the key range split over a cluster (few requests)
   int use_b1_pair = 1;         // single-tile calls: projections on CTA pairs where they fit
   int b1_c[4] = {0, 0, 0, 0};  // cluster sizes of the QKV / O / gate-up / down projections (0 = choose)
   float *ss_a = nullptr, *ss_b = nullptr;   // [D/128 or D/64][64] partial sums of squares of h (after O / after down)
@@ -204,6 +204,45 @@ phyai_status_t check_config(const phyai_expert_config_t* c) {
 bool tc_shape_ok(const phyai_expert_config_t* c) {
   const uint32_t nq = c->n_q_heads * c->head_dim, nqkv = (c->n_q_heads + 2 * c->n_kv_heads) * c->head_dim;
   return c->width % 128 == 0 && c->mlp_dim % 128 == 0 && nq % 128 == 0 && nqkv % 128 == 0;
+}
+
+// ---------------------------------------------------------------------------------------------
+// weight images that only options ask for, made from those of the default paths when the option is set
+// ---------------------------------------------------------------------------------------------
+// Gate and up as matrices of their own, from the image with the two interleaved in groups of 64 channels: half blocks of 64
+// rows (8 KB) move as they are.
+phyai_status_t split_gate_up(phyai_expert* h) {
+  if (!h->pair_ok || h->p_g[0]) return PHYAI_OK;
+  const size_t KC = h->d.D / 64, layer = (size_t)h->d.D * h->d.F, half = 64 * 64, block = 2 * half;
+  __nv_bfloat16 *g = nullptr, *u = nullptr;
+  ST(h->alloc(&g, h->d.L * layer)); ST(h->alloc(&u, h->d.L * layer));
+  for (int l = 0; l < h->d.L; ++l)
+    for (int c = 0; c < h->d.F / 64; ++c)
+      for (int up = 0; up < 2; ++up)
+        CU(cudaMemcpy2DAsync((up ? u : g) + l * layer + (c >> 1) * KC * block + (c & 1) * half, block * 2,
+                             h->p_gu_all + 2 * l * layer + c * KC * block + up * half, block * 2, half * 2, KC, cudaMemcpyDeviceToDevice, h->cap_stream));
+  CU(cudaStreamSynchronize(h->cap_stream));
+  for (int l = 0; l < h->d.L; ++l) h->p_g[l] = g + l * layer, h->p_u[l] = u + l * layer;
+  return PHYAI_OK;
+}
+// Weight codes for the cluster GEMM that decodes them, from the bf16 images (which hold the codes' values exactly).
+phyai_status_t code_blocks(phyai_expert* h) {
+  const bool w4 = h->cfg.dtype == PHYAI_W4A16;
+  if ((h->cfg.dtype != PHYAI_W8E4M3_A16 && !w4) || !h->b1_ok || !h->b_qkv.empty()) return PHYAI_OK;
+  const size_t D = h->d.D, F = h->d.F, L = h->d.L;
+  const size_t n[4] = {D * h->d.Nqkv, (size_t)h->d.Nq * D, D * 2 * F, F * D};
+  const __nv_bfloat16* img[4] = {h->pq_all, h->po_all, h->p_gu_all, h->pd_all};
+  uint8_t* all[4];
+  for (int m = 0; m < 4; ++m) {
+    ST(h->alloc(&all[m], L * n[m] / (w4 ? 2 : 1)));
+    launch_image_codes(img[m], all[m], L * n[m], w4 ? 4 : 8, h->cap_stream);
+  }
+  CU(cudaGetLastError());
+  CU(cudaStreamSynchronize(h->cap_stream));
+  std::vector<uint8_t*>* v[4] = {&h->b_qkv, &h->b_o, &h->b_gu, &h->b_d};
+  for (int m = 0; m < 4; ++m)
+    for (size_t l = 0; l < L; ++l) v[m]->push_back(all[m] + l * n[m] / (w4 ? 2 : 1));
+  return PHYAI_OK;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1050,151 +1089,18 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
         launch_to_f32(bsrc, kind, h->bmod + (size_t)s * 3 * D, (size_t)3 * D, st);
       }
     }
-    // ---- the seven big matrices per layer ----
+    // ---- which kernel families cover this expert ----
     const int Nq = d.Nq, Nkv = d.Hkv * d.dh, Nqkv = d.Nqkv, F = d.F;
-    __nv_bfloat16 *pq_all = nullptr, *po_all = nullptr, *pg_all = nullptr, *pu_all = nullptr, *pd_all = nullptr;
-    if (tc) {   // one allocation per matrix kind, layers at a fixed stride (the persistent kernel indexes by layer)
-      ST(h->alloc(&pq_all, (size_t)L * D * Nqkv)); ST(h->alloc(&po_all, (size_t)L * Nq * D));
-      ST(h->alloc(&pg_all, (size_t)L * D * F)); ST(h->alloc(&pu_all, (size_t)L * D * F));
-      ST(h->alloc(&pd_all, (size_t)L * F * D));
-      h->pq_all = pq_all, h->po_all = po_all, h->pd_all = pd_all;
+    if (tc) {
       h->il_ok = F % 64 == 0 && !a8;   // (W8A8 keeps to the general kernels: no interleaved image, no cluster path)
-      if (h->il_ok) ST(h->alloc(&h->p_gu_all, (size_t)L * D * 2 * F));
       h->pair_ok = h->il_ok && (d.dh == 128 || d.dh == 256) && d.S <= 64 && cfg->max_batch * d.S > 64 && attention_mma_supported(d) &&
                    pair_gemm_supported(Nqkv, D) && pair_gemm_supported(D, Nq) && pair_gemm_supported(2 * F, D) && pair_gemm_supported(D, F);
-      // token counts that use 256-token tiles: the persistent gate / up kernel and its weight image (the pair GEMMs' too)
-      if (h->pair_ok || (pick_nt((int)(cfg->max_batch * d.S)) == 256 && persist_gemm_supported((int)(cfg->max_batch * d.S), 2 * F, D, h->Mpad, a8))) {
-        ST(h->alloc(&h->p_gu16, (size_t)L * D * 2 * F / (a8 ? 2 : 1)));
-        if ((d.dh == 128 || d.dh == 256) && d.S <= 64) ST(h->alloc(&h->p_qkv16, (size_t)L * D * Nqkv / (a8 ? 2 : 1)));
-      }
       // cluster split-K path (one 64-token tile): every projection must fit the kernel's resident stages
       auto fits = [&](int N, int K, bool qkv) {
         return b1_gemm_supported(N, K, b1_pick_cluster(N / 128, K / 64, h->n_sm), h->n_sm, qkv);
       };
       h->b1_ok = h->il_ok && (d.dh == 128 || d.dh == 256) && D % 128 == 0 && d.S <= 64 && fits(Nqkv, D, true) &&
                  fits(D, Nq, false) && fits(2 * F, D, false) && fits(D, F, false);
-      if (w8) {
-        ST(h->alloc(&h->s_qkv_all, (size_t)L * Nqkv)); ST(h->alloc(&h->s_o_all, (size_t)L * D));
-        ST(h->alloc(&h->s_g_all, (size_t)L * F)); ST(h->alloc(&h->s_u_all, (size_t)L * F));
-        ST(h->alloc(&h->s_d_all, (size_t)L * D));
-      }
-    }
-    for (int l = 0; l < L; ++l) {
-      const float* sq = w8 ? w->scales[0][l] : nullptr; const float* sk = w8 ? w->scales[1][l] : nullptr;
-      const float* sv = w8 ? w->scales[2][l] : nullptr; const float* so = w8 ? w->scales[3][l] : nullptr;
-      const float* sg = w8 ? w->scales[4][l] : nullptr; const float* su = w8 ? w->scales[5][l] : nullptr;
-      const float* sd = w8 ? w->scales[6][l] : nullptr;
-      if (tc) {
-        __nv_bfloat16 *pq = pq_all + (size_t)l * D * Nqkv, *po = po_all + (size_t)l * Nq * D;
-        __nv_bfloat16 *pg = pg_all + (size_t)l * D * F, *pu = pu_all + (size_t)l * D * F, *pd = pd_all + (size_t)l * F * D;
-        if (h->p_gu16) {
-          // (bf16 image: 2 bytes per weight; W8A8: the e4m3 codes, 1 byte per weight, in the first half of the layer's slot)
-          __nv_bfloat16* p16 = h->p_gu16 + (size_t)l * D * 2 * F / (a8 ? 2 : 1);
-          if (a8) {
-            launch_pack_bytes(reinterpret_cast<const uint8_t*>(w->wgate[l]), reinterpret_cast<uint8_t*>(p16), D, F, 0, st, 16, 0, 0, 1);
-            launch_pack_bytes(reinterpret_cast<const uint8_t*>(w->wup[l]), reinterpret_cast<uint8_t*>(p16), D, F, 0, st, 16, 1, 0, 1);
-          } else {
-            launch_pack_tiled(w->wgate[l], big_kind, p16, D, F, 0, st, 16, 0);
-            launch_pack_tiled(w->wup[l], big_kind, p16, D, F, 0, st, 16, 1);
-          }
-        }
-        if (h->p_qkv16) {
-          __nv_bfloat16* p16 = h->p_qkv16 + (size_t)l * D * Nqkv / (a8 ? 2 : 1);
-          if (a8) {
-            auto u8 = [](const void* p) { return reinterpret_cast<const uint8_t*>(p); };
-            uint8_t* o8 = reinterpret_cast<uint8_t*>(p16);
-            launch_pack_bytes(u8(w->wq[l]), o8, D, Nq, 0, st, 0, 0, d.dh, 1, 1);
-            launch_pack_bytes(u8(w->wk[l]), o8, D, Nkv, Nq, st, 0, 0, d.dh, 1, 1);
-            launch_pack_bytes(u8(w->wv[l]), o8, D, Nkv, Nq + Nkv, st, 0, 0, 0, 1, 1);
-          } else {
-            launch_pack_tiled(w->wq[l], big_kind, p16, D, Nq, 0, st, 0, 0, d.dh, 1);
-            launch_pack_tiled(w->wk[l], big_kind, p16, D, Nkv, Nq, st, 0, 0, d.dh, 1);
-            launch_pack_tiled(w->wv[l], big_kind, p16, D, Nkv, Nq + Nkv, st, 0, 0, 0, 1);
-          }
-        }
-        if (h->il_ok) {
-          __nv_bfloat16* pgu = h->p_gu_all + (size_t)l * D * 2 * F;
-          launch_pack_tiled(w->wgate[l], big_kind, pgu, D, F, 0, st, 64, 0);
-          launch_pack_tiled(w->wup[l], big_kind, pgu, D, F, 0, st, 64, 1);
-        }
-        if (a8) {
-          // the e4m3 codes themselves as operand images: blocks of 128 channels x 128 k (the allocations are sized
-          // for bf16 images: half of each is used)
-          auto u8 = [](const void* p) { return reinterpret_cast<const uint8_t*>(p); };
-          auto o8 = [](__nv_bfloat16* p) { return reinterpret_cast<uint8_t*>(p); };
-          launch_pack_bytes(u8(w->wq[l]), o8(pq), D, Nq, 0, st, 0, 0, d.dh, 1);
-          launch_pack_bytes(u8(w->wk[l]), o8(pq), D, Nkv, Nq, st, 0, 0, d.dh, 1);
-          launch_pack_bytes(u8(w->wv[l]), o8(pq), D, Nkv, Nq + Nkv, st, 0, 0, 0, 1);
-          launch_pack_bytes(u8(w->wo[l]), o8(po), Nq, D, 0, st, 0, 0, 0, 1);
-          launch_pack_bytes(u8(w->wgate[l]), o8(pg), D, F, 0, st, 0, 0, 0, 1);
-          launch_pack_bytes(u8(w->wup[l]), o8(pu), D, F, 0, st, 0, 0, 0, 1);
-          launch_pack_bytes(u8(w->wdown[l]), o8(pd), F, D, 0, st, 0, 0, 0, 1);
-        } else {
-          launch_pack_tiled(w->wq[l], big_kind, pq, D, Nq, 0, st, 0, 0, d.dh);
-          launch_pack_tiled(w->wk[l], big_kind, pq, D, Nkv, Nq, st, 0, 0, d.dh);
-          launch_pack_tiled(w->wv[l], big_kind, pq, D, Nkv, Nq + Nkv, st);
-          launch_pack_tiled(w->wo[l], big_kind, po, Nq, D, 0, st);
-          launch_pack_tiled(w->wgate[l], big_kind, pg, D, F, 0, st);
-          launch_pack_tiled(w->wup[l], big_kind, pu, D, F, 0, st);
-          launch_pack_tiled(w->wdown[l], big_kind, pd, F, D, 0, st);
-        }
-        h->p_qkv.push_back(pq), h->p_o.push_back(po), h->p_g.push_back(pg), h->p_u.push_back(pu), h->p_d.push_back(pd);
-        if (w8 && !a8 && h->b1_ok) {
-          // one byte per weight for the single-tile (HBM-bound) path; larger batches are tensor-bound and keep using
-          // the bf16 images above
-          uint8_t *bq, *bo, *bgu, *bd;
-          const size_t div = w4 ? 2 : 1;     // int4: half a byte per weight
-          ST(h->alloc(&bq, (size_t)D * Nqkv / div)); ST(h->alloc(&bo, (size_t)Nq * D / div));
-          ST(h->alloc(&bgu, (size_t)D * 2 * F / div)); ST(h->alloc(&bd, (size_t)F * D / div));
-          auto pack = [&](const void* src, uint8_t* dst, int K, int N, int n_off, int il = 0, int second = 0, int perm = 0) {
-            if (w4) launch_pack_nibbles(reinterpret_cast<const uint8_t*>(src), dst, K, N, n_off, st, il, second, perm);
-            else launch_pack_bytes(reinterpret_cast<const uint8_t*>(src), dst, K, N, n_off, st, il, second, perm);
-          };
-          pack(w->wq[l], bq, D, Nq, 0, 0, 0, d.dh);
-          pack(w->wk[l], bq, D, Nkv, Nq, 0, 0, d.dh);
-          pack(w->wv[l], bq, D, Nkv, Nq + Nkv);
-          pack(w->wo[l], bo, Nq, D, 0);
-          pack(w->wgate[l], bgu, D, F, 0, 64, 0);
-          pack(w->wup[l], bgu, D, F, 0, 64, 1);
-          pack(w->wdown[l], bd, F, D, 0);
-          h->b_qkv.push_back(bq), h->b_o.push_back(bo), h->b_gu.push_back(bgu), h->b_d.push_back(bd);
-        }
-        float *cq = nullptr, *co = nullptr, *cg = nullptr, *cu = nullptr, *cd = nullptr;
-        if (w8) {
-          cq = h->s_qkv_all + (size_t)l * Nqkv, co = h->s_o_all + (size_t)l * D, cg = h->s_g_all + (size_t)l * F;
-          cu = h->s_u_all + (size_t)l * F, cd = h->s_d_all + (size_t)l * D;
-          launch_permute_scales(sq, cq, Nq, 0, d.dh, st);
-          launch_permute_scales(sk, cq, Nkv, Nq, d.dh, st);
-          CU(cudaMemcpyAsync(cq + Nq + Nkv, sv, (size_t)Nkv * 4, cudaMemcpyDeviceToDevice, st));
-          CU(cudaMemcpyAsync(co, so, (size_t)D * 4, cudaMemcpyDeviceToDevice, st));
-          CU(cudaMemcpyAsync(cg, sg, (size_t)F * 4, cudaMemcpyDeviceToDevice, st));
-          CU(cudaMemcpyAsync(cu, su, (size_t)F * 4, cudaMemcpyDeviceToDevice, st));
-          CU(cudaMemcpyAsync(cd, sd, (size_t)D * 4, cudaMemcpyDeviceToDevice, st));
-        }
-        h->s_qkv.push_back(cq), h->s_o.push_back(co), h->s_g.push_back(cg), h->s_u.push_back(cu), h->s_d.push_back(cd);
-      } else {
-        float *fq, *fo, *fg, *fu, *fd;
-        ST(h->alloc(&fq, (size_t)D * Nqkv)); ST(h->alloc(&fo, (size_t)Nq * D));
-        ST(h->alloc(&fg, (size_t)D * F)); ST(h->alloc(&fu, (size_t)D * F)); ST(h->alloc(&fd, (size_t)F * D));
-        launch_copy_cols(w->wq[l], big_kind, sq, fq, D, Nq, Nqkv, 0, st);
-        launch_copy_cols(w->wk[l], big_kind, sk, fq, D, Nkv, Nqkv, Nq, st);
-        launch_copy_cols(w->wv[l], big_kind, sv, fq, D, Nkv, Nqkv, Nq + Nkv, st);
-        launch_copy_cols(w->wo[l], big_kind, so, fo, Nq, D, D, 0, st);
-        launch_copy_cols(w->wgate[l], big_kind, sg, fg, D, F, F, 0, st);
-        launch_copy_cols(w->wup[l], big_kind, su, fu, D, F, F, 0, st);
-        launch_copy_cols(w->wdown[l], big_kind, sd, fd, F, D, D, 0, st);
-        h->f_qkv.push_back(fq), h->f_o.push_back(fo), h->f_g.push_back(fg), h->f_u.push_back(fu), h->f_d.push_back(fd);
-      }
-    }
-    // ---- rotary table ----
-    if (cfg->rope_theta > 0.f) {
-      const int npos = (int)cfg->max_prefix_len + d.S;
-      ST(h->alloc(&h->rope, (size_t)npos * (d.dh / 2)));
-      launch_rope_table(h->rope, npos, d.dh, (double)cfg->rope_theta, st);
-      if (h->pair_ok) {
-        ST(h->alloc(&h->rope_il, (size_t)npos * (d.dh / 2)));
-        launch_rope_table(h->rope_il, npos, d.dh, (double)cfg->rope_theta, st, 1);
-      }
     }
     // ---- workspace (zeroed: padding rows of the tiled buffers stay finite) ----
     ST(h->alloc(&h->h, Mp * D, true));
@@ -1254,6 +1160,126 @@ phyai_status_t phyai_expert_create(const phyai_expert_config_t* cfg, const phyai
       ST(h->alloc(&h->attn_f, Mp * Nq, true));
       ST(h->alloc(&h->m_f, Mp * F, true));
       if (!ada) ST(h->alloc(&h->u_f, Mp * D, true));
+    }
+    // ---- the seven big matrices per layer ----
+    __nv_bfloat16 *pq_all = nullptr, *po_all = nullptr, *pg_all = nullptr, *pu_all = nullptr, *pd_all = nullptr;
+    if (tc) {   // one allocation per matrix kind, layers at a fixed stride (the persistent kernel indexes by layer)
+      ST(h->alloc(&pq_all, (size_t)L * D * Nqkv)); ST(h->alloc(&po_all, (size_t)L * Nq * D));
+      ST(h->alloc(&pd_all, (size_t)L * F * D));
+      h->pq_all = pq_all, h->po_all = po_all, h->pd_all = pd_all;
+      if (h->il_ok) ST(h->alloc(&h->p_gu_all, (size_t)L * D * 2 * F));
+      // Gate and up as matrices of their own: calls of more than 64 tokens off the pair path (see split_gate_up)
+      if (!h->il_ok || (!h->pair_ok && cfg->max_batch * d.S > 64)) {
+        ST(h->alloc(&pg_all, (size_t)L * D * F)); ST(h->alloc(&pu_all, (size_t)L * D * F));
+      }
+      // token counts that use 256-token tiles: the persistent gate / up kernel and its weight image (the pair GEMMs' too)
+      if (h->pair_ok || (pick_nt((int)(cfg->max_batch * d.S)) == 256 && persist_gemm_supported((int)(cfg->max_batch * d.S), 2 * F, D, h->Mpad, a8))) {
+        ST(h->alloc(&h->p_gu16, (size_t)L * D * 2 * F / (a8 ? 2 : 1)));
+        if ((d.dh == 128 || d.dh == 256) && d.S <= 64) ST(h->alloc(&h->p_qkv16, (size_t)L * D * Nqkv / (a8 ? 2 : 1)));
+      }
+      if (w8) {
+        ST(h->alloc(&h->s_qkv_all, (size_t)L * Nqkv)); ST(h->alloc(&h->s_o_all, (size_t)L * D));
+        ST(h->alloc(&h->s_g_all, (size_t)L * F)); ST(h->alloc(&h->s_u_all, (size_t)L * F));
+        ST(h->alloc(&h->s_d_all, (size_t)L * D));
+      }
+    }
+    for (int l = 0; l < L; ++l) {
+      const float* sq = w8 ? w->scales[0][l] : nullptr; const float* sk = w8 ? w->scales[1][l] : nullptr;
+      const float* sv = w8 ? w->scales[2][l] : nullptr; const float* so = w8 ? w->scales[3][l] : nullptr;
+      const float* sg = w8 ? w->scales[4][l] : nullptr; const float* su = w8 ? w->scales[5][l] : nullptr;
+      const float* sd = w8 ? w->scales[6][l] : nullptr;
+      if (tc) {
+        __nv_bfloat16 *pq = pq_all + (size_t)l * D * Nqkv, *po = po_all + (size_t)l * Nq * D;
+        __nv_bfloat16 *pg = pg_all ? pg_all + (size_t)l * D * F : nullptr, *pu = pu_all ? pu_all + (size_t)l * D * F : nullptr;
+        __nv_bfloat16* pd = pd_all + (size_t)l * F * D;
+        if (h->p_gu16) {
+          // (bf16 image: 2 bytes per weight; W8A8: the e4m3 codes, 1 byte per weight, in the first half of the layer's slot)
+          __nv_bfloat16* p16 = h->p_gu16 + (size_t)l * D * 2 * F / (a8 ? 2 : 1);
+          if (a8) {
+            launch_pack_bytes(reinterpret_cast<const uint8_t*>(w->wgate[l]), reinterpret_cast<uint8_t*>(p16), D, F, 0, st, 16, 0);
+            launch_pack_bytes(reinterpret_cast<const uint8_t*>(w->wup[l]), reinterpret_cast<uint8_t*>(p16), D, F, 0, st, 16, 1);
+          } else {
+            launch_pack_tiled(w->wgate[l], big_kind, p16, D, F, 0, st, 16, 0);
+            launch_pack_tiled(w->wup[l], big_kind, p16, D, F, 0, st, 16, 1);
+          }
+        }
+        if (h->p_qkv16) {
+          __nv_bfloat16* p16 = h->p_qkv16 + (size_t)l * D * Nqkv / (a8 ? 2 : 1);
+          if (a8) {
+            auto u8 = [](const void* p) { return reinterpret_cast<const uint8_t*>(p); };
+            uint8_t* o8 = reinterpret_cast<uint8_t*>(p16);
+            launch_pack_bytes(u8(w->wq[l]), o8, D, Nq, 0, st, 0, 0, d.dh, 1);
+            launch_pack_bytes(u8(w->wk[l]), o8, D, Nkv, Nq, st, 0, 0, d.dh, 1);
+            launch_pack_bytes(u8(w->wv[l]), o8, D, Nkv, Nq + Nkv, st, 0, 0, 0, 1);
+          } else {
+            launch_pack_tiled(w->wq[l], big_kind, p16, D, Nq, 0, st, 0, 0, d.dh, 1);
+            launch_pack_tiled(w->wk[l], big_kind, p16, D, Nkv, Nq, st, 0, 0, d.dh, 1);
+            launch_pack_tiled(w->wv[l], big_kind, p16, D, Nkv, Nq + Nkv, st, 0, 0, 0, 1);
+          }
+        }
+        if (h->il_ok) {
+          __nv_bfloat16* pgu = h->p_gu_all + (size_t)l * D * 2 * F;
+          launch_pack_tiled(w->wgate[l], big_kind, pgu, D, F, 0, st, 64, 0);
+          launch_pack_tiled(w->wup[l], big_kind, pgu, D, F, 0, st, 64, 1);
+        }
+        if (a8) {
+          // the e4m3 codes themselves as operand images: blocks of 128 channels x 128 k (the allocations are sized
+          // for bf16 images: half of each is used)
+          auto u8 = [](const void* p) { return reinterpret_cast<const uint8_t*>(p); };
+          auto o8 = [](__nv_bfloat16* p) { return reinterpret_cast<uint8_t*>(p); };
+          launch_pack_bytes(u8(w->wq[l]), o8(pq), D, Nq, 0, st, 0, 0, d.dh);
+          launch_pack_bytes(u8(w->wk[l]), o8(pq), D, Nkv, Nq, st, 0, 0, d.dh);
+          launch_pack_bytes(u8(w->wv[l]), o8(pq), D, Nkv, Nq + Nkv, st);
+          launch_pack_bytes(u8(w->wo[l]), o8(po), Nq, D, 0, st);
+          launch_pack_bytes(u8(w->wgate[l]), o8(pg), D, F, 0, st);
+          launch_pack_bytes(u8(w->wup[l]), o8(pu), D, F, 0, st);
+          launch_pack_bytes(u8(w->wdown[l]), o8(pd), F, D, 0, st);
+        } else {
+          launch_pack_tiled(w->wq[l], big_kind, pq, D, Nq, 0, st, 0, 0, d.dh);
+          launch_pack_tiled(w->wk[l], big_kind, pq, D, Nkv, Nq, st, 0, 0, d.dh);
+          launch_pack_tiled(w->wv[l], big_kind, pq, D, Nkv, Nq + Nkv, st);
+          launch_pack_tiled(w->wo[l], big_kind, po, Nq, D, 0, st);
+          if (pg) launch_pack_tiled(w->wgate[l], big_kind, pg, D, F, 0, st);
+          if (pu) launch_pack_tiled(w->wup[l], big_kind, pu, D, F, 0, st);
+          launch_pack_tiled(w->wdown[l], big_kind, pd, F, D, 0, st);
+        }
+        h->p_qkv.push_back(pq), h->p_o.push_back(po), h->p_g.push_back(pg), h->p_u.push_back(pu), h->p_d.push_back(pd);
+        float *cq = nullptr, *co = nullptr, *cg = nullptr, *cu = nullptr, *cd = nullptr;
+        if (w8) {
+          cq = h->s_qkv_all + (size_t)l * Nqkv, co = h->s_o_all + (size_t)l * D, cg = h->s_g_all + (size_t)l * F;
+          cu = h->s_u_all + (size_t)l * F, cd = h->s_d_all + (size_t)l * D;
+          launch_permute_scales(sq, cq, Nq, 0, d.dh, st);
+          launch_permute_scales(sk, cq, Nkv, Nq, d.dh, st);
+          CU(cudaMemcpyAsync(cq + Nq + Nkv, sv, (size_t)Nkv * 4, cudaMemcpyDeviceToDevice, st));
+          CU(cudaMemcpyAsync(co, so, (size_t)D * 4, cudaMemcpyDeviceToDevice, st));
+          CU(cudaMemcpyAsync(cg, sg, (size_t)F * 4, cudaMemcpyDeviceToDevice, st));
+          CU(cudaMemcpyAsync(cu, su, (size_t)F * 4, cudaMemcpyDeviceToDevice, st));
+          CU(cudaMemcpyAsync(cd, sd, (size_t)D * 4, cudaMemcpyDeviceToDevice, st));
+        }
+        h->s_qkv.push_back(cq), h->s_o.push_back(co), h->s_g.push_back(cg), h->s_u.push_back(cu), h->s_d.push_back(cd);
+      } else {
+        float *fq, *fo, *fg, *fu, *fd;
+        ST(h->alloc(&fq, (size_t)D * Nqkv)); ST(h->alloc(&fo, (size_t)Nq * D));
+        ST(h->alloc(&fg, (size_t)D * F)); ST(h->alloc(&fu, (size_t)D * F)); ST(h->alloc(&fd, (size_t)F * D));
+        launch_copy_cols(w->wq[l], big_kind, sq, fq, D, Nq, Nqkv, 0, st);
+        launch_copy_cols(w->wk[l], big_kind, sk, fq, D, Nkv, Nqkv, Nq, st);
+        launch_copy_cols(w->wv[l], big_kind, sv, fq, D, Nkv, Nqkv, Nq + Nkv, st);
+        launch_copy_cols(w->wo[l], big_kind, so, fo, Nq, D, D, 0, st);
+        launch_copy_cols(w->wgate[l], big_kind, sg, fg, D, F, F, 0, st);
+        launch_copy_cols(w->wup[l], big_kind, su, fu, D, F, F, 0, st);
+        launch_copy_cols(w->wdown[l], big_kind, sd, fd, F, D, D, 0, st);
+        h->f_qkv.push_back(fq), h->f_o.push_back(fo), h->f_g.push_back(fg), h->f_u.push_back(fu), h->f_d.push_back(fd);
+      }
+    }
+    // ---- rotary table ----
+    if (cfg->rope_theta > 0.f) {
+      const int npos = (int)cfg->max_prefix_len + d.S;
+      ST(h->alloc(&h->rope, (size_t)npos * (d.dh / 2)));
+      launch_rope_table(h->rope, npos, d.dh, (double)cfg->rope_theta, st);
+      if (h->pair_ok) {
+        ST(h->alloc(&h->rope_il, (size_t)npos * (d.dh / 2)));
+        launch_rope_table(h->rope_il, npos, d.dh, (double)cfg->rope_theta, st, 1);
+      }
     }
     CU(cudaGetLastError());
     CU(cudaStreamSynchronize(st));
@@ -1509,6 +1535,7 @@ phyai_status_t phyai_set_option(phyai_expert_t* h, const char* key, int64_t valu
     return PHYAI_OK;
   }
   if (!strcmp(key, "use_w8_inkernel")) {
+    if (value) ST(code_blocks(h));
     h->use_w8_inkernel = value != 0;
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();
@@ -1523,6 +1550,7 @@ phyai_status_t phyai_set_option(phyai_expert_t* h, const char* key, int64_t valu
   if (!strcmp(key, "use_cluster_gemm") || !strcmp(key, "b1_c_qkv") || !strcmp(key, "b1_c_o") || !strcmp(key, "b1_c_gu") ||
       !strcmp(key, "b1_c_d")) {
     if (!strcmp(key, "use_cluster_gemm")) {
+      if (!value) ST(split_gate_up(h));
       h->use_cluster_gemm = value != 0;
     } else {
       if (value < 0 || value > 8) return fail(PHYAI_ERR_INVALID_ARG, "cluster size out of range 0..8");
@@ -1551,12 +1579,14 @@ phyai_status_t phyai_set_option(phyai_expert_t* h, const char* key, int64_t valu
     return PHYAI_OK;
   }
   if (!strcmp(key, "use_pair_gemm") || !strcmp(key, "use_pair_attention")) {
+    if (!value && !strcmp(key, "use_pair_gemm")) ST(split_gate_up(h));
     (!strcmp(key, "use_pair_gemm") ? h->use_pair_gemm : h->use_pair_attention) = value != 0;
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();
     return PHYAI_OK;
   }
   if (!strcmp(key, "use_persistent_gu") || !strcmp(key, "use_persistent_qkv") || !strcmp(key, "use_attn_splits")) {
+    if (!value && strcmp(key, "use_attn_splits")) ST(split_gate_up(h));
     (!strcmp(key, "use_persistent_gu") ? h->use_persistent_gu : !strcmp(key, "use_attn_splits") ? h->use_attn_splits : h->use_persistent_qkv) = value != 0;
     for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
     h->graphs.clear();

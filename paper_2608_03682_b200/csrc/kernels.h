@@ -89,11 +89,10 @@ void launch_copy_cols(const void* src, int src_kind, const float* scale, float* 
 // row r of the tile goes to row 32 ((r % 64) / 16) + 16 (r / 64) + r % 16 (rows r and r + 64 end up 16 apart).
 void launch_pack_tiled(const void* src, int src_kind, __nv_bfloat16* dst, int K, int N, int n_off, cudaStream_t st,
                        int il_group = 0, int il_second = 0, int perm_dh = 0, int pair16 = 0);
-// e4m3 codes [in=K][out=N] -> byte blocks [N/128][K/64][128][64] in the packed row order of launch_pack_tiled
+// e4m3 codes [in=K][out=N] -> byte blocks [N/128][K/128][128][128] in the packed row order of launch_pack_tiled, the 16-byte
+// chunks of a row XOR-swizzled by row & 7: the e4m3 operand image of the FP8 tensor path
 void launch_pack_bytes(const uint8_t* src, uint8_t* dst, int K, int N, int n_off, cudaStream_t st, int il_group = 0,
-                       int il_second = 0, int perm_dh = 0, int wide = 0, int pair16 = 0);
-// (wide: blocks [N/128][K/128][128][128] instead, the 16-byte chunks of a row XOR-swizzled by row & 7: the e4m3
-// operand image of the FP8 tensor path)
+                       int il_second = 0, int perm_dh = 0, int pair16 = 0);
 // row-major bf16 [M][K] (K a multiple of 8, 16-byte aligned rows) -> the tiled bf16 layout of the GEMM inputs
 void launch_rows_to_tiled(const __nv_bfloat16* x, __nv_bfloat16* tiled, int M, int K, int rows_pad, cudaStream_t st);
 // Per-token e4m3 quantization of a tiled bf16 activation matrix [K/64][rows_pad][64] (W8A8): scale[r] = max|x_r| / 448
@@ -101,10 +100,9 @@ void launch_rows_to_tiled(const __nv_bfloat16* x, __nv_bfloat16* tiled, int M, i
 // [K/128][rows_pad][128] with the same 16-byte chunk swizzle.  Rows >= M are left alone.
 void launch_quant_rows(const int* status, const __nv_bfloat16* x, uint8_t* out, float* scale, int rows_pad, int M, int K,
                        cudaStream_t st);
-// int4 codes [K][N/2] (two neighbouring out channels per byte) -> nibble blocks [N/128][K/64][128][32] in the packed
-// row order of launch_pack_tiled, byte j of a row = codes of k = 2j (low nibble) and 2j + 1 (high nibble)
-void launch_pack_nibbles(const uint8_t* src, uint8_t* dst, int K, int N, int n_off, cudaStream_t st, int il_group = 0,
-                         int il_second = 0, int perm_dh = 0);
+// the codes of n elements of bf16 images (whole blocks): e4m3 (bits = 8) byte blocks [..][128][64] or int4 (4) nibble blocks
+// [..][128][32], byte j of a row = codes of k = 2j (low nibble) and 2j + 1 (high nibble)
+void launch_image_codes(const __nv_bfloat16* img, uint8_t* dst, size_t n, int bits, cudaStream_t st);
 void launch_permute_scales(const float* src, float* dst, int N, int n_off, int perm_dh, cudaStream_t st);
 // Y[r][n] = act( sum_d X[r][d] * W[(w_row_off + d)][n] + bias[n] + add[n] ), r < R
 void launch_rows_gemm(const float* X, int ldx, const void* W, int w_kind, int w_row_off, int N, int K, const float* bias,

@@ -128,11 +128,11 @@ void launch_pack_tiled(const void* src, int kind, __nv_bfloat16* dst, int K, int
   k_pack_tiled<<<blocks, 256, 0, st>>>(src, kind, dst, K, N, n_off, il_group, il_second, perm_dh, pair16);
 }
 
-// e4m3 codes [K][N] -> byte blocks of 128 out channels x 64 k (row order as in k_pack_tiled, no swizzle: the kernel
-// that decodes them writes the swizzled bf16 image itself).  One thread per 8 consecutive k of one out channel.
+// e4m3 codes [K][N] -> byte blocks of 128 out channels x 128 k, the operand image of the FP8 tensor path (row order as in
+// k_pack_tiled).  One thread per 8 consecutive k of one out channel.
 __global__ void k_pack_bytes(const uint8_t* src, uint8_t* dst, int K, int N, int n_off, int il_group, int il_second,
-                             int perm_dh, int wide, int pair16) {
-  const int KC = wide ? K >> 7 : K >> 6;
+                             int perm_dh, int pair16) {
+  const int KC = K >> 7;
   const size_t chunks = (size_t)N * (K >> 3);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < chunks; i += (size_t)gridDim.x * blockDim.x) {
     const int n = (int)(i % N), k0 = (int)(i / N) << 3;
@@ -142,23 +142,17 @@ __global__ void k_pack_bytes(const uint8_t* src, uint8_t* dst, int K, int N, int
     __align__(8) uint8_t v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = src[(size_t)(k0 + j) * N + n];
-    size_t off;
-    if (wide) {
-      // 128-byte rows: 16-byte chunk ((k0 % 128) / 16) XOR (row % 8), then the 8-byte half inside it
-      const int kc = k0 >> 7, w = k0 & 127, r = np & 127;
-      off = (((size_t)(np >> 7) * KC + kc) * 128 + r) * 128 + (size_t)(((w >> 4) ^ (r & 7)) << 4) + (size_t)(w & 8);
-    } else {
-      const int kc = k0 >> 6, c = (k0 & 63) >> 3;
-      off = (((size_t)(np >> 7) * KC + kc) * 128 + (np & 127)) * 64 + (size_t)c * 8;
-    }
+    // 128-byte rows: 16-byte chunk ((k0 % 128) / 16) XOR (row % 8), then the 8-byte half inside it
+    const int kc = k0 >> 7, w = k0 & 127, r = np & 127;
+    const size_t off = (((size_t)(np >> 7) * KC + kc) * 128 + r) * 128 + (size_t)(((w >> 4) ^ (r & 7)) << 4) + (size_t)(w & 8);
     *reinterpret_cast<uint2*>(dst + off) = *reinterpret_cast<const uint2*>(v);
   }
 }
 void launch_pack_bytes(const uint8_t* src, uint8_t* dst, int K, int N, int n_off, cudaStream_t st, int il_group,
-                       int il_second, int perm_dh, int wide, int pair16) {
+                       int il_second, int perm_dh, int pair16) {
   const size_t chunks = (size_t)N * (K >> 3);
   const int blocks = (int)((chunks + 255) / 256 < 16384 ? (chunks + 255) / 256 : 16384);
-  k_pack_bytes<<<blocks, 256, 0, st>>>(src, dst, K, N, n_off, il_group, il_second, perm_dh, wide, pair16);
+  k_pack_bytes<<<blocks, 256, 0, st>>>(src, dst, K, N, n_off, il_group, il_second, perm_dh, pair16);
 }
 
 // row-major bf16 [M][K] -> tiled bf16 [K/64][rows_pad][64] (16-byte chunks XOR-swizzled by row & 7)
@@ -239,33 +233,33 @@ void launch_quant_rows(const int* status, const __nv_bfloat16* x, uint8_t* out, 
   launch_pdl(k_quant_rows, dim3((M + 7) / 8), dim3(256), 0, st, status, x, out, scale, rows_pad, M, K);
 }
 
-// int4 codes: source [K][N/2] with two neighbouring out channels per byte; destination blocks of 128 out channels x
-// 64 k with two neighbouring k per byte (what a row of the MMA's K-major operand needs).  One thread per 8 k of one
-// out channel (4 destination bytes).
-__global__ void k_pack_nibbles(const uint8_t* src, uint8_t* dst, int K, int N, int n_off, int il_group, int il_second,
-                               int perm_dh) {
-  const int KC = K >> 6;
-  const size_t chunks = (size_t)N * (K >> 3);
+// bf16 image blocks of 128 rows x 64 k -> the codes they were made from, in the same row order without a swizzle (the kernel that
+// decodes them writes the swizzled image itself): e4m3 bytes, or 4-bit integers + 8, the lower k in the lower nibble.  The images
+// hold the codes' values exactly.  One thread per 8 consecutive k.
+__global__ void k_image_codes(const uint4* img, uint8_t* dst, size_t chunks, int bits) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < chunks; i += (size_t)gridDim.x * blockDim.x) {
-    const int n = (int)(i % N), k0 = (int)(i / N) << 3;
-    const int np = il_group ? (n / il_group) * (2 * il_group) + (n % il_group) + (il_second ? il_group : 0)
-                            : n_off + (perm_dh ? qkv_channel_to_packed(n, perm_dh) : n);
-    uint32_t w = 0;
+    const int row = (int)(i >> 3) & 127, c = (int)i & 7;
+    const uint4 v = img[(i & ~(size_t)7) + (size_t)(c ^ (row & 7))];
+    const uint32_t p[4] = {v.x, v.y, v.z, v.w};
+    uint32_t w[2] = {0, 0};
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const uint8_t b = src[(size_t)(k0 + j) * (N >> 1) + (n >> 1)];
-      const uint32_t c = (n & 1) ? (b >> 4) : (b & 15);
-      w |= c << (4 * j);
+    for (int j = 0; j < 4; ++j) {
+      const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&p[j]));
+      if (bits == 8) {
+        uint16_t e;
+        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(e) : "f"(x.y), "f"(x.x));
+        w[j >> 1] |= (uint32_t)e << (16 * (j & 1));
+      } else {
+        w[0] |= ((uint32_t)((int)x.x + 8) | (uint32_t)((int)x.y + 8) << 4) << (8 * j);
+      }
     }
-    const int kc = k0 >> 6;
-    *reinterpret_cast<uint32_t*>(dst + (((size_t)(np >> 7) * KC + kc) * 128 + (np & 127)) * 32 + ((k0 & 63) >> 1)) = w;
+    if (bits == 8) reinterpret_cast<uint2*>(dst)[i] = make_uint2(w[0], w[1]);
+    else reinterpret_cast<uint32_t*>(dst)[i] = w[0];
   }
 }
-void launch_pack_nibbles(const uint8_t* src, uint8_t* dst, int K, int N, int n_off, cudaStream_t st, int il_group,
-                         int il_second, int perm_dh) {
-  const size_t chunks = (size_t)N * (K >> 3);
-  const int blocks = (int)((chunks + 255) / 256 < 16384 ? (chunks + 255) / 256 : 16384);
-  k_pack_nibbles<<<blocks, 256, 0, st>>>(src, dst, K, N, n_off, il_group, il_second, perm_dh);
+void launch_image_codes(const __nv_bfloat16* img, uint8_t* dst, size_t n, int bits, cudaStream_t st) {
+  const size_t chunks = n >> 3;
+  k_image_codes<<<(int)((chunks + 255) / 256 < 16384 ? (chunks + 255) / 256 : 16384), 256, 0, st>>>(reinterpret_cast<const uint4*>(img), dst, chunks, bits);
 }
 
 // Row of an adaptive norm's shift through a packed weight matrix: out[n] = scale(n) * sum_k shift[k] * W[n][k].

@@ -64,7 +64,7 @@ extern "C" phyai_status_t phyai_w8a8_project(const void* x_bf16, const uint8_t* 
   cudaMemsetAsync(status, 0, 4, st);
   launch_rows_to_tiled(reinterpret_cast<const __nv_bfloat16*>(x_bf16), xt, (int)M, (int)K, rows_pad, st);
   launch_quant_rows(status, xt, xq, xs, rows_pad, (int)M, (int)K, st);
-  launch_pack_bytes(w_codes, wp, (int)K, (int)N, 0, st, 0, 0, 0, 1);
+  launch_pack_bytes(w_codes, wp, (int)K, (int)N, 0, st);
   TcGemm g{};
   g.W = reinterpret_cast<const __nv_bfloat16*>(wp), g.X = reinterpret_cast<const __nv_bfloat16*>(xq), g.M = (int)M, g.N = (int)N;
   g.K = (int)K, g.epi = TC_STORE, g.scale = w_scales, g.out_f32 = y, g.ldo = (int)N, g.splits = 1, g.rows_pad = rows_pad;
