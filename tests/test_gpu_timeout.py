@@ -13,7 +13,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("cluster_gemm", [1, 0])
-@pytest.mark.parametrize("batch", [1, 40, 80])   # 80 requests = 1120 tokens: the persistent 256-token-tile kernels
+# (beyond 64 tokens cluster_gemm = 1 is the CTA-pair kernels, 0 the general ones: 80 requests = 1120 tokens use the persistent
+# 256-token-tile kernels then)
+@pytest.mark.parametrize("batch", [1, 40, 80])
 def test_expired_wait_is_reported_and_the_handle_recovers(cluster_gemm, batch):
     cfg = small_bf16_config("pi0", max_batch=batch, max_prefix_len=150)
     W = synth.make_weights(cfg, 31, std=0.05)
@@ -44,7 +46,7 @@ def test_expired_wait_is_reported_and_the_handle_recovers(cluster_gemm, batch):
         again = ex.denoise_batched(*args).clone()
         torch.cuda.synchronize()
         assert ex.poll_status() == 0
-        # (beyond 64 tokens the split-K residual adds are atomic, so two runs agree to rounding, not to the bit)
+        # (the general kernels' split-K residual adds beyond 64 tokens are atomic: two runs agree to rounding, not to the bit)
         assert rel_err(again[0].double().cpu().numpy(), ref0) <= BAR["bf16"]
         assert rel_err(again.double().cpu().numpy(), good.double().cpu().numpy()) <= BAR["bf16"]
 
