@@ -29,7 +29,7 @@
 // end and only the global stores are skipped.
 #include "attention.cuh"
 #include "tc.cuh"
-#include "tmap.h"
+#include "tc_pair.cuh"
 
 namespace phyai {
 namespace {
@@ -68,24 +68,12 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
 __device__ __forceinline__ void remote_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void umma2_ss(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d), "l"(da), "l"(db), "r"(idesc), "r"(acc)
-      : "memory");
-}
 __device__ __forceinline__ void umma2_ts(uint32_t d, uint32_t ta, uint64_t db, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n.reg .pred p;\n"
       "setp.ne.b32 p, %4, 0;\n"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d), "r"(ta), "l"(db), "r"(idesc), "r"(acc)
       : "memory");
-}
-// arrives on the barrier at this offset in the CTAs of `mask` once every MMA issued so far has completed
-__device__ __forceinline__ void umma2_commit(uint32_t bar, uint16_t mask) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(mask)
-               : "memory");
 }
 // the two warps that share the rows of a tensor-memory lane quarter
 __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
@@ -133,13 +121,11 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 4) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(512) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    tmem_alloc2(smem_u32(&tmem_slot), 512);
     tc_fence_before();
   }
   __syncthreads();
-  cluster_arrive();                                 // every CTA's barriers exist before a peer can signal them
-  cluster_wait();
+  pair_sync();                                      // every CTA's barriers exist before a peer can signal them
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *reinterpret_cast<volatile uint32_t*>(&tmem_slot), 0);
   const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + 2 * KB;
@@ -160,7 +146,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   const int n_full = n_pre / KB, rem = n_pre - n_full * KB, n_mix = (rem + n_suf + KB - 1) / KB;
   const int T = n_mix + n_full, m0 = n_mix == 1 && n_full > 0 ? 1 : 0;      // mixed tiles: m0 .. m0 + n_mix - 1
   const int lead_rank = crank & ~1;
-  const uint16_t pair_mask = (uint16_t)(3u << lead_rank);
+  const uint32_t pair_mask = 3u << lead_rank;
 
   if (warp < 4) {
     // =========================== loaders: warps 0-1 K, 2-3 V =======================================================
@@ -185,7 +171,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         asm volatile(
             "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(
                 dst + (uint32_t)u * L::PIECE),
-            "l"(a.rq->kv_map), "r"(0), "r"(row), "r"(blk), "r"(plane), "r"(bar & 0xFEFFFFFFu)
+            "l"(a.rq->kv_map), "r"(0), "r"(row), "r"(blk), "r"(plane), "r"(bar & LEADER_MASK)
             : "memory");
       }
     };
@@ -265,7 +251,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         for (int kk = 0; kk < DH / 16; ++kk) {
           const uint64_t da = make_desc(Qs + (uint32_t)(kk >> 2) * (128 * 128) + (uint32_t)(kk & 3) * 32);
           const uint64_t db = make_desc(kb + (uint32_t)(kk >> 2) * L::KBLOCK + (uint32_t)(kk & 3) * 32);
-          if (elect_one()) umma2_ss(tmem_s + (uint32_t)(t & 1) * KB, da, db, IDESC_S, kk > 0 ? 1u : 0u);
+          if (elect_one()) umma2_bf16(tmem_s + (uint32_t)(t & 1) * KB, da, db, IDESC_S, kk > 0 ? 1u : 0u);
         }
         if (elect_one()) umma2_commit(smem_u32(&s_full[t & 1]), pair_mask);
         __syncwarp();
@@ -539,7 +525,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   cluster_wait();
   if (warp == 4) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+    tmem_dealloc2(tmem_base, 512);
     if (lane == 0 && trc) {
       unsigned long long t;
       unsigned sm;

@@ -1,4 +1,4 @@
-// CTA-pair forms of the tensor-core primitives (tcgen05 cta_group::2), shared by the pair GEMM kernels: CTAs 2 i and 2 i + 1
+// CTA-pair forms of the tensor-core primitives (tcgen05 cta_group::2), shared by the kernels on pairs: CTAs 2 i and 2 i + 1
 // of a cluster work on one accumulator tile, the even one (the leader) issues the MMAs, the copies of both signal its barrier.
 #pragma once
 
