@@ -244,14 +244,17 @@ phyai_status_t phyai_poll_status(phyai_expert_t *h);
  * key "b1_attn_hpc": query heads per CTA (1 or 2; 0 = choose) of the cluster attention kernel.  key "use_b1_step":
  * 1 (default) runs the step boundary of those calls (velocity head, Euler update, next embedding) as one cluster kernel.
  * key "use_persistent_gu" / "use_persistent_qkv": 1 (default) runs the gate/up and the q|k|v projection of calls
- * with more than 1024 suffix tokens on the persistent tile kernel (one CTA per SM, two accumulators, a tile's
- * epilogue under the next tile's main loop); 0 keeps them on the one-tile-per-CTA kernel.
+ * with more than 1024 suffix tokens that are not on CTA pairs (see use_pair_gemm; e4m3 activations, widths that are no
+ * multiple of 256) on the persistent tile kernel (one CTA per SM, two accumulators, a tile's epilogue under the next
+ * tile's main loop); 0 keeps them on the one-tile-per-CTA kernel.
  * key "use_attn_splits": 1 (default) lets calls of few requests (at most a quarter of the SMs' worth of head-pair
- * CTAs) split every request's key tiles over up to 8 CTAs of the tcgen05 attention kernel, merged by a second launch.
+ * CTAs) that are not on the pair attention kernel split every request's key tiles over up to 8 CTAs of the tcgen05 attention kernel, merged by a second launch.
  * key "use_pair_gemm": 1 (default) runs the projections of calls with more than 64 suffix tokens on the CTA-pair GEMM
  * with the norms folded in (together with use_cluster_gemm and the two use_persistent options); 0 keeps the general kernels.
  * key "use_pair_attention": 1 (default) lets those calls of few requests use the CTA-pair attention kernel (caches of at
- * least 256 tokens); key "pair_attn_ranges": key ranges per request (1..4, 0 = choose) of that kernel.
+ * least 256 tokens); key "pair_attn_ranges": key ranges per request (1..4, 0 = choose) of that kernel (with heads of
+ * 256 channels at most 3 from 61 suffix rows on, 2 with 64: the partial results have to fit the shared memory).
+ * Options that leave the CTA pairs or decode weight codes make the weight images they need when they are set.
  * key "trace": see phyai_read_trace.
  * key "wait_limit": iteration bound of the device-side waits on other agents' progress (testing).
  * Unknown key -> INVALID_ARG. */

@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(1024) k_kv_scan(const int* lens, int batch, in
 // rows cu[b] + p.  The rows of a request are one contiguous run on both sides: a block moves 16 KB of it (grid.x) of one
 // plane (grid.y) and request (grid.z), its loads issued before the dependency wait (only the destination needs cu).  With
 // `zero_tail` the entry grid.z = batch clears the rows past the last request (after an error: all rows).  Bound by HBM: 258 MB
-// of 8 requests of the pi0 shape 48 us, 5.4 TB/s (a grid-stride loop over padded rows with two divisions per 16 bytes,
+// of 8 requests of the pi0 shape 48 us with the scan, 5.4 TB/s (a grid-stride loop over padded rows with two divisions per 16 bytes,
 // behind a fill of the whole output by the caller: 139 us).
 constexpr int PACK_T = 256, PACK_U = 4, PACK_CHUNK = PACK_T * PACK_U;
 __global__ void __launch_bounds__(PACK_T) k_kv_pack(const uint4* k, const uint4* v, const int* lens, const int* cu, const int* status, uint4* dst,

@@ -317,7 +317,8 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
   a.rope = reinterpret_cast<const float2*>(rope), a.layer = (int)desc->layer, a.out = reinterpret_cast<__nv_bfloat16*>(out);
   a.d = d, a.wait_limit = 1u << 22;
   // The library's choice where shapes and alignment allow it: bf16 operands first (one small kernel), then the tcgen05 kernels
-  // of the denoising loop.  One request of the pi0 shape: 37.6 -> 23 us per call; 16 requests: 70 -> 35 us.
+  // of the denoising loop.  Per call of the pi0 shape, against the mma.sync kernel with its best split: one request 18 - 19 us
+  // against 25, 4 requests 23 / 41, 16 requests 29 / 70.
   const size_t q_elems = (size_t)batch * (d.Hq / 2) * 128 * d.dh, kv_elems = (size_t)batch * d.Hkv * d.S * d.dh;
   const size_t tc_need = sizeof(Request) + (q_elems + 2 * kv_elems) * 2;
   // (a given scratch that cannot hold the operands leaves the call to the mma.sync kernel, which reads the fp32 rows itself)

@@ -603,7 +603,9 @@ int attention_pair_max_ranges(const Dims& d) {
 
 // Key ranges per request: 1 to 4, the least of waves x (fixed cost + tiles of a range), in tiles of 128 keys.  How many
 // clusters of 2 C CTAs the device holds at a time decides the waves (a cluster of 8 needs 8 free SMs in one GPC: 15 on a
-// B200, not 18).
+// B200, not 18).  Against every other choice, ten-step loops of 4 / 8 / 12 / 16 requests: chosen 8.95 / 9.94 / 11.21 / 11.49 ms
+// with 300-token prefixes (best 8.95 / 9.92 / 10.98 / 11.49), 9.18 / 10.17 / 11.56 / 12.15 with 500 (best 9.17 / 10.17 / 11.56 /
+// 12.07).
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
   static PerDeviceCount resident[2][5];
   const int dh = d.dh == 256 ? 1 : 0, items = batch * (d.Hq / 4);

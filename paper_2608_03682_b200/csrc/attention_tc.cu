@@ -1,4 +1,5 @@
-// Suffix -> (prefix U suffix) attention on the tcgen05 tensor cores, for calls with two or more requests.
+// Suffix -> (prefix U suffix) attention on the tcgen05 tensor cores, for calls with about 18 requests or more (fewer: the
+// kernels on CTA pairs and clusters, where their shapes allow).
 //
 // One CTA takes the suffix rows of two query heads that share a kv head (2 x 64 padded rows = the 128
 // rows of one MMA) and walks all key tiles of its request:
@@ -479,9 +480,10 @@ int attention_tc_splits(const Dims& d, int batch, int n_sm, int max_prefix) {
   const int tiles = (max_prefix + KTC - 1) / KTC + 1;
   if (want > tiles) want = tiles;
   if (want > 8) want = 8;
-  // (measured on the pi0-shaped expert, 816-token prefixes: 4 requests 12.2 -> 11.3 ms per call with 8 ranges,
-  // 8 requests 12.9 -> 12.6 ms with 4, 16 requests 16.8 -> 17.6 ms with 2: the merge kernel and the fp32 partials cost
-  // more than two ranges save)
+  // (Serves caches of fewer than 256 tokens, query-head groups that are no multiple of 4, W8A8 and the switched-off pair
+  // kernels.  Measured on the pi0-shaped expert with 816-token prefixes, before the pair kernels took those calls: 4 requests
+  // 12.2 -> 11.3 ms per call with 8 ranges, 8 requests 12.9 -> 12.6 ms with 4, 16 requests 16.8 -> 17.6 ms with 2: the merge
+  // kernel and the fp32 partials cost more than two ranges save.)
   return want < 4 ? 1 : want;
 }
 

@@ -19,8 +19,9 @@
 // per-channel constant shift . W; the residual epilogue writes h, the next projection's operand and its partial sums of
 // squares (one per 64 channels and token).  No split-K and no atomics: a request gives the same bits every time.
 //
-// Measured in the captured ten-step loops, against the one-CTA tile GEMMs and their norm launches: 4 requests 11.0 -> 9.1 ms
-// (with the attention's gains), 8: 12.8 -> 10.4, 64: 32.7 -> 29.4 (power-capped), 256: 117.6 -> 106.
+// Measured in the captured ten-step loops of the pi0 shape, against the one-CTA tile GEMMs and their norm launches (with the
+// pair attention's part): 4 requests of 816 tokens 11.3 -> 9.4 ms, 8: 12.9 -> 10.8, 64 ragged: 33.1 -> 29.9 (power-capped, SM
+// clock 1.73 GHz), 256: 119.6 -> 107.7 (1.55 GHz).
 //
 // Roles: warps 0-3 issue the copies (k-step i by warp i % 4), warp 4 issues the MMAs (leader CTA), the 16 warps from 5
 // on are the epilogue (tensor-memory lane quarter = warp % 4).  Every wait is

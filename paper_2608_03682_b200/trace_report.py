@@ -2,8 +2,8 @@
 
     python -m paper_2608_03682_b200.trace_report [--batch 64] [--dtype bf16] [--first 100] [--last 107] [--option k=v ...]
 
-For every launch index in [first, last) of the call (one layer of the batch-64 loop is seven launches: down of the
-layer before, norm, q|k|v, attention, O, norm, gate/up) the option ``trace_all_from`` makes that launch, if it is a
+For every launch index in [first, last) of the call (one layer is five launches on CTA pairs: q|k|v, attention, O, gate/up,
+down; seven on the general kernels, with a norm before q|k|v and gate/up) the option ``trace_all_from`` makes that launch, if it is a
 tile GEMM or the tcgen05 attention kernel, stamp one slot per CTA (phyai_set_option "trace" / "trace_all_from", phyai_read_trace).  Printed per launch:
 how long the CTAs spend in each phase, when the CTAs of each wave start and end, and the gap between two CTAs on the
 same SM.  Stamps (ns, %globaltimer): 0 start, 1 barriers and tensor memory set up, 2 dependency resolved, 3 first
