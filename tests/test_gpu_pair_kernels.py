@@ -66,6 +66,15 @@ def test_pair_attention_key_ranges(head_dim, n_q, n_kv, ranges):
     check(cfg, [700, 0, 1, 127, 128, 129, 512, 64, 386], 1, range(9), pair_attn_ranges=ranges)
 
 
+@pytest.mark.parametrize("horizon", [59, 60, 62, 63])
+@pytest.mark.parametrize("ranges", [2, 3, 4])
+def test_pair_attention_at_the_most_suffix_rows(ranges, horizon):
+    """The fp32 partials of heads of 256 channels fit the shared memory for four ranges up to 60 rows, three up to 63 (one state
+    token and the horizon): more ranges than that are reduced, and the fullest layouts are right to the last row."""
+    cfg = small_bf16_config("pi0", head_dim=256, n_q_heads=4, max_batch=5, max_prefix_len=400, n_layers=2, horizon=horizon)
+    check(cfg, [400, 0, 129, 256, 33], 1, range(5), pair_attn_ranges=ranges)
+
+
 @pytest.mark.parametrize("head_dim,n_q,n_kv,lens", [(256, 4, 1, [960, 0, 1, 7, 8, 511, 959]), (128, 8, 2, [700, 129, 64]), (128, 4, 1, [256] * 7)])
 def test_attention_of_a_few_requests(head_dim, n_q, n_kv, lens):
     """The library's own choice of key ranges for few requests (63 and 64 suffix rows: with 256 channels not four of them), empty and
@@ -75,10 +84,11 @@ def test_attention_of_a_few_requests(head_dim, n_q, n_kv, lens):
     check(cfg, lens, 1, range(len(lens)))
 
 
-@pytest.mark.parametrize("n_kv,head_dim,suffix,lens", [(1, 256, 51, [700, 0, 129]), (1, 256, 64, [(53 * b) % 300 for b in range(40)]),
+@pytest.mark.parametrize("n_kv,head_dim,suffix,lens", [(1, 256, 51, [700, 0, 129]), (1, 256, 64, [1100]), (1, 256, 1, [0]), (1, 256, 64, [(53 * b) % 300 for b in range(40)]),
                                                       (2, 128, 17, [128] * 45)])
 def test_attention_operator_on_the_pair_kernel(n_kv, head_dim, suffix, lens):
-    """The library's own choice of kernel: split key ranges, one range per request (row-major output), 128-channel heads."""
+    """The library's own choice of kernel: one request (cluster kernel; two key tiles per range, no prefix), split key ranges, one range
+    per request (row-major output), 128-channel heads."""
     from tests.test_gpu_attention_op import make_case, oracle_attention
     qkv, kv, cu, rope = make_case(9, 8, n_kv, head_dim, suffix, lens)
     desc = binding.attention_desc(8, n_kv, head_dim, suffix, n_layers=2, layer=1)
