@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
     // =========================== MMA issuer ======================================================================
     pdl_wait();
     // (this warp never touches the receive area: its part in the cluster barrier that guards it, see the row warps)
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive_relaxed();
     if (lane == 0) suppress = status_set(a.status) ? 1 : 0;
     for (int t = 0; t < T; ++t) {
       const bool trm = lane == 0 && tcta && t == 0;
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
       group_sync<BAR_ROWS, 256>();
       tc_fence_after();
       // (the last logits exist: the Q tile is dead and the receive area free -- see the cluster barrier ahead of the push)
-      if (t == T - 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      if (t == T - 1) cluster_arrive_relaxed();
       if (tr2) trace_stamp(trp, 11);
       // the visible key columns of this row form a prefix of the tile: the keys that exist, and for the state-token row
       // under the block-causal mask only the prefix keys and its own key (suffix key 0, in the first CTA's range)
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
     }
     if (T == 0) {
       if (g == 1) cp_async_wait<0>();
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      cluster_arrive_relaxed();
     }
     // ---- partial out: half an O row into the owner's block of the staging area; group 0 adds (max, sum) --------------
     if (T > 0 && warp == 5) mbar_wait_drain(smem_u32(&pv_done), (uint32_t)(T - 1) & 1u, wc);
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
   // From here on this CTA no longer needs its peers (what they sent has landed); it may leave once every peer says the
   // same, i.e. once every copy out of its own staging area has completed.  Arriving now and waiting at the very end
   // hides the skew between the CTAs behind the merge.
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  cluster_arrive_relaxed();
   if (tracer) trace_stamp(trp, 4);
 
   // ---- merge my rows: the 8 partials in rank order, normalise, store as the output projection's activation tile ----

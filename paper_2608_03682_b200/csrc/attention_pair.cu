@@ -60,25 +60,8 @@ struct ApLayout {
   static_assert(SMEM + 3072 <= 227 * 1024, "partials exceed the shared memory");
 };
 
-__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void remote_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void umma2_ts(uint32_t d, uint32_t ta, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d), "r"(ta), "l"(db), "r"(idesc), "r"(acc)
-      : "memory");
-}
 // the two warps that share the rows of a tensor-memory lane quarter
 __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 template <int DH, int C>
 __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
@@ -234,7 +217,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       }
       __syncwarp();
     }
-    if (C > 1) cluster_arrive();
+    if (C > 1) cluster_arrive_relaxed();
   } else if (warp == 4) {
     // =========================== MMA issuer (leader CTA): S(0), S(1), then P(t) V(t), S(t + 2) ======================
     pdl_wait();
@@ -293,7 +276,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       }
     }
     __syncwarp();
-    if (C > 1) cluster_arrive();
+    if (C > 1) cluster_arrive_relaxed();
   } else {
     // =========================== softmax / correction / output =====================================================
     const int g = (warp - 5) >> 2;            // which half of a row's columns
@@ -324,7 +307,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         __syncwarp();
       }
       tc_fence_after();
-      if (C > 1 && t >= 0 && t == T - 1) cluster_arrive();     // (the last logits exist: Q is dead, its area may receive partials)
+      if (C > 1 && t >= 0 && t == T - 1) cluster_arrive_relaxed();     // (the last logits exist: Q is dead, its area may receive partials)
       // the visible keys of a row form a prefix of a mixed tile: the keys that exist, and for the state-token row under the
       // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
       int nvis = t >= m0 && t < m0 + n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - (t - m0) * KB) : KB;
@@ -381,7 +364,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);      // (of this thread's half of the columns)
       m = m_new;
     }
-    if (C > 1 && T == 0) cluster_arrive();
+    if (C > 1 && T == 0) cluster_arrive_relaxed();
     xch[T & 1][g][row] = l;
     quarter_sync(q);
     l = xch[T & 1][0][row] + xch[T & 1][1][row];
@@ -470,7 +453,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   __syncthreads();
   // From here on this CTA no longer needs its peers; it may leave once every peer says the same (the leader's MMAs have
   // read both CTAs' shared memory, every partial copied out of its staging area has landed).
-  cluster_arrive();
+  cluster_arrive_relaxed();
   if constexpr (C > 1) {
     // ---- merge my rows: the C partials in range order, normalise, store as the output projection's operand ------------
     // A warp per row (rr = hl * n_me + il, every 13th), lane l the four columns of every piece that its l-th 16 bytes hold;

@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(NT, 1) k_gemm_b1(int* status, const B1Gemm g) 
   // From here on this CTA no longer needs its peers: what they sent has landed.  It may leave once every peer says the
   // same (then every copy out of its own staging area has completed): arrive now, wait at the very end, so that the
   // skew between the CTAs hides behind the epilogue.
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  cluster_arrive_relaxed();
   trace_stamp(tr, 4);
   const bool store = !suppress && acc_ok && recv_ok && !*reinterpret_cast<volatile int*>(&abort_flag);
 

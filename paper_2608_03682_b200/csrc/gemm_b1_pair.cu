@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(BP_THREADS, 1)
         tma2d(tiles + (uint32_t)s * chunk + BP_A, &tmx, (kc_begin + s) * 64 + r * HN, smem_u32(&bar_full[s / BP_GROUP]) & LEADER_MASK);
     }
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive_relaxed();
   } else if (warp == 17) {
     // ---------------- MMAs: whole warp in the loop, one elected lane issues -----------------------------------------
     if (r == 0) {
@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(BP_THREADS, 1)
       if (elect_one()) umma2_commit(smem_u32(&bar_accum), 3u << (rank & ~1));
       __syncwarp();
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive_relaxed();
   } else {
     // ---------------- epilogue warps ---------------------------------------------------------------------------------
     // an item: four channels (QKV, gate / up: and their partners) of one token; item i belongs to thread i
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(BP_THREADS, 1)
       }
     }
     // what the peers sent has landed; this CTA leaves once they say the same
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive_relaxed();
     trace_stamp(tr, 4);
     const bool store = mine && !suppress && ok_r > 0 && !*reinterpret_cast<volatile int*>(&abort_flag);
     if constexpr (EPI == B1_RESID) {

@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       // this warp has read its part of the accumulator: the MMAs of the tile after next may overwrite it
       tc_fence_before();
       if (lane == 0)
-        asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(tempty0 + (uint32_t)buf * 8u) : "memory");
+        remote_arrive(tempty0 + (uint32_t)buf * 8u);
       if constexpr (EPI == PG_RESID) {
         if (g.ss_out) {
           asm volatile("bar.sync %0, %1;" ::"n"(BAR_EPI + 1), "n"(PG_EPI) : "memory");
@@ -488,7 +488,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
   __syncthreads();
   // Neither CTA leaves (or gives its tensor memory back) while the other still works: the leader's MMAs read both CTAs'
   // shared memory and write both tensor memories.
-  pair_sync();
+  cluster_arrive_relaxed();
+  cluster_wait();
   if (warp == PG_PROD) {
     tc_fence_after();
     tmem_dealloc2(tmem_base, 512);

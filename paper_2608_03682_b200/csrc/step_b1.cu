@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(SB_THREADS, 1) k_step_b1(int* status, const St
     }
     __syncthreads();
     // what the peers sent has landed; they may leave once every CTA says the same (wait at the very end)
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    cluster_arrive_relaxed();
     trace_stamp(tr, 5);
     // ---- my rows: the partials added in CTA order; Euler update --------------------------------------------------------
     if (my_r >= 0 && lane < A) {
