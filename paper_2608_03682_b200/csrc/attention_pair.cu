@@ -12,7 +12,7 @@
 //   softmax     two threads per row (half of the columns each), straight from tensor memory; P (bf16) over the S buffer
 //   O += P V    M = 256, N = head_dim, K = 128 keys; P is the tensor-memory A operand, V an MN-major B operand; rescaled
 //               only when a row's maximum grows by more than 2^8
-// Small calls split the keys of a request over C = 2 to 4 pairs of one cluster (each range: its share of the prefix and of
+// The keys of a request are split over C = 2 to 4 pairs of one cluster (without a split: attention_persist.cu; each range: its share of the prefix and of
 // the suffix keys); the fp32 partial results are merged over distributed shared memory: row range p of every head belongs to
 // pair p, which is sent its rows of the other C - 1 partials and adds the C in range order.  No partials in global memory, no
 // merge launch.  (Owners that read the partials from the other CTAs instead of being sent them: 4.2 us per launch more.)
@@ -55,8 +55,8 @@ struct ApLayout {
   static constexpr int NP = DH / 128;                        // a block in pieces of 2 x 64 columns, sent as they are staged
   static constexpr int PITCH = 512 + 16;                     // fp32 row of a piece, padded against bank conflicts
   static constexpr int ROW = NP * PITCH + 16;
-  static constexpr int STG = 2 * C * OWN * ROW, RECV = (STG > KV ? STG : KV), PEERS = C > 1 ? 2 * (C - 1) * OWN * ROW : 0;
-  static constexpr size_t SMEM = 1024 + (size_t)(C > 1 && RECV + PEERS > KV + QTILE ? RECV + PEERS : KV + QTILE);
+  static constexpr int STG = 2 * C * OWN * ROW, RECV = (STG > KV ? STG : KV), PEERS = 2 * (C - 1) * OWN * ROW;
+  static constexpr size_t SMEM = 1024 + (size_t)(RECV + PEERS > KV + QTILE ? RECV + PEERS : KV + QTILE);
   static_assert(SMEM + 3072 <= 227 * 1024, "partials exceed the shared memory");
 };
 
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       mbar_init(smem_u32(&s_full[i]), 1), mbar_init(smem_u32(&pv_done[i]), 1);
     }
     mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 8), mbar_init(smem_u32(&q_ready), 1);
-    if (C > 1 && n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * L::ROW));
+    if (n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * L::ROW));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 4) {
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       }
       __syncwarp();
     }
-    if (C > 1) cluster_arrive_relaxed();
+    cluster_arrive_relaxed();
   } else if (warp == 4) {
     // =========================== MMA issuer (leader CTA): S(0), S(1), then P(t) V(t), S(t + 2) ======================
     pdl_wait();
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       }
     }
     __syncwarp();
-    if (C > 1) cluster_arrive_relaxed();
+    cluster_arrive_relaxed();
   } else {
     // =========================== softmax / correction / output =====================================================
     const int g = (warp - 5) >> 2;            // which half of a row's columns
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         __syncwarp();
       }
       tc_fence_after();
-      if (C > 1 && t >= 0 && t == T - 1) cluster_arrive_relaxed();     // (the last logits exist: Q is dead, its area may receive partials)
+      if (t >= 0 && t == T - 1) cluster_arrive_relaxed();     // (the last logits exist: Q is dead, its area may receive partials)
       // the visible keys of a row form a prefix of a mixed tile: the keys that exist, and for the state-token row under the
       // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
       int nvis = t >= m0 && t < m0 + n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - (t - m0) * KB) : KB;
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);      // (of this thread's half of the columns)
       m = m_new;
     }
-    if (C > 1 && T == 0) cluster_arrive_relaxed();
+    if (T == 0) cluster_arrive_relaxed();
     xch[T & 1][g][row] = l;
     quarter_sync(q);
     l = xch[T & 1][0][row] + xch[T & 1][1][row];
@@ -372,89 +372,59 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     group_sync<BAR_ROWS, 256>();
     tc_fence_after();
     if (warp == 5 && lane == 0) trace_stamp(trc, 6);
-    if constexpr (C == 1) {
-      // O / l -> bf16, the O projection's tiled operand: a thread's 128 bytes of a 64-channel chunk go to a staging block of
-      // the warp (the K / V buffers are dead) at the position they have in global memory, then out with coalesced stores
-      const bool okf = !skip && !*reinterpret_cast<volatile int*>(&abort_flag);
-      const float inv = 1.0f / l;
-      const int i0 = (q * 32) & 63, orow = b * S + i0 + lane;
-      const int nrow = okf ? max(0, min(32, S - i0)) : 0;
-      const uint32_t ostage = stg + (uint32_t)(warp - 5) * 4096u;
+    // ---- partial out: half an O row into the owner's block of the staging area; half 0 adds (max, sum) ----------------
+    const int c = i / own, il = i - c * own, n_c = max(0, min(own, S - c * own));
+    const bool wr = i < S;
+    const uint32_t blk = stg + (uint32_t)c * slot;
+    constexpr int PARTS = 8 / (C - 1);       // warps per peer: the bulk copies of one warp complete one after the other
+    const int w8 = warp - 5, pi = w8 % (C - 1), peer = pi < pr ? pi : pi + 1, part = w8 / (C - 1);
+    const int n_p = max(0, min(own, S - peer * own));
 #pragma unroll 1
-      for (int c = g * (DH / 2); c < (g + 1) * (DH / 2); c += 64) {
-        float o[64];
-        tmem_ld64(tmem_o + lane_addr + (uint32_t)c, o);
+    for (int k = 0; k < L::NP; ++k) {
+      float o[64];
+      if (T > 0) {
+        tmem_ld64(tmem_o + lane_addr + (uint32_t)(g * (DH / 2) + k * 64), o);
+      } else {
 #pragma unroll
-        for (int e = 0; e < 64; e += 8)
-          asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ostage + (uint32_t)lane * 128u + (uint32_t)(((e >> 3) ^ (orow & 7)) << 4)),
-                       "r"(pack_bf16(o[e] * inv, o[e + 1] * inv)), "r"(pack_bf16(o[e + 2] * inv, o[e + 3] * inv)),
-                       "r"(pack_bf16(o[e + 4] * inv, o[e + 5] * inv)), "r"(pack_bf16(o[e + 6] * inv, o[e + 7] * inv))
+        for (int e = 0; e < 64; ++e) o[e] = 0.f;
+      }
+      const uint32_t rowp = blk + (uint32_t)((k * 2 * n_c + hl * n_c + il) * L::PITCH + g * 256);
+      if (wr) {
+#pragma unroll
+        for (int e = 0; e < 64; e += 4)
+          asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)e * 4), "f"(o[e]), "f"(o[e + 1]), "f"(o[e + 2]), "f"(o[e + 3])
                        : "memory");
-        __syncwarp();
-        for (int idx = lane; idx < nrow * 8; idx += 32) {
-          const int rr = b * S + i0 + (idx >> 3);
-          uint4 v;
-          asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(ostage + (uint32_t)idx * 16u) : "memory");
-          // (tiled: the chunk's place as staged; row-major, for the operator: the swizzle undone)
-          *reinterpret_cast<uint4*>(a.out + out_index(rr, (head0 + hl) * DH + c + (((idx & 7) ^ (rr & 7)) << 3), a.rows_pad, d.Nq)) = v;
-        }
-        __syncwarp();
+        if (k == 0 && g == 0)
+          asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(blk + (uint32_t)(L::NP * 2 * n_c * L::PITCH + (hl * n_c + il) * 16)), "f"(m), "f"(l)
+                       : "memory");
       }
-    } else {
-      // ---- partial out: half an O row into the owner's block of the staging area; half 0 adds (max, sum) ----------------
-      const int c = i / own, il = i - c * own, n_c = max(0, min(own, S - c * own));
-      const bool wr = i < S;
-      const uint32_t blk = stg + (uint32_t)c * slot;
-      constexpr int PARTS = 8 / (C - 1);       // warps per peer: the bulk copies of one warp complete one after the other
-      const int w8 = warp - 5, pi = w8 % (C - 1), peer = pi < pr ? pi : pi + 1, part = w8 / (C - 1);
-      const int n_p = max(0, min(own, S - peer * own));
-#pragma unroll 1
-      for (int k = 0; k < L::NP; ++k) {
-        float o[64];
-        if (T > 0) {
-          tmem_ld64(tmem_o + lane_addr + (uint32_t)(g * (DH / 2) + k * 64), o);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 64; ++e) o[e] = 0.f;
-        }
-        const uint32_t rowp = blk + (uint32_t)((k * 2 * n_c + hl * n_c + il) * L::PITCH + g * 256);
-        if (wr) {
-#pragma unroll
-          for (int e = 0; e < 64; e += 4)
-            asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(rowp + (uint32_t)e * 4), "f"(o[e]), "f"(o[e + 1]), "f"(o[e + 2]), "f"(o[e + 3])
-                         : "memory");
-          if (k == 0 && g == 0)
-            asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(blk + (uint32_t)(L::NP * 2 * n_c * L::PITCH + (hl * n_c + il) * 16)), "f"(m), "f"(l)
-                         : "memory");
-        }
-        fence_async_smem();                    // generic writes -> visible to the bulk-copy engine
-        group_sync<BAR_ROWS, 256>();
-        if (k == 0) cluster_wait();            // every CTA's Q is dead
-        if (lane == 0 && part < PARTS && n_p > 0) {
-          const uint32_t bytes = (uint32_t)(2 * n_p * (L::PITCH + (k == L::NP - 1 ? 16 : 0))), chunk = (bytes / PARTS + 15) & ~15u;
-          const uint32_t lo = (uint32_t)part * chunk, off = (uint32_t)(k * 2 * n_p * L::PITCH) + lo;
-          if (lo < bytes)
-            asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                             map_rank(recv + (uint32_t)(pr < peer ? pr : pr - 1) * slot + off, peer * 2 + half)),
-                         "r"(stg + (uint32_t)peer * slot + off), "r"(min(chunk, bytes - lo)), "r"(map_rank(smem_u32(&mrg_bar), peer * 2 + half))
-                         : "memory");
-        }
-        __syncwarp();
+      fence_async_smem();                    // generic writes -> visible to the bulk-copy engine
+      group_sync<BAR_ROWS, 256>();
+      if (k == 0) cluster_wait();            // every CTA's Q is dead
+      if (lane == 0 && part < PARTS && n_p > 0) {
+        const uint32_t bytes = (uint32_t)(2 * n_p * (L::PITCH + (k == L::NP - 1 ? 16 : 0))), chunk = (bytes / PARTS + 15) & ~15u;
+        const uint32_t lo = (uint32_t)part * chunk, off = (uint32_t)(k * 2 * n_p * L::PITCH) + lo;
+        if (lo < bytes)
+          asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                           map_rank(recv + (uint32_t)(pr < peer ? pr : pr - 1) * slot + off, peer * 2 + half)),
+                       "r"(stg + (uint32_t)peer * slot + off), "r"(min(chunk, bytes - lo)), "r"(map_rank(smem_u32(&mrg_bar), peer * 2 + half))
+                       : "memory");
       }
-      if (warp == 5) {
-        bool ok = true;
-        if (n_me > 0) ok = mbar_wait_drain(smem_u32(&mrg_bar), 0u, wc) > 0;
-        if (lane == 0) mrg_ok = ok && !skip ? 1 : 0;
-      }
+      __syncwarp();
+    }
+    if (warp == 5) {
+      bool ok = true;
+      if (n_me > 0) ok = mbar_wait_drain(smem_u32(&mrg_bar), 0u, wc) > 0;
+      if (lane == 0) mrg_ok = ok && !skip ? 1 : 0;
     }
     tc_fence_before();
   }
-  if (C > 1 && warp < 5) cluster_wait();
+  if (warp < 5) cluster_wait();
   __syncthreads();
   // From here on this CTA no longer needs its peers; it may leave once every peer says the same (the leader's MMAs have
   // read both CTAs' shared memory, every partial copied out of its staging area has landed).
   cluster_arrive_relaxed();
-  if constexpr (C > 1) {
+  {
     // ---- merge my rows: the C partials in range order, normalise, store as the output projection's operand ------------
     // A warp per row (rr = hl * n_me + il, every 13th), lane l the four columns of every piece that its l-th 16 bytes hold;
     // before that the weights of the warp's rows, a row per lane.
@@ -541,8 +511,8 @@ int max_clusters_one() {
   return cudaOccupancyMaxActiveClusters(&n, k_attn_pair<DH, C>, &cfg) == cudaSuccess ? n : 0;
 }
 int max_clusters(int dh, int c) {
-  if (dh == 256) return c == 1 ? max_clusters_one<256, 1>() : c == 2 ? max_clusters_one<256, 2>() : c == 3 ? max_clusters_one<256, 3>() : max_clusters_one<256, 4>();
-  return c == 1 ? max_clusters_one<128, 1>() : c == 2 ? max_clusters_one<128, 2>() : c == 3 ? max_clusters_one<128, 3>() : max_clusters_one<128, 4>();
+  if (dh == 256) return c == 2 ? max_clusters_one<256, 2>() : c == 3 ? max_clusters_one<256, 3>() : max_clusters_one<256, 4>();
+  return c == 2 ? max_clusters_one<128, 2>() : c == 3 ? max_clusters_one<128, 3>() : max_clusters_one<128, 4>();
 }
 
 template <int DH, int C>
@@ -586,16 +556,16 @@ int attention_pair_max_ranges(const Dims& d) {
 
 // Key ranges per request: 1 to 4, the least of waves x (fixed cost + tiles of a range), in tiles of 128 keys.  How many
 // clusters of 2 C CTAs the device holds at a time decides the waves (a cluster of 8 needs 8 free SMs in one GPC: 15 on a
-// B200, not 18).  Against every other choice, ten-step loops of 4 / 8 / 12 / 16 requests: chosen 8.95 / 9.94 / 11.21 / 11.49 ms
-// with 300-token prefixes (best 8.95 / 9.92 / 10.98 / 11.49), 9.18 / 10.17 / 11.56 / 12.15 with 500 (best 9.17 / 10.17 / 11.56 /
-// 12.07).
+// B200, not 18).  One range: the persistent kernel.  Against every other choice, ten-step loops of 4 / 8 / 12 / 16 / 20 requests:
+// chosen 8.79 / 10.02 / 11.04 / 11.67 / 12.44 ms with 816-token prefixes (best 8.78 / 9.98 / 11.04 / 11.63 / 12.44), 8.50 / 9.30 /
+// 10.29 / 10.94 / 11.69 with 400 (best 8.43 / 9.30 / 10.28 / 10.91 / 11.69).
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
   static PerDeviceCount resident[2][5];
   const int dh = d.dh == 256 ? 1 : 0, items = batch * (d.Hq / 4);
   int best_c = 1;
   double best = 1e30;
   for (int c = 1; c <= 4; ++c) {
-    const int n = resident[dh][c].get([&] { return max_clusters(d.dh, c); });
+    const int n = c == 1 ? attention_persist_pairs(d) : resident[dh][c].get([&] { return max_clusters(d.dh, c); });
     if (n <= 0 || c > attention_pair_max_ranges(d)) continue;
     const double cost = (double)((items + n - 1) / n) * ((c > 1 ? 5.5 : 4.0) + (max_prefix + d.S + c * KB - 1) / (c * KB));
     if (cost < best) best = cost, best_c = c;
@@ -607,15 +577,14 @@ cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfl
                                   const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
                                   int ranges, const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, bool pdl) {
   if (ranges > attention_pair_max_ranges(d)) return cudaErrorInvalidValue;
+  if (ranges == 1) return launch_attention_persist(rq, status, q_tiles, kr, vr, layer, out_tiled, rows_pad, d, batch, order, wait_limit, st, trace, pdl);
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
   a.num_splits = ranges, a.d = d, a.wait_limit = wait_limit, a.order = order, a.trace = trace;
   switch (ranges + (d.dh == 256 ? 4 : 0)) {
-    case 1: return launch_one<128, 1>(a, batch, st, pdl);
     case 2: return launch_one<128, 2>(a, batch, st, pdl);
     case 3: return launch_one<128, 3>(a, batch, st, pdl);
     case 4: return launch_one<128, 4>(a, batch, st, pdl);
-    case 5: return launch_one<256, 1>(a, batch, st, pdl);
     case 6: return launch_one<256, 2>(a, batch, st, pdl);
     case 7: return launch_one<256, 3>(a, batch, st, pdl);
     default: return launch_one<256, 4>(a, batch, st, pdl);

@@ -534,13 +534,16 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     ++cnt;
     return PHYAI_OK;
   };
-  // Attention of the pair path.  Caches of fewer than 256 tokens keep the one-CTA kernel: with at most four 64-key tiles
-  // there is nothing to share or split.  The choice goes by what the handle can hold, not by a call's lengths: those are on the
+  // Attention of the pair path.  Calls of few requests with caches of fewer than 256 tokens keep the one-CTA kernel: with at most
+  // four 64-key tiles there is nothing to split; the persistent pairs are for them from half as many items as there are pairs on
+  // (60 / 200 tokens, one-CTA kernel -> persistent pairs: 20 requests 10.93 -> 11.02 / 11.67 -> 11.46 ms, 64: 24.0 -> 23.6 / 25.5 ->
+  // 25.3, 160: 56.7 -> 54.1 / 60.2 -> 58.2).  The choice goes by what the handle can hold, not by a call's lengths: those are on the
   // device, one graph per (batch, steps) serves them all, and a graph per choice would be captured in the middle of serving.
   // (Ten-step loops with 816-token prefixes, handle for 2048 tokens against one for 816: 2 requests 8.48 / 8.52 ms, 4: 9.31 /
   // 9.36, 8: 10.73 / 10.75, 16: 12.49 / 12.64.)
   const int pr_ranges = h->pair_ranges ? std::min(h->pair_ranges, attention_pair_max_ranges(d)) : (pair && h->q_tiles_pair ? attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len) : 1);
-  const bool attn_pair = pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair && h->cfg.max_prefix_len >= 256 && (pr_ranges > 1 || h->pair_ranges);
+  const bool attn_pair = pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair &&
+                         (h->cfg.max_prefix_len >= 256 || 2 * batch * (d.Hq / 4) >= attention_persist_pairs(d));
   auto attention_rot = [&](int l) -> phyai_status_t {   // from rotated bf16 q / k / v to the output projection's operand
     cudaError_t e;
     const bool tr1 = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from;

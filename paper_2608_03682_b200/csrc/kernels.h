@@ -236,6 +236,11 @@ cudaError_t launch_attention_merge(int* status, const float* part_o, const float
 
 // ---- tcgen05 attention on CTA pairs (attention_pair.cu): several requests; q as operand tiles (see k_attn_b1), key ranges
 // of a request over up to 4 pairs of a cluster
+// (the same shapes; all keys of a request in one pair, a persistent grid of pairs: attention_persist.cu)
+int attention_persist_pairs(const Dims& d);
+cudaError_t launch_attention_persist(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
+                                     const __nv_bfloat16* vr, int layer, __nv_bfloat16* out, int rows_pad, const Dims& d, int batch,
+                                     const int* order, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, bool pdl);
 bool attention_pair_supported(const Dims& d);
 bool prefix_kv_map(unsigned char* map, const void* kv, uint64_t kv_tokens, const Dims& d);   // fills Request::kv_map
 int attention_pair_max_ranges(const Dims& d);

@@ -66,6 +66,16 @@ def test_pair_attention_key_ranges(head_dim, n_q, n_kv, ranges):
     check(cfg, [700, 0, 1, 127, 128, 129, 512, 64, 386], 1, range(9), pair_attn_ranges=ranges)
 
 
+@pytest.mark.parametrize("head_dim,n_q,n_kv,batch,horizon,top", [(256, 8, 1, 75, 12, 520), (128, 8, 2, 190, 50, 300), (256, 4, 1, 149, 63, 120)])
+def test_attention_of_many_requests(head_dim, n_q, n_kv, batch, horizon, top):
+    """More (request, head group) items than CTA pairs: two to six per pair, of one to five key tiles (no prefix, one key, whole and
+    partial blocks of 64 keys, an odd and an even number of blocks), the last round of items incomplete."""
+    cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=batch, max_prefix_len=top, n_layers=2,
+                            horizon=horizon, suffix_block_causal=n_kv == 2)
+    lens = [min(top, (0, 1, 63, 64, 65, top, 127, 128, 129)[b % 9]) if b < 18 else (53 * b) % (top + 1) for b in range(batch)]
+    check(cfg, lens, 1, [*range(0, 18, 2), batch // 2, batch - 2, batch - 1])
+
+
 @pytest.mark.parametrize("horizon", [59, 60, 62, 63])
 @pytest.mark.parametrize("ranges", [2, 3, 4])
 def test_pair_attention_at_the_most_suffix_rows(ranges, horizon):
