@@ -667,6 +667,29 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     ++cnt;
     return PHYAI_OK;
   };
+  // fp32 path with few rows: a block per action row takes the step boundary
+  const bool row_step = !h->tc && simt_norm && step_row_supported(d, batch);
+  auto step_row = [&](int k) -> phyai_status_t {
+    StepRow p{};
+    const float* gate_unused;
+    p.A = d.A, p.H = d.H, p.D = D, p.S = d.S, p.ns = d.ns, p.eps = d.eps, p.dt = dt, p.h = h->h;
+    if (k > 0) {
+      site(k - 1, 2 * d.L, &p.gain, &p.shift, &gate_unused);
+      p.Wout = h->Wout, p.bout = h->bout;
+    }
+    if (k < n) p.Wc = h->Wc, p.bias = h->ada ? h->bcfold : t.tb + (size_t)k * D, p.state_tok = h->state_tok, p.u = h->ada ? nullptr : h->u_f;
+    const cudaError_t e = launch_step_row(h->rq, h->status, p, batch * d.H, st);
+    if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "step boundary launch failed: %s", cudaGetErrorString(e));
+    ++cnt;
+    return PHYAI_OK;
+  };
+  auto mlp2_f32 = [&]() -> phyai_status_t {
+    SimtGemm g{};
+    g.A = h->u_f, g.lda = D, g.B = h->W2f, g.M = batch * d.H, g.N = D, g.K = D, g.epi = EPI_STORE, g.bias = h->b2;
+    g.out = h->h, g.ldo = D, g.rows_in = d.H, g.rows_out = d.S, g.row_off = d.ns;
+    simt_gemm(g);
+    return PHYAI_OK;
+  };
   for (int k = 0; k < n; ++k) {
     // ---- suffix embedding ----
     if (pair) {
@@ -682,6 +705,9 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
         e.xn_out = h->xn64, e.ss_out = h->ss_b;
         ST(b1_gemm(e, 1, M));
       }
+    } else if (row_step) {
+      ST(step_row(k));
+      if (!h->ada) ST(mlp2_f32());
     } else if (!h->ada) {
       launch_embed_pi0(h->rq, h->status, h->Wc, t.tb + (size_t)k * D, h->state_tok, h->h, h->u_f, h->u_t, h->Mpad, d,
                        batch, st);
@@ -697,10 +723,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
         if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "tensor GEMM launch failed: %s", cudaGetErrorString(e));
         ++cnt;
       } else {
-        SimtGemm g{};
-        g.A = h->u_f, g.lda = D, g.B = h->W2f, g.M = rows, g.N = D, g.K = D, g.epi = EPI_STORE, g.bias = h->b2;
-        g.out = h->h, g.ldo = D, g.rows_in = d.H, g.rows_out = d.S, g.row_off = d.ns;
-        simt_gemm(g);
+        ST(mlp2_f32());
       }
     } else {
       launch_embed_pi05(h->rq, h->status, h->Wc, h->bcfold, h->state_tok, h->h, d, batch, st);
@@ -871,6 +894,10 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     }
     if (b1_step) {
       if (k + 1 == n) ST(step_kernel(n, false, true));
+      continue;
+    }
+    if (row_step) {
+      if (k + 1 == n) ST(step_row(n));
       continue;
     }
     const float *gain, *shift, *gate;

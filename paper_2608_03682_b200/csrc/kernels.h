@@ -180,6 +180,16 @@ struct SimtGemm {
 // few token rows (simt_rows.cu)
 bool simt_rows_supported(int M, int K);
 cudaError_t launch_simt_rows(const int* status, const SimtGemm& g, cudaStream_t st);
+// step boundary, a block per action row
+struct StepRow {
+  int A, H, D, S, ns;
+  float eps, dt;
+  const float *gain, *shift, *Wout, *bout;      // the step that ends: final norm (shift or null), velocity head; gain null: none
+  const float *Wc, *bias, *state_tok;           // the step that begins; Wc null: none
+  float *h, *u;                                 // u: pi0's embedding (the MLP's second layer follows), else h
+};
+bool step_row_supported(const Dims& d, int batch);
+cudaError_t launch_step_row(const Request* rq, const int* status, const StepRow& p, int rows, cudaStream_t st);
 bool attention_row_supported(const Dims& d, int max_prefix);
 cudaError_t launch_attention_row(const Request* rq, const int* status, const float* qkv, const float2* rope, int layer, int kv_is_bf16,
                                  float* out, const Dims& d, int batch, int max_prefix, cudaStream_t st);
