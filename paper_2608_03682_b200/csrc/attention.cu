@@ -206,6 +206,7 @@ __global__ void k_check_lens(const int* cu, int batch, uint64_t kv_tokens, int* 
 // also writes the request block and checks the lengths.
 __global__ void __launch_bounds__(256) k_op_operands(Request* rq, const Request src, int* status, const float* qkv, const float2* rope,
                                                      __nv_bfloat16* q_tiles, __nv_bfloat16* kr, __nv_bfloat16* vr, const Dims d, int clear) {
+  pdl_launch_dependents();
   const int i = blockIdx.x, b = blockIdx.y, half = d.dh >> 1, hc = half >> 3;
   if (i == 0 && b == 0) {
     if (threadIdx.x == 0) *rq = src;
@@ -317,8 +318,8 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
   a.rope = reinterpret_cast<const float2*>(rope), a.layer = (int)desc->layer, a.out = reinterpret_cast<__nv_bfloat16*>(out);
   a.d = d, a.wait_limit = 1u << 22;
   // The library's choice where shapes and alignment allow it: bf16 operands first (one small kernel), then the tcgen05 kernels
-  // of the denoising loop.  Per call of the pi0 shape, against the mma.sync kernel with its best split: one request 18 - 19 us
-  // against 25, 4 requests 23 / 41, 16 requests 29 / 70.
+  // of the denoising loop.  Per call of the pi0 shape, against the mma.sync kernel with its best split: one request 14.4 us
+  // against 25, 4 requests 20.5 / 41, 16 requests 26.7 / 70.
   const size_t q_elems = (size_t)batch * (d.Hq / 2) * 128 * d.dh, kv_elems = (size_t)batch * d.Hkv * d.S * d.dh;
   const size_t tc_need = sizeof(Request) + (q_elems + 2 * kv_elems) * 2;
   // (a given scratch that cannot hold the operands leaves the call to the mma.sync kernel, which reads the fp32 rows itself)
@@ -352,9 +353,11 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     if (!b1 && !prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) {
       k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
-      // (the attention kernels read the request block before their dependency wait: no programmatic launch here)
+      // (one wave of clusters: its set-up and the copies of the prefix rows run under the kernel above, 18.5 -> 14.4 us per call of one
+      // request; the kernels on pairs read the request block that the kernel above writes before their dependency wait: no
+      // programmatic launch for them)
       if (b1)
-        e = launch_attention_b1(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch, 1, true, a.wait_limit, st, nullptr, 0, false);
+        e = launch_attention_b1_op(prefix_kv, kv_tokens, cu, status_word, qt, kr, vr, a.layer, a.out, d, (int)batch, a.wait_limit, st);
       else
         e = launch_attention_pair(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch,
                                   attention_pair_ranges(d, (int)batch, (int)(kv_tokens / batch)), nullptr, a.wait_limit, st, nullptr, false);

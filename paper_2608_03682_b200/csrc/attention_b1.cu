@@ -114,8 +114,15 @@ __global__ void __launch_bounds__(288, 1) k_attn_b1(const AttnArgs a) {
   const uint32_t tmem_s = tmem_base, tmem_o = tmem_base + KB;
   const WaitCtx wc{a.status, &abort_flag, a.wait_limit};
 
-  // (the request block is written before the captured loop starts: safe to read ahead of the dependency wait)
-  const Request r = *a.rq;
+  // (the request block is written before the captured loop starts: safe to read ahead of the dependency wait; an operator call
+  // has its cache and lengths in the arguments, complete before the kernel that this one depends on started)
+  struct {
+    const void* prefix_kv;
+    uint64_t kv_tokens;
+    const int* cu_lens;
+  } r;
+  if constexpr (F32) r.prefix_kv = a.op_kv, r.kv_tokens = a.op_kv_tokens, r.cu_lens = a.op_cu;
+  else r.prefix_kv = a.rq->prefix_kv, r.kv_tokens = a.rq->kv_tokens, r.cu_lens = a.rq->cu_lens;
   // (a call whose lengths are invalid stores nothing; the clamps keep its loads inside the cache)
   const int p0 = min(max(r.cu_lens[b], 0), (int)r.kv_tokens), P = min(max(r.cu_lens[b + 1] - p0, 0), (int)r.kv_tokens - p0);
   // Keys of this CTA: an eighth of the prefix keys followed by an eighth of the request's own (suffix) keys -- the
@@ -487,11 +494,11 @@ cudaLaunchConfig_t config_one(const dim3& grid, cudaStream_t st, cudaLaunchAttri
   return cfg;
 }
 template <int DH, int HPC, bool F32>
-cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) {
+cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st) {
   cudaError_t e = setup_one<DH, HPC, F32>();
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at[2];
-  const cudaLaunchConfig_t cfg = config_one<DH, HPC, F32>(dim3(8, a.d.Hq / HPC, batch), st, at, pdl);
+  const cudaLaunchConfig_t cfg = config_one<DH, HPC, F32>(dim3(8, a.d.Hq / HPC, batch), st, at, true);
   return cudaLaunchKernelEx(&cfg, k_attn_b1<DH, HPC, F32>, a);
 }
 // clusters of this kernel that are resident at a time (0 on an error)
@@ -520,14 +527,22 @@ int attention_b1_resident_ctas(const Dims& d) {
 
 cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                 const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d,
-                                int batch, int hpc, bool f32, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, int trace_all, bool pdl) {
+                                int batch, int hpc, unsigned wait_limit, cudaStream_t st, unsigned long long* trace, int trace_all) {
   AttnArgs a{};
   a.rq = rq, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr, a.layer = layer, a.out = out_tiled, a.rows_pad = rows_pad;
   a.num_splits = 8, a.d = d, a.wait_limit = wait_limit, a.trace = trace, a.trace_all = trace_all;
-  if (f32 && hpc != 1) return cudaErrorInvalidValue;
-  if (f32) return d.dh == 256 ? launch_one<256, 1, true>(a, batch, st, pdl) : launch_one<128, 1, true>(a, batch, st, pdl);
-  if (hpc == 1) return d.dh == 256 ? launch_one<256, 1, false>(a, batch, st, pdl) : launch_one<128, 1, false>(a, batch, st, pdl);
-  return d.dh == 256 ? launch_one<256, 2, false>(a, batch, st, pdl) : launch_one<128, 2, false>(a, batch, st, pdl);
+  if (hpc == 1) return d.dh == 256 ? launch_one<256, 1, false>(a, batch, st) : launch_one<128, 1, false>(a, batch, st);
+  return d.dh == 256 ? launch_one<256, 2, false>(a, batch, st) : launch_one<128, 2, false>(a, batch, st);
+}
+
+// operator call: cache and lengths as arguments, row-major output, fp32 partials
+cudaError_t launch_attention_b1_op(const void* prefix_kv, uint64_t kv_tokens, const int* cu_lens, int* status, const __nv_bfloat16* q_tiles,
+                                   const __nv_bfloat16* kr, const __nv_bfloat16* vr, int layer, __nv_bfloat16* out, const Dims& d, int batch,
+                                   unsigned wait_limit, cudaStream_t st) {
+  AttnArgs a{};
+  a.op_kv = prefix_kv, a.op_kv_tokens = kv_tokens, a.op_cu = cu_lens, a.status = status, a.qr = q_tiles, a.kr = kr, a.vr = vr;
+  a.layer = layer, a.out = out, a.num_splits = 8, a.d = d, a.wait_limit = wait_limit;
+  return a.d.dh == 256 ? launch_one<256, 1, true>(a, batch, st) : launch_one<128, 1, true>(a, batch, st);
 }
 
 }  // namespace phyai

@@ -484,7 +484,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
         atr = h->trace + (size_t)trace_cursor * TRACE_STAMPS, all = 1;
         trace_cursor += n_cta;
       }
-      e = launch_attention_b1(h->rq, h->status, h->q_tiles, kr, vr, l, h->attn64, 64, dd, batch, b1_hpc, false, h->wait_limit, st, atr, all);
+      e = launch_attention_b1(h->rq, h->status, h->q_tiles, kr, vr, l, h->attn64, 64, dd, batch, b1_hpc, h->wait_limit, st, atr, all);
     }
     else if (b1_attn_tc)
       e = launch_attention_tc(h->rq, h->status, h->qr_big, kr, vr, l, h->attn64, 64, dd, batch, h->order, h->wait_limit, st);
