@@ -38,9 +38,10 @@ namespace {
 
 constexpr int PG_PROD = 4;
 constexpr int PG_EPI = 512, PG_THREADS = (PG_PROD + 1) * 32 + PG_EPI;
-// tokens an epilogue warp takes at a time: 16 for the rotary epilogue, which then has the registers to hold the (cos, sin)
-// of the next two blocks (one 32-token block ahead on 8 warps: 7 us per tile, bound by the table's latency), else 32
-template <int EPI> constexpr int PG_TB = EPI == PG_QKV ? 16 : 32;
+// tokens an epilogue warp takes at a time: 16, so that the body of the loop is short (its code is fetched once per launch: with 32 in
+// the GeGLU epilogue 2 / 4 requests 7.65 / 8.34 ms, with 16 7.59 / 8.31) and the rotary epilogue has the registers to hold the (cos, sin)
+// of the next two blocks (one 32-token block ahead on 8 warps: 7 us per tile, bound by the table's latency)
+constexpr int PG_TB = 16;
 constexpr int PG_MAXST = 20;
 // one CTA's weight block: 128 rows x 64 k; 64 rows in the half-height form (residual projections of few tokens)
 template <bool HALF> constexpr int PG_A_BYTES = (HALF ? 64 : 128) * 128;
@@ -53,37 +54,19 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
-// 32 columns of 16 tensor-memory lanes in the fragment order of the matrix instructions: registers 4 k .. 4 k + 3 of lane T
+// 16 columns of 16 tensor-memory lanes in the fragment order of the matrix instructions: registers 4 k .. 4 k + 3 of lane T
 // hold (row T / 4, columns 8 k + 2 (T % 4), + 1) and the same columns of row T / 4 + 8
-__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, float* v) {    // 16 columns
+__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, float* v) {
   uint32_t* r = reinterpret_cast<uint32_t*>(v);
   asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr)
                : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait16(float* a, float* b) {
+__device__ __forceinline__ void tmem_ld_wait16(float* a, float* b) {    // the registers pass through, so that no use moves up
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]), "+f"(b[0]), "+f"(b[1]),
                  "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
-               :
-               : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait32(float* a, float* b) {    // the registers pass through, so that no use moves up
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]), "+f"(a[8]), "+f"(a[9]),
-                 "+f"(a[10]), "+f"(a[11]), "+f"(a[12]), "+f"(a[13]), "+f"(a[14]), "+f"(a[15]), "+f"(b[0]), "+f"(b[1]), "+f"(b[2]),
-                 "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7]), "+f"(b[8]), "+f"(b[9]), "+f"(b[10]), "+f"(b[11]),
-                 "+f"(b[12]), "+f"(b[13]), "+f"(b[14]), "+f"(b[15])
                :
                : "memory");
 }
@@ -95,10 +78,16 @@ __device__ __forceinline__ void stmatrix4_t(uint32_t addr, uint32_t r0, uint32_t
 // CPS: k-chunks of 64 per ring stage.  A stage costs the MMA issuer a wait and a commit on top of the chunks' copies; with few
 // tokens per tile that, not bytes or tensor time, set the pace (290 clocks per chunk whatever its size; with four chunks per
 // stage 165, the ingest of the SM: down projection of 204 tokens 9.9 -> 5.6 us).
+// EPI PG_EMBED (internal): PG_RESID of the action MLP, whose rows start from a bias or the state token instead of h.  (A kernel of its
+// own, and the addresses of the residual epilogue as increments: its code is fetched once per launch, between the accumulator and
+// the stores; ten-step loops of 2 / 4 / 8 / 16 requests 7.88 / 8.54 / 9.72 / 11.31 ms before, 7.70 / 8.37 / 9.54 / 11.20 after.)
+constexpr int PG_EMBED = 4;
+
 template <int EPI, bool HALF, int CPS>
 __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
     k_gemm_pair(int* status, const PairGemm g, const __grid_constant__ CUtensorMap tmw, const __grid_constant__ CUtensorMap tmx) {
-  constexpr int EPIW = PG_EPI / 32, TB = PG_TB<EPI>, K8 = TB / 8, A_BYTES = PG_A_BYTES<HALF>;
+  constexpr bool RESID = EPI == PG_RESID || EPI == PG_EMBED;
+  constexpr int EPIW = PG_EPI / 32, TB = PG_TB, K8 = TB / 8, A_BYTES = PG_A_BYTES<HALF>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_full[PG_MAXST];    // leader: both CTAs' operands of a stage have landed
   __shared__ __align__(8) uint64_t bar_empty[PG_MAXST];   // each CTA: the MMAs have read the stage
@@ -109,7 +98,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
   __shared__ __align__(16) float rs_tab[2][256];                        // per token: the folded norm's 1 / rms
   // QKV: (position x dh / 2, element offset of the token's row in q without the head term, the same in k / v, suffix row)
   __shared__ int4 tok_tab[EPI == PG_QKV ? 2 : 1][EPI == PG_QKV ? 256 : 1];
-  __shared__ float ss_tab[EPI == PG_RESID ? 4 : 1][EPI == PG_RESID ? 256 : 1];   // partial sums of squares per lane quarter
+  __shared__ float ss_tab[RESID ? 4 : 1][RESID ? 256 : 1];   // partial sums of squares per lane quarter
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int rank = (int)(blockIdx.x & 1), pair = (int)(blockIdx.x >> 1), n_pairs = (int)(gridDim.x >> 1);
@@ -204,7 +193,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
           }
           if (gi == 0 && lane == 0) trace_stamp(trc, 3);
           uint32_t a0 = tiles + (uint32_t)s * stage_bytes;
-#pragma unroll
+          // (two chunks per turn: unrolled further, more code to fetch at the start of every layer's kernel than the issue rate gains;
+          // ten-step loops of 2 / 8 requests 7.69 / 9.55 ms with all four, 7.64 / 9.47 with two, 7.72 / 9.44 with one, which costs 16 requests 1 %)
+#pragma unroll 2
           for (int c = 0; c < CPS; ++c, a0 += chunk_bytes) {
             const uint64_t da = make_desc(a0), db = make_desc(a0 + A_BYTES);
 #pragma unroll
@@ -277,7 +268,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
           if (g.shift) sh[gr][e & 1] = g.shift[row] * osc;
           sc[gr][e & 1] *= osc;
         }
-      } else if constexpr (EPI == PG_RESID) {
+      } else if constexpr (RESID) {
         const int n = n0 + (HALF ? q & 1 : q) * 32 + lane;
         if (g.scale) scr = g.scale[n];
         if (g.gate) scr *= g.gate[n];
@@ -310,17 +301,19 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       // RESID: in the transposed view a lane takes 4 channels of tokens lane / 8, + 4, + 8, + 12 of the chunk; what is added
       // to (the residual stream, or the MLP's bias / the state token) is requested one chunk ahead
       const int n4 = n0 + (HALF ? q & 1 : q) * 32 + (lane & 7) * 4;
+      const float* const hrow = g.h + (size_t)(tok_base + (lane >> 3)) * g.N + n4;
       float4 old[2][4], gain4 = make_float4(0.f, 0.f, 0.f, 0.f);
       auto fetch_old = [&](int c0, float4* o) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int tok = min(tok_base + c0 + 4 * u + (lane >> 3), g.M - 1);
-          const float* src = g.h + (size_t)tok * g.N + n4;
-          if (g.bias) src = (tok % g.S) < g.ns ? g.state_tok + (size_t)(tok / g.S) * g.N + n4 : g.bias + n4;
-          o[u] = *reinterpret_cast<const float4*>(src);
+          const int tl = c0 + 4 * u + (lane >> 3), tok = tok_base + tl;
+          const float* src = hrow + (size_t)(c0 + 4 * u) * g.N;
+          if (EPI == PG_EMBED) src = (tok % g.S) < g.ns ? g.state_tok + (size_t)(tok / g.S) * g.N + n4 : g.bias + n4;
+          o[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (tl < n_tok) o[u] = *reinterpret_cast<const float4*>(src);
         }
       };
-      if constexpr (EPI == PG_RESID) {
+      if constexpr (RESID) {
         if (g.gain_next) gain4 = __ldg(reinterpret_cast<const float4*>(g.gain_next + n4));
         if (th + cg * 16 < tl_end) fetch_old(th + cg * 16, old[0]);
         if (th + cg * 16 + 64 < tl_end) fetch_old(th + cg * 16 + 64, old[1]);
@@ -350,7 +343,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       const bool ok = !skip && !dead && r > 0 && !*reinterpret_cast<volatile int*>(&abort_flag);
       tc_fence_after();
       if (i == 0 && et == 0) trace_stamp(trc, 5);
-      if constexpr (EPI == PG_RESID) {
+      __nv_bfloat16* const orow = RESID ? g.out + ((size_t)(n4 >> 6) * g.rows_pad + tok_base + (lane >> 3)) * 64 + (n4 & 7) : nullptr;
+      if constexpr (RESID) {
         // 16 token columns at a time: the lane that holds a row scales it and puts it into the warp's staging block [16
         // tokens][32 rows + 4]; then 8 lanes take the 32 channels (128 bytes of h) of one token
 #pragma unroll 1
@@ -365,13 +359,13 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
           for (int u = 0; u < 4; ++u) {
             const int tl = c0 + 4 * u + (lane >> 3), tok = tok_base + tl;
             const float4 a = *reinterpret_cast<const float4*>(sp + 4 * u * PG_PITCH);
-            const bool live = !(g.bias && (tok % g.S) < g.ns);       // (state rows do not pass through the MLP)
+            const bool live = EPI != PG_EMBED || (tok % g.S) >= g.ns;       // (state rows do not pass through the MLP)
             float4 hv = old[0][u];
             if (live) hv.x += a.x, hv.y += a.y, hv.z += a.z, hv.w += a.w;
             if (ok && tl < tl_end) {
-              *reinterpret_cast<float4*>(g.h + (size_t)tok * g.N + n4) = hv;
+              *reinterpret_cast<float4*>(const_cast<float*>(hrow) + (size_t)(c0 + 4 * u) * g.N) = hv;
               if (g.gain_next)
-                *reinterpret_cast<uint2*>(g.out + tiled_index(tok, n4, g.rows_pad)) =
+                *reinterpret_cast<uint2*>(orow + (c0 + 4 * u) * 64 + ((((n4 & 63) >> 3) ^ (tok & 7)) << 3)) =
                     make_uint2(pack_bf16x2(hv.x * gain4.x, hv.y * gain4.y), pack_bf16x2(hv.z * gain4.z, hv.w * gain4.w));
             }
             float s2 = hv.x * hv.x + hv.y * hv.y + hv.z * hv.z + hv.w * hv.w;
@@ -395,13 +389,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
         for (int c0 = cg * TB; c0 < n_tok; c0 += 4 * TB) {
           float a[4 * K8], b[4 * K8];
           const uint32_t ta = tl_addr + (uint32_t)(buf * 256 + c0), tb = ta + (16u << 16);
-          if constexpr (TB == 32) {
-            tmem_ld_frag(ta, a), tmem_ld_frag(tb, b);
-            tmem_ld_wait32(a, b);
-          } else {
-            tmem_ld_frag16(ta, a), tmem_ld_frag16(tb, b);
-            tmem_ld_wait16(a, b);
-          }
+          tmem_ld_frag16(ta, a), tmem_ld_frag16(tb, b);
+          tmem_ld_wait16(a, b);
           const int t2 = c0 + 2 * (lane & 3);            // this lane's tokens: t2 + 8 k and + 1
           if (EPI == PG_GEGLU || EPI == PG_QKV) {
 #pragma unroll
@@ -464,7 +453,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) __cluster_dims__(2, 1, 1)
       tc_fence_before();
       if (lane == 0)
         remote_arrive(tempty0 + (uint32_t)buf * 8u);
-      if constexpr (EPI == PG_RESID) {
+      if constexpr (RESID) {
         if (g.ss_out) {
           asm volatile("bar.sync %0, %1;" ::"n"(BAR_EPI + 1), "n"(PG_EPI) : "memory");
           if (ok && et < n_tok) {     // one partial sum per 64 channels and token
@@ -567,6 +556,7 @@ cudaError_t launch_pair_gemm(int* status, const PairGemm& g_in, int n_sm, int* b
   const int grid = 2 * std::min(n_tiles, n_sm / 2);
   *busy = grid;
   const size_t smem = (size_t)g.stages * stage + 1024 + PG_STG_BYTES;
+  if (g.bias) return t.half ? launch_one<PG_EMBED, true>(status, g, grid, smem, tw, tx, st) : launch_one<PG_EMBED>(status, g, grid, smem, tw, tx, st);
   if (t.half) return launch_one<PG_RESID, true>(status, g, grid, smem, tw, tx, st);
   switch (g.epi) {
     case PG_QKV: return launch_one<PG_QKV>(status, g, grid, smem, tw, tx, st);
