@@ -50,9 +50,8 @@ __global__ void __launch_bounds__(1024) k_kv_scan(const int* lens, int batch, in
 // src [L][B][p_max][row_bytes], dst [L][2][kv_tokens][row_bytes]: plane (l, kv) of request b, rows p < lens[b], go to
 // rows cu[b] + p.  The rows of a request are one contiguous run on both sides: a block moves 16 KB of it (grid.x) of one
 // plane (grid.y) and request (grid.z), its loads issued before the dependency wait (only the destination needs cu).  With
-// `zero_tail` the entry grid.z = batch clears the rows past the last request (after an error: all rows).  Bound by HBM: 258 MB
-// of 8 requests of the pi0 shape 48 us with the scan, 5.4 TB/s (a grid-stride loop over padded rows with two divisions per 16 bytes,
-// behind a fill of the whole output by the caller: 139 us).
+// `zero_tail` the entry grid.z = batch clears the rows past the last request (after an error: all rows).  For more requests than the
+// threads of a block; else k_kv_pack_small.
 constexpr int PACK_T = 256, PACK_U = 4, PACK_CHUNK = PACK_T * PACK_U;
 __global__ void __launch_bounds__(PACK_T) k_kv_pack(const uint4* k, const uint4* v, const int* lens, const int* cu, const int* status, uint4* dst,
                                                     int batch, int p_max, unsigned long long kv_tokens, int row_chunks, int zero_tail) {
@@ -82,6 +81,63 @@ __global__ void __launch_bounds__(PACK_T) k_kv_pack(const uint4* k, const uint4*
     for (int u = 0; u < PACK_U; ++u)
       if (i0 + u * PACK_T < n) o[u * PACK_T] = x[u];
   }
+}
+
+// The same in one launch, for up to PACK_T requests: every block adds the lengths up itself while its loads are on their way, block
+// (0, 0, 0) also writes cu and the status word.  Bound by HBM: with the post-processing launch of the actions 8 requests of the pi0 shape
+// (258 MB moved) 45.8 us, behind a scan kernel 51.7; 1 request 20.8 / 26.8, 32 requests 166 / 175.  (Eight loads per thread instead of
+// four 46.6 / 167.8; streaming stores 45.1 for 8 requests but 171 for 32.)
+__global__ void __launch_bounds__(PACK_T) k_kv_pack_small(const uint4* k, const uint4* v, const int* lens, int* cu, int* status, uint4* dst, int batch,
+                                                          int p_max, unsigned long long kv_tokens, int row_chunks, int clear) {
+  __shared__ long long wsum[2][PACK_T / 32];
+  const int layer = blockIdx.y >> 1, is_v = blockIdx.y & 1, b = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint4* out = dst + (size_t)blockIdx.y * kv_tokens * row_chunks;
+  const int raw = tid < batch ? lens[tid] : 0;
+  const int n = b < batch ? min(max(lens[b], 0), p_max) * row_chunks : 0;
+  const uint4* src = (is_v ? v : k) + ((size_t)layer * batch + b) * p_max * row_chunks;
+  uint4 x[PACK_U];
+  const int i0 = (int)blockIdx.x * PACK_CHUNK + tid;
+  const bool first = blockIdx.x == 0 && blockIdx.y == 0 && b == 0;
+  if (b < batch && (int)blockIdx.x * PACK_CHUNK >= n && !first) return;
+#pragma unroll
+  for (int u = 0; u < PACK_U; ++u)
+    if (i0 + u * PACK_T < n) x[u] = __ldcs(src + i0 + u * PACK_T);
+  // ---- rows ahead of this request, all rows
+  long long run = max(raw, 0);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long up = __shfl_up_sync(0xffffffffu, run, o);
+    if (lane >= o) run += up;
+  }
+  if (lane == 31) wsum[0][warp] = run;
+  bool bad = __syncthreads_or(raw < 0 || raw > p_max);
+  long long total = 0;
+#pragma unroll
+  for (int w = 0; w < PACK_T / 32; ++w) {
+    if (w == warp) run += total;
+    total += wsum[0][w];
+  }
+  if (tid == (b > 0 ? b - 1 : 0)) wsum[1][0] = b > 0 ? run : 0;            // (inclusive sum of the request before)
+  bad |= (unsigned long long)total > kv_tokens;
+  __syncthreads();
+  const long long pre = wsum[1][0];
+  if (first) {
+    if (tid < batch) cu[tid + 1] = (int)min(run, 0x7fffffffLL);
+    if (tid == 0) {
+      cu[0] = 0;
+      if (bad || clear) atomicExch(status, bad ? ST_INVALID_ARG : 0);
+    }
+  }
+  if (b == batch) {
+    const size_t lo = bad ? 0 : (size_t)total * row_chunks, hi = kv_tokens * row_chunks;
+    for (size_t i = lo + (size_t)blockIdx.x * PACK_T + tid; i < hi; i += (size_t)gridDim.x * PACK_T) out[i] = make_uint4(0u, 0u, 0u, 0u);
+    return;
+  }
+  if (bad || (!clear && status_set(status))) return;      // (a word raised before: nothing is copied, unless the call clears it)
+  uint4* o = out + (size_t)pre * row_chunks + i0;
+#pragma unroll
+  for (int u = 0; u < PACK_U; ++u)
+    if (i0 + u * PACK_T < n) o[u * PACK_T] = x[u];
 }
 
 // out[b][h][a] = (clip(x[b][h][a]) + 1) / 2 * (q99[a] - q01[a]) + q01[a] for h < H_out, a < A_out
@@ -124,8 +180,17 @@ static phyai_status_t pack_prefix_kv(const phyai_kv_pack_desc_t* desc, const voi
     return bad("kv_tokens, batch, p_max or n_layers too large");
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int chunks = (int)(row_bytes / 16), B = (int)desc->batch;
-  k_kv_scan<<<1, 1024, 0, st>>>(lens, B, (int)desc->p_max, kv_tokens, cu_prefix_lens, status_word, cleared);
   const unsigned gx = (unsigned)(((size_t)desc->p_max * chunks + PACK_CHUNK - 1) / PACK_CHUNK);
+  if (B <= PACK_T) {
+    k_kv_pack_small<<<dim3(gx, desc->n_layers * 2, B + cleared), PACK_T, 0, st>>>(reinterpret_cast<const uint4*>(k), reinterpret_cast<const uint4*>(v), lens,
+                                                                                  cu_prefix_lens, status_word, reinterpret_cast<uint4*>(prefix_kv), B,
+                                                                                  (int)desc->p_max, (unsigned long long)kv_tokens, chunks, cleared);
+    const cudaError_t es = cudaGetLastError();
+    if (es == cudaSuccess) return PHYAI_OK;
+    snprintf(g_ad_err, sizeof(g_ad_err), "kernel launch failed: %s", cudaGetErrorString(es));
+    return PHYAI_ERR_CUDA;
+  }
+  k_kv_scan<<<1, 1024, 0, st>>>(lens, B, (int)desc->p_max, kv_tokens, cu_prefix_lens, status_word, cleared);
   cudaError_t e = launch_pdl(k_kv_pack, dim3(gx, desc->n_layers * 2, B + cleared < 65535 ? B + cleared : 65535), dim3(PACK_T), 0, st,
                              reinterpret_cast<const uint4*>(k), reinterpret_cast<const uint4*>(v), (const int*)lens, (const int*)cu_prefix_lens,
                              (const int*)status_word, reinterpret_cast<uint4*>(prefix_kv), B, (int)desc->p_max,

@@ -69,6 +69,38 @@ def test_kv_layout_writer_reports_bad_lengths_on_the_device():
                                torch.zeros(1, 1, 4, 1, 4, dtype=torch.bfloat16).cuda(), torch.tensor([1], dtype=torch.int32).cuda())
 
 
+@pytest.mark.parametrize("B", [1, 32, 33, 255, 256, 257])
+def test_kv_layout_writer_over_its_batch_sizes(B):
+    """One launch up to 256 requests (the lengths added up over one warp, several, all threads of a block), two beyond: the gather, the
+    cleared tail, a bad last length, a total that does not fit by one row, and a word that was raised before."""
+    g = torch.Generator().manual_seed(B)
+    k, v = (torch.randn(2, B, 5, 1, 8, generator=g).bfloat16() for _ in range(2))
+    lens = torch.randint(0, 6, (B,), generator=g, dtype=torch.int32)
+    lens[-1] = 5
+    total = int(lens.sum())
+    ref, cu_ref = A.pack_prefix_kv(k.view(torch.int16).numpy(), v.view(torch.int16).numpy(), lens.numpy())
+    for kv_tokens in (total, total + 7):
+        out, cu, status = binding.pack_prefix_kv(k.cuda(), v.cuda(), lens.cuda(), kv_tokens=kv_tokens)
+        got = out.cpu().view(torch.int16).numpy()
+        assert int(status.item()) == 0 and cu.cpu().tolist() == cu_ref.tolist()
+        assert np.array_equal(got[:, :, :total], ref) and not got[:, :, total:].any()
+    bad = lens.clone()
+    bad[-1] = 6
+    for lengths, kv_tokens in ((bad, total + 7), (lens, total - 1)):
+        out, cu, status = binding.pack_prefix_kv(k.cuda(), v.cuda(), lengths.cuda(), kv_tokens=kv_tokens)
+        assert int(status.item()) == binding.ERR_INVALID_ARG and not out.any()
+    # the entry that leaves the word to its caller: raised before, nothing is written; zero, the rows are
+    lib, desc = binding.load_library(), binding.KvPackDesc(binding._KV_PACK_SIZE, 2, 1, 8, 2, B, 5)
+    kd, vd, ld = k.cuda(), v.cuda(), lens.cuda()
+    for word in (binding.ERR_INVALID_ARG, 0):
+        out = torch.zeros(2, 2, total, 1, 8, dtype=torch.bfloat16, device="cuda")
+        cu, status = torch.empty(B + 1, dtype=torch.int32, device="cuda"), torch.tensor([word], dtype=torch.int32, device="cuda")
+        assert lib.phyai_pack_prefix_kv(binding.C.byref(desc), kd.data_ptr(), vd.data_ptr(), ld.data_ptr(), out.data_ptr(), total, cu.data_ptr(),
+                                        status.data_ptr(), None) == binding.OK
+        torch.cuda.synchronize()
+        assert int(status.item()) == word and bool(out.any()) == (word == 0)
+
+
 def test_action_postprocessing_matches_oracle():
     g = torch.Generator().manual_seed(9)
     x = torch.randn(6, 50, 32, generator=g) * 1.3
