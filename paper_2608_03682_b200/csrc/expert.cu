@@ -139,9 +139,11 @@ struct phyai_expert {
   int* status = nullptr;
 
   std::map<int, Tables> tables;
-  std::map<std::pair<int, int>, cudaGraphExec_t> graphs;
+  std::map<std::pair<int, int>, cudaGraphExec_t> graphs;      // by (requests, steps); (requests, -steps): without the first step
   std::map<std::pair<int, int>, uint64_t> launch_counts;
   cudaStream_t cap_stream = nullptr;
+  cudaStream_t copy_stream = nullptr;      // host requests: the prefix caches' way to the device, beside the first step
+  cudaEvent_t copy_events[13] = {};        // [0]: the caller's stream is ready for them; then one per copy
 
   // host-variant staging (allocated on first use)
   void* stg_kv = nullptr; size_t stg_kv_bytes = 0;
@@ -303,6 +305,8 @@ phyai_status_t build_tables(phyai_expert* h, int n, cudaStream_t st, Tables** ou
 // merge pass): from this many CTAs on it beats the split mma.sync kernel + merge.
 constexpr int ATTN_TC_MIN_CTAS = 8;
 constexpr int MAX_SLABS = 16;
+constexpr size_t OVERLAP_KV = (size_t)1 << 20;
+constexpr int HOST_PIECES = 12;
 constexpr int TRACE_SLOTS = 4096, TRACE_STAMPS = 16;
 
 int pick_nt(int M) { return M <= 64 ? 64 : (M <= 1024 ? 128 : 256); }
@@ -336,7 +340,14 @@ int pick_splits(int n_tiles, int tok_tiles, int KC) {
   return s;
 }
 
-phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, cudaStream_t st) {
+// Steps k0 .. k1 - 1 of the call's n, with what comes before the first and after the last.  `gate(l)` is called ahead of layer l of
+// step 0 (host calls: the layer's planes of the prefix cache may still be on their way).
+struct Gate {
+  phyai_status_t (*call)(void*, int);
+  void* self;
+  phyai_status_t operator()(int l) const { return call(self, l); }
+};
+phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, cudaStream_t st, int k0, int k1, const Gate* gate_kv = nullptr) {
   const Dims& d0 = h->d;
   // State-token caching (block-causal suffix mask, plain norms): the state token sees the prefix and itself only, so
   // its hidden states and its rotated key / value of every layer depend neither on x nor on t.  They are computed
@@ -630,9 +641,12 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     return pair_gemm(g);
   };
 
-  launch_begin(h->rq, h->status, h->state_w, h->state_b, h->state_tok, d0, batch, st);
-  ++cnt;
-  if (cache_state) {
+  if (k0 == 0) {
+    launch_begin(h->rq, h->status, h->state_w, h->state_b, h->state_tok, d0, batch, st);
+    ++cnt;
+  }
+  if (cache_state && k0 == 0) {
+    if (gate_kv) ST((*gate_kv)(d.L - 1));
     // the state tokens alone through every layer: row b of h = request b's state token
     Dims dp = d0;
     dp.S = 1, dp.Sk = 1, dp.Sk_stride = d0.S, dp.koff = 0;
@@ -690,7 +704,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     simt_gemm(g);
     return PHYAI_OK;
   };
-  for (int k = 0; k < n; ++k) {
+  for (int k = k0; k < k1; ++k) {
     // ---- suffix embedding ----
     if (pair) {
       ST(pair_step(k));
@@ -731,6 +745,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     }
     // ---- transformer layers ----
     for (int l = 0; l < d.L; ++l) {
+      if (gate_kv && k == 0) ST((*gate_kv)(l));
       if (pair) {
         ST(pair_layer(k, l));
         continue;
@@ -915,27 +930,40 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   return PHYAI_OK;
 }
 
-phyai_status_t run(phyai_expert* h, Request& r, int n, cudaStream_t st) {
+phyai_status_t run(phyai_expert* h, Request& r, int n, cudaStream_t st, const Gate* gate_kv = nullptr) {
   Tables* t = nullptr;
   if (h->q_tiles_pair && r.kv_tokens > 0 && !prefix_kv_map(r.kv_map, r.prefix_kv, r.kv_tokens, h->d))
     return fail(PHYAI_ERR_CUDA, "tensor map of the prefix cache could not be encoded");
   ST(build_tables(h, n, st, &t));
   launch_set_request(h->rq, r, h->cu_internal, st, h->order);
   if (r.cu_lens != nullptr) launch_validate(h->rq, h->status, (int)h->cfg.max_prefix_len, h->order, st);
-  const auto key = std::make_pair(r.batch, n);
+  auto key = std::make_pair(r.batch, n);
   if (!h->use_graph) {
-    ST(enqueue_loop(h, r.batch, n, *t, st));
+    ST(enqueue_loop(h, r.batch, n, *t, st, 0, n, gate_kv));
     h->launch_counts[key] = h->counting;
     return PHYAI_OK;
   }
+  // With a gate the first step is enqueued launch by launch, the others are a graph of their own.
+  int k0 = 0;
+  uint64_t head = 0;
+  if (gate_kv) {
+    ST(enqueue_loop(h, r.batch, n, *t, st, 0, 1, gate_kv));
+    head = h->counting, k0 = 1;
+    if (n == 1) {
+      h->launch_counts[key] = head;
+      return PHYAI_OK;
+    }
+    key.second = -n;
+  }
   auto it = h->graphs.find(key);
   if (it == h->graphs.end()) {
-    if (h->graphs.size() >= 64) return fail(PHYAI_ERR_UNSUPPORTED, "more than 64 captured (batch, n_steps) graphs");
+    const auto same = std::count_if(h->graphs.begin(), h->graphs.end(), [&](const auto& g) { return (g.first.second < 0) == (key.second < 0); });
+    if (same >= 64) return fail(PHYAI_ERR_UNSUPPORTED, "more than 64 captured (batch, n_steps) graphs");
     // tables were enqueued on `st`; the capture stream must not run ahead of them on first replay,
     // which holds because the graph is launched on `st` below.
     cudaGraph_t graph = nullptr;
     CU(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    phyai_status_t s = enqueue_loop(h, r.batch, n, *t, h->cap_stream);
+    phyai_status_t s = enqueue_loop(h, r.batch, n, *t, h->cap_stream, k0, n);
     cudaError_t e = cudaStreamEndCapture(h->cap_stream, &graph);
     if (s != PHYAI_OK) {
       if (graph) cudaGraphDestroy(graph);
@@ -947,7 +975,7 @@ phyai_status_t run(phyai_expert* h, Request& r, int n, cudaStream_t st) {
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
     it = h->graphs.emplace(key, exec).first;
-    h->launch_counts[key] = h->counting;
+    h->launch_counts[std::make_pair(r.batch, n)] = head + h->counting;
   }
   CU(cudaGraphLaunch(it->second, st));
   return PHYAI_OK;
@@ -1336,6 +1364,9 @@ void phyai_expert_destroy(phyai_expert_t* h) {
   cudaDeviceSynchronize();
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+  if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
+  for (cudaEvent_t e : h->copy_events)
+    if (e) cudaEventDestroy(e);
   delete h->packer;
   for (void* p : h->allocs) cudaFree(p);
   delete h;
@@ -1452,26 +1483,53 @@ phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, co
     if (noises[b]) memcpy(pn + b * ha, noises[b], ha * 4);
     else memset(pn + b * ha, 0, ha * 4);
   }
-  phyai_status_t s = [&]() -> phyai_status_t {
-    CU(cudaMemcpyAsync(h->stg_cu, cu, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, st));
-    if (h->cfg.has_state_token) CU(cudaMemcpyAsync(h->stg_states, ps, batch * Ds * 4, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(h->stg_noise, pn, batch * ha * 4, cudaMemcpyHostToDevice, st));
-    // several copies: the engine works on the first planes while the rest is gathered
-    const int pieces = std::min(planes, 12);
-    for (int q = 0; kvb && q < pieces; ++q) {
-      const int p0 = planes * q / pieces, p1 = planes * (q + 1) / pieces;
-      if (p1 == p0) continue;
-      h->packer->wait(p1);
-      CU(cudaMemcpyAsync(static_cast<uint8_t*>(h->stg_kv) + p0 * plane, pin_kv + p0 * plane, (p1 - p0) * plane, cudaMemcpyHostToDevice, st));
-    }
-    return PHYAI_OK;
-  }();
-  if (kvb) h->packer->wait(planes);              // (the caller's memory is not read after this call returns)
-  ST(s);
   Request r{};
   r.prefix_kv = h->stg_kv, r.kv_tokens = total, r.cu_lens = h->stg_cu, r.states = h->cfg.has_state_token ? h->stg_states : nullptr;
   r.noise = h->stg_noise, r.x = h->stg_out, r.batch = (int)batch, r.single_len = 0;
-  ST(run(h, r, (int)n_steps, st));
+  // The caches go in several copies: the engine works on the first planes while the rest is gathered, and, on a stream of their own,
+  // while the first step runs on the layers that have arrived.  (pi0 shape, ten steps, from host tensors to host arrays, us: 1 request
+  // 5190 -> 5040, 2: 8390 -> 7930, 4: 9690 -> 9000, 8: 12070 -> 11350; 1 request of 400 tokens in five steps 2680 -> 2640.)
+  const int pieces = std::min(planes, HOST_PIECES);
+  const bool overlap = kvb >= OVERLAP_KV && h->tc;
+  int issued = 0;
+  cudaStream_t cs = st;
+  auto copy_until = [&](int plane_end) -> phyai_status_t {           // pieces until those planes are on their way
+    while (issued < pieces && planes * issued / pieces < plane_end) {
+      const int p0 = planes * issued / pieces, p1 = planes * (issued + 1) / pieces;
+      h->packer->wait(p1);
+      CU(cudaMemcpyAsync(static_cast<uint8_t*>(h->stg_kv) + p0 * plane, pin_kv + p0 * plane, (p1 - p0) * plane, cudaMemcpyHostToDevice, cs));
+      ++issued;
+      if (overlap) CU(cudaEventRecord(h->copy_events[issued], cs));
+    }
+    return PHYAI_OK;
+  };
+  auto arrived = [&](int l) -> phyai_status_t {                      // layer l waits for its planes (an earlier wait may cover them)
+    const int before = issued;
+    ST(copy_until(2 * l + 2));
+    if (issued > before) CU(cudaStreamWaitEvent(st, h->copy_events[issued], 0));
+    return PHYAI_OK;
+  };
+  const Gate gate{[](void* p, int l) { return (*static_cast<decltype(arrived)*>(p))(l); }, &arrived};
+  phyai_status_t s = [&]() -> phyai_status_t {
+    if (overlap) {
+      if (!h->copy_stream) CU(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
+      for (cudaEvent_t& e : h->copy_events)
+        if (!e) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+      cs = h->copy_stream;
+      CU(cudaEventRecord(h->copy_events[0], st));       // (a call before this one may still read the caches)
+      CU(cudaStreamWaitEvent(cs, h->copy_events[0], 0));
+    }
+    CU(cudaMemcpyAsync(h->stg_cu, cu, (size_t)(batch + 1) * 4, cudaMemcpyHostToDevice, st));
+    if (h->cfg.has_state_token) CU(cudaMemcpyAsync(h->stg_states, ps, batch * Ds * 4, cudaMemcpyHostToDevice, st));
+    CU(cudaMemcpyAsync(h->stg_noise, pn, batch * ha * 4, cudaMemcpyHostToDevice, st));
+    if (!overlap && kvb) ST(copy_until(planes));
+    return run(h, r, (int)n_steps, st, overlap ? &gate : nullptr);
+  }();
+  if (kvb) h->packer->wait(planes);              // (the caller's memory is not read after this call returns)
+  if (s != PHYAI_OK) {
+    if (overlap && cs != st) cudaStreamSynchronize(cs);      // (nor its staging by a copy that no stream of the caller waits for)
+    return s;
+  }
   CU(cudaMemcpyAsync(out, h->stg_out, batch * ha * 4, cudaMemcpyDeviceToHost, st));
   return PHYAI_OK;
 }

@@ -156,6 +156,33 @@ def test_two_workers_prepare_the_next_chunk_while_the_first_is_in_flight():
         assert np.array_equal(got, ref)
 
 
+@pytest.mark.parametrize("cond,batch,top,horizon,n_steps,n_layers", [("pi0", 1, 900, 20, 1, 3), ("pi0", 3, 700, 30, 4, 7), ("pi05", 2, 1000, 12, 2, 1),
+                                                                       ("pi0", 2, 100, 12, 3, 2)])
+def test_host_requests_run_on_layers_as_they_arrive(cond, batch, top, horizon, n_steps, n_layers):
+    """Copies beside the first step (one step and more, fewer and more planes than copies, single-tile and pair kernels) and, with a small
+    cache, ahead of it: call after call with other requests on one stream, each the bits of the call on device memory."""
+    from paper_2608_03682_b200.frontend import ExpertWorker
+    from tests.helpers import small_bf16_config
+    cfg = small_bf16_config(cond, head_dim=256, n_q_heads=4, width=256, max_batch=batch, max_prefix_len=top, horizon=horizon, n_layers=n_layers)
+    W = synth.make_weights(cfg, 27, std=0.05)
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        worker = ExpertWorker(ex, cfg, n_steps)
+        calls = []
+        for c in range(3):
+            lens = [top - (17 * b + 5 * c) % top for b in range(batch)]
+            calls.append([dict(prefix_kv=synth.make_prefix_kv(cfg, 27 + c, p, b), state=synth.make_state(cfg, 27 + c, b) if cfg.has_state_token else None,
+                               noise=synth.make_noise(cfg, 27 + c, b), n_steps=n_steps) for b, p in enumerate(lens)])
+        got = [worker(reqs) for reqs in calls + calls[:1]]
+        for outs, reqs in zip(got, calls + calls[:1]):
+            packed, cu = synth.pack_prefix_kv([r["prefix_kv"] for r in reqs])
+            states = torch.stack([r["state"] for r in reqs]).cuda() if cfg.has_state_token else None
+            ref = ex.denoise_batched(packed.cuda(), torch.from_numpy(cu).cuda(), states, torch.stack([r["noise"] for r in reqs]).cuda(), n_steps)
+            torch.cuda.synchronize()
+            assert ex.poll_status() == 0
+            for b, out in enumerate(outs):
+                assert np.array_equal(np.asarray(out), ref[b].cpu().numpy()), b
+
+
 def test_host_requests_arguments_are_checked():
     """phyai_denoise_requests_host through the C ABI: every bad argument is a status code, and the handle still works."""
     import ctypes as C
