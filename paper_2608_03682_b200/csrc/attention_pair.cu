@@ -64,14 +64,14 @@ struct ApLayout {
 __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
 
 template <int DH, int C>
-__global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
+__global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, const __grid_constant__ CUtensorMap tmq) {
   using L = ApLayout<DH, C>;
   constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(KB >> 3) << 17) | ((256u >> 4) << 24);
   constexpr uint32_t IDESC_PV = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(DH >> 3) << 17) | ((256u >> 4) << 24);
 
   extern __shared__ uint8_t smem_raw[];
-  // leader: operands of a buffer complete in both CTAs; P of a buffer complete in both.  Each CTA: logits / P V complete.
-  __shared__ __align__(8) uint64_t k_full[2], v_full[2], p_full[2][2], s_full[2], pv_done[2], mrg_bar, q_bar, q_ready;
+  // leader: operands of a buffer, Q, P of a buffer complete in both CTAs.  Each CTA: logits / P V complete.
+  __shared__ __align__(8) uint64_t k_full[2], v_full[2], p_full[2][2], s_full[2], pv_done[2], mrg_bar, q_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag, mrg_ok;
   __shared__ float xch[2][2][128];       // the two half-row threads of a row exchange their maximum (by tile parity) and, at the end, sum
@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
   const int S = d.S;
   unsigned long long* const trc = a.trace ? a.trace + (size_t)((blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 16 : nullptr;
   if (tid == 0) trace_stamp(trc, 0);
+  if (tid == 5 * 32) prefetch_tmap(&tmq);
   pdl_launch_dependents();
 
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       mbar_init(smem_u32(&k_full[i]), 2), mbar_init(smem_u32(&v_full[i]), 2), mbar_init(smem_u32(&p_full[i][0]), 8), mbar_init(smem_u32(&p_full[i][1]), 8);
       mbar_init(smem_u32(&s_full[i]), 1), mbar_init(smem_u32(&pv_done[i]), 1);
     }
-    mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 8), mbar_init(smem_u32(&q_ready), 1);
+    mbar_init(smem_u32(&mrg_bar), 1), mbar_init(smem_u32(&q_bar), 1);
     if (n_me > 0) mbar_expect_tx(smem_u32(&mrg_bar), (uint32_t)((C - 1) * 2 * n_me * L::ROW));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -244,7 +245,6 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
       };
       if (T > 0) {
         mbar_wait_drain(smem_u32(&q_bar), 0u, wc);        // both CTAs' Q tiles have landed
-        mbar_wait_drain(smem_u32(&q_ready), 0u, wc);
         issue_s(0);
       }
       if (lane == 0) trace_stamp(trc, 3);
@@ -271,11 +271,6 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
         if (t == 0 && lane == 0) trace_stamp(trc, 4);
       }
       if (lane == 0) trace_stamp(trc, 5);
-    } else if (T > 0) {
-      if (lane == 0) {
-        mbar_wait_drain(smem_u32(&q_bar), 0u, wc);
-        remote_arrive(map_rank(smem_u32(&q_ready), lead_rank));
-      }
     }
     __syncwarp();
     cluster_arrive_relaxed();
@@ -292,11 +287,11 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a) {
     pdl_wait();
     if (T > 0 && lane == 0) {
       // Q (rotated, scaled) was written by the QKV projection as this CTA's operand tile: an eighth per warp (the copies of
-      // one warp complete one after the other)
-      constexpr uint32_t QP = L::QTILE / 8;
-      const uint32_t off = (uint32_t)(warp - 5) * QP;
-      mbar_expect_tx(smem_u32(&q_bar), QP);
-      bulk_g2s(Qs + off, reinterpret_cast<const uint8_t*>(a.qr) + (size_t)(b * (d.Hq >> 1) + (head0 >> 1)) * L::QTILE + off, QP, smem_u32(&q_bar));
+      // one warp complete one after the other), both CTAs' counted on the leader's barrier (with own
+      // barriers and a relay ten-step loops of 2 / 8 / 16 requests 7.61 / 9.45 / 11.14 ms, so 7.57 / 9.42 / 11.06)
+      const uint32_t bar = smem_u32(&q_bar);
+      if (half == 0 && warp == 5) mbar_expect_tx(bar, 2u * L::QTILE);
+      tma2d(Qs + (uint32_t)(warp - 5) * (L::QTILE / 8), &tmq, (b * (d.Hq >> 1) + (head0 >> 1)) * (DH * 2) + (warp - 5) * (DH / 4), bar & LEADER_MASK);
     }
     __syncwarp();
     const bool skip = status_set(a.status);
@@ -529,7 +524,9 @@ cudaError_t launch_one(const AttnArgs& a, int batch, cudaStream_t st, bool pdl) 
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at, cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_attn_pair<DH, C>, a);
+  CUtensorMap tq;      // q tiles: rows of 64 channels, an eighth of a CTA's tile at a time
+  if (!row_map(&tq, a.qr, (uint64_t)batch * (a.d.Hq / 2) * (DH * 2), DH / 4)) return cudaErrorInvalidValue;
+  return cudaLaunchKernelEx(&cfg, k_attn_pair<DH, C>, a, tq);
 }
 
 }  // namespace
