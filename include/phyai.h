@@ -146,7 +146,7 @@ size_t phyai_prefix_kv_bytes(const phyai_expert_config_t *cfg, uint64_t total_pr
  *   prefix_kv   device, layout [n_layers][2 (K,V)][kv_tokens][n_kv_heads][head_dim], head_dim
  *               contiguous, float32 for PHYAI_F32 else bfloat16, 16-byte aligned; K is used as
  *               given (already rotated by the producer).  kv_tokens is the token capacity of the
- *               buffer (>= prefix_len); rows >= prefix_len are never read.
+ *               buffer (>= prefix_len); rows >= prefix_len have no part in a result (a kernel may fetch and mask them).
  *   prefix_len  0 <= prefix_len <= min(kv_tokens, max_prefix_len); 0 = suffix-only attention.
  *   state       device float32 [state_dim] (NULL iff has_state_token == 0)
  *   noise       device float32 [horizon, action_dim]: x at t = 1

@@ -17,8 +17,9 @@
 // pair p, which is sent its rows of the other C - 1 partials and adds the C in range order.  No partials in global memory, no
 // merge launch.  (Owners that read the partials from the other CTAs instead of being sent them: 4.2 us per launch more.)
 //
-// Measured at 8 requests of 816 + 51 keys and 8 heads (C = 3), from the projection's end to the merged output: 15 us (split
-// ranges of the one-CTA kernel 21 us, their merge launch 8): operands 2 - 3, 1.2 - 2 per key tile, merge 4.7.  What bounds
+// Measured at 8 requests of 816 + 51 keys and 8 heads (C = 3), from the projection's end to the merged output: 11.3 us (with
+// arrivals that release at cluster scope 15; split ranges of the one-CTA kernel 21, their merge launch 8): operands 1.2 - 3, first
+// tile 2.9, 1.25 per further tile, merge and output 4.2.  What bounds
 // the merge is the way between SMs, 28 bytes per ns for one: a CTA sends (C - 1) / C of its 102 KB, in two pieces, the first
 // while the second is staged (in one piece 0.7 us per launch more; as bf16, half the bytes, the merge took 3.7; through
 // global memory, which all clusters share, 3 us more at 8 requests).

@@ -100,8 +100,8 @@ struct phyai_expert {
   __nv_bfloat16 *kr_st = nullptr, *vr_st = nullptr;   // [L][max 64 tokens worth of requests][Hkv][S][dh] suffix K / V per layer
   // Weight codes of single-tile calls: 0 = the bf16 images made at create (the other token counts need them as well), 1 = the
   // GEMM kernels decode blocks of codes.  The loop is bound by its chain of kernels, not by bytes, and the decode (about 1 us
-  // of shared-memory traffic) lies on it for every CTA that starts late: pi0 with e4m3 codes 5.09 ms with images, 5.76 with
-  // codes, 5.15 with codes in the QKV projection alone.
+  // of shared-memory traffic) lies on it for every CTA that starts late: pi0 with e4m3 codes 4.74 ms with images, 5.36 with
+  // codes.
   int use_w8_inkernel = 0;
   int use_b1_pair = 1;         // single-tile calls: projections on CTA pairs where they fit
   int b1_c[4] = {0, 0, 0, 0};  // cluster sizes of the QKV / O / gate-up / down projections (0 = choose)
@@ -550,8 +550,8 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   // (60 / 200 tokens, one-CTA kernel -> persistent pairs: 20 requests 10.93 -> 11.02 / 11.67 -> 11.46 ms, 64: 24.0 -> 23.6 / 25.5 ->
   // 25.3, 160: 56.7 -> 54.1 / 60.2 -> 58.2).  The choice goes by what the handle can hold, not by a call's lengths: those are on the
   // device, one graph per (batch, steps) serves them all, and a graph per choice would be captured in the middle of serving.
-  // (Ten-step loops with 816-token prefixes, handle for 2048 tokens against one for 816: 2 requests 8.48 / 8.52 ms, 4: 9.31 /
-  // 9.36, 8: 10.73 / 10.75, 16: 12.49 / 12.64.)
+  // (Ten-step loops with 816-token prefixes, handle for 2048 tokens against one for 816: 2 requests 7.60 / 7.55 ms, 4: 8.29 / 8.28,
+  // 8: 9.45 / 9.42, 16: 11.20 / 11.18.)
   const int pr_ranges = h->pair_ranges ? std::min(h->pair_ranges, attention_pair_max_ranges(d)) : (pair && h->q_tiles_pair ? attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len) : 1);
   const bool attn_pair = pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair &&
                          (h->cfg.max_prefix_len >= 256 || 2 * batch * (d.Hq / 4) >= attention_persist_pairs(d));

@@ -21,7 +21,8 @@
 //
 // Measured in the captured ten-step loops of the pi0 shape, against the one-CTA tile GEMMs and their norm launches (with the
 // pair attention's part): 4 requests of 816 tokens 11.3 -> 9.4 ms, 8: 12.9 -> 10.8, 64 ragged: 33.1 -> 29.9 (power-capped, SM
-// clock 1.73 GHz), 256: 119.6 -> 107.7 (1.55 GHz).
+// clock 1.73 GHz), 256: 119.6 -> 107.7 (1.55 GHz).  With cluster arrivals that do not release at cluster scope, shorter epilogues and the
+// persistent pair attention since: 8.3, 9.4, 28.0 (1.65 GHz), 100 (1.4 - 1.5 GHz).
 //
 // Roles: warps 0-3 issue the copies (k-step i by warp i % 4), warp 4 issues the MMAs (leader CTA), the 16 warps from 5
 // on are the epilogue (tensor-memory lane quarter = warp % 4).  Every wait is

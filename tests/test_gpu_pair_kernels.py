@@ -76,6 +76,31 @@ def test_attention_of_many_requests(head_dim, n_q, n_kv, batch, horizon, top):
     check(cfg, lens, 1, [*range(0, 18, 2), batch // 2, batch - 2, batch - 1])
 
 
+@pytest.mark.parametrize("head_dim,n_q,n_kv,batch", [(256, 8, 1, 45), (128, 8, 2, 60)])
+def test_rows_past_a_prefix_have_no_part_in_its_request(head_dim, n_q, n_kv, batch):
+    """The persistent kernel fetches whole blocks of 64 keys: what follows a prefix (every third request's cache is NaN or infinite, and so
+    are the rows behind the last one) leaves the other requests' actions as they are, to the bit."""
+    cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=batch, max_prefix_len=300, n_layers=2, horizon=12)
+    W = synth.make_weights(cfg, 53, std=0.05)
+    lens = [(1, 63, 64, 65, 130, 300, 0, 191)[b % 8] for b in range(batch)]
+    packed, cu = synth.pack_prefix_kv([synth.make_prefix_kv(cfg, 53, p, b) for b, p in enumerate(lens)])
+    packed = torch.cat([packed, torch.zeros_like(packed[:, :, :70])], dim=2)
+    dirty = packed.clone()
+    dirty[:, :, int(cu[-1]):] = float("nan")
+    for b in range(1, batch, 3):
+        dirty[:, :, cu[b]:cu[b + 1]] = float("nan") if b % 2 else float("inf")
+    states = torch.stack([synth.make_state(cfg, 53, b) for b in range(batch)]).cuda()
+    noise = torch.stack([synth.make_noise(cfg, 53, b) for b in range(batch)]).cuda()
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        clean = ex.denoise_batched(packed.cuda(), torch.from_numpy(cu).cuda(), states, noise, 2).clone()
+        out = ex.denoise_batched(dirty.cuda(), torch.from_numpy(cu).cuda(), states, noise, 2)
+        torch.cuda.synchronize()
+        assert ex.poll_status() == 0 and clean.isfinite().all()
+    for b in range(batch):
+        if b % 3 != 1 or lens[b] == 0:
+            assert torch.equal(out[b], clean[b]), (b, lens[b])
+
+
 @pytest.mark.parametrize("horizon", [59, 60, 62, 63])
 @pytest.mark.parametrize("ranges", [2, 3, 4])
 def test_pair_attention_at_the_most_suffix_rows(ranges, horizon):
