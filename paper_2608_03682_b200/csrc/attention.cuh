@@ -93,6 +93,79 @@ __device__ __forceinline__ void group_sync() {
   asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
 }
 
+// the two warps that share the rows of a tensor-memory lane quarter (named barriers 4 to 7)
+__device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
+
+// Softmax of a tile of 128 keys in the kernels on CTA pairs.  Two threads per row (its two warps: lane quarter q, column half g);
+// logits in tensor memory at `sb`, the thread's are columns [64 g, 64 g + 64), of which the first `nvis` are visible; P = 2^(S - m)
+// goes over them as bf16 pairs, 32 columns per half.  m: running maximum (log2 units) of the row, l: sum over this thread's
+// columns, acc: the accumulator's rows of this warp.  `prev_done` returns once every P V so far has completed.  Without
+// `effect` nothing is written (a rehearsal of the code).
+//
+// P of the two halves is published by half, and the product of the first 64 keys starts with the first half alone, over all
+// channels of the accumulator.  So the warps of a quarter, which rescale half of the channels each and take that branch
+// together (same maxima), meet at its end: no half is published while the other one still rescales.
+constexpr float PAIR_RESCALE = 8.0f;          // log2 units by which a maximum grows before the accumulator is rescaled
+template <int DH, typename PrevDone>
+__device__ __forceinline__ void pair_softmax_tile(float& m, float& l, float (*xch)[128], uint32_t sb, uint32_t acc, int g, int q, int row, int nvis,
+                                                  bool effect, PrevDone prev_done) {
+  float s[64];
+  tmem_ld64(sb + (uint32_t)(g * 64), s);
+  if (nvis < 64) {
+#pragma unroll
+    for (int c = 0; c < 64; ++c) s[c] = c < nvis ? s[c] : -INFINITY;
+  }
+  float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int c = 0; c < 64; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], s[c]);
+  xch[g][row] = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+  quarter_sync(q);                            // (also: both halves of these S rows have been read -> P may overwrite them)
+  const float mx = fmaxf(xch[0][row], xch[1][row]) * LOG2E;
+  // keep the old maximum unless the new one exceeds it by more than the threshold (exact algebra, no rescaling)
+  float m_new = m;
+  if (mx > m + PAIR_RESCALE || m == -INFINITY) m_new = fmaxf(m, mx);
+  const bool rescale = m_new != m && m != -INFINITY;
+  const float corr = rescale ? exp2f(m - m_new) : 1.0f;
+  const float nsub = m_new == -INFINITY ? 0.f : -m_new;
+  float rs4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int c16 = 0; c16 < 2; ++c16) {
+    uint32_t w[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const int c = c16 * 32 + 2 * e;
+      const float e0 = ex2_fast(fmaf(s[c], LOG2E, nsub)), e1 = ex2_fast(fmaf(s[c + 1], LOG2E, nsub));
+      rs4[e & 3] += e0 + e1;
+      w[e] = pack_bf16(e0, e1);
+    }
+    if (effect) tmem_st16u(sb + (uint32_t)(g * 32 + c16 * 16), w);
+  }
+  if (__any_sync(0xffffffffu, rescale)) {     // rare: rescale this warp's half rows of the accumulator
+    prev_done();
+    __syncwarp();
+    tc_fence_after();
+#pragma unroll 1
+    for (int c = g * (DH / 2); c < (g + 1) * (DH / 2); c += 16) {
+      float o[16];
+      tmem_ld16(acc + (uint32_t)c, o);
+#pragma unroll
+      for (int e = 0; e < 16; ++e) o[e] *= corr;
+      tmem_st16(acc + (uint32_t)c, o);
+    }
+    tmem_st_wait();
+    tc_fence_before();
+    quarter_sync(q);
+    tc_fence_after();
+  }
+  tmem_st_wait();
+  tc_fence_before();
+  __syncwarp();
+  if (effect) {
+    l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
+    m = m_new;
+  }
+}
+
 // One attention role: the suffix rows of HPC query heads (head group `hgrp`) of request `b` against
 // key tiles [T*split/num_splits, T*(split+1)/num_splits).  Executed by HPC*128 threads (`tid` is the
 // thread's index within that group) that synchronise on named barrier BAR.  DH: head_dim; NBUF: K/V

@@ -38,7 +38,6 @@ namespace {
 constexpr int KB = 128;                       // keys per tile
 constexpr int AP_THREADS = 13 * 32;
 constexpr int BAR_ROWS = 1, BAR_K = 2, BAR_V = 3;
-constexpr float RESCALE_THRESHOLD = 8.0f;     // log2 units
 
 template <int DH, int C>
 struct ApLayout {
@@ -60,9 +59,6 @@ struct ApLayout {
   static constexpr size_t SMEM = 1024 + (size_t)(RECV + PEERS > KV + QTILE ? RECV + PEERS : KV + QTILE);
   static_assert(SMEM + 3072 <= 227 * 1024, "partials exceed the shared memory");
 };
-
-// the two warps that share the rows of a tensor-memory lane quarter
-__device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
 
 template <int DH, int C>
 __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, const __grid_constant__ CUtensorMap tmq) {
@@ -284,7 +280,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, c
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
     const bool causal_row = d.block_causal && d.ns && i == 0;
     const uint32_t pfull0 = map_rank(smem_u32(&p_full[0][g]), lead_rank);
-    float m = -INFINITY, l = 0.f;             // running maximum (log2 units) and sum
+    float m = -INFINITY, l = 0.f;             // running maximum (log2 units) and sum (of this thread's half of the columns)
     pdl_wait();
     if (T > 0 && lane == 0) {
       // Q (rotated, scaled) was written by the QKV projection as this CTA's operand tile: an eighth per warp (the copies of
@@ -310,57 +306,10 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, c
       // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
       int nvis = t >= m0 && t < m0 + n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - (t - m0) * KB) : KB;
       nvis -= g * 64;
-      float s[64];
-      tmem_ld64(sb + (uint32_t)(g * 64), s);
-      if (nvis < 64) {
-#pragma unroll
-        for (int c = 0; c < 64; ++c) s[c] = c < nvis ? s[c] : -INFINITY;
-      }
-      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-      for (int c = 0; c < 64; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], s[c]);
-      xch[t & 1][g][row] = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-      quarter_sync(q);                        // (also: both halves of these S rows have been read -> P may overwrite them)
-      const float mx = fmaxf(xch[t & 1][0][row], xch[t & 1][1][row]) * LOG2E;
-      // keep the old maximum unless the new one exceeds it by more than the threshold (exact algebra, no rescaling)
-      float m_new = m;
-      if (mx > m + RESCALE_THRESHOLD || m == -INFINITY) m_new = fmaxf(m, mx);
-      const bool rescale = m_new != m && m != -INFINITY;
-      const float corr = rescale ? exp2f(m - m_new) : 1.0f;
-      const float nsub = m_new == -INFINITY ? 0.f : -m_new;
-      float rs4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int c16 = 0; c16 < 2; ++c16) {
-        uint32_t w[16];
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const int c = c16 * 32 + 2 * e;
-          const float e0 = ex2_fast(fmaf(s[c], LOG2E, nsub)), e1 = ex2_fast(fmaf(s[c + 1], LOG2E, nsub));
-          rs4[e & 3] += e0 + e1;
-          w[e] = pack_bf16(e0, e1);
-        }
-        if (t >= 0) tmem_st16u(sb + (uint32_t)(g * 32 + c16 * 16), w);
-      }
-      if (__any_sync(0xffffffffu, rescale)) {     // rare: rescale this warp's half rows of the accumulator
-        if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(t - 1) & 1]), (uint32_t)((t - 1) >> 1) & 1u, wc);   // every P V so far
-        __syncwarp();
-        tc_fence_after();
-#pragma unroll 1
-        for (int c = g * (DH / 2); c < (g + 1) * (DH / 2); c += 16) {
-          float o[16];
-          tmem_ld16(tmem_o + lane_addr + (uint32_t)c, o);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) o[e] *= corr;
-          tmem_st16(tmem_o + lane_addr + (uint32_t)c, o);
-        }
-      }
-      tmem_st_wait();
-      tc_fence_before();
-      __syncwarp();
-      if (t < 0) continue;
-      if (lane == 0) remote_arrive(pfull0 + (uint32_t)(t & 1) * 16u);
-      l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);      // (of this thread's half of the columns)
-      m = m_new;
+      pair_softmax_tile<DH>(m, l, xch[t & 1], sb, tmem_o + lane_addr, g, q, row, nvis, t >= 0, [&] {
+        if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(t - 1) & 1]), (uint32_t)((t - 1) >> 1) & 1u, wc);
+      });
+      if (t >= 0 && lane == 0) remote_arrive(pfull0 + (uint32_t)(t & 1) * 16u);
     }
     if (T == 0) cluster_arrive_relaxed();
     xch[T & 1][g][row] = l;

@@ -34,7 +34,6 @@ namespace {
 
 constexpr int KB = 128;                       // keys per tile: two blocks of 64
 constexpr int AS_THREADS = 12 * 32;
-constexpr float RESCALE_THRESHOLD = 8.0f;     // log2 units
 
 template <int DH>
 struct AsLayout {
@@ -328,65 +327,16 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
         // mask sees only the first
         const int blk = 2 * t + g;
         const int nvis = blk < it.nsp ? it.P - blk * 64 : blk == it.nsp ? (causal_row ? 1 : S) : 0;
-        float s[64];
-        tmem_ld64(sb + (uint32_t)(g * 64), s);
-        if (nvis < 64) {
-#pragma unroll
-          for (int c = 0; c < 64; ++c) s[c] = c < nvis ? s[c] : -INFINITY;
-        }
-        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-        for (int c = 0; c < 64; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], s[c]);
-        xch[n & 1][g][row] = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-        // the two warps of a lane quarter (also: both halves of these S rows have been read -> P may overwrite them)
-        asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory");
-        const float mx = fmaxf(xch[n & 1][0][row], xch[n & 1][1][row]) * LOG2E;
-        // keep the old maximum unless the new one exceeds it by more than the threshold (exact algebra, no rescaling)
-        float m_new = m;
-        if (mx > m + RESCALE_THRESHOLD || m == -INFINITY) m_new = fmaxf(m, mx);
-        const bool rescale = m_new != m && m != -INFINITY;
-        const float corr = rescale ? exp2f(m - m_new) : 1.0f;
-        const float nsub = m_new == -INFINITY ? 0.f : -m_new;
-        float rs4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int c16 = 0; c16 < 2; ++c16) {
-          uint32_t w[16];
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const int c = c16 * 32 + 2 * e;
-            const float e0 = ex2_fast(fmaf(s[c], LOG2E, nsub)), e1 = ex2_fast(fmaf(s[c + 1], LOG2E, nsub));
-            rs4[e & 3] += e0 + e1;
-            w[e] = pack_bf16(e0, e1);
-          }
-          if (!rehearsal) tmem_st16u(sb + (uint32_t)(g * 32 + c16 * 16), w);
-        }
-        if (__any_sync(0xffffffffu, rescale)) {     // rare: rescale this warp's half rows of the accumulator
-          if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(n - 1) & 1]), (uint32_t)((n - 1) >> 1) & 1u, wc);   // every P V so far
-          __syncwarp();
-          tc_fence_after();
-#pragma unroll 1
-          for (int c = g * (DH / 2); c < (g + 1) * (DH / 2); c += 16) {
-            float o[16];
-            tmem_ld16(tmem_o + lane_addr + (uint32_t)c, o);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) o[e] *= corr;
-            tmem_st16(tmem_o + lane_addr + (uint32_t)c, o);
-          }
-        }
-        tmem_st_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (!rehearsal) {
-          if (lane == 0) remote_arrive(pfull0 + (uint32_t)(n & 1) * 16u);
-          l = l * corr + (rs4[0] + rs4[1]) + (rs4[2] + rs4[3]);
-          m = m_new;
-        }
+        pair_softmax_tile<DH>(m, l, xch[n & 1], sb, tmem_o + lane_addr, g, q, row, nvis, !rehearsal, [&] {
+          if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(n - 1) & 1]), (uint32_t)((n - 1) >> 1) & 1u, wc);
+        });
+        if (!rehearsal && lane == 0) remote_arrive(pfull0 + (uint32_t)(n & 1) * 16u);
       }
       if ((t == 0 && k > 0) || rehearsal) {
         // ---- the item before: O / l -> bf16, 32 columns at a time through a staging block of the warp, out with coalesced stores
         // (tiled: the chunk's place as staged; row-major, for the operator: the swizzle undone)
         xsum[g][row] = l_prev;
-        asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory");
+        quarter_sync(q);
         const float inv = 1.0f / (xsum[0][row] + xsum[1][row]);
         if (lane == 0 && !rehearsal) mbar_wait_drain(smem_u32(&pv_done[(n - 1) & 1]), (uint32_t)((n - 1) >> 1) & 1u, wc);
         __syncwarp();

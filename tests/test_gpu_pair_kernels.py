@@ -1,6 +1,7 @@
 """The kernels on CTA pairs (calls of more than 64 suffix tokens) against the oracle, at the edges of their tiles: token
 counts around the 32-token steps of the tile width, one and several tiles per pair, every key-range split of the attention
 kernel, prefixes with no full key tile, exactly one, and empty ranges; reproducible to the bit."""
+import numpy as np
 import pytest
 import torch
 
@@ -132,6 +133,42 @@ def test_attention_operator_on_the_pair_kernel(n_kv, head_dim, suffix, lens):
     assert int(status.item()) == 0
     ref = oracle_attention(qkv, kv, cu, 8, n_kv, head_dim, suffix, 1, 10000.0)
     assert abs(out.double().cpu().numpy() - ref).max() <= 2e-2 * abs(ref).max()
+
+
+@pytest.mark.parametrize("n_q,n_kv,head_dim,suffix,lens", [
+    (8, 1, 256, 51, [816, 400, 130]), (8, 2, 128, 17, [700, 64, 1, 513, 250]), (8, 1, 256, 51, [(97 * b) % 900 for b in range(8)]),
+    (8, 1, 256, 33, [600 + 13 * b for b in range(14)]),
+    (4, 1, 256, 51, [(67 * b) % 500 for b in range(100)] + [(5 * b) % 65 for b in range(60)]), (8, 2, 128, 64, [(41 * b) % 420 for b in range(90)])])
+def test_logits_that_grow_over_the_keys(n_q, n_kv, head_dim, suffix, lens):
+    """Half of the rows see logits that grow by 11.5 (log2) with every 64 keys, up to the request's own: their accumulators are rescaled in
+    every tile, beside rows that keep theirs.  Split key ranges, and several items per pair with prefixes of less than a tile last."""
+    from tests.test_gpu_attention_op import oracle_attention
+    rng = np.random.default_rng(12)
+    B, T, scale = len(lens), sum(lens), head_dim ** -0.5
+    u = rng.choice([-1.0, 1.0], head_dim)
+    level = np.concatenate([8.0 * (np.arange(p) // 64) for p in lens])
+    kv = rng.standard_normal((1, 2, T, n_kv, head_dim))
+    kv[0, 0] += level[:, None, None] * u
+    qkv = rng.standard_normal((B * suffix, n_q + 2 * n_kv, head_dim))
+    qkv[:, :n_q] = rng.choice([-1.0, 1.0], (B * suffix, n_q, 1)) * u / (head_dim * scale)    # (scaled: exact in bf16; logit = +-level + noise)
+    qkv[:, n_q:n_q + n_kv] += np.repeat([8.0 * ((p + 63) // 64) for p in lens], suffix)[:, None, None] * u
+    kv = torch.from_numpy(kv).bfloat16()
+    qkv = torch.from_numpy(qkv.reshape(B * suffix, -1)).float()
+    qkv[:, n_q * head_dim:] = qkv[:, n_q * head_dim:].bfloat16().float()
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    desc = binding.attention_desc(n_q, n_kv, head_dim, suffix, n_layers=1, layer=0)
+    args = (desc, qkv.cuda(), kv.cuda(), torch.from_numpy(cu).cuda(), None)
+    outs = [binding.suffix_attention(*args) for _ in range(8)]
+    torch.cuda.synchronize()
+    for out, status in outs:
+        assert int(status.item()) == 0 and torch.equal(out, outs[0][0])
+    ref = oracle_attention(qkv, kv, cu, n_q, n_kv, head_dim, suffix, 0, 0.0)
+    qkv[:, (n_q + n_kv) * head_dim:].abs_(), kv[:, 1].abs_()
+    mean_abs = oracle_attention(qkv, kv, cu, n_q, n_kv, head_dim, suffix, 0, 0.0)
+    # P: one bf16 rounding (2^-9); logits of at most 2^7 in 16 truncated accumulations (2^-16 each, in product and sum: 2^-11); the result: one
+    # bf16 rounding
+    bound = mean_abs * 2.0 ** -8 + np.abs(ref) * 2.0 ** -8
+    assert (np.abs(outs[0][0].double().cpu().numpy() - ref) <= bound).all(), (np.abs(outs[0][0].double().cpu().numpy() - ref) / bound).max()
 
 
 @pytest.mark.parametrize("tokens,n_kv,dh,layers,shift", [(1, 1, 64, 3, 0), (65, 3, 64, 1, 4), (641, 1, 128, 5, 0), (200, 1, 192, 2, 4)])
