@@ -73,7 +73,9 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
   __shared__ __align__(8) uint64_t k_full[2], v_full[2], p_full[2][2], q_full, o_free, s_full[2], pv_done[2], q_free, v_own;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  __shared__ float xch[2][2][128], xsum[2][128];   // the two half-row threads of a row: maximum (by tile parity), sum of an item
+  // what the two half-row threads of a row exchange: maximum (by tile parity), sum of an item (by item parity: after a last item of one
+  // tile two outputs follow one another with no barrier between the reading of one's sums and the writing of the other's)
+  __shared__ float xch[2][2][128], xsum[2][2][128];
 
   const Dims& d = a.d;
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
@@ -335,9 +337,9 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
       if ((t == 0 && k > 0) || rehearsal) {
         // ---- the item before: O / l -> bf16, 32 columns at a time through a staging block of the warp, out with coalesced stores
         // (tiled: the chunk's place as staged; row-major, for the operator: the swizzle undone)
-        xsum[g][row] = l_prev;
+        xsum[k & 1][g][row] = l_prev;
         quarter_sync(q);
-        const float inv = 1.0f / (xsum[0][row] + xsum[1][row]);
+        const float inv = 1.0f / (xsum[k & 1][0][row] + xsum[k & 1][1][row]);
         if (lane == 0 && !rehearsal) mbar_wait_drain(smem_u32(&pv_done[(n - 1) & 1]), (uint32_t)((n - 1) >> 1) & 1u, wc);
         __syncwarp();
         tc_fence_after();

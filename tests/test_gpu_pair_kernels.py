@@ -171,6 +171,26 @@ def test_logits_that_grow_over_the_keys(n_q, n_kv, head_dim, suffix, lens):
     assert (np.abs(outs[0][0].double().cpu().numpy() - ref) <= bound).all(), (np.abs(outs[0][0].double().cpu().numpy() - ref) / bound).max()
 
 
+@pytest.mark.parametrize("head_dim,n_kv,batch", [(256, 1, 150), (128, 1, 150), (256, 1, 301)])
+def test_items_of_one_tile_at_the_end_of_a_pairs_list(head_dim, n_kv, batch):
+    """The last two or three items of a pair are a long prefix and ones of a single tile: their outputs follow one another without a
+    softmax in between.  Zero queries: every sum is the number of keys, 17 to 81 in the last items and 400 and more in those before."""
+    from tests.test_gpu_attention_op import make_case, oracle_attention
+    lens = [400 + b % 60 if b < batch // 2 else (b * 5) % 65 for b in range(batch)]
+    qkv, kv, cu, _ = make_case(13, 4, n_kv, head_dim, 17, lens, theta=0.0)
+    qkv[:, :4 * head_dim] = 0.0
+    qkv[:, 4 * head_dim:] = qkv[:, 4 * head_dim:].bfloat16().float()
+    desc = binding.attention_desc(4, n_kv, head_dim, 17, n_layers=2, layer=1)
+    args = (desc, qkv.cuda(), kv.cuda(), torch.from_numpy(cu).cuda(), None)
+    outs = [binding.suffix_attention(*args) for _ in range(8)]
+    torch.cuda.synchronize()
+    for out, status in outs:
+        assert int(status.item()) == 0 and torch.equal(out, outs[0][0])
+    ref = oracle_attention(qkv, kv, cu, 4, n_kv, head_dim, 17, 1, 0.0)
+    # (P is exactly 1; at most 36 truncated additions of at most 2^9 x 4: 2^-12 each, over at least 17 keys; one bf16 rounding)
+    assert (np.abs(outs[0][0].double().cpu().numpy() - ref) <= np.abs(ref) * 2.0 ** -8 + 36 * 2.0 ** -12 / 17).all()
+
+
 @pytest.mark.parametrize("tokens,n_kv,dh,layers,shift", [(1, 1, 64, 3, 0), (65, 3, 64, 1, 4), (641, 1, 128, 5, 0), (200, 1, 192, 2, 4)])
 def test_feature_projection_of_all_layers(tokens, n_kv, dh, layers, shift):
     """Row counts that leave the last 256 padded, warps whose 32 rows end a plane, planes at an 8-byte-aligned address."""
