@@ -323,8 +323,13 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
   const size_t q_elems = (size_t)batch * (d.Hq / 2) * 128 * d.dh, kv_elems = (size_t)batch * d.Hkv * d.S * d.dh;
   const size_t tc_need = sizeof(Request) + (q_elems + 2 * kv_elems) * 2;
   // (a given scratch that cannot hold the operands leaves the call to the mma.sync kernel, which reads the fp32 rows itself)
-  bool tc = splits == 0 && !((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(qkv)) & 15u) && kv_tokens > 0 &&
-            attention_pair_supported(d) && (!scratch || tc_need <= scratch_bytes);
+  const bool tc_form = splits == 0 && !((reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(qkv)) & 15u) && kv_tokens > 0 &&
+                       attention_pair_supported(d) && (!scratch || tc_need <= scratch_bytes);
+  // One wave of clusters of eight (15 on a B200), else CTA pairs with fewer key ranges, which read the cache through a tensor map; a
+  // device that holds neither at a time leaves the call to the mma.sync kernel as well.
+  const bool b1 = tc_form && attention_b1_ctas(d, (int)batch, 1) <= attention_b1_resident_ctas(d);
+  const int ranges = tc_form && !b1 ? attention_pair_ranges(d, (int)batch, (int)(kv_tokens / batch)) : 0;
+  bool tc = b1 || ranges > 0;
   if (splits == 0) splits = attention_pick_splits(d, (int)batch, (int)(kv_tokens < 4096 ? kv_tokens : 4096));
   const size_t mma_need = attention_scratch_floats(d, (int)batch, splits) * sizeof(float);
   size_t need = tc ? tc_need : mma_need;
@@ -348,8 +353,6 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     __nv_bfloat16 *qt = reinterpret_cast<__nv_bfloat16*>(rq + 1), *kr = qt + q_elems, *vr = kr + kv_elems;
     Request r{};
     r.prefix_kv = prefix_kv, r.kv_tokens = kv_tokens, r.cu_lens = cu, r.batch = (int)batch;
-    // One wave of clusters of eight (15 on a B200), else CTA pairs with fewer key ranges, which read the cache through a tensor map.
-    const bool b1 = attention_b1_ctas(d, (int)batch, 1) <= attention_b1_resident_ctas(d);
     if (!b1 && !prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) {
       k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
@@ -359,8 +362,7 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
       if (b1)
         e = launch_attention_b1_op(prefix_kv, kv_tokens, cu, status_word, qt, kr, vr, a.layer, a.out, d, (int)batch, a.wait_limit, st);
       else
-        e = launch_attention_pair(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch,
-                                  attention_pair_ranges(d, (int)batch, (int)(kv_tokens / batch)), nullptr, a.wait_limit, st, nullptr, false);
+        e = launch_attention_pair(rq, status_word, qt, kr, vr, a.layer, a.out, 0, d, (int)batch, ranges, nullptr, a.wait_limit, st, nullptr, false);
     }
   } else {
     if (splits > 1) {

@@ -29,13 +29,14 @@
 // (leader CTA), 5-12 fetch Q, softmax, correction, output.  Every wait is bounded; after a give-up the protocol runs to its
 // end and only the global stores are skipped.
 #include "attention.cuh"
+#include "attention_choice.h"
 #include "tc.cuh"
 #include "tc_pair.cuh"
 
 namespace phyai {
 namespace {
 
-constexpr int KB = 128;                       // keys per tile
+constexpr int KB = PAIR_TILE;                 // keys per tile
 constexpr int AP_THREADS = 13 * 32;
 constexpr int BAR_ROWS = 1, BAR_K = 2, BAR_V = 3;
 
@@ -503,23 +504,21 @@ int attention_pair_max_ranges(const Dims& d) {
   return d.dh != 256 || d.S <= ApLayout<256, 4>::S_MAX ? 4 : (d.S <= ApLayout<256, 3>::S_MAX ? 3 : 2);
 }
 
-// Key ranges per request: 1 to 4, the least of waves x (fixed cost + tiles of a range), in tiles of 128 keys.  How many
-// clusters of 2 C CTAs the device holds at a time decides the waves (a cluster of 8 needs 8 free SMs in one GPC: 15 on a
-// B200, not 18).  One range: the persistent kernel.  Against every other choice, ten-step loops of 4 / 8 / 12 / 16 / 20 requests:
-// chosen 8.79 / 10.02 / 11.04 / 11.67 / 12.44 ms with 816-token prefixes (best 8.78 / 9.98 / 11.04 / 11.63 / 12.44), 8.50 / 9.30 /
-// 10.29 / 10.94 / 11.69 with 400 (best 8.43 / 9.30 / 10.28 / 10.91 / 11.69).
+// clusters of `ranges` pairs that are resident at a time; <= 0: none
+int attention_pair_resident(const Dims& d, int ranges) {
+  static PerDeviceCount resident[2][MAX_PAIR_RANGES + 1];
+  if (ranges == 1) return attention_persist_pairs(d);
+  return resident[d.dh == 256 ? 1 : 0][ranges].get([&] { return max_clusters(d.dh, ranges); });
+}
+
+// Key ranges per request (see choose_pair_ranges), 0 if no kernel on pairs can run.  A cluster of 8 CTAs needs 8 free SMs in one
+// GPC: 15 on a B200, not 18.  One range: the persistent kernel.  Against every other choice, ten-step loops of 4 / 8 / 12 / 16 / 20
+// requests: chosen 8.79 / 10.02 / 11.04 / 11.67 / 12.44 ms with 816-token prefixes (best 8.78 / 9.98 / 11.04 / 11.63 / 12.44), 8.50 /
+// 9.30 / 10.29 / 10.94 / 11.69 with 400 (best 8.43 / 9.30 / 10.28 / 10.91 / 11.69).
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
-  static PerDeviceCount resident[2][5];
-  const int dh = d.dh == 256 ? 1 : 0, items = batch * (d.Hq / 4);
-  int best_c = 1;
-  double best = 1e30;
-  for (int c = 1; c <= 4; ++c) {
-    const int n = c == 1 ? attention_persist_pairs(d) : resident[dh][c].get([&] { return max_clusters(d.dh, c); });
-    if (n <= 0 || c > attention_pair_max_ranges(d)) continue;
-    const double cost = (double)((items + n - 1) / n) * ((c > 1 ? 5.5 : 4.0) + (max_prefix + d.S + c * KB - 1) / (c * KB));
-    if (cost < best) best = cost, best_c = c;
-  }
-  return best_c;
+  int resident[MAX_PAIR_RANGES + 1] = {};
+  for (int c = 1; c <= MAX_PAIR_RANGES; ++c) resident[c] = attention_pair_resident(d, c);
+  return choose_pair_ranges(resident, batch * (d.Hq / 4), max_prefix + d.S, attention_pair_max_ranges(d));
 }
 
 cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,

@@ -552,9 +552,13 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   // device, one graph per (batch, steps) serves them all, and a graph per choice would be captured in the middle of serving.
   // (Ten-step loops with 816-token prefixes, handle for 2048 tokens against one for 816: 2 requests 7.60 / 7.55 ms, 4: 8.29 / 8.28,
   // 8: 9.45 / 9.42, 16: 11.20 / 11.18.)
-  const int pr_ranges = h->pair_ranges ? std::min(h->pair_ranges, attention_pair_max_ranges(d)) : (pair && h->q_tiles_pair ? attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len) : 1);
-  const bool attn_pair = pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair &&
-                         (h->cfg.max_prefix_len >= 256 || 2 * batch * (d.Hq / 4) >= attention_persist_pairs(d));
+  // (A device that holds no cluster of a form at a time: no choice of that form, and none at all, the kernels without clusters.)
+  int pr_ranges = 0;
+  if (pair && h->use_pair_attention && h->use_tc_attention && h->q_tiles_pair) {
+    pr_ranges = h->pair_ranges ? std::min(h->pair_ranges, attention_pair_max_ranges(d)) : attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len);
+    if (pr_ranges > 0 && attention_pair_resident(d, pr_ranges) <= 0) pr_ranges = 0;
+  }
+  const bool attn_pair = pr_ranges > 0 && (h->cfg.max_prefix_len >= 256 || 2 * batch * (d.Hq / 4) >= attention_persist_pairs(d));
   auto attention_rot = [&](int l) -> phyai_status_t {   // from rotated bf16 q / k / v to the output projection's operand
     cudaError_t e;
     const bool tr1 = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from;

@@ -37,7 +37,10 @@ struct PerDeviceCount {
     int v = n[dev].load(std::memory_order_acquire);
     if (v == 0) {
       v = ask();
-      if (v == 0) v = -1;
+      if (v <= 0) {
+        v = -1;
+        cudaGetLastError();      // (the answer is no: not an error of the call that asked)
+      }
       n[dev].store(v, std::memory_order_release);
     }
     return v;
@@ -257,6 +260,7 @@ cudaError_t launch_attention_persist(const Request* rq, int* status, const __nv_
 bool attention_pair_supported(const Dims& d);
 bool prefix_kv_map(unsigned char* map, const void* kv, uint64_t kv_tokens, const Dims& d);   // fills Request::kv_map
 int attention_pair_max_ranges(const Dims& d);
+int attention_pair_resident(const Dims& d, int ranges);
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix);
 cudaError_t launch_attention_pair(const Request* rq, int* status, const __nv_bfloat16* q_tiles, const __nv_bfloat16* kr,
                                   const __nv_bfloat16* vr, int layer, __nv_bfloat16* out_tiled, int rows_pad, const Dims& d, int batch,
