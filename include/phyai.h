@@ -146,7 +146,7 @@ size_t phyai_prefix_kv_bytes(const phyai_expert_config_t *cfg, uint64_t total_pr
  *   prefix_kv   device, layout [n_layers][2 (K,V)][kv_tokens][n_kv_heads][head_dim], head_dim
  *               contiguous, float32 for PHYAI_F32 else bfloat16, 16-byte aligned; K is used as
  *               given (already rotated by the producer).  kv_tokens is the token capacity of the
- *               buffer (>= prefix_len); rows >= prefix_len have no part in a result (a kernel may fetch and mask them).
+ *               buffer (>= prefix_len); rows >= prefix_len are never read.
  *   prefix_len  0 <= prefix_len <= min(kv_tokens, max_prefix_len); 0 = suffix-only attention.
  *   state       device float32 [state_dim] (NULL iff has_state_token == 0)
  *   noise       device float32 [horizon, action_dim]: x at t = 1
@@ -170,6 +170,8 @@ phyai_status_t phyai_denoise(phyai_expert_t *h, const void *prefix_kv, uint64_t 
  *
  *   batch           1 <= batch <= max_batch
  *   prefix_kv       device, [n_layers][2][kv_tokens][n_kv_heads][head_dim]
+ *                   Rows >= cu[batch] are never read; of a cache with cu[0] > 0, up to 63 rows before cu[0] may be fetched
+ *                   (with a first prefix of fewer than 64 tokens), and have no part in a result.
  *   cu_prefix_lens  device int32 [batch+1], non-decreasing, cu[0] >= 0, cu[batch] <= kv_tokens,
  *                   every difference <= max_prefix_len (checked on the device: a violation sets
  *                   the status word to INVALID_ARG and the call writes nothing)

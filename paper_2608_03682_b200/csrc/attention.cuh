@@ -97,7 +97,7 @@ __device__ __forceinline__ void group_sync() {
 __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0, 64;" ::"r"(4 + q) : "memory"); }
 
 // Softmax of a tile of 128 keys in the kernels on CTA pairs.  Two threads per row (its two warps: lane quarter q, column half g);
-// logits in tensor memory at `sb`, the thread's are columns [64 g, 64 g + 64), of which the first `nvis` are visible; P = 2^(S - m)
+// logits in tensor memory at `sb`, the thread's are columns [64 g, 64 g + 64), visible those with a bit in `vis`; P = 2^(S - m)
 // goes over them as bf16 pairs, 32 columns per half.  m: running maximum (log2 units) of the row, l: sum over this thread's
 // columns, acc: the accumulator's rows of this warp.  `prev_done` returns once every P V so far has completed.  Without
 // `effect` nothing is written (a rehearsal of the code).
@@ -107,13 +107,14 @@ __device__ __forceinline__ void quarter_sync(int q) { asm volatile("bar.sync %0,
 // together (same maxima), meet at its end: no half is published while the other one still rescales.
 constexpr float PAIR_RESCALE = 8.0f;          // log2 units by which a maximum grows before the accumulator is rescaled
 template <int DH, typename PrevDone>
-__device__ __forceinline__ void pair_softmax_tile(float& m, float& l, float (*xch)[128], uint32_t sb, uint32_t acc, int g, int q, int row, int nvis,
+__device__ __forceinline__ void pair_softmax_tile(float& m, float& l, float (*xch)[128], uint32_t sb, uint32_t acc, int g, int q, int row, uint64_t vis,
                                                   bool effect, PrevDone prev_done) {
   float s[64];
   tmem_ld64(sb + (uint32_t)(g * 64), s);
-  if (nvis < 64) {
+  const uint32_t v0 = (uint32_t)vis, v1 = (uint32_t)(vis >> 32);
+  if (~(v0 & v1)) {        // (one instruction tests a bit; two bounds take two, in code that is fetched cold: 1 % of a loop of 16 requests)
 #pragma unroll
-    for (int c = 0; c < 64; ++c) s[c] = c < nvis ? s[c] : -INFINITY;
+    for (int c = 0; c < 64; ++c) s[c] = ((c < 32 ? v0 : v1) >> (c & 31)) & 1u ? s[c] : -INFINITY;
   }
   float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll

@@ -1,7 +1,30 @@
-// Which attention kernel on CTA pairs serves a call, from what the host knows of it (no device code).
+// Attention on CTA pairs, what needs no GPU: which kernel serves a call, which rows of the cache a block of keys is fetched from.
 #pragma once
 
+#include <cstdint>
+
+#ifdef __CUDACC__
+#define PHYAI_HOST_DEVICE __host__ __device__ __forceinline__
+#else
+#define PHYAI_HOST_DEVICE inline
+#endif
+
 namespace phyai {
+
+// the first n columns of 64, a bit each (n below 0 as 0, above 64 as 64)
+PHYAI_HOST_DEVICE uint64_t first_columns(int n) { return n <= 0 ? 0 : ~0ull >> (n < 64 ? 64 - n : 0); }
+
+// Block `sb` of the (P + 63) / 64 blocks of a prefix of P keys: 64 rows of the cache from the prefix's row `row` on, of which those
+// with a bit in `keys` are the block's keys.  A last block that is not full ends where the prefix ends, so that no row past it is
+// read: its first rows are keys of the block before it, or, of a prefix of fewer than 64 keys, what lies before the prefix (row < 0).
+struct PrefixBlock {
+  int row;
+  uint64_t keys;
+};
+PHYAI_HOST_DEVICE PrefixBlock prefix_block(int P, int sb) {
+  const int left = P - sb * 64;
+  return left >= 64 ? PrefixBlock{sb * 64, ~0ull} : PrefixBlock{P - 64, ~0ull << (64 - left)};
+}
 
 constexpr int MAX_PAIR_RANGES = 4;
 constexpr int PAIR_TILE = 128;      // keys per tile of the kernels on pairs

@@ -297,17 +297,17 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, c
     // has left the instruction caches by the next layer, and the first softmax took 3.4 us instead of 1.7.
     for (int t = T > 0 ? -1 : 0; t < T; ++t) {
       const uint32_t sb = tmem_s + (uint32_t)(t & 1) * KB + lane_addr;
+      // the visible keys of a row form a prefix of a mixed tile: the keys that exist, and for the state-token row under the
+      // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
+      const int nvis = t >= m0 && t < m0 + n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - (t - m0) * KB) : KB;
+      const uint64_t vis = first_columns(nvis - g * 64);
       if (t >= 0) {
         if (lane == 0) mbar_wait_drain(smem_u32(&s_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
         __syncwarp();
       }
       tc_fence_after();
       if (t >= 0 && t == T - 1) cluster_arrive_relaxed();     // (the last logits exist: Q is dead, its area may receive partials)
-      // the visible keys of a row form a prefix of a mixed tile: the keys that exist, and for the state-token row under the
-      // block-causal mask the prefix keys and its own key (suffix key 0, in the first range)
-      int nvis = t >= m0 && t < m0 + n_mix ? min(KB, (causal_row ? rem + (suf_lo == 0 && n_suf > 0 ? 1 : 0) : rem + n_suf) - (t - m0) * KB) : KB;
-      nvis -= g * 64;
-      pair_softmax_tile<DH>(m, l, xch[t & 1], sb, tmem_o + lane_addr, g, q, row, nvis, t >= 0, [&] {
+      pair_softmax_tile<DH>(m, l, xch[t & 1], sb, tmem_o + lane_addr, g, q, row, vis, t >= 0, [&] {
         if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(t - 1) & 1]), (uint32_t)((t - 1) >> 1) & 1u, wc);
       });
       if (t >= 0 && lane == 0) remote_arrive(pfull0 + (uint32_t)(t & 1) * 16u);

@@ -11,8 +11,9 @@
 //   O += P V    M = 256, N = head_dim, K = 128 keys; P is the tensor-memory A operand, V an MN-major B operand
 // A tile is two blocks of 64 keys.  The blocks of an item are its prefix (the last one possibly in part) and, at the end, the
 // request's own keys; all come by tensor-map copies.  K: block h of a tile belongs to CTA h of the pair (the tensor cores read the
-// other half of the tile from the peer); V: each CTA fetches its half of the channels of both blocks.  Rows past the end of the
-// prefix hold another request's keys and values: their logits are masked; their values are overwritten with zeros (0 x NaN).
+// other half of the tile from the peer); V: each CTA fetches its half of the channels of both blocks.  No row past the end of a
+// prefix is read: a partial last block is the 64 rows that end there, behind keys of the block before (or, of a prefix of fewer than
+// 64 keys, behind what lies before it): those rows' logits are masked, their values overwritten with zeros (0 x infinity, 0 x NaN).
 //
 // What bounds it is the tensor pipe (2048 clocks per tile of 128 keys) and, close behind, the chain logits -> softmax (MUFU: 1024
 // clocks) -> P V, which the second S buffer overlaps with the other products.
@@ -26,13 +27,14 @@
 // Warps of a CTA: 0 fetches K, 1 V, 2 Q, 3 issues the MMAs (leader CTA), 4-11 softmax, correction, output.  Every wait is
 // bounded; after a give-up the protocol runs to its end and only the global stores are skipped.
 #include "attention.cuh"
+#include "attention_choice.h"
 #include "tc.cuh"
 #include "tc_pair.cuh"
 
 namespace phyai {
 namespace {
 
-constexpr int KB = 128;                       // keys per tile: two blocks of 64
+constexpr int KB = PAIR_TILE;                 // keys per tile: two blocks of 64
 constexpr int AS_THREADS = 12 * 32;
 
 template <int DH>
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
           const void* map = own ? (const void*)&tmk : (const void*)a.rq->kv_map;
 #pragma unroll
           for (int u = 0; u < 2; ++u)
-            kv_copy(dst + (uint32_t)u * L::PIECE, map, own ? 0 : it.p0 + sb * 64, (own ? 0 : hk * (DH / 64)) + u * (DH / 128),
+            kv_copy(dst + (uint32_t)u * L::PIECE, map, own ? 0 : it.p0 + prefix_block(it.P, sb).row, (own ? 0 : hk * (DH / 64)) + u * (DH / 128),
                     own ? it.b * d.Hkv + hk : a.layer * 2, bar & LEADER_MASK);
         }
         it = nx;
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
       const int hk = it.group * 4 / (d.Hq / d.Hkv), rem = it.P & 63;
       for (int t = 0; t < it.T; ++t, ++n) {
         const int nb = min(2, it.nsp + 1 - 2 * t);                       // blocks of this tile
-        const int part = rem ? it.nsp - 1 - 2 * t : -1;                  // its block that ends with the prefix, if 0 or 1
+        const int part = rem ? it.nsp - 1 - 2 * t : -1;                  // its block that is not full, if 0 or 1
         const bool clear = part == 0 || part == 1;
         const uint32_t dst = Vs + (uint32_t)(n & 1) * L::TILE;
         if (lane == 0) {
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
             const int sb = 2 * t + u;
             const bool own = sb == it.nsp;
             if (own && !waited) pdl_wait(), waited = true;
-            kv_copy(dst + (uint32_t)u * L::PIECE, own ? (const void*)&tmv : (const void*)a.rq->kv_map, own ? 0 : it.p0 + sb * 64,
+            kv_copy(dst + (uint32_t)u * L::PIECE, own ? (const void*)&tmv : (const void*)a.rq->kv_map, own ? 0 : it.p0 + prefix_block(it.P, sb).row,
                     (own ? 0 : hk * (DH / 64)) + half * (DH / 128), own ? it.b * d.Hkv + hk : a.layer * 2 + 1, bar);
           }
           if (clear) mbar_wait_drain(bar, ph_own, wl);
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
           ph_own ^= 1u;
           const uint32_t z = dst + (uint32_t)part * L::PIECE;
           for (int i = lane; i < (64 - rem) * (DH / 16); i += 32) {      // (a row: 8 x 16 bytes in each of DH / 128 blocks)
-            const int row = rem + i / (DH / 16), c = i % (DH / 16);
+            const int row = i / (DH / 16), c = i % (DH / 16);
             asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(z + (uint32_t)((c >> 3) * L::KBLOCK + row * 128 + (c & 7) * 16)), "r"(0u) : "memory");
           }
           fence_async_smem();                    // generic-proxy writes, read next by the tensor cores
@@ -320,16 +322,16 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
     for (int k = 0, t = 0, n = 0;;) {
       if (k < n_my) {
         const uint32_t sb = tmem_s + (uint32_t)(n & 1) * KB + lane_addr;
+        // the visible keys of a block: its own of the prefix's; of the request's own keys the state-token row under the block-causal
+        // mask sees only the first
+        const int blk = 2 * t + g;
+        const uint64_t vis = blk < it.nsp ? prefix_block(it.P, blk).keys : blk == it.nsp ? first_columns(causal_row ? 1 : S) : 0;
         if (!rehearsal) {
           if (lane == 0) mbar_wait_drain(smem_u32(&s_full[n & 1]), (uint32_t)(n >> 1) & 1u, wc);
           __syncwarp();
         }
         tc_fence_after();
-        // the visible keys of a block: those that exist; of the request's own keys the state-token row under the block-causal
-        // mask sees only the first
-        const int blk = 2 * t + g;
-        const int nvis = blk < it.nsp ? it.P - blk * 64 : blk == it.nsp ? (causal_row ? 1 : S) : 0;
-        pair_softmax_tile<DH>(m, l, xch[n & 1], sb, tmem_o + lane_addr, g, q, row, nvis, !rehearsal, [&] {
+        pair_softmax_tile<DH>(m, l, xch[n & 1], sb, tmem_o + lane_addr, g, q, row, vis, !rehearsal, [&] {
           if (lane == 0) mbar_wait_drain(smem_u32(&pv_done[(n - 1) & 1]), (uint32_t)((n - 1) >> 1) & 1u, wc);
         });
         if (!rehearsal && lane == 0) remote_arrive(pfull0 + (uint32_t)(n & 1) * 16u);

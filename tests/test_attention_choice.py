@@ -11,11 +11,17 @@ PROGRAM = r"""
 #include <cstdlib>
 #include "attention_choice.h"
 
-// resident[1..4] items keys most -> ranges
+// resident[1..4] items keys most -> ranges; prefix -> row, keys of its blocks
 int main(int argc, char** argv) {
   if (argc == 8) {
     const int resident[5] = {0, atoi(argv[1]), atoi(argv[2]), atoi(argv[3]), atoi(argv[4])};
     printf("%d\n", phyai::choose_pair_ranges(resident, atoi(argv[5]), atoi(argv[6]), atoi(argv[7])));
+  } else {
+    const int P = atoi(argv[1]);
+    for (int sb = 0; sb < (P + 63) / 64; ++sb) {
+      const phyai::PrefixBlock k = phyai::prefix_block(P, sb);
+      printf("%d %llx\n", k.row, (unsigned long long)k.keys);
+    }
   }
 }
 """
@@ -39,3 +45,13 @@ def test_key_ranges(program, resident, items, keys, most, ranges):
     options = [c for c in range(1, most + 1) if resident[c - 1] > 0]
     assert ranges == (min(options, key=cost) if options else 0)
     assert program(*resident, items, keys, most) == [str(ranges)]
+
+
+@pytest.mark.parametrize("prefix", [*range(0, 200), 255, 256, 257, 816, 967, 968])
+def test_blocks_of_a_prefix(program, prefix):
+    """Every key is in one block; the 64 rows of a block end in the prefix, and begin there unless it has fewer."""
+    v = program(prefix)
+    blocks = [(int(row), int(keys, 16)) for row, keys in zip(v[::2], v[1::2])]
+    assert [row + c for row, keys in blocks for c in range(64) if keys >> c & 1] == list(range(prefix))
+    for row, keys in blocks:
+        assert keys and row + 64 <= prefix and (row >= 0 or prefix < 64)

@@ -78,16 +78,17 @@ def test_attention_of_many_requests(head_dim, n_q, n_kv, batch, horizon, top):
 
 
 @pytest.mark.parametrize("head_dim,n_q,n_kv,batch", [(256, 8, 1, 45), (128, 8, 2, 60)])
-def test_rows_past_a_prefix_have_no_part_in_its_request(head_dim, n_q, n_kv, batch):
-    """The persistent kernel fetches whole blocks of 64 keys: what follows a prefix (every third request's cache is NaN or infinite, and so
-    are the rows behind the last one) leaves the other requests' actions as they are, to the bit."""
+def test_rows_around_a_prefix_have_no_part_in_its_request(head_dim, n_q, n_kv, batch):
+    """What lies around a prefix (every third request's cache is NaN or infinite, and so are the rows before the first one and behind the
+    last) leaves the other requests' actions as they are, to the bit; a first block that would begin before the cache."""
     cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=batch, max_prefix_len=300, n_layers=2, horizon=12)
     W = synth.make_weights(cfg, 53, std=0.05)
     lens = [(1, 63, 64, 65, 130, 300, 0, 191)[b % 8] for b in range(batch)]
     packed, cu = synth.pack_prefix_kv([synth.make_prefix_kv(cfg, 53, p, b) for b, p in enumerate(lens)])
-    packed = torch.cat([packed, torch.zeros_like(packed[:, :, :70])], dim=2)
+    packed = torch.cat([torch.zeros_like(packed[:, :, :30]), packed, torch.zeros_like(packed[:, :, :70])], dim=2)
+    cu = cu + np.int32(30)
     dirty = packed.clone()
-    dirty[:, :, int(cu[-1]):] = float("nan")
+    dirty[:, :, :30], dirty[:, :, int(cu[-1]):] = float("nan"), float("nan")
     for b in range(1, batch, 3):
         dirty[:, :, cu[b]:cu[b + 1]] = float("nan") if b % 2 else float("inf")
     states = torch.stack([synth.make_state(cfg, 53, b) for b in range(batch)]).cuda()
@@ -100,6 +101,25 @@ def test_rows_past_a_prefix_have_no_part_in_its_request(head_dim, n_q, n_kv, bat
     for b in range(batch):
         if b % 3 != 1 or lens[b] == 0:
             assert torch.equal(out[b], clean[b]), (b, lens[b])
+
+
+@pytest.mark.parametrize("head_dim,n_kv", [(256, 1), (128, 2)])
+def test_infinite_values_among_the_keys_of_a_partial_block(head_dim, n_kv):
+    """The 64 rows that a partial last block is fetched from begin with keys of the block before: an infinite value there (and one among the
+    block's own keys, and in a prefix of fewer than 64) gives its channel an infinite result and leaves the others as they are."""
+    from tests.test_gpu_attention_op import make_case
+    lens = [(130, 65, 191, 40, 127)[b % 5] for b in range(90)]
+    qkv, kv, cu, _ = make_case(14, 4 * n_kv, n_kv, head_dim, 33, lens, theta=0.0)
+    dirty = kv.clone()
+    for b in range(0, 90, 2):
+        dirty[1, 1, cu[b] + (100, 5, 180, 20, 64)[b % 5], :, 3] = float("inf")
+        dirty[1, 1, cu[b + 1] - 1, :, 70] = float("-inf")
+    desc = binding.attention_desc(4 * n_kv, n_kv, head_dim, 33, n_layers=2, layer=1)
+    clean, out = (binding.suffix_attention(desc, qkv.cuda(), x.cuda(), torch.from_numpy(cu).cuda(), None)[0].view(90, 33, 4 * n_kv, head_dim) for x in (kv, dirty))
+    torch.cuda.synchronize()
+    want = clean.clone()
+    want[::2, :, :, 3], want[::2, :, :, 70] = float("inf"), float("-inf")
+    assert clean.isfinite().all() and torch.equal(out, want)
 
 
 @pytest.mark.parametrize("horizon", [59, 60, 62, 63])
