@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, c
         if (is_v) group_sync<BAR_V, 64>(); else group_sync<BAR_K, 64>();
       }
       if (lt == 0) {
-        for (int t = m0; t < m0 + n_mix; ++t) remote_arrive(full0 + (uint32_t)t * 8u);
+        for (int t = m0; t < m0 + n_mix; ++t) remote_arrive_stores(full0 + (uint32_t)t * 8u);
         for (int t = 2; t < T; ++t) {
           mbar_wait_drain(smem_u32(is_v ? &pv_done[t & 1] : &s_full[t & 1]), (uint32_t)((t - 2) >> 1) & 1u, wc);
           issue_full(t);
@@ -225,8 +225,13 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, c
       if (half == 1) trace_stamp(trc, 3), trace_stamp(trc, 4), trace_stamp(trc, 5);
     }
     if (half == 0) {
+      // operands of tile t; the rows of a mixed tile were stored by threads of both CTAs
+      auto wait_tile = [&](const uint64_t* full, int t) {
+        mbar_wait_drain(smem_u32(&full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        if (t >= m0 && t < m0 + n_mix) pair_acquire(smem_u32(&full[t & 1]), (uint32_t)(t >> 1) & 1u);
+      };
       auto issue_s = [&](int t) {
-        mbar_wait_drain(smem_u32(&k_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        wait_tile(k_full, t);
         tc_fence_after();
         const uint32_t kb = Ks + (uint32_t)(t & 1) * L::KTILE;
         // (rolled loops: most of the time of a first pass is the fetch of its code, which has left the instruction caches since the
@@ -248,7 +253,7 @@ __global__ void __launch_bounds__(AP_THREADS, 1) k_attn_pair(const AttnArgs a, c
       if (lane == 0) trace_stamp(trc, 3);
       if (T > 1) issue_s(1);
       for (int t = 0; t < T; ++t) {
-        mbar_wait_drain(smem_u32(&v_full[t & 1]), (uint32_t)(t >> 1) & 1u, wc);
+        wait_tile(v_full, t);
         const uint32_t vb = Vs + (uint32_t)(t & 1) * L::VTILE;
         // (the first 64 keys' probabilities are ready before the others': their half of the product hides under the rest of
         // the softmax)

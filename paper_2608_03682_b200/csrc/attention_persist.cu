@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
           }
           fence_async_smem();                    // generic-proxy writes, read next by the tensor cores
           __syncwarp();
-          if (lane == 0) remote_arrive(full_lead + (uint32_t)(n & 1) * 8u);
+          if (lane == 0) remote_arrive_stores(full_lead + (uint32_t)(n & 1) * 8u);
         }
       }
       it = nx;
@@ -275,6 +275,8 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
             go = true;
           }
           if (__all_sync(0xffffffffu, go)) {
+            // (the tile with the block that is not full: rows of it were cleared by a warp of each CTA)
+            if ((it.P & 63) && tp == (it.nsp - 1) >> 1) pair_acquire(smem_u32(&v_full[np & 1]), par);
             const uint32_t vb = Vs + (uint32_t)(np & 1) * L::TILE;
 #pragma unroll 1
             for (int kh = 0; kh < 2; ++kh) {

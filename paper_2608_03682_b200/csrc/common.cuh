@@ -34,8 +34,9 @@ __device__ __forceinline__ void pdl_enter() {
 
 // ---------------------------------------------------------------------------------------------
 // Cluster barrier that publishes no data: "this CTA no longer needs what it reads (or awaits) there".  What crosses CTAs goes by
-// bulk copies that are counted on an mbarrier, and is observed there, so the arrival needs no release: one at cluster scope waits
-// for every store of the thread, in the middle of a chain of kernels that take 3 - 7 us.  (Ten-step loops with arrivals that
+// bulk copies that are counted on an mbarrier, or is announced on one by an arrival that releases it, and is observed there, so this
+// arrival needs no release: one at cluster scope waits for every store of the thread, in the middle of a chain of kernels that take
+// 3 - 7 us.  (Ten-step loops with arrivals that
 // release at cluster scope -> without: 1 request 5.08 -> 4.79 ms, 4: 9.38 -> 8.79, 16: 12.66 -> 11.73; the same bits.)
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }

@@ -46,11 +46,26 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// arrives on a barrier of this or another CTA of the cluster.  (Release at CTA scope: what the arrivals announce is tensor memory,
-// fenced by tcgen05.fence, or shared memory behind a proxy fence.  At cluster scope the arrival of a softmax warp took 1500
+// arrives on a barrier of this or another CTA of the cluster.  (Release at CTA scope: for arrivals that announce tensor memory, which is
+// fenced by tcgen05.fence, or copies that the barrier counts itself.  At cluster scope the arrival of a softmax warp took 1500
 // clocks per key tile, between the probabilities and their product.)
 __device__ __forceinline__ void remote_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// The same for stores to shared memory (each behind the writer's own proxy fence) that the leader's MMAs read in this CTA: the release
+// reaches the leader, whose MMA warp acquires it with pair_acquire on the completed phase.
+__device__ __forceinline__ void remote_arrive_stores(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void pair_acquire(uint32_t bar, uint32_t parity) {
+  uint32_t done;      // (the phase is complete, or the call has been given up)
+  asm volatile(
+      "{\n.reg .pred p;\n"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
 }
 // A operand in tensor memory
 __device__ __forceinline__ void umma2_ts(uint32_t d, uint32_t ta, uint64_t db, uint32_t idesc, uint32_t acc) {

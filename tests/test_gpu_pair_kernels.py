@@ -77,10 +77,11 @@ def test_attention_of_many_requests(head_dim, n_q, n_kv, batch, horizon, top):
     check(cfg, lens, 1, [*range(0, 18, 2), batch // 2, batch - 2, batch - 1])
 
 
-@pytest.mark.parametrize("head_dim,n_q,n_kv,batch", [(256, 8, 1, 45), (128, 8, 2, 60)])
+@pytest.mark.parametrize("head_dim,n_q,n_kv,batch", [(256, 8, 1, 45), (128, 8, 2, 60), (256, 8, 1, 8), (128, 8, 2, 13)])
 def test_rows_around_a_prefix_have_no_part_in_its_request(head_dim, n_q, n_kv, batch):
     """What lies around a prefix (every third request's cache is NaN or infinite, and so are the rows before the first one and behind the
-    last) leaves the other requests' actions as they are, to the bit; a first block that would begin before the cache."""
+    last) leaves the other requests' actions as they are, to the bit; a first block that would begin before the cache.  Rows that threads of
+    both CTAs of a pair clear or store themselves, with one key range per request and with several."""
     cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=n_q, n_kv_heads=n_kv, max_batch=batch, max_prefix_len=300, n_layers=2, horizon=12)
     W = synth.make_weights(cfg, 53, std=0.05)
     lens = [(1, 63, 64, 65, 130, 300, 0, 191)[b % 8] for b in range(batch)]
