@@ -136,6 +136,8 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
         const Item nx = item(k + 1);
         const int hk = it.group * 4 / (d.Hq / d.Hkv);
         for (int t = 0; t < it.T; ++t, ++n) {
+          // (these products need what the kernel before writes: its time is not to count against the limit of the wait)
+          if (n >= 2 && !waited) pdl_wait(), waited = true;
           if (n >= 2) mbar_wait_drain(smem_u32(&s_full[n & 1]), (uint32_t)((n - 2) >> 1) & 1u, wl);
           const int sb = 2 * t + half;
           const uint32_t bar = smem_u32(&k_full[n & 1]), dst = Ks + (uint32_t)(n & 1) * L::TILE;
@@ -169,6 +171,7 @@ __global__ void __launch_bounds__(AS_THREADS, 1) __cluster_dims__(2, 1, 1)
         const bool clear = part == 0 || part == 1;
         const uint32_t dst = Vs + (uint32_t)(n & 1) * L::TILE;
         if (lane == 0) {
+          if (n >= 2 && !waited) pdl_wait(), waited = true;
           if (n >= 2) mbar_wait_drain(smem_u32(&pv_done[n & 1]), (uint32_t)((n - 2) >> 1) & 1u, wl);
           uint32_t bar = smem_u32(&v_full[n & 1]);
           if (clear) {
