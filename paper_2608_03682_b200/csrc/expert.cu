@@ -155,6 +155,7 @@ struct phyai_expert {
   int use_graph = 1;
   unsigned wait_limit = 1u << 22;
   uint64_t counting = 0;  // launches counted by the last enqueue
+  int trace_cursor = 0;   // trace slots they were given (trace_all_from)
 
   template <typename T>
   phyai_status_t alloc(T** p, size_t count, bool zero = false) {
@@ -371,7 +372,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
   const int nt = pick_nt(M);
   const int tok_tiles = (M + nt - 1) / nt;
   const float dt = -1.0f / (float)n;
-  uint64_t cnt = 0;
+  uint64_t cnt = k0 > 0 ? h->counting : 0;        // (the steps before were enqueued just now)
   auto site = [&](int k, int s, const float** gain, const float** shift, const float** gate) {
     if (h->ada) {
       const float* base = t.mod + ((size_t)k * h->sites + s) * 3 * D;
@@ -423,7 +424,8 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
 
   const int kcb = h->a8 ? 128 : 64;   // contraction elements per 128-byte operand row (k-chunk of the tile GEMM)
   int ss_na = D / 128, ss_nb = D / 128;   // partial sums of squares per token that the last writer of ss_a / ss_b left
-  int trace_cursor = 0;
+  int& trace_cursor = h->trace_cursor;
+  if (k0 == 0) trace_cursor = 0;
   const bool use_w8 = h->use_w8_inkernel && !h->b_qkv.empty();
   auto b1_gemm = [&](B1Gemm g, int which, int Mloc) -> phyai_status_t {
     g.M = Mloc, g.wait_limit = h->wait_limit, g.gelu_exact = d.gelu_exact, g.inv_D = 1.0f / (float)D, g.eps = d.eps;
@@ -941,28 +943,27 @@ phyai_status_t run(phyai_expert* h, Request& r, int n, cudaStream_t st, const Ga
   ST(build_tables(h, n, st, &t));
   launch_set_request(h->rq, r, h->cu_internal, st, h->order);
   if (r.cu_lens != nullptr) launch_validate(h->rq, h->status, (int)h->cfg.max_prefix_len, h->order, st);
-  auto key = std::make_pair(r.batch, n);
   if (!h->use_graph) {
     ST(enqueue_loop(h, r.batch, n, *t, st, 0, n, gate_kv));
-    h->launch_counts[key] = h->counting;
+    h->launch_counts[std::make_pair(r.batch, n)] = h->counting;
     return PHYAI_OK;
   }
   // With a gate the first step is enqueued launch by launch, the others are a graph of their own.
-  int k0 = 0;
-  uint64_t head = 0;
-  if (gate_kv) {
-    ST(enqueue_loop(h, r.batch, n, *t, st, 0, 1, gate_kv));
-    head = h->counting, k0 = 1;
-    if (n == 1) {
-      h->launch_counts[key] = head;
-      return PHYAI_OK;
-    }
-    key.second = -n;
-  }
+  const int k0 = gate_kv ? 1 : 0;
+  const auto key = std::make_pair(r.batch, gate_kv ? -n : n);
   auto it = h->graphs.find(key);
-  if (it == h->graphs.end()) {
+  if (it == h->graphs.end() && k0 < n) {
     const auto same = std::count_if(h->graphs.begin(), h->graphs.end(), [&](const auto& g) { return (g.first.second < 0) == (key.second < 0); });
     if (same >= 64) return fail(PHYAI_ERR_UNSUPPORTED, "more than 64 captured (batch, n_steps) graphs");
+  }
+  if (gate_kv) {
+    ST(enqueue_loop(h, r.batch, n, *t, st, 0, 1, gate_kv));
+    if (n == 1) {
+      h->launch_counts[std::make_pair(r.batch, n)] = h->counting;
+      return PHYAI_OK;
+    }
+  }
+  if (it == h->graphs.end()) {
     // tables were enqueued on `st`; the capture stream must not run ahead of them on first replay,
     // which holds because the graph is launched on `st` below.
     cudaGraph_t graph = nullptr;
@@ -979,7 +980,7 @@ phyai_status_t run(phyai_expert* h, Request& r, int n, cudaStream_t st, const Ga
     cudaGraphDestroy(graph);
     if (e != cudaSuccess) return fail(PHYAI_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
     it = h->graphs.emplace(key, exec).first;
-    h->launch_counts[std::make_pair(r.batch, n)] = head + h->counting;
+    h->launch_counts[std::make_pair(r.batch, n)] = h->counting;
   }
   CU(cudaGraphLaunch(it->second, st));
   return PHYAI_OK;

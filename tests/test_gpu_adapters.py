@@ -183,6 +183,87 @@ def test_host_requests_run_on_layers_as_they_arrive(cond, batch, top, horizon, n
                 assert np.array_equal(np.asarray(out), ref[b].cpu().numpy()), b
 
 
+def one_layer_overlapped(cfg_id, batch):
+    """An expert whose calls' caches are large enough to go beside the first step, and requests for it."""
+    from tests.helpers import small_bf16_config
+    cfg = small_bf16_config("pi0", head_dim=256, width=256, n_layers=1, max_batch=batch, max_prefix_len=1100, horizon=12)
+    reqs = [(synth.make_prefix_kv(cfg, cfg_id, 1100, b), synth.make_state(cfg, cfg_id, b), synth.make_noise(cfg, cfg_id, b)) for b in range(batch)]
+    return cfg, synth.make_weights(cfg, cfg_id, std=0.05), reqs
+
+
+def test_host_requests_refused_for_their_graph_run_no_step():
+    """Sixty-four graphs without a first step (8 batch sizes x 8 numbers of steps); a call that would need another one is refused, with none
+    of its launches on the way (the time stamps of the call before stay), and what has a graph still runs."""
+    cfg, W, reqs = one_layer_overlapped(29, 9)
+    out = torch.zeros(9, cfg.horizon, cfg.action_dim).pin_memory()
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        ex.set_option("trace", 1)
+        for batch in range(1, 9):
+            for n in range(2, 10):
+                ex.denoise_requests_host(reqs[:batch], n, out[:batch])
+        ex.denoise_requests_host(reqs[:2], 3, out[:2])
+        torch.cuda.synchronize()
+        good, stamps = out[:2].clone(), ex.read_trace()
+        for refused in (lambda: ex.denoise_requests_host(reqs, 3, out), lambda: ex.denoise_requests_host(reqs[:2], 10, out[:2])):
+            with pytest.raises(binding.PhyaiError, match="graphs"):
+                refused()
+            torch.cuda.synchronize()
+            assert stamps.any() and np.array_equal(ex.read_trace(), stamps)
+        ex.denoise_requests_host(reqs[:1], 1, out[:1])           # (a single step needs no graph)
+        ex.denoise_requests_host(reqs[:2], 3, out[:2])
+        torch.cuda.synchronize()
+        assert ex.poll_status() == 0 and torch.equal(out[:2], good)
+
+
+def test_host_requests_count_and_stamp_their_launches_as_one_call():
+    """The launches of the first step and of the graph behind it count on: as many, and as many time stamps, as from device memory."""
+    cfg, W, reqs = one_layer_overlapped(30, 1)
+    kv, state, noise = reqs[0]
+    out = torch.zeros(1, cfg.horizon, cfg.action_dim).pin_memory()
+    stamped, launches = [], []
+    for host in (False, True):
+        for first in (0, 6):                # (every kernel of the call; the launches 6 .. 10 on all of their CTAs: they begin in the first step)
+            with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+                ex.set_option("trace", 1)
+                ex.set_option("trace_all_from", first)
+                if host:
+                    ex.denoise_requests_host(reqs, 4, out)
+                else:
+                    ref = ex.denoise(kv.cuda(), 1100, state.cuda(), noise.cuda(), 4)
+                torch.cuda.synchronize()
+                stamped.append(ex.read_trace().any(axis=1).nonzero()[0].tolist())
+                launches.append(ex.launches_per_call(1, 4))
+    assert stamped[0] and stamped[1] and stamped[2:] == stamped[:2] and len(set(launches)) == 1
+    assert torch.equal(out[0], ref.cpu())
+
+
+@pytest.mark.parametrize("kind,batch,option", [("pi0", 1, ("use_graph", 0)), ("pi05", 3, ("use_graph", 0)), ("block causal", 1, ("use_state_cache", 1)),
+                                              ("w8a8", 1, None), ("w8a8", 9, None), ("two heads", 6, None)])
+def test_host_requests_of_the_other_kernels(kind, batch, option):
+    """Layers as they arrive, without a graph, behind the cached pass of the state tokens, and on the kernels of W8A8 and of head groups that the
+    pairs do not take: the bits of the call on device memory (W8A8 of several token tiles adds with atomics: to rounding)."""
+    from tests.helpers import rel_err, small_bf16_config
+    more = {"block causal": dict(suffix_block_causal=True, head_dim=256, width=1024, mlp_dim=4096, n_q_heads=8), "w8a8": dict(dtype="w8a8e4m3", head_dim=256)}
+    cfg = small_bf16_config("pi05" if kind == "pi05" else "pi0", **{**dict(max_batch=batch, max_prefix_len=900), **more.get(kind, {})})
+    W = synth.make_weights(cfg, 31, std=0.05)
+    lens = [900 - 17 * b for b in range(batch)]
+    reqs = [(synth.make_prefix_kv(cfg, 31, p, b), synth.make_state(cfg, 31, b) if cfg.has_state_token else None, synth.make_noise(cfg, 31, b)) for b, p in enumerate(lens)]
+    packed, cu = synth.pack_prefix_kv([r[0] for r in reqs])
+    assert packed.numel() * 2 > 1 << 20
+    out = torch.zeros(batch, cfg.horizon, cfg.action_dim).pin_memory()
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        if option:
+            ex.set_option(*option)
+        ref = ex.denoise_batched(packed.cuda(), torch.from_numpy(cu).cuda(), torch.stack([r[1] for r in reqs]).cuda() if cfg.has_state_token else None,
+                                 torch.stack([r[2] for r in reqs]).cuda(), 3).cpu()
+        for _ in range(2):
+            out.zero_()
+            ex.denoise_requests_host(reqs, 3, out)
+            torch.cuda.synchronize()
+            assert ex.poll_status() == 0
+            assert torch.equal(out, ref) or (kind == "w8a8" and batch > 1 and rel_err(out.double().numpy(), ref.double().numpy()) <= 0.15)
+
+
 def test_host_requests_arguments_are_checked():
     """phyai_denoise_requests_host through the C ABI: every bad argument is a status code, and the handle still works."""
     import ctypes as C
