@@ -45,4 +45,12 @@ inline int choose_pair_ranges(const int (&resident)[MAX_PAIR_RANGES + 1], int it
   return best_c;
 }
 
+// Whether calls of caches of at most `keys` tokens take the kernels on pairs (`pairs` of them resident at a time) or the one-CTA kernel.
+// From 256 tokens on always; with less there are at most four 64-key tiles, nothing to split, and the persistent pairs have to win by their
+// longer tiles: from half as many items as pairs on, and, where the whole cache is one block of 64 keys, from seven eighths on.  Ten-step
+// loops of 19 / 20 / 24 / 28 / 32 / 36 requests (two items each, 74 pairs), one-CTA kernel -> persistent pairs, ms: 60 tokens 10.68 -> 10.89,
+// 10.75 -> 10.81, 11.91 -> 12.03, 13.16 -> 13.21, 14.50 -> 14.52, 15.75 -> 15.50; 120: 10.93 -> 11.00, 11.01 -> 10.95, 12.15 -> 12.30, 13.61 -> 13.58,
+// 14.91 -> 14.76, 16.04 -> 15.91; 200: 11.32 -> 11.30, 11.40 -> 11.24, 12.66 -> 12.62, 14.08 -> 13.92, 15.48 -> 15.21.
+inline bool pairs_pay(int keys, int items, int pairs) { return keys >= 256 || (keys > 64 ? 2 * items >= pairs : 8 * items >= 7 * pairs); }
+
 }  // namespace phyai

@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/phyai.h"
+#include "attention_choice.h"
 #include "host_pack.h"
 #include "kernels.h"
 
@@ -547,11 +548,9 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     ++cnt;
     return PHYAI_OK;
   };
-  // Attention of the pair path.  Calls of few requests with caches of fewer than 256 tokens keep the one-CTA kernel: with at most
-  // four 64-key tiles there is nothing to split; the persistent pairs are for them from half as many items as there are pairs on
-  // (60 / 200 tokens, one-CTA kernel -> persistent pairs: 20 requests 10.93 -> 11.02 / 11.67 -> 11.46 ms, 64: 24.0 -> 23.6 / 25.5 ->
-  // 25.3, 160: 56.7 -> 54.1 / 60.2 -> 58.2).  The choice goes by what the handle can hold, not by a call's lengths: those are on the
-  // device, one graph per (batch, steps) serves them all, and a graph per choice would be captured in the middle of serving.
+  // Attention of the pair path, where it pays (see pairs_pay).  The choice goes by what the handle can hold, not by a call's lengths:
+  // those are on the device, one graph per (batch, steps) serves them all, and a graph per choice would be captured in the middle of
+  // serving.
   // (Ten-step loops with 816-token prefixes, handle for 2048 tokens against one for 816: 2 requests 7.60 / 7.55 ms, 4: 8.29 / 8.28,
   // 8: 9.45 / 9.42, 16: 11.20 / 11.18.)
   // (A device that holds no cluster of a form at a time: no choice of that form, and none at all, the kernels without clusters.)
@@ -560,7 +559,7 @@ phyai_status_t enqueue_loop(phyai_expert* h, int batch, int n, const Tables& t, 
     pr_ranges = h->pair_ranges ? std::min(h->pair_ranges, attention_pair_max_ranges(d)) : attention_pair_ranges(d, batch, (int)h->cfg.max_prefix_len);
     if (pr_ranges > 0 && attention_pair_resident(d, pr_ranges) <= 0) pr_ranges = 0;
   }
-  const bool attn_pair = pr_ranges > 0 && (h->cfg.max_prefix_len >= 256 || 2 * batch * (d.Hq / 4) >= attention_persist_pairs(d));
+  const bool attn_pair = pr_ranges > 0 && pairs_pay((int)h->cfg.max_prefix_len, batch * (d.Hq / 4), attention_persist_pairs(d));
   auto attention_rot = [&](int l) -> phyai_status_t {   // from rotated bf16 q / k / v to the output projection's operand
     cudaError_t e;
     const bool tr1 = h->trace && h->trace_all_from > 0 && cnt == h->trace_all_from;

@@ -11,11 +11,13 @@ PROGRAM = r"""
 #include <cstdlib>
 #include "attention_choice.h"
 
-// resident[1..4] items keys most -> ranges; prefix -> row, keys of its blocks
+// resident[1..4] items keys most -> ranges; keys items pairs -> whether pairs pay; prefix -> row, keys of its blocks
 int main(int argc, char** argv) {
   if (argc == 8) {
     const int resident[5] = {0, atoi(argv[1]), atoi(argv[2]), atoi(argv[3]), atoi(argv[4])};
     printf("%d\n", phyai::choose_pair_ranges(resident, atoi(argv[5]), atoi(argv[6]), atoi(argv[7])));
+  } else if (argc == 4) {
+    printf("%d\n", phyai::pairs_pay(atoi(argv[1]), atoi(argv[2]), atoi(argv[3])) ? 1 : 0);
   } else {
     const int P = atoi(argv[1]);
     for (int sb = 0; sb < (P + 63) / 64; ++sb) {
@@ -45,6 +47,12 @@ def test_key_ranges(program, resident, items, keys, most, ranges):
     options = [c for c in range(1, most + 1) if resident[c - 1] > 0]
     assert ranges == (min(options, key=cost) if options else 0)
     assert program(*resident, items, keys, most) == [str(ranges)]
+
+
+@pytest.mark.parametrize("keys,items,pays", [(60, 38, 0), (64, 40, 0), (60, 56, 0), (0, 60, 0), (64, 72, 1), (65, 36, 0), (65, 38, 1), (255, 37, 1),
+                                              (255, 36, 0), (256, 2, 1), (968, 2, 1)])
+def test_small_caches_take_the_pairs_where_they_are_faster(program, keys, items, pays):
+    assert program(keys, items, 74) == [str(pays)]
 
 
 @pytest.mark.parametrize("prefix", [*range(0, 200), 255, 256, 257, 816, 967, 968])
