@@ -79,3 +79,31 @@ def test_expired_waits_in_the_full_width_single_tile_kernels(cond, dtype):
         torch.cuda.synchronize()
         assert ex.poll_status() == 0
         assert torch.equal(again, good)              # the single-tile path is bit-reproducible
+
+
+@pytest.mark.parametrize("head_dim,batch", [(256, 5), (256, 160), (128, 80)])
+def test_expired_waits_in_the_attention_on_pairs(head_dim, batch):
+    """Split key ranges (5 requests) and the persistent pairs (one to three items per pair): after a wait that gave up the issuing warp goes on
+    in a fixed order, to the end of its items."""
+    cfg = small_bf16_config("pi0", head_dim=head_dim, n_q_heads=4, max_batch=batch, max_prefix_len=300, n_layers=2)
+    W = synth.make_weights(cfg, 33, std=0.05)
+    lens = [300 - (37 * b) % 290 for b in range(batch)]
+    kvs = [synth.make_prefix_kv(cfg, 33, p, b) for b, p in enumerate(lens)]
+    packed, cu = synth.pack_prefix_kv(kvs)
+    states = torch.stack([synth.make_state(cfg, 33, b) for b in range(batch)])
+    noise = torch.stack([synth.make_noise(cfg, 33, b) for b in range(batch)])
+    args = (packed.cuda(), torch.from_numpy(cu).cuda(), states.cuda(), noise.cuda(), 2)
+    ref = O.denoise(cfg, W, kvs[0], lens[0], states[0], noise[0], 2)
+    with binding.Expert(cfg, binding.weights_to_device(W)) as ex:
+        good = ex.denoise_batched(*args).clone()
+        torch.cuda.synchronize()
+        assert ex.poll_status() == 0
+        assert rel_err(good[0].double().cpu().numpy(), ref) <= BAR["bf16"]
+        ex.set_option("wait_limit", 1)
+        ex.denoise_batched(*args)
+        torch.cuda.synchronize()
+        assert ex.poll_status() == binding.ERR_TIMEOUT
+        ex.set_option("wait_limit", 1 << 22)
+        again = ex.denoise_batched(*args)
+        torch.cuda.synchronize()
+        assert ex.poll_status() == 0 and torch.equal(again, good)
