@@ -203,13 +203,13 @@ __global__ void k_check_lens(const int* cu, int batch, uint64_t kv_tokens, int* 
 // Operands of the tcgen05 kernels from an operator call's fp32 q | k | v rows: q rotated, scaled and rounded into the operand
 // tiles [request][head pair][dh / 64][128 rows][64] (rows past the suffix are zero), k rotated, v as is: bf16 rows
 // [request][Hkv][S][dh].  One block per (suffix row < 64, request), a thread 8 channels and their rotary partners.  Block 0
-// also writes the request block and checks the lengths.
+// also checks the lengths and writes the request block, if the attention kernel reads one.
 __global__ void __launch_bounds__(256) k_op_operands(Request* rq, const Request src, int* status, const float* qkv, const float2* rope,
                                                      __nv_bfloat16* q_tiles, __nv_bfloat16* kr, __nv_bfloat16* vr, const Dims d, int clear) {
   pdl_launch_dependents();
   const int i = blockIdx.x, b = blockIdx.y, half = d.dh >> 1, hc = half >> 3;
   if (i == 0 && b == 0) {
-    if (threadIdx.x == 0) *rq = src;
+    if (threadIdx.x == 0 && rq) *rq = src;
     check_lens(src.cu_lens, src.batch, src.kv_tokens, status, clear);
   }
   const int nq = d.Hq * hc, nk = d.Hkv * hc;               // items of 8 + 8 channels: q, k, v
@@ -355,7 +355,7 @@ phyai_status_t attention_op(const phyai_attention_desc_t* desc, uint32_t batch, 
     r.prefix_kv = prefix_kv, r.kv_tokens = kv_tokens, r.cu_lens = cu, r.batch = (int)batch;
     if (!b1 && !prefix_kv_map(r.kv_map, prefix_kv, kv_tokens, d)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) {
-      k_op_operands<<<dim3(64, batch), 256, 0, st>>>(rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
+      k_op_operands<<<dim3(64, batch), 256, 0, st>>>(b1 ? nullptr : rq, r, status_word, qkv, a.rope, qt, kr, vr, d, clear);
       // (one wave of clusters: its set-up and the copies of the prefix rows run under the kernel above, 18.5 -> 14.4 us per call of one
       // request; the kernels on pairs read the request block that the kernel above writes before their dependency wait: no
       // programmatic launch for them)
