@@ -205,7 +205,9 @@ phyai_status_t phyai_denoise_batched_host(phyai_expert_t *h, uint32_t batch, con
  *                call's copies have run on `stream` (a buffer per call lets the next call gather while this one computes)
  * The call gathers the requests into `staging` (on a few threads of the handle's own, the copies to the device following
  * plane by plane), runs the batched kernels and copies the actions back on `stream`.  The inputs are not read after it
- * returns; the result is valid after the stream is synchronised.
+ * returns; the result is valid after the stream is synchronised.  Caches of 1 MB and more in all (not of the fp32 engine) are copied on
+ * a stream of the handle's own, made by the first such call with its events, behind what `stream` holds at the call and ahead of the
+ * layers that read them: once `stream` has run the call, those copies have run too.
  */
 uint64_t phyai_requests_staging_bytes(const phyai_expert_t* h, uint32_t batch, uint64_t kv_tokens);
 phyai_status_t phyai_denoise_requests_host(phyai_expert_t* h, uint32_t batch, const void* const* prefix_kvs,
@@ -253,8 +255,8 @@ phyai_status_t phyai_poll_status(phyai_expert_t *h);
  * CTAs) that are not on the pair attention kernel split every request's key tiles over up to 8 CTAs of the tcgen05 attention kernel, merged by a second launch.
  * key "use_pair_gemm": 1 (default) runs the projections of calls with more than 64 suffix tokens on the CTA-pair GEMM
  * with the norms folded in (together with use_cluster_gemm and the two use_persistent options); 0 keeps the general kernels.
- * key "use_pair_attention": 1 (default) lets those calls of few requests use the CTA-pair attention kernel (caches of at
- * least 256 tokens); key "pair_attn_ranges": key ranges per request (1..4, 0 = choose) of that kernel (with heads of
+ * key "use_pair_attention": 1 (default) lets those calls use the CTA-pair attention kernels (with caches of fewer than 256 tokens
+ * only calls of many requests); key "pair_attn_ranges": key ranges per request (1..4, 0 = choose; 1 is the persistent kernel; with heads of
  * 256 channels at most 3 from 61 suffix rows on, 2 with 64: the partial results have to fit the shared memory).
  * Options that leave the CTA pairs or decode weight codes make the weight images they need when they are set.
  * key "trace": see phyai_read_trace.

@@ -518,8 +518,8 @@ int attention_pair_resident(const Dims& d, int ranges) {
 
 // Key ranges per request (see choose_pair_ranges), 0 if no kernel on pairs can run.  A cluster of 8 CTAs needs 8 free SMs in one
 // GPC: 15 on a B200, not 18.  One range: the persistent kernel.  Against every other choice, ten-step loops of 4 / 8 / 12 / 16 / 20
-// requests: chosen 8.79 / 10.02 / 11.04 / 11.67 / 12.44 ms with 816-token prefixes (best 8.78 / 9.98 / 11.04 / 11.63 / 12.44), 8.50 /
-// 9.30 / 10.29 / 10.94 / 11.69 with 400 (best 8.43 / 9.30 / 10.28 / 10.91 / 11.69).
+// requests: chosen 8.35 / 9.47 / 10.51 / 11.18 / 12.40 ms with 816-token prefixes (best 8.33 / 9.47 / 10.51 / 11.13 / 12.40), 8.19 /
+// 8.89 / 9.90 / 10.55 / 11.72 with 400 (best 8.01, two ranges instead of four / 8.89 / 9.90 / 10.52 / 11.72).
 int attention_pair_ranges(const Dims& d, int batch, int max_prefix) {
   int resident[MAX_PAIR_RANGES + 1] = {};
   for (int c = 1; c <= MAX_PAIR_RANGES; ++c) resident[c] = attention_pair_resident(d, c);

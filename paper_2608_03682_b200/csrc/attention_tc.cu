@@ -1,5 +1,5 @@
 // Suffix -> (prefix U suffix) attention on the tcgen05 tensor cores, one CTA per request and pair of heads: for W8A8, head
-// groups that are no multiple of four and few requests with caches under 256 tokens (others: the kernels on CTA pairs and clusters).
+// groups that are no multiple of four and few requests with caches under 256 tokens (pairs_pay; others: the kernels on CTA pairs and clusters).
 //
 // One CTA takes the suffix rows of two query heads that share a kv head (2 x 64 padded rows = the 128
 // rows of one MMA) and walks all key tiles of its request:

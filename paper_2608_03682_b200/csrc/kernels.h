@@ -236,7 +236,7 @@ cudaError_t launch_attention_b1(const Request* rq, int* status, const __nv_bfloa
                                 int trace_all = 0);
 cudaError_t launch_attention_b1_op(const void* prefix_kv, uint64_t kv_tokens, const int* cu_lens, int* status, const __nv_bfloat16* q_tiles,
                                    const __nv_bfloat16* kr, const __nv_bfloat16* vr, int layer, __nv_bfloat16* out, const Dims& d, int batch,
-                                   unsigned wait_limit, cudaStream_t st);   // f32: fp32 partial results (one head per CTA only)
+                                   unsigned wait_limit, cudaStream_t st);   // operator calls: one head per CTA, fp32 partial results
 // CTAs of one launch with `hpc` (1 or 2) query heads per CTA, and how many of the fp32 form are resident at a time
 int attention_b1_ctas(const Dims& d, int batch, int hpc);
 int attention_b1_resident_ctas(const Dims& d);
